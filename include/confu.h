@@ -128,9 +128,9 @@ int confu_set_paging(confu_ctx* ctx, const int32_t* block_table, int32_t max_pag
  *   CONFU_OPT_ATTENTION_PATH  which kernel confu_tree_plan prepares for and confu_tree_attention
  *                             launches: CONFU_ATTENTION_AUTO (default: the fastest path that
  *                             supports the dims), _GENERIC (CUDA cores, every dtype and shape),
- *                             _TENSOR (tcgen05, one CTA per SM; bf16, D = 128, Hq/Hkv <= 4),
+ *                             _TENSOR (tcgen05, one CTA per SM; bf16, Hq/Hkv <= 32, S <= 128),
  *                             _TENSOR_PAIR (tcgen05 two-SM instructions, one CTA pair per two SMs;
- *                             as _TENSOR, and more than 32 query rows).  A path that does not
+ *                             as _TENSOR, D = 128, and more than 32 or 128 / (Hq/Hkv) query rows).  A path that does not
  *                             support the dims makes the calls return CONFU_ERR_UNSUPPORTED.  Set
  *                             it before confu_tree_plan: a plan only fits the path it was built
  *                             for (status CONFU_ST_BAD_PLAN otherwise).
@@ -206,9 +206,9 @@ int confu_tree_plan(confu_ctx* ctx, const confu_dims* dims,
  * denominators.  plan: a buffer filled by confu_tree_plan for these dims, lengths
  * and trees, or NULL to have the call build one in the workspace (then parent,
  * con_owner are read; otherwise they may be NULL).  Accumulation is fp32; bf16
- * inputs use the tensor-core path when D == 128 and Hq/Hkv <= 4; it takes the
- * query rows in groups of 64, so R > 64 streams the keys twice (the two groups walk
- * the same keys at the same time: the second read is served by L2).
+ * inputs use the tensor-core path when Hq/Hkv <= 32 and S <= 128; it takes the
+ * query rows in groups of 2 * (128 / (Hq/Hkv)), so more rows than that stream the keys once
+ * per group (the groups walk the same keys at the same time: the later reads are served by L2).
  * Needs the workspace.  All pointers device.  Ordinary stream order holds: the kernels are
  * launched as programmatic dependents (their blocks may be scheduled while the kernel before them
  * drains) but wait for all earlier work of the stream before their first global memory access,

@@ -32,7 +32,7 @@ int cuda_fail(confu_ctx* ctx, cudaError_t e)
 
 // workspace carving: [plan built by the attention call itself][split-KV partial slots]
 size_t ws_plan_offset() { return 0; }
-size_t ws_partial_offset(const confu_dims* d) { return align_up(plan_bytes(d->B, d->Hkv), 256); }
+size_t ws_partial_offset(const confu_dims* d) { return align_up(plan_bytes(d->B, d->Hkv, row_groups(d->T + d->C, d->Hq / d->Hkv)), 256); }
 size_t ws_total(const confu_ctx* ctx, const confu_dims* d)
 {
     return ws_partial_offset(d) + (size_t)2 * ctx->sm_count * partial_slot_bytes();
@@ -43,7 +43,7 @@ size_t ws_total(const confu_ctx* ctx, const confu_dims* d)
 namespace confu {
 cudaError_t launch_bounded_wait(unsigned long long limit_ns, int32_t* status, cudaStream_t st);
 bool tc_attention_supported(const confu_dims& d);
-bool pair_attention_supported(const confu_dims& d, int sm_count);
+bool pair_attention_supported(const confu_dims& d);
 bool fp8_attention_supported(const confu_dims& d);
 cudaError_t launch_attention_fp8(const Ctx* ctx, const confu_dims& d, const void* q, const void* k_cache,
                                  const void* v_cache, int64_t n_slots, const SlotMap& map,
@@ -68,11 +68,13 @@ namespace {
 // (never _AUTO), or a negative error code when a forced path cannot take them.
 int resolve_attention_path(const confu_ctx* ctx, const confu_dims& d)
 {
-    // (a share of the work is walked by one CTA, or CTA pair, per group of 64 query rows: at least two of them)
-    const bool tc = tc_attention_supported(d) && ctx->sm_count >= 2, pair = pair_attention_supported(d, ctx->sm_count);
+    // (a share of the work is walked by one CTA, or CTA pair, per group of query rows: at least that many of them)
+    const int n_rg = row_groups(d.T + d.C, d.Hq / d.Hkv);
+    const bool tc = tc_attention_supported(d) && ctx->sm_count >= n_rg;
+    const bool pair = pair_attention_supported(d) && ctx->sm_count / 2 >= n_rg;
     if (d.kv_dtype == CONFU_FP8_E4M3) {         // one kernel serves E4M3 caches
         const bool ok = ctx->attention_path == CONFU_ATTENTION_AUTO || ctx->attention_path == CONFU_ATTENTION_TENSOR;
-        return ok && fp8_attention_supported(d) && ctx->sm_count >= 2 ? (int)CONFU_ATTENTION_TENSOR : (int)CONFU_ERR_UNSUPPORTED;
+        return ok && fp8_attention_supported(d) && ctx->sm_count >= n_rg ? (int)CONFU_ATTENTION_TENSOR : (int)CONFU_ERR_UNSUPPORTED;
     }
     switch (ctx->attention_path) {
         case CONFU_ATTENTION_GENERIC: return CONFU_ATTENTION_GENERIC;
@@ -82,9 +84,10 @@ int resolve_attention_path(const confu_ctx* ctx, const confu_dims& d)
             // The two-SM kernel wins where a (sequence, kv head, row group) is split over many work units
             // (small batches: half as many, twice as long runs, half the partial results to merge); with
             // more such pairs than units the one-CTA kernel is the faster one.
-            const int n_rg = (d.T + d.C + kGroupRows - 1) / kGroupRows;
             const bool few_pairs = (int64_t)d.B * d.Hkv * n_rg <= ctx->sm_count / 2;
-            if (pair && few_pairs) return CONFU_ATTENTION_TENSOR_PAIR;
+            // (and with all query rows in one M tile the second CTA of a pair would only see padding)
+            const bool two_tiles = d.T + d.C > rows_per_tile(d.Hq / d.Hkv);
+            if (pair && few_pairs && two_tiles) return CONFU_ATTENTION_TENSOR_PAIR;
             return tc ? (int)CONFU_ATTENTION_TENSOR : (int)CONFU_ATTENTION_GENERIC;
         }
     }
@@ -223,7 +226,7 @@ const char* confu_last_cuda_error(const confu_ctx* ctx)
 size_t confu_plan_bytes(const confu_ctx* ctx, const confu_dims* dims)
 {
     if (!ctx || check_dims(dims) != CONFU_OK) return 0;
-    return plan_bytes(dims->B, dims->Hkv);
+    return plan_bytes(dims->B, dims->Hkv, row_groups(dims->T + dims->C, dims->Hq / dims->Hkv));
 }
 
 int confu_tree_plan(confu_ctx* ctx, const confu_dims* dims, const int64_t* seq_start, const int32_t* prefix_len,

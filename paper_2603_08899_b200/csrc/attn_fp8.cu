@@ -156,7 +156,7 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
     Segment s;
     uint32_t stage = 0, seg = 0;       // running stage / pair counters
     const int R = prm.d.T + prm.d.C;
-    const uint32_t q_box_bytes = 32u * prm.G * 128u;
+    const uint32_t q_box_bytes = (uint32_t)(prm.rpt * prm.G) * 128u;
     TileRef prev = {0, 0, false};
     bool have_prev = false;
     // fills stage `stage` with V of `prev` (if any) and K of `cur` (if any)
@@ -186,7 +186,7 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
                 mbar_arrive_expect_tx(&sh.q_full, 2u * prm.n_mt * q_box_bytes);
                 for (int mt = 0; mt < prm.n_mt; ++mt)
                     for (int kb = 0; kb < 2; ++kb)
-                        tma_load_3d(sh.q + (mt * 2 + kb) * kHalfTile, q_map, &sh.q_full, kb * 64, s.g * prm.G, s.b * R + kGroupRows * s.rg + 32 * mt);
+                        tma_load_3d(sh.q + (mt * 2 + kb) * kHalfTile, q_map, &sh.q_full, kb * 64, s.g * prm.G, s.b * R + prm.rpt * (2 * s.rg + mt));
             }
             prev = cur;
             have_prev = true;
@@ -328,8 +328,8 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
     Segment s;
     uint32_t n_s = 0, seg = 0;
     while (w.next(s)) {
-        const int r = kGroupRows * s.rg + 32 * t + lane_row / G;            // query row of this thread in this pair
-        const bool row_valid = lane_row < 32 * G && r < R;
+        const int r = prm.rpt * (2 * s.rg + t) + lane_row / G;            // query row of this thread in this pair
+        const bool row_valid = lane_row < prm.rpt * G && r < R;
         const uint64_t mask = row_valid ? pv.mask[(size_t)s.b * kMaxRows + r] : 0ull;
         // this run's Q has landed as bf16: this thread's row becomes E4M3 for the tensor pipe
         if (!mbar_wait(&sh.q_full, seg & 1, &sh.abort, prm.wait_ns)) return;
@@ -412,8 +412,8 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
                 const int lr = warp_in_wg * 32 + 8 * kk + (lane >> 2);
-                const int rk = kGroupRows * s.rg + 32 * t + lr / G;
-                o_ptr[kk] = (lr < 32 * G && rk < R)
+                const int rk = prm.rpt * (2 * s.rg + t) + lr / G;
+                o_ptr[kk] = (lr < prm.rpt * G && rk < R)
                                 ? prm.out + (((size_t)s.b * R + rk) * Hq + s.g * G + lr % G) * kD + 8 * (lane & 3)
                                 : nullptr;
             }
@@ -573,7 +573,7 @@ static bool make_byte_map(CUtensorMap* map, const void* base, uint64_t rows, uin
 
 }  // namespace f8
 
-bool make_tile_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t heads, uint32_t box_rows, uint32_t box_heads);
+bool make_tile_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t heads, uint32_t box_rows, uint32_t box_heads, uint32_t head_dim);
 
 }  // namespace tc
 
@@ -592,7 +592,7 @@ cudaError_t launch_attention_fp8(const Ctx* ctx, const confu_dims& d, const void
     using namespace tc::f8;
     const int R = d.T + d.C, G = d.Hq / d.Hkv;
     CUtensorMap q_map, k_map, v_map, ks_map, vs_map;
-    bool ok = make_tile_map(&q_map, q, (uint64_t)d.B * R, d.Hq, 32, G) && make_byte_map(&k_map, k_cache, n_slots, d.Hkv) &&
+    bool ok = make_tile_map(&q_map, q, (uint64_t)d.B * R, d.Hq, rows_per_tile(G), G, kD) && make_byte_map(&k_map, k_cache, n_slots, d.Hkv) &&
               make_byte_map(&v_map, v_cache, n_slots, d.Hkv);
     if (d.S > 0) ok = ok && make_byte_map(&ks_map, k_soft, d.S, d.Hkv) && make_byte_map(&vs_map, v_soft, d.S, d.Hkv);
     else { ks_map = k_map; vs_map = v_map; }
@@ -606,9 +606,7 @@ cudaError_t launch_attention_fp8(const Ctx* ctx, const confu_dims& d, const void
     prm.out = (__nv_bfloat16*)out;
     prm.lse = lse;
     prm.status = status;
-    prm.n_mt = R > 32 ? 2 : 1;
-    prm.n_rg = (R + kGroupRows - 1) / kGroupRows;
-    prm.G = G;
+    set_rows(prm, d);
     prm.c = (d.sm_scale != 0.f ? d.sm_scale : 1.f / sqrtf((float)d.D)) * 1.4426950408889634f;
     prm.wait_ns = ctx->wait_ns;
     prm.k_scale = ctx->k_scale;

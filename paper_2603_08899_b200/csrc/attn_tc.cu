@@ -3,7 +3,7 @@
 //
 // One persistent CTA per SM walks a contiguous range of the flat list of 128-key tiles of all
 // (sequence, kv head) pairs.  For a pair the query block is the R rows x G heads that share the kv
-// head: two M tiles of 128 rows (32 rows x G heads each, padded when G < 4).  Per key tile:
+// head: up to two M tiles of 128 rows (128 / G query rows x G heads each) per row group.  Per key tile:
 //     S_t = Q_t K^T           tcgen05.mma, A and B from shared memory (K-major, 128B swizzle)
 //     P_t = exp2(S_t*c - m)   one thread per row: tcgen05.ld, mask (last tiles only), tcgen05.st as bf16
 //                             over the S columns
@@ -33,16 +33,20 @@ namespace confu {
 namespace tc {
 
 constexpr int kThreads = 384;            // warps 0-3: softmax of M tile 0, 4-7: of M tile 1, 8: TMA, 9: MMA, 10: ragged tail of V
-constexpr int kStages = 2;               // ring of stages; stage g = [V of the CTA's g-1st key tile | K of its g-th]
-constexpr int kQBytes = 2 * kTileBytes;             // two M tiles
+// Per head dim: a 128-row tile of Q, K or V is D / 64 swizzled halves of 16 KB ([128 rows][128 B] each).
+// ring of stages; stage g = [V of the CTA's g-1st key tile | K of its g-th]: two of 64 KB at D = 128 (all
+// that is left beside Q), four of 32 KB at D = 64
+template <int D> constexpr int kTile = kTileKeys * D * 2;
+template <int D> constexpr int kStages = D == 128 ? 2 : 4;
 constexpr uint32_t kTmemCols = 512;                 // S0 | S1 | O0 | O1, 128 columns each; P_t overlays S_t
 constexpr float kRescaleThreshold = 8.f;            // lazy rescale: move the reference max only past 2^8
 
+template <int D>
 struct SharedStorage {
-    alignas(1024) uint8_t q[kQBytes];
-    alignas(1024) uint8_t kv[kStages][2][kTileBytes];    // [stage][0: V tile, 1: K tile]
+    alignas(1024) uint8_t q[2 * kTile<D>];               // two M tiles
+    alignas(1024) uint8_t kv[kStages<D>][2][kTile<D>];   // [stage][0: V tile, 1: K tile]
     alignas(8) uint64_t q_full, q_empty;
-    uint64_t kv_full[kStages], kv_empty[kStages];
+    uint64_t kv_full[kStages<D>], kv_empty[kStages<D>];
     uint64_t s_full[2], p_full[2], o_done[2];
     uint64_t v_fixed;                     // the rows of a V tile past the sequence's last slot have been zeroed
     uint32_t tmem_base;
@@ -60,7 +64,8 @@ struct TileRef {                       // where a key tile's K and V come from
     bool soft;                         // the soft-prompt tile
 };
 
-__device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanView& pv, const CUtensorMap* q_map,
+template <int D>
+__device__ void producer_role(SharedStorage<D>& sh, const Params& prm, const PlanView& pv, const CUtensorMap* q_map,
                               const CUtensorMap* k_map, const CUtensorMap* v_map, const CUtensorMap* ks_map,
                               const CUtensorMap* vs_map)
 {
@@ -69,23 +74,23 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
     Segment s;
     uint32_t stage = 0, seg = 0;       // running stage / pair counters
     const int R = prm.d.T + prm.d.C;
-    const uint32_t q_box_bytes = 32u * prm.G * 128u;
+    const uint32_t q_box_bytes = (uint32_t)(prm.rpt * prm.G) * 128u;
     TileRef prev = {0, 0, false};
     bool have_prev = false;
     // fills stage `stage` with V of `prev` (if any) and K of `cur` (if any)
     auto fill = [&](const TileRef* cur) -> bool {
-        const uint32_t st = stage % kStages;
-        if (!mbar_wait(&sh.kv_empty[st], ((stage / kStages) & 1) ^ 1, &sh.abort, prm.wait_ns)) return false;
-        mbar_arrive_expect_tx(&sh.kv_full[st], (have_prev ? kTileBytes : 0) + (cur ? kTileBytes : 0));
+        const uint32_t st = stage % kStages<D>;
+        if (!mbar_wait(&sh.kv_empty[st], ((stage / kStages<D>) & 1) ^ 1, &sh.abort, prm.wait_ns)) return false;
+        mbar_arrive_expect_tx(&sh.kv_full[st], (have_prev ? kTile<D> : 0) + (cur ? kTile<D> : 0));
         if (have_prev) {
             const CUtensorMap* m = prev.soft ? vs_map : v_map;
             tma_load_3d(sh.kv[st][0], m, &sh.kv_full[st], 0, prev.g, prev.z);
-            tma_load_3d(sh.kv[st][0] + kHalfTile, m, &sh.kv_full[st], 64, prev.g, prev.z);
+            if (D > 64) tma_load_3d(sh.kv[st][0] + kHalfTile, m, &sh.kv_full[st], 64, prev.g, prev.z);
         }
         if (cur) {
             const CUtensorMap* m = cur->soft ? ks_map : k_map;
             tma_load_3d(sh.kv[st][1], m, &sh.kv_full[st], 0, cur->g, cur->z);
-            tma_load_3d(sh.kv[st][1] + kHalfTile, m, &sh.kv_full[st], 64, cur->g, cur->z);
+            if (D > 64) tma_load_3d(sh.kv[st][1] + kHalfTile, m, &sh.kv_full[st], 64, cur->g, cur->z);
         }
         ++stage;
         return true;
@@ -104,10 +109,10 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
             if (!fill(&cur)) return;
             if (t == s.t0) {
                 if (!mbar_wait(&sh.q_empty, (seg & 1) ^ 1, &sh.abort, prm.wait_ns)) return;
-                mbar_arrive_expect_tx(&sh.q_full, 2u * prm.n_mt * q_box_bytes);
+                mbar_arrive_expect_tx(&sh.q_full, (D / 64) * prm.n_mt * q_box_bytes);
                 for (int mt = 0; mt < prm.n_mt; ++mt)
-                    for (int kb = 0; kb < 2; ++kb)
-                        tma_load_3d(sh.q + (mt * 2 + kb) * kHalfTile, q_map, &sh.q_full, kb * 64, s.g * prm.G, s.b * R + kGroupRows * s.rg + 32 * mt);
+                    for (int kb = 0; kb < D / 64; ++kb)
+                        tma_load_3d(sh.q + mt * kTile<D> + kb * kHalfTile, q_map, &sh.q_full, kb * 64, s.g * prm.G, s.b * R + prm.rpt * (2 * s.rg + mt));
             }
             prev = cur;
             have_prev = true;
@@ -119,8 +124,8 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
 
 // One thread issues all tensor-core work.  Per stage g: P V of key tile g-1 for both M tiles (each
 // as soon as its P is there), Q K^T of key tile g for both, then the stage is released.
-template <bool kTwo>
-__device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& pv, uint32_t tmem)
+template <int D, bool kTwo>
+__device__ void mma_role(SharedStorage<D>& sh, const Params& prm, const PlanView& pv, uint32_t tmem)
 {
     constexpr int kMt = kTwo ? 2 : 1;
     Walker w(pv, prm, blockIdx.x);
@@ -130,12 +135,13 @@ __device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& p
     // two 64-column halves kHalfTile apart) = stage 0's words + stage * stage size
     const uint32_t q_lo = desc_lo(smem_u32(sh.q), 16);
     const uint32_t v_lo0 = desc_lo(smem_u32(sh.kv[0][0]), kHalfTile), k_lo0 = desc_lo(smem_u32(sh.kv[0][1]), 16);
-    constexpr uint32_t kTileStep = kTileBytes >> 4, kStageStep = 2 * kTileStep;
+    constexpr uint32_t kTileStep = kTile<D> >> 4, kStageStep = 2 * kTileStep;
+    constexpr uint32_t kIdescO = D == 128 ? kIdescPV : kIdescPV64;
 
-    // S_t = Q_t K^T: 8 steps of 16 head dims; step i sits in 64-column half i/4 at byte 32*(i%4) of the swizzled row
+    // S_t = Q_t K^T: D / 16 steps of 16 head dims; step i sits in 64-column half i/4 at byte 32*(i%4) of the swizzled row
     auto issue_qk = [&](int t, uint32_t kl) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < D / 16; ++i) {
             const uint32_t off = ((uint32_t)(i >> 2) * kHalfTile + (uint32_t)(i & 3) * 32u) >> 4;
             mma_ss(tmem + t * 128, q_lo + t * kTileStep + off, kl + off, kIdescQK, i > 0 ? 1u : 0u);
         }
@@ -146,15 +152,15 @@ __device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& p
     auto issue_pv = [&](int t, uint32_t vl, bool first_of_segment) {
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-            mma_ts(tmem + 256 + t * 128, tmem + t * 128 + i * 8, vl + i * (2048u >> 4), kIdescPV,
+            mma_ts(tmem + 256 + t * 128, tmem + t * 128 + i * 8, vl + i * (2048u >> 4), kIdescO,
                    (first_of_segment && i == 0) ? 0u : 1u);
     };
     // one stage: P V of the previous key tile (if any), Q K^T of the current one (if any)
     bool have_prev = false, prev_first = false, prev_last = false, prev_ragged = false;
     uint32_t n_fix = 0;
     auto run_stage = [&](bool have_cur, bool cur_first, bool cur_last, bool cur_ragged) -> bool {
-        const uint32_t st = stage % kStages;
-        if (!mbar_wait(&sh.kv_full[st], (stage / kStages) & 1, &sh.abort, prm.wait_ns)) return false;
+        const uint32_t st = stage % kStages<D>;
+        if (!mbar_wait(&sh.kv_full[st], (stage / kStages<D>) & 1, &sh.abort, prm.wait_ns)) return false;
         if (have_cur && cur_first && !mbar_wait(&sh.q_full, seg & 1, &sh.abort, prm.wait_ns)) return false;
         // the V tile of a sequence's last key tile: wait until its rows past the last slot are zero
         if (have_prev && prev_ragged) {
@@ -199,7 +205,8 @@ __device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& p
 // of a sequence's last key tile, zeroes the rows past the sequence's last slot (generic-proxy
 // stores, made visible to the tensor pipe by a proxy fence) before it lets the issuing thread go on.
 // It arrives on every stage's empty barrier, so a stage is never refilled before it has seen it.
-__device__ void tail_role(SharedStorage& sh, const Params& prm, const PlanView& pv)
+template <int D>
+__device__ void tail_role(SharedStorage<D>& sh, const Params& prm, const PlanView& pv)
 {
     Walker w(pv, prm, blockIdx.x);
     Segment s;
@@ -208,11 +215,11 @@ __device__ void tail_role(SharedStorage& sh, const Params& prm, const PlanView& 
     int prev_valid = 0;                 // > 0: the previous tile's V needs rows [prev_valid, 128) zeroed
     bool have_prev = false;
     auto run_stage = [&](int cur_valid) -> bool {
-        const uint32_t st = stage % kStages;
-        if (!mbar_wait(&sh.kv_full[st], (stage / kStages) & 1, &sh.abort, prm.wait_ns)) return false;
+        const uint32_t st = stage % kStages<D>;
+        if (!mbar_wait(&sh.kv_full[st], (stage / kStages<D>) & 1, &sh.abort, prm.wait_ns)) return false;
         if (have_prev && prev_valid > 0) {
             const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-            for (int half = 0; half < 2; ++half)
+            for (int half = 0; half < D / 64; ++half)
                 for (int off = prev_valid * 128 + lane * 16; off < kHalfTile; off += 32 * 16)
                     *reinterpret_cast<uint4*>(sh.kv[st][0] + half * kHalfTile + off) = zero;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -232,7 +239,8 @@ __device__ void tail_role(SharedStorage& sh, const Params& prm, const PlanView& 
     if (have_prev) run_stage(0);
 }
 
-__device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanView& pv, uint32_t tmem, int t /*M tile*/)
+template <int D>
+__device__ void softmax_role(SharedStorage<D>& sh, const Params& prm, const PlanView& pv, uint32_t tmem, int t /*M tile*/)
 {
     const int lane_row = threadIdx.x & 127;                 // row of the M tile = TMEM lane
     const int warp_in_wg = (threadIdx.x >> 5) & 3;
@@ -247,8 +255,8 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
     Segment s;
     uint32_t n_s = 0, seg = 0;
     while (w.next(s)) {
-        const int r = kGroupRows * s.rg + 32 * t + lane_row / G;            // query row of this thread in this pair
-        const bool row_valid = lane_row < 32 * G && r < R;
+        const int r = prm.rpt * (2 * s.rg + t) + lane_row / G;            // query row of this thread in this pair
+        const bool row_valid = lane_row < prm.rpt * G && r < R;
         const uint64_t mask = row_valid ? pv.mask[(size_t)s.b * kMaxRows + r] : 0ull;
         float m_ref = -INFINITY, l = 0.f;
         for (int tile = s.t0; tile < s.t1; ++tile) {
@@ -279,7 +287,7 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
                     if (move) { m_ref = m_new; l *= alpha; }
                     // S_full of this tile implies the previous PV of this M tile has completed
 #pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4) {
+                    for (int q4 = 0; q4 < D / 32; ++q4) {
                         uint32_t ov[32];
                         tmem_ld32(o_addr + q4 * 32, ov);
                         tc_wait_ld();
@@ -321,9 +329,9 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
                 const int lr = warp_in_wg * 32 + 8 * kk + (lane >> 2);
-                const int rk = kGroupRows * s.rg + 32 * t + lr / G;
-                o_ptr[kk] = (lr < 32 * G && rk < R)
-                                ? prm.out + (((size_t)s.b * R + rk) * Hq + s.g * G + lr % G) * kD + 8 * (lane & 3)
+                const int rk = prm.rpt * (2 * s.rg + t) + lr / G;
+                o_ptr[kk] = (lr < prm.rpt * G && rk < R)
+                                ? prm.out + (((size_t)s.b * R + rk) * Hq + s.g * G + lr % G) * D + 8 * (lane & 3)
                                 : nullptr;
             }
         } else {
@@ -331,7 +339,7 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
                     (size_t)(t * 128 + warp_in_wg * 32 + (lane >> 3)) * kPartD + 4 * (lane & 7);
         }
 #pragma unroll 1
-        for (int q4 = 0; q4 < 4; ++q4) {
+        for (int q4 = 0; q4 < D / 32; ++q4) {
             uint32_t ov[32];
             tmem_ld32(o_addr + q4 * 32, ov);
             tc_wait_ld();
@@ -374,20 +382,21 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
     }
 }
 
+template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 attention_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                     const __grid_constant__ CUtensorMap v_map, const __grid_constant__ CUtensorMap ks_map,
                     const __grid_constant__ CUtensorMap vs_map, const Params prm)
 {
     extern __shared__ uint8_t smem_raw[];
-    SharedStorage& sh = *reinterpret_cast<SharedStorage*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    SharedStorage<D>& sh = *reinterpret_cast<SharedStorage<D>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int warp = threadIdx.x >> 5;
 
     if (threadIdx.x == 0) {
         mbar_init(&sh.q_full, 1);
         mbar_init(&sh.q_empty, 1);
         // a stage is free again when its MMAs have completed and the tail warp has seen it
-        for (int i = 0; i < kStages; ++i) { mbar_init(&sh.kv_full[i], 1); mbar_init(&sh.kv_empty[i], 2); }
+        for (int i = 0; i < kStages<D>; ++i) { mbar_init(&sh.kv_full[i], 1); mbar_init(&sh.kv_empty[i], 2); }
         mbar_init(&sh.v_fixed, 1);
         for (int t = 0; t < 2; ++t) {
             mbar_init(&sh.s_full[t], 1);
@@ -426,8 +435,8 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
             if ((threadIdx.x & 31) == 0) producer_role(sh, prm, pv, &q_map, &k_map, &v_map, &ks_map, &vs_map);
         } else if (warp == 9) {
             if ((threadIdx.x & 31) == 0) {
-                if (prm.n_mt > 1) mma_role<true>(sh, prm, pv, tmem);
-                else mma_role<false>(sh, prm, pv, tmem);
+                if (prm.n_mt > 1) mma_role<D, true>(sh, prm, pv, tmem);
+                else mma_role<D, false>(sh, prm, pv, tmem);
             }
         } else if (warp == 10) {
             tail_role(sh, prm, pv);
@@ -469,14 +478,14 @@ static EncodeTiledFn encode_fn()
     return fn;
 }
 
-// [rows][heads][128] bf16 tensor, box = box_rows x box_heads x 64 elements, 128-byte swizzle
+// [rows][heads][head_dim] bf16 tensor, box = box_rows x box_heads x 64 elements, 128-byte swizzle
 bool make_tile_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t heads, uint32_t box_rows,
-                   uint32_t box_heads)
+                   uint32_t box_heads, uint32_t head_dim)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
-    const cuuint64_t dims[3] = {(cuuint64_t)kD, heads, rows};
-    const cuuint64_t strides[2] = {(cuuint64_t)kD * 2, heads * kD * 2};
+    const cuuint64_t dims[3] = {(cuuint64_t)head_dim, heads, rows};
+    const cuuint64_t strides[2] = {(cuuint64_t)head_dim * 2, heads * head_dim * 2};
     const cuuint32_t box[3] = {64, box_heads, box_rows};
     const cuuint32_t estr[3] = {1, 1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
@@ -489,20 +498,21 @@ bool make_tile_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t h
 bool tc_attention_supported(const confu_dims& d)
 {
     const int G = d.Hq / d.Hkv;
-    return d.kv_dtype == CONFU_BF16 && d.D == 128 && G <= 4 && d.S <= 128;
+    return d.kv_dtype == CONFU_BF16 && G <= kMaxTcGroup && d.S <= 128;
 }
 
-cudaError_t launch_attention_tc(const Ctx* ctx, const confu_dims& d, const void* q, const void* k_cache,
-                                const void* v_cache, int64_t n_slots, const SlotMap& map,
-                                const int32_t* prefix_len, const void* k_soft, const void* v_soft, const void* plan,
-                                void* partials, void* out, float* lse, int32_t* status, cudaStream_t st)
+template <int D>
+static cudaError_t launch_tc(const Ctx* ctx, const confu_dims& d, const void* q, const void* k_cache,
+                             const void* v_cache, int64_t n_slots, const SlotMap& map, const int32_t* prefix_len,
+                             const void* k_soft, const void* v_soft, const void* plan, void* partials, void* out,
+                             float* lse, int32_t* status, cudaStream_t st)
 {
     using namespace tc;
     const int R = d.T + d.C, G = d.Hq / d.Hkv;
     CUtensorMap q_map, k_map, v_map, ks_map, vs_map;
-    bool ok = make_tile_map(&q_map, q, (uint64_t)d.B * R, d.Hq, 32, G) && make_tile_map(&k_map, k_cache, n_slots, d.Hkv, kTileKeys, 1) &&
-              make_tile_map(&v_map, v_cache, n_slots, d.Hkv, kTileKeys, 1);
-    if (d.S > 0) ok = ok && make_tile_map(&ks_map, k_soft, d.S, d.Hkv, kTileKeys, 1) && make_tile_map(&vs_map, v_soft, d.S, d.Hkv, kTileKeys, 1);
+    bool ok = make_tile_map(&q_map, q, (uint64_t)d.B * R, d.Hq, rows_per_tile(G), G, D) && make_tile_map(&k_map, k_cache, n_slots, d.Hkv, kTileKeys, 1, D) &&
+              make_tile_map(&v_map, v_cache, n_slots, d.Hkv, kTileKeys, 1, D);
+    if (d.S > 0) ok = ok && make_tile_map(&ks_map, k_soft, d.S, d.Hkv, kTileKeys, 1, D) && make_tile_map(&vs_map, v_soft, d.S, d.Hkv, kTileKeys, 1, D);
     else { ks_map = k_map; vs_map = v_map; }
     if (!ok) return cudaErrorInvalidValue;
     Params prm;
@@ -514,17 +524,15 @@ cudaError_t launch_attention_tc(const Ctx* ctx, const confu_dims& d, const void*
     prm.out = (__nv_bfloat16*)out;
     prm.lse = lse;
     prm.status = status;
-    prm.n_mt = R > 32 ? 2 : 1;
-    prm.n_rg = (R + kGroupRows - 1) / kGroupRows;
-    prm.G = G;
+    set_rows(prm, d);
     prm.c = (d.sm_scale != 0.f ? d.sm_scale : 1.f / sqrtf((float)d.D)) * 1.4426950408889634f;
     prm.wait_ns = ctx->wait_ns;
     prm.k_scale = prm.v_scale = nullptr;
-    const size_t smem = sizeof(SharedStorage) + 1024;
+    const size_t smem = sizeof(SharedStorage<D>) + 1024;
     static OncePerDevice attr_done;
     {
         cudaError_t e = attr_done.run([&] {
-            return cudaFuncSetAttribute(attention_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            return cudaFuncSetAttribute(attention_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         });
         if (e != cudaSuccess) return e;
     }
@@ -542,9 +550,18 @@ cudaError_t launch_attention_tc(const Ctx* ctx, const confu_dims& d, const void*
     cfg.stream = st;
     cfg.attrs = pdl;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, attention_tc_kernel, q_map, k_map, v_map, ks_map, vs_map, prm);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, attention_tc_kernel<D>, q_map, k_map, v_map, ks_map, vs_map, prm);
     if (e != cudaSuccess) return e;
     return launch_combine(prm, ctx->sm_count, st);
+}
+
+cudaError_t launch_attention_tc(const Ctx* ctx, const confu_dims& d, const void* q, const void* k_cache,
+                                const void* v_cache, int64_t n_slots, const SlotMap& map,
+                                const int32_t* prefix_len, const void* k_soft, const void* v_soft, const void* plan,
+                                void* partials, void* out, float* lse, int32_t* status, cudaStream_t st)
+{
+    return (d.D == 64 ? launch_tc<64> : launch_tc<128>)(ctx, d, q, k_cache, v_cache, n_slots, map, prefix_len, k_soft, v_soft,
+                                                        plan, partials, out, lse, status, st);
 }
 
 }  // namespace confu

@@ -7,7 +7,7 @@
 namespace confu {
 namespace tc {
 
-constexpr int kD = 128;
+constexpr int kD = 128;         // largest head dim of the tensor-core kernels
 
 struct Params {
     confu_dims d;
@@ -18,9 +18,10 @@ struct Params {
     __nv_bfloat16* out;
     float* lse;
     int32_t* status;
-    int n_mt;            // M tiles in use (R > 32 ? 2 : 1)
-    int n_rg;            // groups of 64 query rows (R > 64 ? 2 : 1); a pair = (sequence, kv head, row group)
-    int G;
+    int n_mt;            // M tiles in use (2 unless one holds all rows)
+    int n_rg;            // groups of query rows; a pair = (sequence, kv head, row group)
+    int G;               // query heads per kv head
+    int rpt;             // query rows per M tile (128 / G); a row group is two M tiles
     float c;             // sm_scale * log2(e)
     unsigned long long wait_ns;   // limit of every wait on an mbarrier (wall clock)
     const float* k_scale;         // E4M3 cache: value = code * scale[kv head] (device, [Hkv]); unused otherwise
@@ -32,6 +33,15 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
     uint32_t r;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
+}
+
+// The row packing of a launch (see rows_per_tile).
+inline void set_rows(Params& p, const confu_dims& d)
+{
+    p.G = d.Hq / d.Hkv;
+    p.rpt = rows_per_tile(p.G);
+    p.n_mt = d.T + d.C > p.rpt ? 2 : 1;
+    p.n_rg = row_groups(d.T + d.C, p.G);
 }
 
 // Enqueues the merge of the partial results that the attention launch with the same parameters

@@ -1,8 +1,8 @@
 // Tensor-core tree attention on CTA pairs: the two-SM form of tcgen05.mma (cta_group::2).
 //
 // Two CTAs of a cluster (two neighbouring SMs) work on one (sequence, kv head, row group) at a time.
-// The 256 query rows that share the kv head (64 rows x 4 heads of the GQA group) are one M = 256
-// operand: rows 0-127 (query rows 0-31 of the group) live in CTA 0, rows 128-255 in CTA 1.  Per
+// The 256 query rows that share the kv head (2 x 128 / G query rows x G heads of the GQA group) are one M = 256
+// operand: rows 0-127 (the first 128 / G query rows of the group) live in CTA 0, rows 128-255 in CTA 1.  Per
 // 128-key tile
 //     S = Q K^T      one M256 N128 K16 instruction per 16 head dims: each CTA supplies its 128 rows of
 //                    Q and 64 of the 128 keys, and receives its 128 rows of S in its own tensor memory
@@ -180,7 +180,7 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
     Segment s;
     uint32_t g = 0, seg = 0;
     const int R = prm.d.T + prm.d.C;
-    const uint32_t q_box_bytes = 32u * prm.G * 128u;
+    const uint32_t q_box_bytes = (uint32_t)(prm.rpt * prm.G) * 128u;
     TileRef hist[kVLag];               // the tiles of the last kVLag stages, oldest first: hist[0]'s V travels with this stage's K
 #pragma unroll
     for (int i = 0; i < kVLag; ++i) hist[i].present = false;
@@ -221,7 +221,7 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
                 mbar_arrive_expect_tx(&sh.q_full[qb], 2u * q_box_bytes);
                 for (int kb = 0; kb < 2; ++kb)
                     tma_load_3d(sh.q[qb] + kb * kHalfTile, q_map, &sh.q_full[qb], kb * 64, s.g * prm.G,
-                                s.b * R + kGroupRows * s.rg + 32 * (int)rank);
+                                s.b * R + prm.rpt * (2 * s.rg + (int)rank));
             }
         }
         ++seg;
@@ -376,8 +376,8 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
     Segment s;
     uint32_t g = 0, seg = 0;
     while (w.next(s)) {
-        const int r = kGroupRows * s.rg + 32 * (int)rank + lane_row / G;      // query row of this thread in this run
-        const bool row_valid = lane_row < 32 * G && r < R;
+        const int r = prm.rpt * (2 * s.rg + (int)rank) + lane_row / G;      // query row of this thread in this run
+        const bool row_valid = lane_row < prm.rpt * G && r < R;
         const uint64_t mask = row_valid ? pv.mask[(size_t)s.b * kMaxRows + r] : 0ull;
         // this thread's share of the row's sum of weights, relative to the reference maximum m_mine
         // (the row's reference as of the last tile this thread worked on)
@@ -484,8 +484,8 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) {
                 const int lr = wq * 32 + 8 * kk + (lane >> 2);
-                const int rk = kGroupRows * s.rg + 32 * (int)rank + lr / G;
-                o_ptr[kk] = (lr < 32 * G && rk < R)
+                const int rk = prm.rpt * (2 * s.rg + (int)rank) + lr / G;
+                o_ptr[kk] = (lr < prm.rpt * G && rk < R)
                                 ? prm.out + (((size_t)s.b * R + rk) * Hq + s.g * G + lr % G) * kD + 8 * (lane & 3)
                                 : nullptr;
             }
@@ -634,14 +634,14 @@ attention_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
 
 }  // namespace pair
 
-bool make_tile_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t heads, uint32_t box_rows, uint32_t box_heads);
+bool make_tile_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t heads, uint32_t box_rows, uint32_t box_heads, uint32_t head_dim);
 
 }  // namespace tc
 
-bool pair_attention_supported(const confu_dims& d, int sm_count)
+bool pair_attention_supported(const confu_dims& d)
 {
     const int G = d.Hq / d.Hkv;
-    return d.kv_dtype == CONFU_BF16 && d.D == 128 && G <= 4 && d.S <= 128 && d.T + d.C > 32 && sm_count >= 4;
+    return d.kv_dtype == CONFU_BF16 && d.D == 128 && G <= kMaxTcGroup && d.S <= 128 && (d.T + d.C > 32 || d.T + d.C > rows_per_tile(G));
 }
 
 cudaError_t launch_attention_pair(const Ctx* ctx, const confu_dims& d, const void* q, const void* k_cache,
@@ -654,9 +654,9 @@ cudaError_t launch_attention_pair(const Ctx* ctx, const confu_dims& d, const voi
     const int R = d.T + d.C, G = d.Hq / d.Hkv;
     CUtensorMap q_map, k_map, v_map, ks_map, vs_map;
     // K: 64 keys x 64 head dims per box (this CTA's keys, one half of the head dim); V: 128 keys x 64 head dims
-    bool ok = make_tile_map(&q_map, q, (uint64_t)d.B * R, d.Hq, 32, G) && make_tile_map(&k_map, k_cache, n_slots, d.Hkv, 64, 1) &&
-              make_tile_map(&v_map, v_cache, n_slots, d.Hkv, kTileKeys, 1);
-    if (d.S > 0) ok = ok && make_tile_map(&ks_map, k_soft, d.S, d.Hkv, 64, 1) && make_tile_map(&vs_map, v_soft, d.S, d.Hkv, kTileKeys, 1);
+    bool ok = make_tile_map(&q_map, q, (uint64_t)d.B * R, d.Hq, rows_per_tile(G), G, kD) && make_tile_map(&k_map, k_cache, n_slots, d.Hkv, 64, 1, kD) &&
+              make_tile_map(&v_map, v_cache, n_slots, d.Hkv, kTileKeys, 1, kD);
+    if (d.S > 0) ok = ok && make_tile_map(&ks_map, k_soft, d.S, d.Hkv, 64, 1, kD) && make_tile_map(&vs_map, v_soft, d.S, d.Hkv, kTileKeys, 1, kD);
     else { ks_map = k_map; vs_map = v_map; }
     if (!ok) return cudaErrorInvalidValue;
     Params prm;
@@ -668,9 +668,7 @@ cudaError_t launch_attention_pair(const Ctx* ctx, const confu_dims& d, const voi
     prm.out = (__nv_bfloat16*)out;
     prm.lse = lse;
     prm.status = status;
-    prm.n_mt = 2;
-    prm.n_rg = (R + kGroupRows - 1) / kGroupRows;
-    prm.G = G;
+    set_rows(prm, d);
     prm.c = (d.sm_scale != 0.f ? d.sm_scale : 1.f / sqrtf((float)d.D)) * 1.4426950408889634f;
     prm.wait_ns = ctx->wait_ns;
     prm.k_scale = prm.v_scale = nullptr;

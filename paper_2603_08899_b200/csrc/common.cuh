@@ -12,9 +12,21 @@ namespace confu {
 
 constexpr int kMaxRows = CONFU_MAX_ROWS;        // R = T + C <= 128
 constexpr int kMaxTree = CONFU_MAX_TREE;        // T <= 64: one 64-bit word of visible tree slots per row
-constexpr int kGroupRows = 64;                  // query rows the tensor-core kernel handles per pass over a pair's keys
 constexpr int kPathLen = CONFU_MAX_DEPTH + 1;
 constexpr int kTileKeys = 128;                  // keys per attention tile (tensor-core path)
+
+// How the tensor-core kernels pack query rows: the G query heads that share a kv head stand side by
+// side in an M tile of 128, so a tile holds 128 / G query rows, and a pass over a pair's keys (two M
+// tiles) a group of twice as many.  (Filling the tile whatever G is, instead of 32 rows x G heads,
+// halves the tensor and exponential work of a group of 64 rows at G <= 2 and is what lets G > 4 in.  One
+// layer, own plan, bf16: B 4, 64 / 8 heads of 128, R 64, prefixes 500..4000: 49 us, on CUDA cores 15270 us;
+// B 2, 32 / 8 heads of 64, R 64, prefixes 1500..2500: 27 us, on CUDA cores 2820 us.)
+constexpr int kMaxTcGroup = 32;                 // query heads per kv head the tensor-core kernels take (groups of 8 rows at G = 32)
+__host__ __device__ inline int rows_per_tile(int G) { return 128 / G; }
+__host__ __device__ inline int row_groups(int R, int G)
+{
+    return G > kMaxTcGroup ? 1 : (R + 2 * rows_per_tile(G) - 1) / (2 * rows_per_tile(G));
+}
 
 // ---------------------------------------------------------------------------
 // Plan buffer (device).  Built once per step by plan_kernel, read by every layer.
@@ -25,14 +37,14 @@ constexpr int kTileKeys = 128;                  // keys per attention tile (tens
 //   int32  tiles[B]           key tiles of one (sequence, kv head) pair, soft-prompt tile included
 //   int64  tile_base[B + 1]   position of sequence b's first (sequence, kv head) stretch on the flat cost line (exclusive scan)
 //   int32  seg_begin[kPlanMaxCtas + 1]   CTA c of the tensor-core kernel walks segs[seg_begin[c] .. seg_begin[c+1])
-//   SegDesc segs[B * Hkv * 2 + kPlanMaxCtas]   the runs of key tiles, one pair at a time, of every CTA in walking order
+//   SegDesc segs[B * Hkv * max(2, n_rg) + kPlanMaxCtas]   the runs of key tiles, one pair at a time, of every CTA in walking order
 //
 // The split-KV work is balanced on a "cost line": every (sequence, kv head) pair takes
 // tiles + kPairOverheadTiles consecutive positions (the overhead stands for loading Q, draining
 // the pipeline and writing the output once per pair), pairs in (sequence, head) order.  The line is
 // cut into n equal shares; share c covers positions [c*N/n, (c+1)*N/n); position q of a pair means
 // key tile q - kPairOverheadTiles, so a share that ends inside a pair's overhead zone takes none of
-// its tiles.  With n_rg groups of 64 query rows (n_rg = 1 or 2) there are n = n_ctas / n_rg shares and
+// its tiles.  With n_rg groups of query rows (row_groups above) there are n = n_ctas / n_rg shares and
 // CTA c * n_rg + rg walks share c for row group rg: the CTAs of a share read the same K/V tiles at
 // about the same time, so that only the first read of a tile goes to DRAM.
 // ---------------------------------------------------------------------------
@@ -47,7 +59,7 @@ struct PlanHeader {
 // One run of key tiles of one pair inside a CTA's share of the cost line.
 constexpr int kPlanMaxCtas = 256;
 struct alignas(16) SegDesc {
-    int32_t b, g_rg;           // sequence; kv head | group of 64 query rows << 16
+    int32_t b, g_rg;           // sequence; kv head | group of query rows << 16
     int32_t t0, t1;            // tiles [t0, t1) of the pair
     int32_t nt, P;             // tiles of the pair (soft-prompt tile included); prefix length
     int32_t part_slot;         // -1: the run covers the whole pair; else the CTA's partial slot
@@ -69,7 +81,7 @@ struct PlanView {
 
 __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-__host__ __device__ inline size_t plan_bytes(int B, int Hkv)
+__host__ __device__ inline size_t plan_bytes(int B, int Hkv, int n_rg)
 {
     size_t n = align_up(sizeof(PlanHeader), 256);
     n += align_up((size_t)B * kMaxRows * sizeof(uint64_t), 256);
@@ -77,7 +89,7 @@ __host__ __device__ inline size_t plan_bytes(int B, int Hkv)
     n += align_up((size_t)B * sizeof(int32_t), 256);
     n += align_up((size_t)(B + 1) * sizeof(int64_t), 256);
     n += align_up((size_t)(kPlanMaxCtas + 1) * sizeof(int32_t), 256);
-    n += align_up(((size_t)B * Hkv * 2 + kPlanMaxCtas) * sizeof(SegDesc), 256);
+    n += align_up(((size_t)B * Hkv * (n_rg > 2 ? n_rg : 2) + kPlanMaxCtas) * sizeof(SegDesc), 256);
     return n;
 }
 

@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(256) plan_kernel(confu_dims d, int units, int 
         int64_t acc = 0;
         for (int b = 0; b < B; ++b) {
             pv.tile_base[b] = acc;
-            // one stretch of the line per (sequence, kv head); its groups of 64 query rows are walked side by side
+            // one stretch of the line per (sequence, kv head); its groups of query rows are walked side by side
             if (pv.tiles[b] > 0) acc += (int64_t)(pv.tiles[b] + kPairOverheadTiles) * d.Hkv;
         }
         pv.tile_base[B] = acc;
@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(256) plan_kernel(confu_dims d, int units, int 
         h.n_tiles = acc;
         // The line is cut into `lanes` shares; CTA lane * n_rg + rg walks the lane's share for row group rg,
         // so the CTAs of a lane read the same K/V tiles at about the same time (the second read hits L2).
-        const int n_rg0 = (R + kGroupRows - 1) / kGroupRows;
+        const int n_rg0 = row_groups(R, d.Hq / d.Hkv);
         int cap = units < kPlanMaxCtas ? units : kPlanMaxCtas;
         int lanes = cap / n_rg0;
         if ((int64_t)lanes > acc) lanes = (int)acc;
@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(256) plan_kernel(confu_dims d, int units, int 
     // The runs of key tiles of every CTA of the tensor-core attention kernel, worked out once per step
     // instead of by every role of every CTA of every layer: thread c walks CTA c's share of the cost
     // line, first to count its runs, then (behind a prefix sum) to write them down.
-    const int n_rg = (R + kGroupRows - 1) / kGroupRows;
+    const int n_rg = row_groups(R, d.Hq / d.Hkv);
     const int64_t N = pv.hdr->n_tiles;
     const int n_ctas = pv.hdr->n_ctas, n_lanes = n_ctas / n_rg;
     for (int pass = 0; pass < 2; ++pass) {

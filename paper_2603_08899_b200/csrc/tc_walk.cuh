@@ -11,7 +11,7 @@ constexpr int kTileBytes = kTileKeys * kD * 2;      // one 128-key tile of K or 
 constexpr int kHalfTile = kTileBytes / 2;           // one 64-wide half of the head dim: [128 rows][128 B]
 
 struct Segment {
-    int b, g, rg;      // sequence, kv head, group of 64 query rows
+    int b, g, rg;      // sequence, kv head, group of query rows
     int t0, t1;        // tiles [t0, t1) of this pair
     int nt, nkt;       // tiles of the pair; key tiles (the soft-prompt tile, if any, is tile nkt)
     int64_t P;         // prefix length

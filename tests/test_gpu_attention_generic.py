@@ -1,0 +1,40 @@
+"""CUDA-core attention at the edges of its blocks (16, 32 or 64 row-head pairs) and of its 64-key tiles, with
+clusters of every size, against the fp64 oracle; and that slots a row does not see may hold anything."""
+import pytest
+import torch
+
+from paper_2603_08899_b200 import binding as cb
+from paper_2603_08899_b200 import inputs
+from tests import harness as H
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gpu():
+    g = H.Gpu()
+    yield g
+    g.close()
+
+
+def _cfg(B, Hq, Hkv, D, T, C, S, prefix, dtype):
+    return inputs.VerifyConfig("generic", B=B, L=1, Hq=Hq, Hkv=Hkv, D=D, T=T, C=C, S=S, V=32, prefix=prefix, tree="random",
+                               kv_dtype=dtype, logit_dtype=torch.float32, sigma_logit=1.0, draft="independent",
+                               temperatures=(1.0,), seed=700 + B + D + T, max_depth=7, fanout=(1, 4))
+
+
+F, H16 = torch.float32, torch.bfloat16
+CASES = [_cfg(1, 1, 1, 64, 1, 0, 0, 0, F), _cfg(1, 1, 1, 128, 16, 0, 0, 48, F), _cfg(1, 1, 1, 128, 17, 0, 3, 44, F),
+         _cfg(1, 4, 2, 64, 8, 2, 2, 700, F), _cfg(2, 32, 4, 64, 33, 31, 16, (1, 600), F), _cfg(12, 16, 8, 128, 30, 30, 16, (1, 300), F),
+         _cfg(3, 8, 8, 128, 64, 64, 130, (60, 200), F), _cfg(2, 4, 2, 128, 20, 20, 150, (60, 200), H16),
+         _cfg(1, 40, 1, 64, 5, 3, 2, 333, H16)]
+
+
+@pytest.mark.parametrize("cfg", CASES, ids=lambda c: f"B{c.B}_{c.Hq}x{c.Hkv}x{c.D}_R{c.R}_S{c.S}")
+def test_generic_matches_oracle(gpu, cfg):
+    parent, owner, plen, seq_start, n_slots, t = H.setup_case(cfg)
+    assert cb.confu_attention_path(gpu.ctx, H.dims_of(cfg)) == cb.ATTENTION_GENERIC
+    out, lse, st = H.gpu_attention(gpu, cfg, t, seq_start, plen, parent, owner, n_slots)
+    want, want_lse, _ = H.oracle_attention(cfg, t, seq_start, plen, parent, owner)
+    assert st.tolist() == [0] * cfg.B
+    H.assert_attention_close(out, lse, want, want_lse, cfg.kv_dtype, cfg.name)

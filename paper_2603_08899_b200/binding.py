@@ -1,4 +1,5 @@
-"""Thin ctypes binding of the C-ABI library (libconfu.so): argument marshalling only.
+"""Thin binding of the C-ABI library (libconfu.so): argument marshalling only.  The calls that enqueue
+work go through a small native module (csrc/python_calls.cpp), everything else through ctypes.
 
 Every function here has the name of the C entry point it forwards to and does nothing but
 turn torch CUDA tensors into pointers; every step of the path runs in the CUDA kernels.
@@ -63,6 +64,19 @@ def lib():
     return _lib
 
 
+_calls = None
+
+
+def _native():
+    """The native module with the calls that enqueue work, behind the library itself."""
+    global _calls
+    if _calls is None:
+        lib()
+        from . import _calls as module
+        _calls = module
+    return _calls
+
+
 class ConfuError(RuntimeError):
     def __init__(self, fn, code, detail=""):
         self.code = code
@@ -90,8 +104,16 @@ def _check(fn, rc, ctx=None):
         raise ConfuError(fn, rc, detail)
 
 
+def _done(fn, rc, ctx):
+    if rc:
+        _check(fn, rc, ctx)
+
+
+_DTYPES = {torch.bfloat16: BF16, torch.float32: F32, torch.uint8: FP8_E4M3, torch.float8_e4m3fn: FP8_E4M3}
+
+
 def dtype_code(dt):
-    return {torch.bfloat16: BF16, torch.float32: F32, torch.uint8: FP8_E4M3, torch.float8_e4m3fn: FP8_E4M3}[dt]
+    return _DTYPES[dt]
 
 
 def make_dims(B, Hq, Hkv, D, T, Cn, S, dtype, sm_scale=0.0):
@@ -150,18 +172,14 @@ def confu_plan_bytes(ctx, dims):
 
 
 def confu_tree_plan(ctx, dims, seq_start, prefix_len, parent, con_owner, plan, status, stream=None):
-    _check("confu_tree_plan",
-           lib().confu_tree_plan(ctx, C.byref(dims), _ptr(seq_start), _ptr(prefix_len), _ptr(parent),
-                                 _ptr(con_owner), _ptr(plan), _ptr(status), _stream(stream)), ctx)
+    _done("confu_tree_plan", _native().tree_plan(ctx, dims, seq_start, prefix_len, parent, con_owner, plan, status, stream), ctx)
 
 
 def confu_tree_attention(ctx, dims, q, k_cache, v_cache, n_slots, seq_start, prefix_len, k_soft, v_soft, parent,
                          con_owner, plan, out, lse, status, stream=None):
-    _check("confu_tree_attention",
-           lib().confu_tree_attention(ctx, C.byref(dims), _ptr(q), _ptr(k_cache), _ptr(v_cache), C.c_int64(n_slots),
-                                      _ptr(seq_start), _ptr(prefix_len), _ptr(k_soft), _ptr(v_soft), _ptr(parent),
-                                      _ptr(con_owner), _ptr(plan), _ptr(out), _ptr(lse), _ptr(status),
-                                      _stream(stream)), ctx)
+    _done("confu_tree_attention",
+          _native().tree_attention(ctx, dims, q, k_cache, v_cache, n_slots, seq_start, prefix_len, k_soft, v_soft, parent,
+                                   con_owner, plan, out, lse, status, stream), ctx)
 
 
 def confu_accept_workspace_bytes(B, T, V):
@@ -171,37 +189,26 @@ def confu_accept_workspace_bytes(B, T, V):
 def confu_tree_accept(ctx, B, T, Cn, V, logit_dtype, target_logits, draft_logits, tokens, parent, con_owner, uniforms,
                       temperature, sibling_mode, accept_len, path, next_token, future_row, counters, workspace,
                       status, stream=None):
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check("confu_tree_accept",
-           lib().confu_tree_accept(ctx, C.c_int32(B), C.c_int32(T), C.c_int32(Cn), C.c_int32(V),
-                                   C.c_int32(dtype_code(logit_dtype)), _ptr(target_logits), _ptr(draft_logits),
-                                   _ptr(tokens), _ptr(parent), _ptr(con_owner), _ptr(uniforms),
-                                   C.c_float(temperature), C.c_int32(sibling_mode), _ptr(accept_len), _ptr(path),
-                                   _ptr(next_token), _ptr(future_row), _ptr(counters), _ptr(workspace),
-                                   C.c_size_t(ws_bytes), _ptr(status), _stream(stream)), ctx)
+    _done("confu_tree_accept",
+          _native().tree_accept(ctx, B, T, Cn, V, _DTYPES[logit_dtype], target_logits, draft_logits, tokens, parent, con_owner,
+                                uniforms, temperature, sibling_mode, accept_len, path, next_token, future_row, counters,
+                                workspace, status, stream), ctx)
 
 
 def confu_tree_accept_match(ctx, B, T, Cn, V, logit_dtype, target_logits, tokens, parent, con_owner, uniforms,
                             temperature, accept_len, path, next_token, future_row, counters, status, stream=None):
     """Acceptance by the sample-and-match rule; reads only the target rows of the walked path."""
-    _check("confu_tree_accept_match",
-           lib().confu_tree_accept_match(ctx, C.c_int32(B), C.c_int32(T), C.c_int32(Cn), C.c_int32(V),
-                                         C.c_int32(dtype_code(logit_dtype)), _ptr(target_logits), _ptr(tokens),
-                                         _ptr(parent), _ptr(con_owner), _ptr(uniforms), C.c_float(temperature),
-                                         _ptr(accept_len), _ptr(path), _ptr(next_token), _ptr(future_row),
-                                         _ptr(counters), _ptr(status), _stream(stream)), ctx)
+    _done("confu_tree_accept_match",
+          _native().tree_accept_match(ctx, B, T, Cn, V, _DTYPES[logit_dtype], target_logits, tokens, parent, con_owner, uniforms,
+                                      temperature, accept_len, path, next_token, future_row, counters, status, stream), ctx)
 
 
 def confu_con_embedding(ctx, hidden, router_w, router_b, experts, k_expert, renormalize, out, sel=None, gate=None,
                         status=None, stream=None):
     """Contemplate-token embedding: router -> softmax -> top-k experts -> weighted sum of their embeddings."""
-    B, H_in = hidden.shape
-    n_expert, H_out = experts.shape
-    _check("confu_con_embedding",
-           lib().confu_con_embedding(ctx, C.c_int32(B), C.c_int32(H_in), C.c_int32(H_out), C.c_int32(n_expert),
-                                     C.c_int32(k_expert), C.c_int32(dtype_code(hidden.dtype)), _ptr(hidden),
-                                     _ptr(router_w), _ptr(router_b), _ptr(experts), C.c_int32(1 if renormalize else 0),
-                                     _ptr(out), _ptr(sel), _ptr(gate), _ptr(status), _stream(stream)), ctx)
+    _done("confu_con_embedding",
+          _native().con_embedding(ctx, _DTYPES[hidden.dtype], hidden, router_w, router_b, experts, k_expert,
+                                  1 if renormalize else 0, out, sel, gate, status, stream), ctx)
 
 
 def confu_tree_accept_static_max_rows():
@@ -225,13 +232,11 @@ def confu_tree_accept_static(B, T, Cn, V, logit_dtype, target_logits, draft_logi
 def confu_kv_compact(ctx, dims, n_layers, k_layer_ptrs, v_layer_ptrs, seq_start, prefix_len, accept_len, path,
                      new_prefix_len, status, stream=None):
     """k_layer_ptrs / v_layer_ptrs: int64 CUDA tensors holding the per-layer pool addresses."""
-    _check("confu_kv_compact",
-           lib().confu_kv_compact(ctx, C.byref(dims), C.c_int32(n_layers), _ptr(k_layer_ptrs), _ptr(v_layer_ptrs),
-                                  _ptr(seq_start), _ptr(prefix_len), _ptr(accept_len), _ptr(path),
-                                  _ptr(new_prefix_len), _ptr(status), _stream(stream)), ctx)
+    _done("confu_kv_compact",
+          _native().kv_compact(ctx, dims, n_layers, k_layer_ptrs, v_layer_ptrs, seq_start, prefix_len, accept_len, path,
+                               new_prefix_len, status, stream), ctx)
 
 
 def confu_kv_append(ctx, dims, k_rows, v_rows, k_cache, v_cache, seq_start, prefix_len, stream=None):
-    _check("confu_kv_append",
-           lib().confu_kv_append(ctx, C.byref(dims), _ptr(k_rows), _ptr(v_rows), _ptr(k_cache), _ptr(v_cache),
-                                 _ptr(seq_start), _ptr(prefix_len), _stream(stream)), ctx)
+    _done("confu_kv_append",
+          _native().kv_append(ctx, dims, k_rows, v_rows, k_cache, v_cache, seq_start, prefix_len, stream), ctx)

@@ -1,7 +1,9 @@
-"""Build libconfu.so (the C-ABI CUDA library) in-tree for sm_100a with nvcc."""
+"""Build libconfu.so (the C-ABI CUDA library) in-tree for sm_100a with nvcc, and the native module its Python calls go
+through (_calls*.so, g++)."""
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -13,6 +15,28 @@ HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "attn_tc.cuh"), 
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
+
+
+CALLS_SRC = os.path.join(CSRC, "python_calls.cpp")
+CALLS = os.path.join(HERE, "_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
+
+
+def build_calls(force: bool = False) -> str:
+    """The native module behind binding.py; links to libconfu.so next to it and to torch's Python library."""
+    header = os.path.join(ROOT, "include", "confu.h")
+    if not force and os.path.exists(CALLS) and os.path.getmtime(CALLS) >= max(os.path.getmtime(p) for p in (CALLS_SRC, header)):
+        return CALLS
+    import torch
+    from torch.utils import cpp_extension
+    nvcc = _nvcc()
+    cuda = os.path.dirname(os.path.dirname(nvcc)) if os.path.isabs(nvcc) else "/usr/local/cuda"
+    inc = cpp_extension.include_paths() + [sysconfig.get_paths()["include"], os.path.join(cuda, "include"), os.path.join(ROOT, "include")]
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-w", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    cmd += [f"-I{d}" for d in inc] + [CALLS_SRC, "-o", CALLS, f"-L{HERE}", "-lconfu", "-Wl,-rpath,$ORIGIN", f"-L{lib}",
+                                      "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    subprocess.run(cmd, check=True)
+    return CALLS
 
 
 def _nvcc():
@@ -27,6 +51,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if not force and os.path.exists(LIB):
         newest = max(os.path.getmtime(p) for p in srcs + HEADERS)
         if os.path.getmtime(LIB) >= newest:
+            build_calls()
             return LIB
     objdir = os.path.join(HERE, "_build")
     os.makedirs(objdir, exist_ok=True)
@@ -45,6 +70,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
             raise RuntimeError("nvcc failed: " + " ".join(cmd))
     link = [_nvcc(), "-shared", "-o", LIB] + objs + ["-gencode", "arch=compute_100a,code=sm_100a", "-cudart", "static"]
     subprocess.run(link, check=True)
+    build_calls(force)
     return LIB
 
 

@@ -4,87 +4,127 @@
 // branch): a tree row sees itself and its ancestors; a contemplate row sees itself, its owner
 // and the owner's ancestors.  Bit j < T of mask[b][r] says "row r sees the slot of tree row j";
 // that a contemplate row sees its own slot (and no other contemplate row's) is implied.
+//
+// One CTA, a chain of short phases: what it costs is latency (global loads that depend on one another, barriers,
+// 64-bit divisions), and every step waits for it.  A warp takes a sequence: parents go through shared memory, so that
+// walking to the root is a few shared loads; the cost line is a warp scan; each CTA's share is found by bisection in
+// shared memory.  B 32: 35 -> 10 us, B 8: 12 -> 7 us; at B 1 the step is 5 us shorter: the attention kernel of the first
+// layer sets itself up meanwhile.
 #include "common.cuh"
 
 namespace confu {
 
-__global__ void __launch_bounds__(256) plan_kernel(confu_dims d, int units, int paired, const int64_t* __restrict__ seq_start,
-                                                   const int32_t* __restrict__ prefix_len,
-                                                   const int32_t* __restrict__ parent,
-                                                   const int32_t* __restrict__ con_owner, void* plan_raw,
-                                                   int32_t* status)
+constexpr int kPlanThreads = 1024, kPlanWarps = kPlanThreads / 32;      // at most; at least kPlanMaxCtas threads
+constexpr int kPlanCached = 1024;                    // sequences whose tile counts and positions fit shared memory
+
+__global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int units, int paired, const int64_t* __restrict__ seq_start,
+                                                            const int32_t* __restrict__ prefix_len,
+                                                            const int32_t* __restrict__ parent,
+                                                            const int32_t* __restrict__ con_owner, void* plan_raw,
+                                                            int32_t* status)
 {
     const int B = d.B, T = d.T, C = d.C, R = d.T + d.C;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    __shared__ int8_t s_par[kPlanWarps][kMaxTree];
+    __shared__ uint64_t s_mask[kPlanWarps][kMaxTree];
+    __shared__ int32_t s_tiles[kPlanCached];
+    __shared__ int64_t s_base[kPlanCached + 1];
+    __shared__ int s_warp[kPlanMaxCtas / 32];
     PlanView pv = plan_view(plan_raw, B);
-    __shared__ int s_bad[2];
-    __shared__ uint64_t s_mask[2][kMaxTree];
-    const int grp = threadIdx.x >> 7, r = threadIdx.x & 127;     // two sequences at a time, one thread per row
+    const bool cached = B <= kPlanCached;
 
-    for (int b0 = 0; b0 < B; b0 += 2) {
-        const int b = b0 + grp;
-        if (r == 0) s_bad[grp] = 0;
-        __syncthreads();
-        if (b < B) {
-            const int32_t* par = parent + (size_t)b * T;
-            int code = 0;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // ---- validation, masks, tile counts: a warp per sequence ----
+    for (int b = warp; b < B; b += (int)(blockDim.x >> 5)) {
+        int p[2], o[2];
+        bool bad_parent = false, bad_owner = false;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = lane + 32 * h;
+            p[h] = r < T ? parent[(size_t)b * T + r] : 0;
+            o[h] = r < C ? con_owner[(size_t)b * C + r] : 0;
+        }
+        const int P = prefix_len[b];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = lane + 32 * h;
             if (r < T) {
-                const int p = par[r];
-                if (r == 0 ? (p != -1) : (p < 0 || p >= r)) code = CONFU_ST_BAD_PARENT;
-            } else if (r < R) {
-                const int o = con_owner[(size_t)b * C + (r - T)];
-                if (o < 0 || o >= T) code = CONFU_ST_BAD_OWNER;
+                bad_parent = bad_parent || (r == 0 ? p[h] != -1 : (p[h] < 0 || p[h] >= r));
+                s_par[warp][r] = (int8_t)p[h];
             }
-            if (code) atomicMax(&s_bad[grp], code == CONFU_ST_BAD_PARENT ? 2 : 1);
+            bad_owner = bad_owner || (r < C && (o[h] < 0 || o[h] >= T));
         }
-        __syncthreads();
-        if (b < B && r < T) {
-            // a tree row sees itself and its ancestors
-            const int32_t* par = parent + (size_t)b * T;
-            uint64_t m = 1ull << r;
-            if (!s_bad[grp]) {
-                int a = par[r];
-                for (int it = 0; it < T && a >= 0; ++it) { m |= 1ull << a; a = par[a]; }
-            }
-            s_mask[grp][r] = m;
-        }
-        __syncthreads();
-        if (b < B) {
-            const int bad = s_bad[grp];
-            uint64_t m = 0;
-            if (r < T) m = s_mask[grp][r];
-            else if (r < R && !bad) m = s_mask[grp][con_owner[(size_t)b * C + (r - T)]];   // owner and its ancestors (+ its own slot, implied)
-            pv.mask[(size_t)b * kMaxRows + r] = m;
-            if (r == 0) {
-                const int code = bad == 2 ? CONFU_ST_BAD_PARENT : (bad == 1 ? CONFU_ST_BAD_OWNER : 0);
-                pv.bad[b] = code;
-                if (code && status) status[b] = code;
-                const int64_t keys = (int64_t)prefix_len[b] + R;
-                pv.tiles[b] = code ? 0 : (int32_t)((keys + kTileKeys - 1) / kTileKeys) + (d.S > 0 ? 1 : 0);
+        bad_parent = __any_sync(0xffffffffu, bad_parent);
+        bad_owner = __any_sync(0xffffffffu, bad_owner);
+        const int code = bad_parent ? CONFU_ST_BAD_PARENT : bad_owner ? CONFU_ST_BAD_OWNER : 0;
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {                // a tree row sees itself and its ancestors
+            const int r = lane + 32 * h;
+            if (r < T) {
+                uint64_t m = 1ull << r;
+                if (!code)
+                    for (int a = s_par[warp][r]; a >= 0; a = s_par[warp][a]) m |= 1ull << a;
+                s_mask[warp][r] = m;
             }
         }
-        __syncthreads();
+        __syncwarp();
+        // tree rows, then contemplate rows (owner and its ancestors; its own slot is implied), then nothing
+        uint64_t* mask = pv.mask + (size_t)b * kMaxRows;
+        for (int r = lane; r < T; r += 32) mask[r] = s_mask[warp][r];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int k = lane + 32 * h;
+            if (k < C) mask[T + k] = code ? 0 : s_mask[warp][o[h]];
+        }
+        for (int r = R + lane; r < kMaxRows; r += 32) mask[r] = 0;
+        if (lane == 0) {
+            pv.bad[b] = code;
+            if (code && status) status[b] = code;
+            const int64_t keys = (int64_t)P + R;
+            const int tiles = code ? 0 : (int32_t)((keys + kTileKeys - 1) / kTileKeys) + (d.S > 0 ? 1 : 0);
+            pv.tiles[b] = tiles;
+            if (cached) s_tiles[b] = tiles;
+        }
+        __syncwarp();
     }
-    __shared__ int s_count[kPlanMaxCtas + 1];
-    if (threadIdx.x == 0) {
+    __syncthreads();
+    // ---- the cost line: one stretch per (sequence, kv head); its groups of query rows are walked side by side ----
+    if (warp == 0) {
         int64_t acc = 0;
-        for (int b = 0; b < B; ++b) {
-            pv.tile_base[b] = acc;
-            // one stretch of the line per (sequence, kv head); its groups of query rows are walked side by side
-            if (pv.tiles[b] > 0) acc += (int64_t)(pv.tiles[b] + kPairOverheadTiles) * d.Hkv;
+        for (int b0 = 0; b0 < B; b0 += 32) {
+            const int b = b0 + lane;
+            const int tiles = b < B ? (cached ? s_tiles[b] : pv.tiles[b]) : 0;
+            const int64_t own = tiles > 0 ? (int64_t)(tiles + kPairOverheadTiles) * d.Hkv : 0;
+            int64_t incl = own;
+#pragma unroll
+            for (int k = 1; k < 32; k <<= 1) {
+                const int64_t t = __shfl_up_sync(0xffffffffu, incl, k);
+                if (lane >= k) incl += t;
+            }
+            if (b < B) {
+                pv.tile_base[b] = acc + incl - own;
+                if (cached) s_base[b] = acc + incl - own;
+            }
+            acc += __shfl_sync(0xffffffffu, incl, 31);
         }
-        pv.tile_base[B] = acc;
-        PlanHeader h;
-        h.B = B; h.Hkv = d.Hkv; h.T = T; h.C = C; h.S = d.S; h.R = R;
-        h.n_tiles = acc;
-        // The line is cut into `lanes` shares; CTA lane * n_rg + rg walks the lane's share for row group rg,
-        // so the CTAs of a lane read the same K/V tiles at about the same time (the second read hits L2).
-        const int n_rg0 = row_groups(R, d.Hq / d.Hkv);
-        int cap = units < kPlanMaxCtas ? units : kPlanMaxCtas;
-        int lanes = cap / n_rg0;
-        if ((int64_t)lanes > acc) lanes = (int)acc;
-        h.n_ctas = lanes * n_rg0;
-        h.paired = paired;
-        *pv.hdr = h;
+        if (lane == 0) {
+            pv.tile_base[B] = acc;
+            if (cached) s_base[B] = acc;
+            PlanHeader h;
+            h.B = B; h.Hkv = d.Hkv; h.T = T; h.C = C; h.S = d.S; h.R = R;
+            h.n_tiles = acc;
+            // The line is cut into `lanes` shares; CTA lane * n_rg + rg walks the lane's share for row group rg,
+            // so the CTAs of a lane read the same K/V tiles at about the same time (the second read hits L2).
+            const int n_rg0 = row_groups(R, d.Hq / d.Hkv);
+            const int cap = units < kPlanMaxCtas ? units : kPlanMaxCtas;
+            int lanes = cap / n_rg0;
+            if ((int64_t)lanes > acc) lanes = (int)acc;
+            h.n_ctas = lanes * n_rg0;
+            h.paired = paired;
+            *pv.hdr = h;
+        }
     }
     __syncthreads();
     // The runs of key tiles of every CTA of the tensor-core attention kernel, worked out once per step
@@ -93,53 +133,74 @@ __global__ void __launch_bounds__(256) plan_kernel(confu_dims d, int units, int 
     const int n_rg = row_groups(R, d.Hq / d.Hkv);
     const int64_t N = pv.hdr->n_tiles;
     const int n_ctas = pv.hdr->n_ctas, n_lanes = n_ctas / n_rg;
+    auto base_of = [&](int b) { return cached ? s_base[b] : pv.tile_base[b]; };
+    const int c = tid;
+    int64_t f0 = 0, f1 = 0;
+    int seq0 = 0;
+    if (c < n_ctas) {
+        f0 = (int64_t)(c / n_rg) * N / n_lanes;
+        f1 = (int64_t)(c / n_rg + 1) * N / n_lanes;
+        for (int hi = B; seq0 + 1 < hi;) {           // the last sequence whose stretch starts at or before f0
+            const int mid = (seq0 + hi) / 2;
+            if (base_of(mid) <= f0) seq0 = mid;
+            else hi = mid;
+        }
+    }
+    int first = 0;
     for (int pass = 0; pass < 2; ++pass) {
-        const int c = threadIdx.x;
+        int n = 0;
         if (c < n_ctas) {
-            const int lane = c / n_rg, rg = c % n_rg;
-            int64_t f = (int64_t)lane * N / n_lanes;
-            const int64_t f1 = (int64_t)(lane + 1) * N / n_lanes;
-            int n = 0;
-            SegDesc* out = pv.segs + (pass ? s_count[c] : 0);
-            int lo = 0;
-            while (f < f1) {
-                while (lo + 1 < B && pv.tile_base[lo + 1] <= f) ++lo;         // the sequence position f falls into
-                const int nt = pv.tiles[lo];
-                const int cost = nt + kPairOverheadTiles;
-                const int64_t local = f - pv.tile_base[lo];
-                const int pos = (int)(local % cost);
+            SegDesc* out = pv.segs + first;
+            int seq = seq0;
+            int64_t base = base_of(seq), next = base_of(seq + 1);
+            for (int64_t f = f0; f < f1;) {
+                while (next <= f) {                  // (f < f1 <= N: ends at the last sequence with tiles at the latest)
+                    base = next;
+                    next = base_of(++seq + 1);
+                }
+                const int nt = cached ? s_tiles[seq] : pv.tiles[seq];
+                const uint32_t cost = (uint32_t)(nt + kPairOverheadTiles), local = (uint32_t)(f - base);
+                const int head = (int)(local / cost), pos = (int)(local - head * cost);
                 const int64_t room = f1 - f;
-                const int take = (int)((int64_t)(cost - pos) <= room ? cost - pos : room);
+                const int take = (int64_t)(cost - pos) <= room ? (int)cost - pos : (int)room;
                 f += take;
                 const int t0 = pos > kPairOverheadTiles ? pos - kPairOverheadTiles : 0;
                 const int t1 = pos + take > kPairOverheadTiles ? pos + take - kPairOverheadTiles : 0;
-                if (t1 <= t0) continue;                    // the share ended inside this pair's overhead zone
+                if (t1 <= t0) continue;              // the share ended inside this pair's overhead zone
                 if (pass) {
-                    SegDesc d;
-                    d.b = lo;
-                    d.g_rg = (int)(local / cost) | (rg << 16);       // the stretches of a sequence are in kv-head order
-                    d.t0 = t0;
-                    d.t1 = t1;
-                    d.nt = nt;
-                    d.P = prefix_len[lo];
-                    d.part_slot = (t0 == 0 && t1 == nt) ? -1 : 2 * c + (t1 < nt ? 1 : 0);
-                    d.pad0 = 0;
-                    d.slot0 = seq_start ? seq_start[lo] : 0;
-                    d.pad1 = 0;
-                    out[n] = d;
+                    SegDesc s;
+                    s.b = seq;
+                    s.g_rg = head | ((c % n_rg) << 16);          // the stretches of a sequence are in kv-head order
+                    s.t0 = t0;
+                    s.t1 = t1;
+                    s.nt = nt;
+                    s.P = prefix_len[seq];
+                    s.part_slot = (t0 == 0 && t1 == nt) ? -1 : 2 * c + (t1 < nt ? 1 : 0);
+                    s.pad0 = 0;
+                    s.slot0 = seq_start ? seq_start[seq] : 0;
+                    s.pad1 = 0;
+                    out[n] = s;
                 }
                 ++n;
             }
-            if (!pass) s_count[c] = n;
         }
-        __syncthreads();
-        if (!pass && threadIdx.x == 0) {
-            int acc = 0;
-            for (int c2 = 0; c2 < n_ctas; ++c2) { const int n = s_count[c2]; s_count[c2] = acc; acc += n; }
-            s_count[n_ctas] = acc;
-            for (int c2 = 0; c2 <= n_ctas; ++c2) pv.seg_begin[c2] = s_count[c2];
+        if (!pass) {                                 // exclusive scan of the counts over the first kPlanMaxCtas threads
+            int incl = n;
+#pragma unroll
+            for (int k = 1; k < 32; k <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, incl, k);
+                if (lane >= k) incl += t;
+            }
+            if (warp < kPlanMaxCtas / 32 && lane == 31) s_warp[warp] = incl;
+            __syncthreads();
+            if (c < kPlanMaxCtas) {
+                int before = 0;
+                for (int w = 0; w < warp; ++w) before += s_warp[w];
+                first = before + incl - n;
+                if (c < n_ctas) pv.seg_begin[c] = first;
+                if (c + 1 == n_ctas || (c == 0 && n_ctas == 0)) pv.seg_begin[n_ctas] = first + n;
+            }
         }
-        __syncthreads();
     }
 }
 
@@ -149,8 +210,10 @@ cudaError_t launch_plan(const Ctx* ctx, const confu_dims& d, const int64_t* seq_
 {
     // work units of the attention launch the plan is for: one CTA per SM, or one CTA pair per two SMs
     const int units = paired ? ctx->sm_count / 2 : ctx->sm_count;
-    plan_kernel<<<1, 256, 0, st>>>(d, units, paired ? 1 : 0, seq_start, prefix_len, parent, con_owner, plan, status);
-    return cudaGetLastError();
+    // a warp per sequence, no more threads than that needs (a CTA of 1024 starts 0.5 us later than one of 256)
+    const int threads = d.B <= 8 ? 256 : d.B <= 16 ? 512 : kPlanThreads;
+    return launch_pdl(plan_kernel, dim3(1), dim3((unsigned)threads), st, d, units, paired ? 1 : 0, seq_start, prefix_len, parent, con_owner,
+                      plan, status);
 }
 
 }  // namespace confu

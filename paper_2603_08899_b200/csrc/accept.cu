@@ -88,6 +88,8 @@ __global__ void __launch_bounds__(256) row_stats_kernel(const T* __restrict__ tl
                                                         int n_rows, int nch, int chunk_elems, float k2,
                                                         RowStat* __restrict__ stats)
 {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int row = blockIdx.x, chunk = blockIdx.y, mat = blockIdx.z;
     const T* base = (mat == 0 ? tl : dl) + (size_t)row * V;
     const bool vec_ok = ((size_t)V * sizeof(T)) % 16 == 0;
@@ -185,9 +187,8 @@ static cudaError_t launch_accept_t(int sm_count, int B, int Tn, int C, int V, co
     const float k2 = (greedy ? 1.f : 1.f / temperature) * kLog2e;
     RowStat* stats = (RowStat*)workspace;
     if (!lazy) {
-        row_stats_kernel<T><<<dim3(n_rows, nch, nmat), 256, 0, st>>>((const T*)tl, (const T*)dl, V, n_rows, nch,
-                                                                     chunk_elems, k2, stats);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_pdl(row_stats_kernel<T>, dim3(n_rows, nch, nmat), dim3(256), st, (const T*)tl, (const T*)dl, V,
+                                         n_rows, nch, chunk_elems, k2, stats);
         if (e != cudaSuccess) return e;
     }
     return launch_walk(sizeof(T) == 4 ? CONFU_F32 : CONFU_BF16, B, Tn, C, V, tl, dl, tokens, parent, con_owner, uniforms, temperature,

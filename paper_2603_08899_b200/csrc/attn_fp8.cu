@@ -2,7 +2,7 @@
 //
 // The structure is that of the bf16 kernel (attn_tc.cu: one persistent CTA per SM, a TMA thread, an
 // MMA thread, one softmax warpgroup per 128-row M tile, a warp that zeroes the ragged tail of a V
-// tile, stream-K split of the ragged batch, partial results merged by combine_kernel).  What differs:
+// tile, stream-K split of the ragged batch, partial results merged by merge_kernel).  What differs:
 //   - K and V tiles are E4M3 bytes: a 128-key tile of one kv head is 16 KB, its 128 head dims are one
 //     128-byte swizzled row, and one MMA covers 32 of them (4 per product instead of 8);
 //   - Q arrives as bf16: at the start of a run each softmax thread turns its row into E4M3 with a
@@ -151,8 +151,7 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
                               const CUtensorMap* k_map, const CUtensorMap* v_map, const CUtensorMap* ks_map,
                               const CUtensorMap* vs_map)
 {
-    Walker w(pv, prm, blockIdx.x);
-    const int n_total = (int)(w.end - w.cur);                 // runs; every run has at least one tile
+    Walker w;
     Segment s;
     uint32_t stage = 0, seg = 0;       // running stage / pair counters
     const int R = prm.d.T + prm.d.C;
@@ -169,7 +168,7 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
         ++stage;
         return true;
     };
-    while (w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x, false, s); run; run = w.next(s)) {
         for (int t = s.t0; t < s.t1; ++t) {
             TileRef cur;
             cur.g = s.g;
@@ -193,7 +192,7 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
         }
         ++seg;
     }
-    if (n_total > 0 && !fill(nullptr)) return;
+    if (have_prev && !fill(nullptr)) return;
 }
 
 // One thread issues all tensor-core work.  Per stage g: P V of key tile g-1 for both M tiles (each
@@ -202,7 +201,7 @@ template <bool kTwo>
 __device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& pv, uint32_t tmem)
 {
     constexpr int kMt = kTwo ? 2 : 1;
-    Walker w(pv, prm, blockIdx.x);
+    Walker w;
     Segment s;
     uint32_t stage = 0, seg = 0;
     // descriptor low words: Q tiles (K-major); a stage's K tile (K-major) and V tile (MN-major, its
@@ -269,7 +268,7 @@ __device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& p
     };
 
     const int R = prm.d.T + prm.d.C;
-    while (w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x, false, s); run; run = w.next(s)) {
         const int n_tiles = s.t1 - s.t0;
         for (int j = 0; j < n_tiles; ++j)
             if (!run_stage(true, j == 0, j + 1 == n_tiles, ragged_rows(s, s.t0 + j, R) > 0)) return;
@@ -284,7 +283,7 @@ __device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& p
 // It arrives on every stage's empty barrier, so a stage is never refilled before it has seen it.
 __device__ void tail_role(SharedStorage& sh, const Params& prm, const PlanView& pv)
 {
-    Walker w(pv, prm, blockIdx.x);
+    Walker w;
     Segment s;
     const int R = prm.d.T + prm.d.C, lane = threadIdx.x & 31;
     uint32_t stage = 0;
@@ -308,7 +307,7 @@ __device__ void tail_role(SharedStorage& sh, const Params& prm, const PlanView& 
         prev_valid = cur_valid;
         return true;
     };
-    while (w.next(s))
+    for (bool run = w.begin(pv, prm, blockIdx.x, false, s); run; run = w.next(s))
         for (int tile = s.t0; tile < s.t1; ++tile)
             if (!run_stage(ragged_rows(s, tile, R))) return;
     if (have_prev) run_stage(0);
@@ -324,10 +323,10 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
     const int G = prm.G, T = prm.d.T, R = prm.d.T + prm.d.C, S = prm.d.S, Hq = prm.d.Hq;
     const int hl = lane_row % G;
 
-    Walker w(pv, prm, blockIdx.x);
+    Walker w;
     Segment s;
     uint32_t n_s = 0, seg = 0;
-    while (w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x, false, s); run; run = w.next(s)) {
         const int r = prm.rpt * (2 * s.rg + t) + lane_row / G;            // query row of this thread in this pair
         const bool row_valid = lane_row < prm.rpt * G && r < R;
         const uint64_t mask = row_valid ? pv.mask[(size_t)s.b * kMaxRows + r] : 0ull;
@@ -505,11 +504,9 @@ attention_fp8_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
     // kernel before this one in the stream drains.  From here on global memory is read and written:
     // every CTA waits until the kernels before this one have completed.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const PlanView pv = plan_view(const_cast<void*>(prm.plan), prm.d.B);
+    const PlanView pv = plan_view(const_cast<void*>(prm.plan), prm.d.B, prm.d.Hkv);
 
-    if ((int)blockIdx.x >= pv.hdr->n_ctas) {
-        // nothing to do: straight to the teardown, which releases tensor memory
-    } else if (warp < 8) {
+    if (warp < 8) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
         const int t = warp >> 2;
         if (t < prm.n_mt) softmax_role(sh, prm, pv, tmem, t);

@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(M / 4 * kGroupThreads<M>, 1) attention_generic
     auto out_at = [&](int i) { const int f = block * M + i; return ((size_t)b * R + f / G) * Hq + g * G + f % G; };
 
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    PlanView pv = plan_view(const_cast<void*>(plan_raw), dm.B);
+    PlanView pv = plan_view(const_cast<void*>(plan_raw), dm.B, dm.Hkv);
     if (pv.bad[b]) {                                 // malformed tree: zero rows (the whole cluster leaves)
         if (rank == 0) {
             for (int i = tid; i < n_rows * (D / 4); i += NT) store4(out + out_at(i / (D / 4)) * D + 4 * (i % (D / 4)), make_float4(0.f, 0.f, 0.f, 0.f));

@@ -15,7 +15,7 @@
 // one empty barrier each, which leaves the issuing thread three waits and three commits per key
 // tile.  Prefix tiles need no mask; the ancestor bitmask (one 64-bit word per row, in a register) is applied only to
 // the tiles that hold the tree slots, the ragged tail and the soft-prompt entries.  A range that
-// does not cover a whole pair writes an unnormalised partial (O, m, l) that combine_kernel merges
+// does not cover a whole pair writes an unnormalised partial (O, m, l) that merge_kernel merges
 // in a fixed order.
 //
 // The last key tile of a sequence reaches past its last slot, into slots that belong to another
@@ -69,8 +69,7 @@ __device__ void producer_role(SharedStorage<D>& sh, const Params& prm, const Pla
                               const CUtensorMap* k_map, const CUtensorMap* v_map, const CUtensorMap* ks_map,
                               const CUtensorMap* vs_map)
 {
-    Walker w(pv, prm, blockIdx.x);
-    const int n_total = (int)(w.end - w.cur);                 // runs; every run has at least one tile
+    Walker w;
     Segment s;
     uint32_t stage = 0, seg = 0;       // running stage / pair counters
     const int R = prm.d.T + prm.d.C;
@@ -95,7 +94,7 @@ __device__ void producer_role(SharedStorage<D>& sh, const Params& prm, const Pla
         ++stage;
         return true;
     };
-    while (w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x, false, s); run; run = w.next(s)) {
         for (int t = s.t0; t < s.t1; ++t) {
             TileRef cur;
             cur.g = s.g;
@@ -119,7 +118,7 @@ __device__ void producer_role(SharedStorage<D>& sh, const Params& prm, const Pla
         }
         ++seg;
     }
-    if (n_total > 0 && !fill(nullptr)) return;
+    if (have_prev && !fill(nullptr)) return;
 }
 
 // One thread issues all tensor-core work.  Per stage g: P V of key tile g-1 for both M tiles (each
@@ -128,7 +127,7 @@ template <int D, bool kTwo>
 __device__ void mma_role(SharedStorage<D>& sh, const Params& prm, const PlanView& pv, uint32_t tmem)
 {
     constexpr int kMt = kTwo ? 2 : 1;
-    Walker w(pv, prm, blockIdx.x);
+    Walker w;
     Segment s;
     uint32_t stage = 0, seg = 0;
     // descriptor low words: Q tiles (K-major); a stage's K tile (K-major) and V tile (MN-major, its
@@ -192,7 +191,7 @@ __device__ void mma_role(SharedStorage<D>& sh, const Params& prm, const PlanView
     };
 
     const int R = prm.d.T + prm.d.C;
-    while (w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x, false, s); run; run = w.next(s)) {
         const int n_tiles = s.t1 - s.t0;
         for (int j = 0; j < n_tiles; ++j)
             if (!run_stage(true, j == 0, j + 1 == n_tiles, ragged_rows(s, s.t0 + j, R) > 0)) return;
@@ -208,7 +207,7 @@ __device__ void mma_role(SharedStorage<D>& sh, const Params& prm, const PlanView
 template <int D>
 __device__ void tail_role(SharedStorage<D>& sh, const Params& prm, const PlanView& pv)
 {
-    Walker w(pv, prm, blockIdx.x);
+    Walker w;
     Segment s;
     const int R = prm.d.T + prm.d.C, lane = threadIdx.x & 31;
     uint32_t stage = 0;
@@ -233,7 +232,7 @@ __device__ void tail_role(SharedStorage<D>& sh, const Params& prm, const PlanVie
         prev_valid = cur_valid;
         return true;
     };
-    while (w.next(s))
+    for (bool run = w.begin(pv, prm, blockIdx.x, false, s); run; run = w.next(s))
         for (int tile = s.t0; tile < s.t1; ++tile)
             if (!run_stage(ragged_rows(s, tile, R))) return;
     if (have_prev) run_stage(0);
@@ -251,10 +250,10 @@ __device__ void softmax_role(SharedStorage<D>& sh, const Params& prm, const Plan
     const int hl = lane_row % G;
     const float c = prm.c;
 
-    Walker w(pv, prm, blockIdx.x);
+    Walker w;
     Segment s;
     uint32_t n_s = 0, seg = 0;
-    while (w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x, false, s); run; run = w.next(s)) {
         const int r = prm.rpt * (2 * s.rg + t) + lane_row / G;            // query row of this thread in this pair
         const bool row_valid = lane_row < prm.rpt * G && r < R;
         const uint64_t mask = row_valid ? pv.mask[(size_t)s.b * kMaxRows + r] : 0ull;
@@ -421,11 +420,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
     // kernel before this one in the stream drains.  From here on global memory is read and written:
     // every CTA waits until the kernels before this one have completed.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const PlanView pv = plan_view(const_cast<void*>(prm.plan), prm.d.B);
+    const PlanView pv = plan_view(const_cast<void*>(prm.plan), prm.d.B, prm.d.Hkv);
 
-    if ((int)blockIdx.x >= pv.hdr->n_ctas) {
-        // nothing to do: straight to the teardown, which releases tensor memory
-    } else if (warp < 8) {
+    if (warp < 8) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
         const int t = warp >> 2;
         if (t < prm.n_mt) softmax_role(sh, prm, pv, tmem, t);

@@ -46,7 +46,7 @@ inline void set_rows(Params& p, const confu_dims& d)
 
 // Enqueues the merge of the partial results that the attention launch with the same parameters
 // left in prm.partials (pairs whose key tiles were split over several CTAs).
-cudaError_t launch_combine(const Params& prm, int sm_count, cudaStream_t st);
+cudaError_t launch_combine(const Params& prm, int units, cudaStream_t st);
 
 }  // namespace tc
 }  // namespace confu

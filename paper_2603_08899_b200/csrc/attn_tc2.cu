@@ -175,8 +175,7 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
                               const CUtensorMap* q_map, const CUtensorMap* k_map, const CUtensorMap* v_map,
                               const CUtensorMap* ks_map, const CUtensorMap* vs_map)
 {
-    Walker w(pv, prm, blockIdx.x >> 1);
-    const int n_total = (int)(w.end - w.cur);
+    Walker w;
     Segment s;
     uint32_t g = 0, seg = 0;
     const int R = prm.d.T + prm.d.C;
@@ -205,7 +204,7 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
         ++g;
         return true;
     };
-    while (w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x >> 1, true, s); run; run = w.next(s)) {
         for (int t = s.t0; t < s.t1; ++t) {
             TileRef cur;
             cur.present = true;
@@ -228,7 +227,7 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
     }
     // kVLag more stages: they carry the V tiles of the last key tiles (a stage may be empty when the
     // whole walk is shorter than kVLag tiles)
-    for (int i = 0; i < (n_total > 0 ? kVLag : 0); ++i)
+    for (int i = 0; i < (g > 0 ? kVLag : 0); ++i)
         if (!fill(nullptr)) return;
 }
 
@@ -236,7 +235,7 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
 // last V tile that lie past its last slot, and reports to the issuing thread in CTA 0.
 __device__ void relay_role(SharedStorage& sh, const Params& prm, const PlanView& pv)
 {
-    Walker w(pv, prm, blockIdx.x >> 1);
+    Walker w;
     Segment s;
     const int R = prm.d.T + prm.d.C, lane = threadIdx.x & 31;
     uint32_t g = 0, seg = 0;
@@ -265,7 +264,7 @@ __device__ void relay_role(SharedStorage& sh, const Params& prm, const PlanView&
         ++g;
         return true;
     };
-    while (w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x >> 1, true, s); run; run = w.next(s)) {
         for (int tile = s.t0; tile < s.t1; ++tile) {
             if (!run_stage(true, ragged_rows(s, tile, R))) return;
             if (tile == s.t0) {
@@ -290,14 +289,14 @@ __device__ void relay_role(SharedStorage& sh, const Params& prm, const PlanView&
 // A stage [K of tile h | V of tile h - kVLag] is free again when both threads' instructions on it have completed.
 __device__ void qk_role(SharedStorage& sh, const Params& prm, const PlanView& pv, uint32_t tmem)
 {
-    Walker w(pv, prm, blockIdx.x >> 1);
+    Walker w;
     Segment s;
     uint32_t g = 0, seg = 0;
     uint32_t q_lo[kQBufs];
     for (int i = 0; i < kQBufs; ++i) q_lo[i] = desc_lo(smem_u32(sh.q[i]), 16);
     const uint32_t k_lo0 = desc_lo(smem_u32(sh.kv[0]), 16);
     constexpr uint32_t kStageStep = kStageBytes >> 4;
-    while (w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x >> 1, true, s); run; run = w.next(s)) {
         const int n_tiles = s.t1 - s.t0;
         for (int j = 0; j < n_tiles; ++j, ++g) {
             const uint32_t st = g % kStages;
@@ -329,14 +328,16 @@ __device__ void qk_role(SharedStorage& sh, const Params& prm, const PlanView& pv
 
 __device__ void pv_role(SharedStorage& sh, const Params& prm, const PlanView& pv, uint32_t tmem)
 {
-    Walker w(pv, prm, blockIdx.x >> 1);
+    Walker w;
     Segment s;
     uint32_t g = 0;
     const uint32_t v_lo0 = desc_lo(smem_u32(sh.kv[0] + kKBytes), 16);
     constexpr uint32_t kStageStep = kStageBytes >> 4;
     // the first kVLag stages carry no V tile: this thread has nothing to wait for on them
-    for (int i = 0; i < kVLag; ++i) commit_both(&sh.kv_empty[i]);
-    while (w.next(s)) {
+    bool run = w.begin(pv, prm, blockIdx.x >> 1, true, s);
+    if (run)
+        for (int i = 0; i < kVLag; ++i) commit_both(&sh.kv_empty[i]);
+    for (; run; run = w.next(s)) {
         const int n_tiles = s.t1 - s.t0;
         for (int j = 0; j < n_tiles; ++j, ++g) {
             const uint32_t st = (g + kVLag) % kStages, pb = g & 1;      // V of tile g travels with K of tile g + kVLag
@@ -372,10 +373,10 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
     const uint32_t s_addr = tmem + lane_base + kColS + buf * 128, p_addr = tmem + lane_base + kColP + buf * 64;
     const uint32_t ref_mine = smem_u32(&sh.xref[set][lane_row]), ref_theirs = smem_u32(&sh.xref[set ^ 1][lane_row]);
 
-    Walker w(pv, prm, blockIdx.x >> 1);
+    Walker w;
     Segment s;
     uint32_t g = 0, seg = 0;
-    while (w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x >> 1, true, s); run; run = w.next(s)) {
         const int r = prm.rpt * (2 * s.rg + (int)rank) + lane_row / G;      // query row of this thread in this run
         const bool row_valid = lane_row < prm.rpt * G && r < R;
         const uint64_t mask = row_valid ? pv.mask[(size_t)s.b * kMaxRows + r] : 0ull;
@@ -588,16 +589,12 @@ attention_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
     // kernel before this one in the stream drains.  From here on global memory is read and written:
     // every CTA waits until the kernels before this one have completed.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const PlanView pv = plan_view(const_cast<void*>(prm.plan), prm.d.B);
-    // (both CTAs of a pair take the same way through the next two tests)
-    const bool listed = (int)(blockIdx.x >> 1) < pv.hdr->n_ctas;
-    const bool pair_plan = pv.hdr->paired == 1;             // the plan lists runs per CTA pair, not per CTA
-    if (!pair_plan && blockIdx.x == 0 && prm.status)
-        for (int b = threadIdx.x; b < prm.d.B; b += kThreads) prm.status[b] = CONFU_ST_BAD_PLAN;
+    const PlanView pv = plan_view(const_cast<void*>(prm.plan), prm.d.B, prm.d.Hkv);
+    // a plan that lists runs per CTA, not per CTA pair, is refused: no role finds anything to do
+    if (warp == 11 && blockIdx.x == 0 && prm.status && pv.hdr->paired == 0)
+        for (int b = threadIdx.x & 31; b < prm.d.B; b += 32) prm.status[b] = CONFU_ST_BAD_PLAN;
 
-    if (!listed || !pair_plan) {
-        // nothing to do: straight to the teardown, which releases tensor memory
-    } else if (warp < 8) {
+    if (warp < 8) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
         softmax_role(sh, prm, pv, tmem, rank);
     } else if (warp == 8) {

@@ -36,7 +36,9 @@ __host__ __device__ inline int row_groups(int R, int G)
 //   int32  bad[B]             non-zero: malformed tree, sequence skipped
 //   int32  tiles[B]           key tiles of one (sequence, kv head) pair, soft-prompt tile included
 //   int64  tile_base[B + 1]   position of sequence b's first (sequence, kv head) stretch on the flat cost line (exclusive scan)
-//   int32  seg_begin[kPlanMaxCtas + 1]   CTA c of the tensor-core kernel walks segs[seg_begin[c] .. seg_begin[c+1])
+//   CtaPlan cta[kPlanMaxCtas]   work unit c of the tensor-core kernel: its first run of key tiles, how many it has and where
+//                             the others are (one 64-byte read tells a CTA what to start with)
+//   int32  parts[B * Hkv]     who walked a (sequence, kv head): first share | number of shares << 16 (0: malformed tree)
 //   SegDesc segs[B * Hkv * max(2, n_rg) + kPlanMaxCtas]   the runs of key tiles, one pair at a time, of every CTA in walking order
 //
 // The split-KV work is balanced on a "cost line": every (sequence, kv head) pair takes
@@ -69,13 +71,23 @@ struct alignas(16) SegDesc {
 };
 static_assert(sizeof(SegDesc) == 48, "SegDesc is read as three 16-byte words");
 
+struct alignas(64) CtaPlan {
+    SegDesc first;
+    int32_t n_runs;            // 0: nothing to do
+    int32_t begin;             // its runs are segs[begin .. begin + n_runs)
+    int32_t paired;            // as in the header
+    int32_t pad;
+};
+static_assert(sizeof(CtaPlan) == 64, "CtaPlan is read as four 16-byte words");
+
 struct PlanView {
     PlanHeader* hdr;
     uint64_t* mask;
     int32_t* bad;
     int32_t* tiles;
     int64_t* tile_base;
-    int32_t* seg_begin;
+    CtaPlan* cta;
+    int32_t* parts;
     SegDesc* segs;
 };
 
@@ -88,12 +100,13 @@ __host__ __device__ inline size_t plan_bytes(int B, int Hkv, int n_rg)
     n += align_up((size_t)B * sizeof(int32_t), 256);
     n += align_up((size_t)B * sizeof(int32_t), 256);
     n += align_up((size_t)(B + 1) * sizeof(int64_t), 256);
-    n += align_up((size_t)(kPlanMaxCtas + 1) * sizeof(int32_t), 256);
+    n += align_up((size_t)kPlanMaxCtas * sizeof(CtaPlan), 256);
+    n += align_up((size_t)B * Hkv * sizeof(int32_t), 256);
     n += align_up(((size_t)B * Hkv * (n_rg > 2 ? n_rg : 2) + kPlanMaxCtas) * sizeof(SegDesc), 256);
     return n;
 }
 
-__host__ __device__ inline PlanView plan_view(void* base, int B)
+__host__ __device__ inline PlanView plan_view(void* base, int B, int Hkv)
 {
     char* p = (char*)base;
     PlanView v;
@@ -102,7 +115,8 @@ __host__ __device__ inline PlanView plan_view(void* base, int B)
     v.bad = (int32_t*)p;                     p += align_up((size_t)B * sizeof(int32_t), 256);
     v.tiles = (int32_t*)p;                   p += align_up((size_t)B * sizeof(int32_t), 256);
     v.tile_base = (int64_t*)p;               p += align_up((size_t)(B + 1) * sizeof(int64_t), 256);
-    v.seg_begin = (int32_t*)p;               p += align_up((size_t)(kPlanMaxCtas + 1) * sizeof(int32_t), 256);
+    v.cta = (CtaPlan*)p;                     p += align_up((size_t)kPlanMaxCtas * sizeof(CtaPlan), 256);
+    v.parts = (int32_t*)p;                   p += align_up((size_t)B * Hkv * sizeof(int32_t), 256);
     v.segs = (SegDesc*)p;
     return v;
 }

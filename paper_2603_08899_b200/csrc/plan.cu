@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
     __shared__ int32_t s_tiles[kPlanCached];
     __shared__ int64_t s_base[kPlanCached + 1];
     __shared__ int s_warp[kPlanMaxCtas / 32];
-    PlanView pv = plan_view(plan_raw, B);
+    PlanView pv = plan_view(plan_raw, B, d.Hkv);
     const bool cached = B <= kPlanCached;
 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -146,6 +146,18 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
             else hi = mid;
         }
     }
+    // Key tile q of (sequence, kv head) sits at position F + q of the line; position x belongs to share
+    // floor(((x + 1) * n - 1) / N) of n.
+    for (int u = tid; u < B * d.Hkv; u += (int)blockDim.x) {
+        const int b = u / d.Hkv, nt = cached ? s_tiles[b] : pv.tiles[b];
+        int32_t parts = 0;
+        if (nt > 0) {
+            const int64_t F = base_of(b) + (int64_t)(u % d.Hkv) * (nt + kPairOverheadTiles) + kPairOverheadTiles;
+            const int lo = (int)(((F + 1) * n_lanes - 1) / N), hi = (int)(((F + nt) * n_lanes - 1) / N);
+            parts = lo | ((hi - lo + 1) << 16);
+        }
+        pv.parts[u] = parts;
+    }
     int first = 0;
     for (int pass = 0; pass < 2; ++pass) {
         int n = 0;
@@ -180,6 +192,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
                     s.slot0 = seq_start ? seq_start[seq] : 0;
                     s.pad1 = 0;
                     out[n] = s;
+                    if (n == 0) pv.cta[c].first = s;
                 }
                 ++n;
             }
@@ -197,8 +210,9 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
                 int before = 0;
                 for (int w = 0; w < warp; ++w) before += s_warp[w];
                 first = before + incl - n;
-                if (c < n_ctas) pv.seg_begin[c] = first;
-                if (c + 1 == n_ctas || (c == 0 && n_ctas == 0)) pv.seg_begin[n_ctas] = first + n;
+                pv.cta[c].n_runs = n;                // (0 past the last unit)
+                pv.cta[c].begin = first;
+                pv.cta[c].paired = paired;
             }
         }
     }

@@ -19,22 +19,35 @@ struct Segment {
     int part_slot;     // -1: the range covers the whole pair, write the output directly
 };
 
-// A CTA's runs of key tiles come from the plan: one 48-byte descriptor each, in walking order.
+// The runs of key tiles of a work unit (CTA or CTA pair), in walking order: the first from the unit's own record in
+// the plan (one read tells a role what to start with), the others from 48-byte descriptors.
 struct Walker {
     const SegDesc* cur;
-    const SegDesc* end;
+    int left;
     bool soft;
-    __device__ Walker(const PlanView& v, const Params& p, int cta) : soft(p.d.S > 0)
+    // The unit's first run; false when it has nothing to do, or when the plan is for the other kind of unit.
+    __device__ bool begin(const PlanView& v, const Params& p, int unit, bool paired, Segment& s)
     {
-        cur = v.segs + v.seg_begin[cta];
-        end = v.segs + v.seg_begin[cta + 1];
+        const uint4* q = reinterpret_cast<const uint4*>(v.cta + unit);
+        const uint4 w0 = __ldg(q), w1 = __ldg(q + 1), w2 = __ldg(q + 2), w3 = __ldg(q + 3);
+        soft = p.d.S > 0;
+        cur = v.segs + (int)w3.y;
+        left = paired && w3.z == 0 ? 0 : (int)w3.x;
+        take(s, w0, w1, w2);
+        return left > 0;
     }
-    // Next run of key tiles of one pair inside the share; false when the share is used up.
+    // The next run; false when the share is used up.
     __device__ bool next(Segment& s)
     {
-        if (cur >= end) return false;
-        const uint4* q = reinterpret_cast<const uint4*>(cur);
-        const uint4 w0 = __ldg(q), w1 = __ldg(q + 1), w2 = __ldg(q + 2);
+        if (--left <= 0) return false;
+        const uint4* q = reinterpret_cast<const uint4*>(++cur);
+        take(s, __ldg(q), __ldg(q + 1), __ldg(q + 2));
+        return true;
+    }
+
+private:
+    __device__ void take(Segment& s, const uint4& w0, const uint4& w1, const uint4& w2) const
+    {
         s.b = (int)w0.x;
         s.g = (int)(w0.y & 0xffffu);
         s.rg = (int)(w0.y >> 16);
@@ -45,8 +58,6 @@ struct Walker {
         s.P = (int)w1.y;
         s.part_slot = (int)w1.z;
         s.slot0 = (int64_t)(((uint64_t)w2.y << 32) | w2.x);
-        ++cur;
-        return true;
     }
 };
 

@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
     __shared__ uint64_t s_mask[kPlanWarps][kMaxTree];
     __shared__ int32_t s_tiles[kPlanCached];
     __shared__ int64_t s_base[kPlanCached + 1];
-    __shared__ int s_warp[kPlanMaxCtas / 32];
+    __shared__ int s_warp[kPlanMaxCtas / 32], s_own;
     PlanView pv = plan_view(plan_raw, B, d.Hkv);
     const bool cached = B <= kPlanCached;
 
@@ -109,18 +109,51 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
             }
             acc += __shfl_sync(0xffffffffu, incl, 31);
         }
+        // The line is cut into `lanes` shares; CTA lane * n_rg + rg walks the lane's share for row group rg,
+        // so the CTAs of a lane read the same K/V tiles at about the same time (the second read hits L2).
+        const int n_rg0 = row_groups(R, d.Hq / d.Hkv);
+        const int cap = units < kPlanMaxCtas ? units : kPlanMaxCtas;
+        int lanes = cap / n_rg0;
+        // With few enough stretches every one can have shares of its own, of at most `own` tiles: where that is no
+        // longer than a share of the line, no work unit changes from one pair to the next.  (A layer at batch 1, prefix 4096:
+        // 34 tiles in 9 shares of at most 4 instead of a line cut into shares of 4.1, some of which span two pairs: 17.5 ->
+        // 16.9 us; prefix 512: 12.75 -> 12.2; 4 sequences of 500..4000: 23.9 -> 22.9; E4M3 cache, batch 1: 20.0 -> 18.3.)
+        int own = 0;
+        if (cached && acc > 0 && (int64_t)B * d.Hkv <= lanes) {
+            const int longest = (int)((acc + lanes - 1) / lanes);
+            for (own = 1; own <= longest; ++own) {
+                int shares = 0;
+                for (int b = lane; b < B; b += 32) shares += (s_tiles[b] + own - 1) / own;
+#pragma unroll
+                for (int k = 16; k > 0; k >>= 1) shares += __shfl_xor_sync(0xffffffffu, shares, k);
+                if (shares * d.Hkv <= lanes) break;
+            }
+            if (own > longest) own = 0;
+        }
+        if (own) {                                   // positions are share numbers now
+            acc = 0;
+            for (int b0 = 0; b0 < B; b0 += 32) {
+                const int b = b0 + lane;
+                const int mine = b < B ? (s_tiles[b] + own - 1) / own * d.Hkv : 0;
+                int incl = mine;
+#pragma unroll
+                for (int k = 1; k < 32; k <<= 1) {
+                    const int t = __shfl_up_sync(0xffffffffu, incl, k);
+                    if (lane >= k) incl += t;
+                }
+                if (b < B) s_base[b] = acc + incl - mine;
+                acc += __shfl_sync(0xffffffffu, incl, 31);
+            }
+            __syncwarp();
+        }
+        if ((int64_t)lanes > acc) lanes = (int)acc;
         if (lane == 0) {
+            s_own = own;
             pv.tile_base[B] = acc;
             if (cached) s_base[B] = acc;
             PlanHeader h;
             h.B = B; h.Hkv = d.Hkv; h.T = T; h.C = C; h.S = d.S; h.R = R;
             h.n_tiles = acc;
-            // The line is cut into `lanes` shares; CTA lane * n_rg + rg walks the lane's share for row group rg,
-            // so the CTAs of a lane read the same K/V tiles at about the same time (the second read hits L2).
-            const int n_rg0 = row_groups(R, d.Hq / d.Hkv);
-            const int cap = units < kPlanMaxCtas ? units : kPlanMaxCtas;
-            int lanes = cap / n_rg0;
-            if ((int64_t)lanes > acc) lanes = (int)acc;
             h.n_ctas = lanes * n_rg0;
             h.paired = paired;
             *pv.hdr = h;
@@ -145,6 +178,33 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
             if (base_of(mid) <= f0) seq0 = mid;
             else hi = mid;
         }
+    }
+    if (s_own) {                                     // shares of their own: one run each, a stretch's tiles dealt out evenly
+        for (int u = tid; u < B * d.Hkv; u += (int)blockDim.x) {
+            const int b = u / d.Hkv, k = (s_tiles[b] + s_own - 1) / s_own;
+            pv.parts[u] = k ? ((int)s_base[b] + u % d.Hkv * k) | (k << 16) : 0;
+        }
+        if (c < n_ctas) {
+            const int nt = s_tiles[seq0], k = (nt + s_own - 1) / s_own, local = c / n_rg - (int)s_base[seq0], p = local % k;
+            SegDesc s;
+            s.b = seq0;
+            s.g_rg = (local / k) | ((c % n_rg) << 16);
+            s.t0 = p * nt / k;
+            s.t1 = (p + 1) * nt / k;
+            s.nt = nt;
+            s.P = prefix_len[seq0];
+            s.part_slot = k == 1 ? -1 : 2 * c + (p + 1 < k ? 1 : 0);
+            s.pad0 = 0;
+            s.slot0 = seq_start ? seq_start[seq0] : 0;
+            s.pad1 = 0;
+            pv.cta[c].first = s;
+        }
+        if (c < kPlanMaxCtas) {
+            pv.cta[c].n_runs = c < n_ctas ? 1 : 0;
+            pv.cta[c].begin = 0;
+            pv.cta[c].paired = paired;
+        }
+        return;
     }
     // Key tile q of (sequence, kv head) sits at position F + q of the line; position x belongs to share
     // floor(((x + 1) * n - 1) / N) of n.

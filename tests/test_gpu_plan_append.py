@@ -52,3 +52,25 @@ def test_append_writes_the_rows_and_nothing_else(gpu, R, Hkv, D, dtype):
             lo = int(start[b]) + int(plen[b])
             p[lo:lo + R] = r[b]
         assert torch.equal(d.cpu(), p)
+
+
+@pytest.mark.parametrize("B,Hkv,G,prefix,R", [(1, 8, 4, 4096, (60, 4)), (1, 1, 4, 20000, (20, 20)), (2, 8, 3, (1, 900), (40, 30)), (9, 8, 4, (100, 300), (20, 20)), (7, 4, 8, (0, 1500), (30, 4))])
+def test_shares_of_their_own(gpu, B, Hkv, G, prefix, R):
+    """Few (sequence, kv head) pairs for the machine: each gets a number of equal shares; an uneven one per pair, one tile per
+    share, and batches that just fit or just do not."""
+    cfg = inputs.VerifyConfig("own", B=B, L=1, Hq=G * Hkv, Hkv=Hkv, D=128, T=R[0], C=R[1], S=3, V=32, prefix=prefix, tree="random",
+                              kv_dtype=torch.bfloat16, logit_dtype=torch.float32, sigma_logit=1.0, draft="independent",
+                              temperatures=(1.0,), seed=560 + B, max_depth=7, fanout=(1, 4))
+    parent, owner, plen, seq_start, n_slots, t = H.setup_case(cfg)
+    if B > 1:
+        parent[1, 1] = 7
+    want, want_lse, want_st = H.oracle_attention(cfg, t, seq_start, plen, parent, owner)
+    for path in (cb.ATTENTION_TENSOR, cb.ATTENTION_TENSOR_PAIR):
+        gpu.set_path(path)
+        try:
+            out, lse, st = H.gpu_attention(gpu, cfg, t, seq_start, plen, parent, owner, n_slots, use_plan=True)
+        finally:
+            gpu.set_path(cb.ATTENTION_AUTO)
+        assert st.tolist() == want_st.tolist()
+        ok = [b for b in range(B) if want_st[b] == 0]
+        H.assert_attention_close(out[ok], lse[ok], want[ok], want_lse[ok], cfg.kv_dtype, "own shares")

@@ -461,8 +461,6 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
             if (lane == 0) mbar_arrive_remote(p_full_leader);
         }
         // ---- end of the run: this thread's 64 head dims of the row of O ----
-        if (!wait_warp(sh, &sh.o_done, seg & 1, prm.wait_ns)) return;
-        tc_fence_after();
         // the row's sum of weights: the shares of the two threads of the row, each brought to the larger
         // (= the final) reference maximum (bounded wait, like every other)
         sh.xsum[set][lane_row] = l;
@@ -494,6 +492,9 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
             p_ptr = prm.partials + (size_t)s.part_slot * (partial_slot_bytes() / sizeof(float)) +
                     (size_t)(rank * 128 + wq * 32 + (lane >> 3)) * kPartD + 4 * (lane & 7);
         }
+        // (everything above goes on while the last P V does)
+        if (!wait_warp(sh, &sh.o_done, seg & 1, prm.wait_ns)) return;
+        tc_fence_after();
 #pragma unroll 1
         for (int q4 = 2 * half; q4 < 2 * half + 2; ++q4) {
             uint32_t ov[32];

@@ -178,8 +178,9 @@ __global__ void __launch_bounds__(kMergeThreads, 4) merge_kernel(const Params pr
         return;
     }
     if (row0 >= rows || query_row(prm, u, t, row0) >= prm.d.T + prm.d.C) return;
-    if (u.n == 2)
-        for (int i = row0; i < end; i += 4) merge_rows<D, 2, 4>(prm, u, t, i, end, lane);
+    if (u.n <= 4 && per_warp == 1) merge_rows<D, 4, 1>(prm, u, t, row0, end, lane);
+    else if (u.n == 2 && per_warp == 4) merge_rows<D, 2, 4>(prm, u, t, row0, end, lane);
+    else if (u.n == 2) merge_rows<D, 2, 2>(prm, u, t, row0, end, lane);
     else if (u.n <= 4)
         for (int i = row0; i < end; i += 2) merge_rows<D, 4, 2>(prm, u, t, i, end, lane);
     else
@@ -190,9 +191,11 @@ __global__ void __launch_bounds__(kMergeThreads, 4) merge_kernel(const Params pr
 
 cudaError_t launch_combine(const Params& prm, int units, cudaStream_t st)
 {
-    // few pairs, each spread over many units: a row per warp, to have every row in flight; many pairs: four rows per
-    // warp, a quarter of the blocks
-    const int n_pairs = prm.d.B * prm.d.Hkv * prm.n_rg, per_warp = units >= n_pairs * prm.n_mt ? 1 : 4;
+    // Rows per warp: one where that leaves every warp's rows in flight together, more where there are many pairs (a
+    // quarter of the blocks, two to four parts each).  B 8, prefixes 101..3001, per layer: 2 rows 27.2 us, 4 rows 27.9; B 4,
+    // 500..4000: 1 row 20.7 us, and 22.7 with the loads of rows that the warp does not have repeated instead of left out.
+    const int n_pairs = prm.d.B * prm.d.Hkv * prm.n_rg, tiles = n_pairs * prm.n_mt;
+    const int per_warp = tiles <= units ? 1 : tiles <= 2 * units ? 2 : 4;
     const dim3 grid((unsigned)n_pairs, (unsigned)prm.n_mt, (unsigned)(128 / (kMergeWarps * per_warp)));
     return prm.d.D == 64 ? launch_pdl(merge_kernel<64>, grid, dim3(kMergeThreads), st, prm, per_warp)
                          : launch_pdl(merge_kernel<kD>, grid, dim3(kMergeThreads), st, prm, per_warp);

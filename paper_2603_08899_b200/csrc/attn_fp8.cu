@@ -195,7 +195,9 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
     if (have_prev && !fill(nullptr)) return;
 }
 
-// One thread issues all tensor-core work.  Per stage g: P V of key tile g-1 for both M tiles (each
+// One warp drives the tensor pipe, one lane of it issues.  (The warp stays together, so that what an instruction's
+// descriptors are made of can live in uniform registers: with a lone thread the same loop took 12 % longer,
+// and the kernel 2-3 % at 32 sequences.)  Per stage g: P V of key tile g-1 for both M tiles (each
 // as soon as its P is there), Q K^T of key tile g for both, then the stage is released.
 template <bool kTwo>
 __device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& pv, uint32_t tmem)
@@ -204,6 +206,7 @@ __device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& p
     Walker w;
     Segment s;
     uint32_t stage = 0, seg = 0;
+    const bool issuer = elect_lane();
     // descriptor low words: Q tiles (K-major); a stage's K tile (K-major) and V tile (MN-major, its
     // two 64-column halves kHalfTile apart) = stage 0's words + stage * stage size
     const uint32_t q_lo = desc_lo(smem_u32(sh.q8[0]), 16);
@@ -212,6 +215,7 @@ __device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& p
 
     // S_t = Q_t K^T: 4 steps of 32 head dims; step i sits at byte 32 i of the swizzled 128-byte row
     auto issue_qk = [&](int t, uint32_t kl) {
+        if (!issuer) return;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const uint32_t off = ((uint32_t)i * 32u) >> 4;
@@ -222,6 +226,7 @@ __device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& p
     // O_t += P_t V: 4 steps of 32 keys (4096 B of the V tile and 8 TMEM columns of four E4M3 weights each);
     // P sits in the first 32 columns of the S_t block
     auto issue_pv = [&](int t, uint32_t vl, bool first_of_segment) {
+        if (!issuer) return;
 #pragma unroll
         for (int i = 0; i < 4; ++i)
             mma8_ts(tmem + 256 + t * 128, tmem + t * 128 + i * 8, vl + i * (4096u >> 4), kIdescPV8,
@@ -248,7 +253,7 @@ __device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& p
                 if (!mbar_wait(&sh.p_full[t], (stage - 1) & 1, &sh.abort, prm.wait_ns)) return false;
                 tc_fence_after();
                 issue_pv(t, vl, prev_first);
-                if (prev_last) tc_commit(&sh.o_done[t]);
+                if (prev_last && issuer) tc_commit(&sh.o_done[t]);
             }
             if (have_cur) {
                 // at the start of a run: the E4M3 rows of this M tile's Q have been written
@@ -257,8 +262,8 @@ __device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& p
                 issue_qk(t, kl);
             }
         }
-        tc_commit(&sh.kv_empty[st]);
-        if (have_cur && cur_last) tc_commit(&sh.q_empty);               // last Q K^T of the pair has been issued
+        if (issuer) tc_commit(&sh.kv_empty[st]);
+        if (have_cur && cur_last && issuer) tc_commit(&sh.q_empty);               // last Q K^T of the pair has been issued
         ++stage;
         have_prev = have_cur;
         prev_first = cur_first;
@@ -515,10 +520,8 @@ attention_fp8_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
         if (warp == 8) {
             if ((threadIdx.x & 31) == 0) producer_role(sh, prm, pv, &q_map, &k_map, &v_map, &ks_map, &vs_map);
         } else if (warp == 9) {
-            if ((threadIdx.x & 31) == 0) {
-                if (prm.n_mt > 1) mma_role<true>(sh, prm, pv, tmem);
-                else mma_role<false>(sh, prm, pv, tmem);
-            }
+            if (prm.n_mt > 1) mma_role<true>(sh, prm, pv, tmem);
+            else mma_role<false>(sh, prm, pv, tmem);
         } else if (warp == 10) {
             tail_role(sh, prm, pv);
         }

@@ -280,7 +280,8 @@ __device__ void relay_role(SharedStorage& sh, const Params& prm, const PlanView&
         if (!run_stage(false, 0)) return;
 }
 
-// Two threads of CTA 0 issue the tensor-core work of the pair, each waiting only for what its own
+// Two warps of CTA 0 drive the tensor pipe of the pair (one lane of each issues; the warp stays together, so that the
+// descriptors can live in uniform registers: about 1 % of a layer), each waiting only for what its own
 // instructions need (the pipe takes instructions from both without loss), so that neither product
 // waits behind a wake-up that belongs to the other:
 //   qk_role   S[g & 1] = Q K^T of key tile g as soon as K has landed in both CTAs and the softmax
@@ -290,6 +291,7 @@ __device__ void relay_role(SharedStorage& sh, const Params& prm, const PlanView&
 __device__ void qk_role(SharedStorage& sh, const Params& prm, const PlanView& pv, uint32_t tmem)
 {
     Walker w;
+    const bool issuer = elect_lane();
     Segment s;
     uint32_t g = 0, seg = 0;
     uint32_t q_lo[kQBufs];
@@ -310,11 +312,11 @@ __device__ void qk_role(SharedStorage& sh, const Params& prm, const PlanView& pv
             for (int i = 0; i < 8; ++i) {
                 const uint32_t q_off = ((uint32_t)(i >> 2) * kHalfTile + (uint32_t)(i & 3) * 32u) >> 4;
                 const uint32_t k_off = ((uint32_t)(i >> 2) * kKHalf + (uint32_t)(i & 3) * 32u) >> 4;
-                mma2_ss(tmem + kColS + (g & 1) * 128, ql + q_off, kl + k_off, kIdescQK2, i > 0 ? 1u : 0u);
+                if (issuer) mma2_ss(tmem + kColS + (g & 1) * 128, ql + q_off, kl + k_off, kIdescQK2, i > 0 ? 1u : 0u);
             }
-            commit_both(&sh.s_full[g & 1]);
-            commit_both(&sh.kv_empty[st]);
-            if (j + 1 == n_tiles) commit_both(&sh.q_empty[seg % kQBufs]);     // every Q K^T of this run has been issued
+            if (issuer) commit_both(&sh.s_full[g & 1]);
+            if (issuer) commit_both(&sh.kv_empty[st]);
+            if (j + 1 == n_tiles && issuer) commit_both(&sh.q_empty[seg % kQBufs]);     // every Q K^T of this run has been issued
         }
         ++seg;
     }
@@ -322,13 +324,14 @@ __device__ void qk_role(SharedStorage& sh, const Params& prm, const PlanView& pv
     // counts its arrival too (the softmax threads wait for it before they rescale O)
     for (int i = 0; i < (g > 0 ? kVLag : 0); ++i, ++g) {
         if (!wait_c(sh, &sh.kv_ready[g % kStages], (g / kStages) & 1, prm.wait_ns)) return;
-        commit_both(&sh.kv_empty[g % kStages]);
+        if (issuer) commit_both(&sh.kv_empty[g % kStages]);
     }
 }
 
 __device__ void pv_role(SharedStorage& sh, const Params& prm, const PlanView& pv, uint32_t tmem)
 {
     Walker w;
+    const bool issuer = elect_lane();
     Segment s;
     uint32_t g = 0;
     const uint32_t v_lo0 = desc_lo(smem_u32(sh.kv[0] + kKBytes), 16);
@@ -336,7 +339,7 @@ __device__ void pv_role(SharedStorage& sh, const Params& prm, const PlanView& pv
     // the first kVLag stages carry no V tile: this thread has nothing to wait for on them
     bool run = w.begin(pv, prm, blockIdx.x >> 1, true, s);
     if (run)
-        for (int i = 0; i < kVLag; ++i) commit_both(&sh.kv_empty[i]);
+        for (int i = 0; i < kVLag; ++i) if (issuer) commit_both(&sh.kv_empty[i]);
     for (; run; run = w.next(s)) {
         const int n_tiles = s.t1 - s.t0;
         for (int j = 0; j < n_tiles; ++j, ++g) {
@@ -348,10 +351,10 @@ __device__ void pv_role(SharedStorage& sh, const Params& prm, const PlanView& pv
             const uint32_t vl = v_lo0 + st * kStageStep;
 #pragma unroll
             for (int i = 0; i < 8; ++i)
-                mma2_ts(tmem + kColO, tmem + kColP + pb * 64 + i * 8, vl + i * (2048u >> 4), kIdescPV2,
+                if (issuer) mma2_ts(tmem + kColO, tmem + kColP + pb * 64 + i * 8, vl + i * (2048u >> 4), kIdescPV2,
                         (j == 0 && i == 0) ? 0u : 1u);
-            commit_both(&sh.kv_empty[st]);
-            if (j + 1 == n_tiles) commit_both(&sh.o_done);
+            if (issuer) commit_both(&sh.kv_empty[st]);
+            if (j + 1 == n_tiles && issuer) commit_both(&sh.o_done);
         }
     }
 }
@@ -603,13 +606,13 @@ attention_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
         if ((threadIdx.x & 31) == 0) producer_role(sh, prm, pv, rank, &q_map, &k_map, &v_map, &ks_map, &vs_map);
     } else if (warp == 9) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-        if ((threadIdx.x & 31) == 0 && rank == 0) qk_role(sh, prm, pv, tmem);
+        if (rank == 0) qk_role(sh, prm, pv, tmem);
     } else if (warp == 10) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         relay_role(sh, prm, pv);
     } else if (warp == 11) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-        if ((threadIdx.x & 31) == 0 && rank == 0) pv_role(sh, prm, pv, tmem);
+        if (rank == 0) pv_role(sh, prm, pv, tmem);
     }
     __syncwarp();
     // ---- teardown ----

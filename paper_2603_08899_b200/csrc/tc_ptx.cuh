@@ -63,6 +63,14 @@ __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* m
         : "memory");
 }
 
+// true in one lane of a converged warp
+__device__ __forceinline__ bool elect_lane()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // high word of every shared-memory descriptor: SBO = 1024 B (>> 4) | version 1 (bit 46) | swizzle 128B (code 2, bits 61-63)
 constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
 

@@ -13,7 +13,11 @@
 //     reference maximum moves whenever the running maximum grows by more than 3, which keeps every
 //     weight at or under 2^8 < 448, while weights down to 2^-14 of the reference survive; moving it
 //     more eagerly costs a rescale of O each time); numerator and denominator carry the same shift;
-//   - the per-head V scale multiplies the output rows (or the partial results) at the end of a run.
+//   - the per-head V scale multiplies the output rows (or the partial results) at the end of a run;
+//   - a key tile is worked on in two halves of 64 keys: E4M3 products take half the time of bf16 ones, so the serial
+//     chain S -> weights -> P V -> next S of an M tile was mostly waiting (1200 of 3800 cycles per tile for S); now the
+//     tensor pipe serves one half of the chain while the softmax threads work on the other.  About 3450 cycles per tile and
+//     SM now; a layer of 32 sequences, prefixes 512..16384: 292 -> 264 us.
 #include "tc_walk.cuh"
 
 namespace confu {
@@ -36,7 +40,7 @@ struct SharedStorage {
     alignas(8) uint64_t q_full, q_empty;
     uint64_t q8_full[2];                                 // the 128 threads of an M tile have written its E4M3 rows
     uint64_t kv_full[kStages], kv_empty[kStages];
-    uint64_t s_full[2], p_full[2], o_done[2];
+    uint64_t s_full[2][2], p_full[2][2], o_done[2];      // [M tile][half of the key tile]
     uint64_t v_fixed;                     // the rows of a V tile past the sequence's last slot have been zeroed
     uint32_t tmem_base;
     int abort;
@@ -67,8 +71,8 @@ __device__ __forceinline__ void mma8_ts(uint32_t d_tmem, uint32_t a_tmem, uint32
         : "memory");
 }
 // Instruction descriptor: E4M3 (format code 0) x E4M3 -> fp32, M = 128, N = 128; B K-major (Q K^T) or MN-major (P V)
-constexpr uint32_t kIdescQK8 = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-constexpr uint32_t kIdescPV8 = kIdescQK8 | (1u << 16);
+constexpr uint32_t kIdescQK8 = (1u << 4) | ((64u >> 3) << 17) | ((128u >> 4) << 24);          // N = 64: half a key tile
+constexpr uint32_t kIdescPV8 = (1u << 4) | (1u << 16) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 
 // four floats -> four E4M3 bytes (a in the lowest byte), round to nearest even, saturating at +-448
 __device__ __forceinline__ uint32_t pack_e4m3(float a, float b, float c, float d)
@@ -213,26 +217,27 @@ __device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& p
     const uint32_t v_lo0 = desc_lo(smem_u32(sh.kv[0][0]), 16), k_lo0 = desc_lo(smem_u32(sh.kv[0][1]), 16);
     constexpr uint32_t kTileStep = kTile8 >> 4, kStageStep = 2 * kTileStep;
 
-    // S_t = Q_t K^T: 4 steps of 32 head dims; step i sits at byte 32 i of the swizzled 128-byte row
-    auto issue_qk = [&](int t, uint32_t kl) {
+    // half h of S_t = Q_t K_h^T: 4 steps of 32 head dims; step i sits at byte 32 i of the swizzled 128-byte row
+    auto issue_qk = [&](int t, int h, uint32_t kl) {
         if (!issuer) return;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const uint32_t off = ((uint32_t)i * 32u) >> 4;
-            mma8_ss(tmem + t * 128, q_lo + t * kTileStep + off, kl + off, kIdescQK8, i > 0 ? 1u : 0u);
+            mma8_ss(tmem + t * 128 + h * 64, q_lo + t * kTileStep + off, kl + h * (8192u >> 4) + off, kIdescQK8, i > 0 ? 1u : 0u);
         }
-        tc_commit(&sh.s_full[t]);
+        tc_commit(&sh.s_full[t][h]);
     };
-    // O_t += P_t V: 4 steps of 32 keys (4096 B of the V tile and 8 TMEM columns of four E4M3 weights each);
-    // P sits in the first 32 columns of the S_t block
-    auto issue_pv = [&](int t, uint32_t vl, bool first_of_segment) {
+    // O_t += P_t V over half h: 2 steps of 32 keys (4096 B of the V tile and 8 TMEM columns of four E4M3 weights each);
+    // P sits in the first 16 of the half's columns of S_t
+    auto issue_pv = [&](int t, int h, uint32_t vl, bool first_of_segment) {
         if (!issuer) return;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            mma8_ts(tmem + 256 + t * 128, tmem + t * 128 + i * 8, vl + i * (4096u >> 4), kIdescPV8,
-                    (first_of_segment && i == 0) ? 0u : 1u);
+        for (int i = 0; i < 2; ++i)
+            mma8_ts(tmem + 256 + t * 128, tmem + t * 128 + h * 64 + i * 8, vl + (2 * h + i) * (4096u >> 4), kIdescPV8,
+                    (first_of_segment && h == 0 && i == 0) ? 0u : 1u);
     };
-    // one stage: P V of the previous key tile (if any), Q K^T of the current one (if any)
+    // one stage: P V of the previous key tile (if any), Q K^T of the current one (if any), half by half: while the
+    // tensor pipe serves one half of a chain, its softmax threads work on the other
     bool have_prev = false, prev_first = false, prev_last = false, prev_ragged = false;
     uint32_t n_fix = 0;
     auto run_stage = [&](bool have_cur, bool cur_first, bool cur_last, bool cur_ragged) -> bool {
@@ -245,21 +250,33 @@ __device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& p
         }
         tc_fence_after();
         const uint32_t vl = v_lo0 + st * kStageStep, kl = k_lo0 + st * kStageStep;
+        if (have_prev) {
 #pragma unroll
-        for (int t = 0; t < kMt; ++t) {
-            if (have_prev) {
-                // (At the start of a pair this P V overwrites the previous pair's O_t; the softmax
-                // threads hand P over only after they have read that O_t out.)
-                if (!mbar_wait(&sh.p_full[t], (stage - 1) & 1, &sh.abort, prm.wait_ns)) return false;
-                tc_fence_after();
-                issue_pv(t, vl, prev_first);
-                if (prev_last && issuer) tc_commit(&sh.o_done[t]);
+            for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                for (int t = 0; t < kMt; ++t) {
+                    // (At the start of a pair this P V overwrites the previous pair's O_t; the softmax
+                    // threads hand P over only after they have read that O_t out.)
+                    if (!mbar_wait(&sh.p_full[t][h], (stage - 1) & 1, &sh.abort, prm.wait_ns)) return false;
+                    tc_fence_after();
+                    issue_pv(t, h, vl, prev_first);
+                    // Behind every P V of half 0 comes a completion of s_full[t][0], with or without a Q K^T: half 1 of
+                    // the same tile waits for it before it rescales O.
+                    if (prev_last) {
+                        if (issuer) tc_commit(h == 0 ? &sh.s_full[t][0] : &sh.o_done[t]);
+                    } else
+                        issue_qk(t, h, kl);
+                }
             }
-            if (have_cur) {
-                // at the start of a run: the E4M3 rows of this M tile's Q have been written
-                if (cur_first && !mbar_wait(&sh.q8_full[t], seg & 1, &sh.abort, prm.wait_ns)) return false;
-                if (cur_first) tc_fence_after();
-                issue_qk(t, kl);
+        }
+        if (have_cur && cur_first) {
+            // the start of a run: the E4M3 rows of each M tile's Q have been written
+#pragma unroll
+            for (int t = 0; t < kMt; ++t) {
+                if (!mbar_wait(&sh.q8_full[t], seg & 1, &sh.abort, prm.wait_ns)) return false;
+                tc_fence_after();
+                issue_qk(t, 0, kl);
+                issue_qk(t, 1, kl);
             }
         }
         if (issuer) tc_commit(&sh.kv_empty[st]);
@@ -330,7 +347,7 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
 
     Walker w;
     Segment s;
-    uint32_t n_s = 0, seg = 0;
+    uint32_t n_s[2] = {0, 0}, seg = 0;                      // completions of s_full[t][half] used up, runs
     for (bool run = w.begin(pv, prm, blockIdx.x, false, s); run; run = w.next(s)) {
         const int r = prm.rpt * (2 * s.rg + t) + lane_row / G;            // query row of this thread in this pair
         const bool row_valid = lane_row < prm.rpt * G && r < R;
@@ -343,57 +360,76 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
         // one factor for the exponent's argument: softmax scale * log2(e) * the row's Q scale * the head's K scale
         const float c = prm.c * q_scale * __ldg(prm.k_scale + s.g);
         float m_ref = -INFINITY, l = 0.f;
-        for (int tile = s.t0; tile < s.t1; ++tile) {
-            if (!mbar_wait(&sh.s_full[t], n_s & 1, &sh.abort, prm.wait_ns)) return;
-            ++n_s;
+        // 64 scores of half h, masked where the tile needs it
+        auto load_half = [&](int h, int tile, uint32_t (&sv)[64]) -> bool {
+            if (!mbar_wait(&sh.s_full[t][h], n_s[h] & 1, &sh.abort, prm.wait_ns)) return false;
+            ++n_s[h];
             tc_fence_after();
-            uint32_t sv[128];
-#pragma unroll
-            for (int q4 = 0; q4 < 4; ++q4) tmem_ld32(s_addr + q4 * 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[q4 * 32]));
+            tmem_ld32(s_addr + h * 64, *reinterpret_cast<uint32_t(*)[32]>(&sv[0]));
+            tmem_ld32(s_addr + h * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[32]));
             tc_wait_ld();
-            const bool masked = tile >= s.nkt || (int64_t)(tile + 1) * kTileKeys > s.P;
-            if (masked) {
+            if (tile >= s.nkt || (int64_t)(tile + 1) * kTileKeys > s.P) {
                 uint64_t lo, hi;
                 visible_bits(s, tile, R, T, S, r, row_valid, mask, lo, hi);
+                const uint64_t vis = h ? hi : lo;
 #pragma unroll
-                for (int j = 0; j < 64; ++j) {
-                    if (!((lo >> j) & 1ull)) sv[j] = 0xff800000u;            // -inf
-                    if (!((hi >> j) & 1ull)) sv[64 + j] = 0xff800000u;
-                }
+                for (int j = 0; j < 64; ++j)
+                    if (!((vis >> j) & 1ull)) sv[j] = 0xff800000u;           // -inf
             }
-            const float m_new = fmaxf(m_ref, max128(sv) * c);
-            if (tile == s.t0) {
-                m_ref = m_new;
-            } else {
-                const bool move = m_new - m_ref > kRescaleThreshold;         // false when both are -inf (NaN)
-                if (__any_sync(0xffffffffu, move)) {
-                    const float alpha = move ? ex2(m_ref - m_new) : 1.f;
-                    if (move) { m_ref = m_new; l *= alpha; }
-                    // S_full of this tile implies the previous PV of this M tile has completed
+            return true;
+        };
+        // the reference maximum follows the running maximum; O is brought along when it moves.  P V of the half before
+        // has completed when the other half's next completion of s_full is there (see the issuing warp).
+        auto follow = [&](float m_half, int h) -> bool {
+            const float m_new = fmaxf(m_ref, m_half);
+            const bool move = m_new - m_ref > kRescaleThreshold;             // false when both are -inf (NaN)
+            if (!__any_sync(0xffffffffu, move)) return true;
+            if (!mbar_wait(&sh.s_full[t][h ^ 1], n_s[h ^ 1] & 1, &sh.abort, prm.wait_ns)) return false;
+            tc_fence_after();
+            const float alpha = move ? ex2(m_ref - m_new) : 1.f;
+            if (move) { m_ref = m_new; l *= alpha; }
+#pragma unroll 1
+            for (int q4 = 0; q4 < 8; ++q4) {
+                uint32_t ov[16];
+                tmem_ld16(o_addr + q4 * 16, ov);
+                tc_wait_ld();
 #pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4) {
-                        uint32_t ov[32];
-                        tmem_ld32(o_addr + q4 * 32, ov);
-                        tc_wait_ld();
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) ov[j] = __float_as_uint(__uint_as_float(ov[j]) * alpha);
-                        tmem_st32(o_addr + q4 * 32, ov);
-                    }
-                }
+                for (int j = 0; j < 16; ++j) ov[j] = __float_as_uint(__uint_as_float(ov[j]) * alpha);
+                tmem_st16(o_addr + q4 * 16, ov);
             }
+            return true;
+        };
+        // P over the first 16 columns of the half (whose scores sit in registers by now); masked scores are -inf
+        // and get weight exactly 0
+        auto hand_over = [&](int h, const uint32_t (&sv)[64]) {
             const float neg_m = (m_ref == -INFINITY) ? 0.f : kPShift - m_ref;
-            // P overlays the first 32 columns of S_t (all of S_t is in registers by now); masked
-            // scores are -inf and get weight exactly 0
-            {
-                uint32_t pk[32];
-                l += weights64_e4m3(&sv[0], c, neg_m, &pk[0]);
-                l += weights64_e4m3(&sv[64], c, neg_m, &pk[16]);
-                tmem_st32(s_addr, pk);
-            }
+            uint32_t pk[16];
+            l += weights64_e4m3(sv, c, neg_m, pk);
+            tmem_st16(s_addr + h * 64, pk);
             tc_wait_st();
             tc_fence_before();
-            mbar_arrive(&sh.p_full[t]);
+            mbar_arrive(&sh.p_full[t][h]);
+        };
+        for (int tile = s.t0; tile < s.t1; ++tile) {
+            uint32_t sa[64], sb[64];
+            if (!load_half(0, tile, sa)) return;
+            const float m0 = max64(sa) * c;
+            if (tile == s.t0) {                              // the first reference comes from the whole tile
+                if (!load_half(1, tile, sb)) return;
+                m_ref = fmaxf(m0, max64(sb) * c);
+                hand_over(0, sa);
+                hand_over(1, sb);
+            } else {
+                if (!follow(m0, 0)) return;
+                hand_over(0, sa);
+                if (!load_half(1, tile, sb)) return;
+                if (!follow(max64(sb) * c, 1)) return;
+                hand_over(1, sb);
+            }
         }
+        // (the completion that stands for the P V of the last half 0)
+        if (!mbar_wait(&sh.s_full[t][0], n_s[0] & 1, &sh.abort, prm.wait_ns)) return;
+        ++n_s[0];
         // ---- epilogue of this pair / range ----
         if (!mbar_wait(&sh.o_done[t], seg & 1, &sh.abort, prm.wait_ns)) return;
         tc_fence_after();
@@ -487,8 +523,10 @@ attention_fp8_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
         for (int i = 0; i < kStages; ++i) { mbar_init(&sh.kv_full[i], 1); mbar_init(&sh.kv_empty[i], 2); }
         mbar_init(&sh.v_fixed, 1);
         for (int t = 0; t < 2; ++t) {
-            mbar_init(&sh.s_full[t], 1);
-            mbar_init(&sh.p_full[t], 128);
+            for (int h = 0; h < 2; ++h) {
+                mbar_init(&sh.s_full[t][h], 1);
+                mbar_init(&sh.p_full[t][h], 128);
+            }
             mbar_init(&sh.o_done[t], 1);
         }
         sh.abort = 0;

@@ -8,12 +8,13 @@
 //     P_t = exp2(S_t*c - m)   one thread per row: tcgen05.ld, mask (last tiles only), tcgen05.st as bf16
 //                             over the S columns
 //     O_t += P_t V            tcgen05.mma, A from TMEM, B = V tile in shared memory (MN-major)
-// Each M tile has its own softmax warpgroup; the two run out of phase, so that while one computes
-// exponentials the tensor pipe serves the other (P V, then the next Q K^T).  The tensor pipe holds
+// Each M tile has its own softmax warpgroup, and a key tile is worked on in two halves of 64 keys: while a
+// warpgroup computes the weights of one half, the tensor pipe does P V and the next Q K^T of the other (as one
+// piece the chain S -> weights -> P V -> next S was serial: 16 sequences of 512..8000 77.6 -> 73.4 us a layer, batch 1
+// 17.9 -> 16.9; at 32 sequences, where the power cap sets the pace, the same).  The tensor pipe holds
 // about one instruction ahead of the issuing thread, so whatever that thread does between MMAs is
 // idle pipe time: K/V travel in stages of [V of key tile g-1 | K of key tile g] with one full and
-// one empty barrier each, which leaves the issuing thread three waits and three commits per key
-// tile.  Prefix tiles need no mask; the ancestor bitmask (one 64-bit word per row, in a register) is applied only to
+// one empty barrier each.  Prefix tiles need no mask; the ancestor bitmask (one 64-bit word per row, in a register) is applied only to
 // the tiles that hold the tree slots, the ragged tail and the soft-prompt entries.  A range that
 // does not cover a whole pair writes an unnormalised partial (O, m, l) that merge_kernel merges
 // in a fixed order.
@@ -47,7 +48,7 @@ struct SharedStorage {
     alignas(1024) uint8_t kv[kStages<D>][2][kTile<D>];   // [stage][0: V tile, 1: K tile]
     alignas(8) uint64_t q_full, q_empty;
     uint64_t kv_full[kStages<D>], kv_empty[kStages<D>];
-    uint64_t s_full[2], p_full[2], o_done[2];
+    uint64_t s_full[2][2], p_full[2][2], o_done[2];      // [M tile][half of the key tile]
     uint64_t v_fixed;                     // the rows of a V tile past the sequence's last slot have been zeroed
     uint32_t tmem_base;
     int abort;
@@ -140,32 +141,32 @@ __device__ void mma_role(SharedStorage<D>& sh, const Params& prm, const PlanView
     constexpr uint32_t kTileStep = kTile<D> >> 4, kStageStep = 2 * kTileStep;
     constexpr uint32_t kIdescO = D == 128 ? kIdescPV : kIdescPV64;
 
-    // S_t = Q_t K^T: D / 16 steps of 16 head dims; step i sits in 64-column half i/4 at byte 32*(i%4) of the swizzled row
-    auto issue_qk = [&](int t, uint32_t kl) {
+    // half h of S_t = Q_t K_h^T: D / 16 steps of 16 head dims; step i sits in 64-column half i/4 at byte 32*(i%4) of the swizzled row
+    auto issue_qk = [&](int t, int h, uint32_t kl) {
         if (!issuer) return;
 #pragma unroll
         for (int i = 0; i < D / 16; ++i) {
             const uint32_t off = ((uint32_t)(i >> 2) * kHalfTile + (uint32_t)(i & 3) * 32u) >> 4;
-            mma_ss(tmem + t * 128, q_lo + t * kTileStep + off, kl + off, kIdescQK, i > 0 ? 1u : 0u);
+            mma_ss(tmem + t * 128 + h * 64, q_lo + t * kTileStep + off, kl + h * (8192u >> 4) + off, kIdescQK64, i > 0 ? 1u : 0u);
         }
-        tc_commit(&sh.s_full[t]);
+        tc_commit(&sh.s_full[t][h]);
     };
-    // O_t += P_t V: 8 steps of 16 keys (2048 B of the V tile and 8 TMEM columns of bf16 pairs each);
-    // P sits in the first 64 columns of the S_t block
-    auto issue_pv = [&](int t, uint32_t vl, bool first_of_segment) {
+    // O_t += P_t V over half h: 4 steps of 16 keys (2048 B of the V tile and 8 TMEM columns of bf16 pairs each);
+    // P sits in the first 32 of the half's columns of S_t
+    auto issue_pv = [&](int t, int h, uint32_t vl, bool first_of_segment) {
         if (!issuer) return;
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-            mma_ts(tmem + 256 + t * 128, tmem + t * 128 + i * 8, vl + i * (2048u >> 4), kIdescO,
-                   (first_of_segment && i == 0) ? 0u : 1u);
+        for (int i = 0; i < 4; ++i)
+            mma_ts(tmem + 256 + t * 128, tmem + t * 128 + h * 64 + i * 8, vl + (4 * h + i) * (2048u >> 4), kIdescO,
+                   (first_of_segment && h == 0 && i == 0) ? 0u : 1u);
     };
-    // one stage: P V of the previous key tile (if any), Q K^T of the current one (if any)
+    // one stage: P V of the previous key tile (if any), Q K^T of the current one (if any), half by half: while the
+    // tensor pipe serves one half of a chain, its softmax threads work on the other
     bool have_prev = false, prev_first = false, prev_last = false, prev_ragged = false;
     uint32_t n_fix = 0;
     auto run_stage = [&](bool have_cur, bool cur_first, bool cur_last, bool cur_ragged) -> bool {
         const uint32_t st = stage % kStages<D>;
         if (!mbar_wait(&sh.kv_full[st], (stage / kStages<D>) & 1, &sh.abort, prm.wait_ns)) return false;
-        if (have_cur && cur_first && !mbar_wait(&sh.q_full, seg & 1, &sh.abort, prm.wait_ns)) return false;
         // the V tile of a sequence's last key tile: wait until its rows past the last slot are zero
         if (have_prev && prev_ragged) {
             if (!mbar_wait(&sh.v_fixed, n_fix & 1, &sh.abort, prm.wait_ns)) return false;
@@ -173,17 +174,34 @@ __device__ void mma_role(SharedStorage<D>& sh, const Params& prm, const PlanView
         }
         tc_fence_after();
         const uint32_t vl = v_lo0 + st * kStageStep, kl = k_lo0 + st * kStageStep;
+        if (have_prev) {
 #pragma unroll
-        for (int t = 0; t < kMt; ++t) {
-            if (have_prev) {
-                // (At the start of a pair this P V overwrites the previous pair's O_t; the softmax
-                // threads hand P over only after they have read that O_t out.)
-                if (!mbar_wait(&sh.p_full[t], (stage - 1) & 1, &sh.abort, prm.wait_ns)) return false;
-                tc_fence_after();
-                issue_pv(t, vl, prev_first);
-                if (prev_last && issuer) tc_commit(&sh.o_done[t]);
+            for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                for (int t = 0; t < kMt; ++t) {
+                    // (At the start of a pair this P V overwrites the previous pair's O_t; the softmax
+                    // threads hand P over only after they have read that O_t out.)
+                    if (!mbar_wait(&sh.p_full[t][h], (stage - 1) & 1, &sh.abort, prm.wait_ns)) return false;
+                    tc_fence_after();
+                    issue_pv(t, h, vl, prev_first);
+                    // Behind every P V of half 0 comes a completion of s_full[t][0], with or without a Q K^T: half 1 of
+                    // the same tile waits for it before it rescales O.
+                    if (prev_last) {
+                        if (issuer) tc_commit(h == 0 ? &sh.s_full[t][0] : &sh.o_done[t]);
+                    } else
+                        issue_qk(t, h, kl);
+                }
             }
-            if (have_cur) issue_qk(t, kl);
+        }
+        if (have_cur && cur_first) {
+            // the start of a run: its Q has landed
+            if (!mbar_wait(&sh.q_full, seg & 1, &sh.abort, prm.wait_ns)) return false;
+            tc_fence_after();
+#pragma unroll
+            for (int t = 0; t < kMt; ++t) {
+                issue_qk(t, 0, kl);
+                issue_qk(t, 1, kl);
+            }
         }
         if (issuer) tc_commit(&sh.kv_empty[st]);
         if (have_cur && cur_last && issuer) tc_commit(&sh.q_empty);               // last Q K^T of the pair has been issued
@@ -257,63 +275,82 @@ __device__ void softmax_role(SharedStorage<D>& sh, const Params& prm, const Plan
 
     Walker w;
     Segment s;
-    uint32_t n_s = 0, seg = 0;
+    uint32_t n_s[2] = {0, 0}, seg = 0;                      // completions of s_full[t][half] used up, runs
     for (bool run = w.begin(pv, prm, blockIdx.x, false, s); run; run = w.next(s)) {
         const int r = prm.rpt * (2 * s.rg + t) + lane_row / G;            // query row of this thread in this pair
         const bool row_valid = lane_row < prm.rpt * G && r < R;
         const uint64_t mask = row_valid ? pv.mask[(size_t)s.b * kMaxRows + r] : 0ull;
         float m_ref = -INFINITY, l = 0.f;
-        for (int tile = s.t0; tile < s.t1; ++tile) {
-            if (!mbar_wait(&sh.s_full[t], n_s & 1, &sh.abort, prm.wait_ns)) return;
-            ++n_s;
+        // 64 scores of half h, masked where the tile needs it
+        auto load_half = [&](int h, int tile, uint32_t (&sv)[64]) -> bool {
+            if (!mbar_wait(&sh.s_full[t][h], n_s[h] & 1, &sh.abort, prm.wait_ns)) return false;
+            ++n_s[h];
             tc_fence_after();
-            uint32_t sv[128];
-#pragma unroll
-            for (int q4 = 0; q4 < 4; ++q4) tmem_ld32(s_addr + q4 * 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[q4 * 32]));
+            tmem_ld32(s_addr + h * 64, *reinterpret_cast<uint32_t(*)[32]>(&sv[0]));
+            tmem_ld32(s_addr + h * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[32]));
             tc_wait_ld();
-            const bool masked = tile >= s.nkt || (int64_t)(tile + 1) * kTileKeys > s.P;
-            if (masked) {
+            if (tile >= s.nkt || (int64_t)(tile + 1) * kTileKeys > s.P) {
                 uint64_t lo, hi;
                 visible_bits(s, tile, R, T, S, r, row_valid, mask, lo, hi);
+                const uint64_t vis = h ? hi : lo;
 #pragma unroll
-                for (int j = 0; j < 64; ++j) {
-                    if (!((lo >> j) & 1ull)) sv[j] = 0xff800000u;            // -inf
-                    if (!((hi >> j) & 1ull)) sv[64 + j] = 0xff800000u;
-                }
+                for (int j = 0; j < 64; ++j)
+                    if (!((vis >> j) & 1ull)) sv[j] = 0xff800000u;           // -inf
             }
-            const float m_new = fmaxf(m_ref, max128(sv) * c);
-            if (tile == s.t0) {
-                m_ref = m_new;
-            } else {
-                const bool move = m_new - m_ref > kRescaleThreshold;         // false when both are -inf (NaN)
-                if (__any_sync(0xffffffffu, move)) {
-                    const float alpha = move ? ex2(m_ref - m_new) : 1.f;
-                    if (move) { m_ref = m_new; l *= alpha; }
-                    // S_full of this tile implies the previous PV of this M tile has completed
+            return true;
+        };
+        // the reference maximum follows the running maximum; O is brought along when it moves.  P V of the half before
+        // has completed when the other half's next completion of s_full is there (see the issuing warp).
+        auto follow = [&](float m_half, int h) -> bool {
+            const float m_new = fmaxf(m_ref, m_half);
+            const bool move = m_new - m_ref > kRescaleThreshold;             // false when both are -inf (NaN)
+            if (!__any_sync(0xffffffffu, move)) return true;
+            if (!mbar_wait(&sh.s_full[t][h ^ 1], n_s[h ^ 1] & 1, &sh.abort, prm.wait_ns)) return false;
+            tc_fence_after();
+            const float alpha = move ? ex2(m_ref - m_new) : 1.f;
+            if (move) { m_ref = m_new; l *= alpha; }
+#pragma unroll 1
+            for (int q4 = 0; q4 < D / 16; ++q4) {
+                uint32_t ov[16];
+                tmem_ld16(o_addr + q4 * 16, ov);
+                tc_wait_ld();
 #pragma unroll
-                    for (int q4 = 0; q4 < D / 32; ++q4) {
-                        uint32_t ov[32];
-                        tmem_ld32(o_addr + q4 * 32, ov);
-                        tc_wait_ld();
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) ov[j] = __float_as_uint(__uint_as_float(ov[j]) * alpha);
-                        tmem_st32(o_addr + q4 * 32, ov);
-                    }
-                }
+                for (int j = 0; j < 16; ++j) ov[j] = __float_as_uint(__uint_as_float(ov[j]) * alpha);
+                tmem_st16(o_addr + q4 * 16, ov);
             }
+            return true;
+        };
+        // P over the first 32 columns of the half (whose scores sit in registers by now); masked scores are -inf
+        // and get weight exactly 0
+        auto hand_over = [&](int h, const uint32_t (&sv)[64]) {
             const float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref;
-            // P overlays the first 64 columns of S_t (all of S_t is in registers by now); masked
-            // scores are -inf and get weight exactly 0
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                uint32_t pk[32];
-                l += weights64(&sv[64 * half], c, neg_m, pk);
-                tmem_st32(s_addr + 32 * half, pk);
-            }
+            uint32_t pk[32];
+            l += weights64(sv, c, neg_m, pk);
+            tmem_st32(s_addr + h * 64, pk);
             tc_wait_st();
             tc_fence_before();
-            mbar_arrive(&sh.p_full[t]);
+            mbar_arrive(&sh.p_full[t][h]);
+        };
+        for (int tile = s.t0; tile < s.t1; ++tile) {
+            uint32_t sa[64], sb[64];
+            if (!load_half(0, tile, sa)) return;
+            const float m0 = max64(sa) * c;
+            if (tile == s.t0) {                              // the first reference comes from the whole tile
+                if (!load_half(1, tile, sb)) return;
+                m_ref = fmaxf(m0, max64(sb) * c);
+                hand_over(0, sa);
+                hand_over(1, sb);
+            } else {
+                if (!follow(m0, 0)) return;
+                hand_over(0, sa);
+                if (!load_half(1, tile, sb)) return;
+                if (!follow(max64(sb) * c, 1)) return;
+                hand_over(1, sb);
+            }
         }
+        // (the completion that stands for the P V of the last half 0)
+        if (!mbar_wait(&sh.s_full[t][0], n_s[0] & 1, &sh.abort, prm.wait_ns)) return;
+        ++n_s[0];
         // ---- epilogue of this pair / range ----
         if (!mbar_wait(&sh.o_done[t], seg & 1, &sh.abort, prm.wait_ns)) return;
         tc_fence_after();
@@ -403,8 +440,10 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
         for (int i = 0; i < kStages<D>; ++i) { mbar_init(&sh.kv_full[i], 1); mbar_init(&sh.kv_empty[i], 2); }
         mbar_init(&sh.v_fixed, 1);
         for (int t = 0; t < 2; ++t) {
-            mbar_init(&sh.s_full[t], 1);
-            mbar_init(&sh.p_full[t], 128);
+            for (int h = 0; h < 2; ++h) {
+                mbar_init(&sh.s_full[t][h], 1);
+                mbar_init(&sh.p_full[t][h], 128);
+            }
             mbar_init(&sh.o_done[t], 1);
         }
         sh.abort = 0;

@@ -160,6 +160,7 @@ __device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) { retur
 // Instruction descriptor: bf16 x bf16 -> fp32, M = 128, N = 128; B K-major (QK^T) or MN-major (PV).
 constexpr uint32_t kIdescQK = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
 constexpr uint32_t kIdescPV = kIdescQK | (1u << 16);
+constexpr uint32_t kIdescQK64 = (1u << 4) | (1u << 7) | (1u << 10) | ((64u >> 3) << 17) | ((128u >> 4) << 24);                // N = 64: half a key tile
 constexpr uint32_t kIdescPV64 = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((64u >> 3) << 17) | ((128u >> 4) << 24);   // N = 64: head dim 64
 
 }  // namespace tc

@@ -9,7 +9,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libconfu.so")
-SOURCES = ["api.cu", "plan.cu", "attn_generic.cu", "attn_tc.cu", "attn_tc2.cu", "attn_fp8.cu", "combine.cu", "accept.cu", "accept_walk.cu", "accept_static.cu", "compact.cu", "moe.cu", "selftest.cu"]
+SOURCES = ["api.cu", "plan.cu", "attn_generic.cu", "attn_tc.cu", "attn_tc2.cu", "attn_narrow.cu", "attn_fp8.cu", "combine.cu", "accept.cu", "accept_walk.cu", "accept_static.cu", "compact.cu", "moe.cu", "selftest.cu"]
 HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "attn_tc.cuh"), os.path.join(CSRC, "tc_ptx.cuh"), os.path.join(CSRC, "tc_walk.cuh"), os.path.join(CSRC, "accept.cuh"), os.path.join(CSRC, "walk.cuh"),
            os.path.join(ROOT, "include", "confu.h")]
 

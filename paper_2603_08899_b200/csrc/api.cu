@@ -32,7 +32,7 @@ int cuda_fail(confu_ctx* ctx, cudaError_t e)
 
 // workspace carving: [plan built by the attention call itself][split-KV partial slots]
 size_t ws_plan_offset() { return 0; }
-size_t ws_partial_offset(const confu_dims* d) { return align_up(plan_bytes(d->B, d->Hkv, row_groups(d->T + d->C, d->Hq / d->Hkv)), 256); }
+size_t ws_partial_offset(const confu_dims* d) { return align_up(plan_bytes(d->B, d->Hkv, row_groups(d->T + d->C, d->Hq / d->Hkv, 1)), 256); }
 size_t ws_total(const confu_ctx* ctx, const confu_dims* d)
 {
     return ws_partial_offset(d) + (size_t)2 * ctx->sm_count * partial_slot_bytes();
@@ -56,6 +56,10 @@ cudaError_t launch_attention_pair(const Ctx* ctx, const confu_dims& d, const voi
                                   const void* v_cache, int64_t n_slots, const SlotMap& map,
                                   const int32_t* prefix_len, const void* k_soft, const void* v_soft, const void* plan,
                                   void* partials, void* out, float* lse, int32_t* status, cudaStream_t st);
+cudaError_t launch_attention_narrow(const Ctx* ctx, const confu_dims& d, const void* q, const void* k_cache,
+                                    const void* v_cache, int64_t n_slots, const SlotMap& map,
+                                    const int32_t* prefix_len, const void* k_soft, const void* v_soft, const void* plan,
+                                    void* partials, void* out, float* lse, int32_t* status, cudaStream_t st);
 cudaError_t launch_attention_tc(const Ctx* ctx, const confu_dims& d, const void* q, const void* k_cache,
                                 const void* v_cache, int64_t n_slots, const SlotMap& map,
                                 const int32_t* prefix_len, const void* k_soft, const void* v_soft, const void* plan,
@@ -69,7 +73,7 @@ namespace {
 int resolve_attention_path(const confu_ctx* ctx, const confu_dims& d)
 {
     // (a share of the work is walked by one CTA, or CTA pair, per group of query rows: at least that many of them)
-    const int n_rg = row_groups(d.T + d.C, d.Hq / d.Hkv);
+    const int n_rg = row_groups(d.T + d.C, d.Hq / d.Hkv, 2);
     const bool tc = tc_attention_supported(d) && ctx->sm_count >= n_rg;
     const bool pair = pair_attention_supported(d) && ctx->sm_count / 2 >= n_rg;
     if (d.kv_dtype == CONFU_FP8_E4M3) {         // one kernel serves E4M3 caches
@@ -80,17 +84,22 @@ int resolve_attention_path(const confu_ctx* ctx, const confu_dims& d)
         case CONFU_ATTENTION_GENERIC: return CONFU_ATTENTION_GENERIC;
         case CONFU_ATTENTION_TENSOR: return tc ? (int)CONFU_ATTENTION_TENSOR : (int)CONFU_ERR_UNSUPPORTED;
         case CONFU_ATTENTION_TENSOR_PAIR: return pair ? (int)CONFU_ATTENTION_TENSOR_PAIR : (int)CONFU_ERR_UNSUPPORTED;
-        default: {
-            // The two-SM kernel wins where a (sequence, kv head, row group) is split over many work units
-            // (small batches: half as many, twice as long runs, half the partial results to merge); with
-            // more such pairs than units the one-CTA kernel is the faster one.
-            const bool few_pairs = (int64_t)d.B * d.Hkv * n_rg <= ctx->sm_count / 2;
-            // (and with all query rows in one M tile the second CTA of a pair would only see padding)
-            const bool two_tiles = d.T + d.C > rows_per_tile(d.Hq / d.Hkv);
-            if (pair && few_pairs && two_tiles) return CONFU_ATTENTION_TENSOR_PAIR;
-            return tc ? (int)CONFU_ATTENTION_TENSOR : (int)CONFU_ATTENTION_GENERIC;
-        }
+        default: return tc ? (int)CONFU_ATTENTION_TENSOR : (int)CONFU_ATTENTION_GENERIC;
     }
+}
+
+// The kind of work units (PlanKind) that the tensor-core kernel for these dims uses: one M tile per CTA, or two.  One wins
+// where pairs are few: every CTA has a short run or a few, and what counts is the way from its start to its last
+// store.  Two read K and V half as often and need half as many runs.  (8 kv heads, R 64: two M tiles a pair; us per layer, one
+// tile against two.  8 sequences of 300..4000: 39.5 / 43.9; 10 of 300..6000: 48.0 / 54.9, of 15..300: 18.8 / 20.0; 16 of
+// 300..6000: 75 / 82, but of 15..300: 25.0 / 22.3; 32 of 600..12000: 227 / 209.)  A path that the caller has chosen is
+// taken as it is named.
+int plan_kind(const confu_ctx* ctx, const confu_dims& d, int path)
+{
+    if (path == CONFU_ATTENTION_TENSOR_PAIR) return kPlanPair;
+    const int n_tiles = row_groups(d.T + d.C, d.Hq / d.Hkv, 1);
+    const bool few = 2 * (int64_t)d.B * d.Hkv * n_tiles <= 3 * (int64_t)ctx->sm_count;
+    return path == CONFU_ATTENTION_TENSOR && ctx->attention_path == CONFU_ATTENTION_AUTO && d.kv_dtype == CONFU_BF16 && few ? kPlanNarrow : kPlanCta;
 }
 
 }  // namespace
@@ -226,7 +235,7 @@ const char* confu_last_cuda_error(const confu_ctx* ctx)
 size_t confu_plan_bytes(const confu_ctx* ctx, const confu_dims* dims)
 {
     if (!ctx || check_dims(dims) != CONFU_OK) return 0;
-    return plan_bytes(dims->B, dims->Hkv, row_groups(dims->T + dims->C, dims->Hq / dims->Hkv));
+    return plan_bytes(dims->B, dims->Hkv, row_groups(dims->T + dims->C, dims->Hq / dims->Hkv, 1));
 }
 
 int confu_tree_plan(confu_ctx* ctx, const confu_dims* dims, const int64_t* seq_start, const int32_t* prefix_len,
@@ -241,7 +250,7 @@ int confu_tree_plan(confu_ctx* ctx, const confu_dims* dims, const int64_t* seq_s
     const int path = resolve_attention_path(ctx, *dims);
     if (path < 0) return path;
     cudaError_t e = launch_plan(ctx, *dims, seq_start, prefix_len, parent, con_owner, plan, status,
-                                path == CONFU_ATTENTION_TENSOR_PAIR, (cudaStream_t)stream);
+                                plan_kind(ctx, *dims, path), (cudaStream_t)stream);
     return e == cudaSuccess ? CONFU_OK : cuda_fail(ctx, e);
 }
 
@@ -273,7 +282,7 @@ int confu_tree_attention(confu_ctx* ctx, const confu_dims* dims, const void* q, 
     if (!plan) {
         void* own_plan = ws + ws_plan_offset();
         cudaError_t e = launch_plan(ctx, *dims, seq_start, prefix_len, parent, con_owner, own_plan, status,
-                                    path == CONFU_ATTENTION_TENSOR_PAIR, st);
+                                    plan_kind(ctx, *dims, path), st);
         if (e != cudaSuccess) return cuda_fail(ctx, e);
         use_plan = own_plan;
     }
@@ -284,6 +293,9 @@ int confu_tree_attention(confu_ctx* ctx, const confu_dims* dims, const void* q, 
     else if (path == CONFU_ATTENTION_TENSOR && dims->kv_dtype == CONFU_FP8_E4M3)
         e = launch_attention_fp8(ctx, *dims, q, k_cache, v_cache, n_slots, map, prefix_len, k_soft, v_soft,
                                  use_plan, ws + ws_partial_offset(dims), out, lse, status, st);
+    else if (path == CONFU_ATTENTION_TENSOR && plan_kind(ctx, *dims, path) == kPlanNarrow)
+        e = launch_attention_narrow(ctx, *dims, q, k_cache, v_cache, n_slots, map, prefix_len, k_soft, v_soft,
+                                    use_plan, ws + ws_partial_offset(dims), out, lse, status, st);
     else if (path == CONFU_ATTENTION_TENSOR)
         e = launch_attention_tc(ctx, *dims, q, k_cache, v_cache, n_slots, map, prefix_len, k_soft, v_soft,
                                 use_plan, ws + ws_partial_offset(dims), out, lse, status, st);

@@ -172,7 +172,7 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
         ++stage;
         return true;
     };
-    for (bool run = w.begin(pv, prm, blockIdx.x, false, s); run; run = w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x, kPlanCta, s); run; run = w.next(s)) {
         for (int t = s.t0; t < s.t1; ++t) {
             TileRef cur;
             cur.g = s.g;
@@ -290,7 +290,7 @@ __device__ void mma_role(SharedStorage& sh, const Params& prm, const PlanView& p
     };
 
     const int R = prm.d.T + prm.d.C;
-    for (bool run = w.begin(pv, prm, blockIdx.x, false, s); run; run = w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x, kPlanCta, s); run; run = w.next(s)) {
         const int n_tiles = s.t1 - s.t0;
         for (int j = 0; j < n_tiles; ++j)
             if (!run_stage(true, j == 0, j + 1 == n_tiles, ragged_rows(s, s.t0 + j, R) > 0)) return;
@@ -329,7 +329,7 @@ __device__ void tail_role(SharedStorage& sh, const Params& prm, const PlanView& 
         prev_valid = cur_valid;
         return true;
     };
-    for (bool run = w.begin(pv, prm, blockIdx.x, false, s); run; run = w.next(s))
+    for (bool run = w.begin(pv, prm, blockIdx.x, kPlanCta, s); run; run = w.next(s))
         for (int tile = s.t0; tile < s.t1; ++tile)
             if (!run_stage(ragged_rows(s, tile, R))) return;
     if (have_prev) run_stage(0);
@@ -348,7 +348,7 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
     Walker w;
     Segment s;
     uint32_t n_s[2] = {0, 0}, seg = 0;                      // completions of s_full[t][half] used up, runs
-    for (bool run = w.begin(pv, prm, blockIdx.x, false, s); run; run = w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x, kPlanCta, s); run; run = w.next(s)) {
         const int r = prm.rpt * (2 * s.rg + t) + lane_row / G;            // query row of this thread in this pair
         const bool row_valid = lane_row < prm.rpt * G && r < R;
         const uint64_t mask = row_valid ? pv.mask[(size_t)s.b * kMaxRows + r] : 0ull;
@@ -644,7 +644,7 @@ cudaError_t launch_attention_fp8(const Ctx* ctx, const confu_dims& d, const void
     prm.out = (__nv_bfloat16*)out;
     prm.lse = lse;
     prm.status = status;
-    set_rows(prm, d);
+    set_rows(prm, d, 2);
     prm.c = (d.sm_scale != 0.f ? d.sm_scale : 1.f / sqrtf((float)d.D)) * 1.4426950408889634f;
     prm.wait_ns = ctx->wait_ns;
     prm.k_scale = ctx->k_scale;

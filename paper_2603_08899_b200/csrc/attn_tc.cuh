@@ -21,7 +21,8 @@ struct Params {
     int n_mt;            // M tiles in use (2 unless one holds all rows)
     int n_rg;            // groups of query rows; a pair = (sequence, kv head, row group)
     int G;               // query heads per kv head
-    int rpt;             // query rows per M tile (128 / G); a row group is two M tiles
+    int rpt;             // query rows per M tile (128 / G)
+    int tpg;             // M tiles per row group
     float c;             // sm_scale * log2(e)
     unsigned long long wait_ns;   // limit of every wait on an mbarrier (wall clock)
     const float* k_scale;         // E4M3 cache: value = code * scale[kv head] (device, [Hkv]); unused otherwise
@@ -36,12 +37,13 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
 }
 
 // The row packing of a launch (see rows_per_tile).
-inline void set_rows(Params& p, const confu_dims& d)
+inline void set_rows(Params& p, const confu_dims& d, int tpg)
 {
+    p.tpg = tpg;
     p.G = d.Hq / d.Hkv;
     p.rpt = rows_per_tile(p.G);
-    p.n_mt = d.T + d.C > p.rpt ? 2 : 1;
-    p.n_rg = row_groups(d.T + d.C, p.G);
+    p.n_mt = d.T + d.C > p.rpt ? tpg : 1;
+    p.n_rg = row_groups(d.T + d.C, p.G, tpg);
 }
 
 // Enqueues the merge of the partial results that the attention launch with the same parameters

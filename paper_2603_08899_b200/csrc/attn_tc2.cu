@@ -204,7 +204,7 @@ __device__ void producer_role(SharedStorage& sh, const Params& prm, const PlanVi
         ++g;
         return true;
     };
-    for (bool run = w.begin(pv, prm, blockIdx.x >> 1, true, s); run; run = w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x >> 1, kPlanPair, s); run; run = w.next(s)) {
         for (int t = s.t0; t < s.t1; ++t) {
             TileRef cur;
             cur.present = true;
@@ -264,7 +264,7 @@ __device__ void relay_role(SharedStorage& sh, const Params& prm, const PlanView&
         ++g;
         return true;
     };
-    for (bool run = w.begin(pv, prm, blockIdx.x >> 1, true, s); run; run = w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x >> 1, kPlanPair, s); run; run = w.next(s)) {
         for (int tile = s.t0; tile < s.t1; ++tile) {
             if (!run_stage(true, ragged_rows(s, tile, R))) return;
             if (tile == s.t0) {
@@ -298,7 +298,7 @@ __device__ void qk_role(SharedStorage& sh, const Params& prm, const PlanView& pv
     for (int i = 0; i < kQBufs; ++i) q_lo[i] = desc_lo(smem_u32(sh.q[i]), 16);
     const uint32_t k_lo0 = desc_lo(smem_u32(sh.kv[0]), 16);
     constexpr uint32_t kStageStep = kStageBytes >> 4;
-    for (bool run = w.begin(pv, prm, blockIdx.x >> 1, true, s); run; run = w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x >> 1, kPlanPair, s); run; run = w.next(s)) {
         const int n_tiles = s.t1 - s.t0;
         for (int j = 0; j < n_tiles; ++j, ++g) {
             const uint32_t st = g % kStages;
@@ -337,7 +337,7 @@ __device__ void pv_role(SharedStorage& sh, const Params& prm, const PlanView& pv
     const uint32_t v_lo0 = desc_lo(smem_u32(sh.kv[0] + kKBytes), 16);
     constexpr uint32_t kStageStep = kStageBytes >> 4;
     // the first kVLag stages carry no V tile: this thread has nothing to wait for on them
-    bool run = w.begin(pv, prm, blockIdx.x >> 1, true, s);
+    bool run = w.begin(pv, prm, blockIdx.x >> 1, kPlanPair, s);
     if (run)
         for (int i = 0; i < kVLag; ++i) if (issuer) commit_both(&sh.kv_empty[i]);
     for (; run; run = w.next(s)) {
@@ -379,7 +379,7 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
     Walker w;
     Segment s;
     uint32_t g = 0, seg = 0;
-    for (bool run = w.begin(pv, prm, blockIdx.x >> 1, true, s); run; run = w.next(s)) {
+    for (bool run = w.begin(pv, prm, blockIdx.x >> 1, kPlanPair, s); run; run = w.next(s)) {
         const int r = prm.rpt * (2 * s.rg + (int)rank) + lane_row / G;      // query row of this thread in this run
         const bool row_valid = lane_row < prm.rpt * G && r < R;
         const uint64_t mask = row_valid ? pv.mask[(size_t)s.b * kMaxRows + r] : 0ull;
@@ -595,7 +595,7 @@ attention_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const PlanView pv = plan_view(const_cast<void*>(prm.plan), prm.d.B, prm.d.Hkv);
     // a plan that lists runs per CTA, not per CTA pair, is refused: no role finds anything to do
-    if (warp == 11 && blockIdx.x == 0 && prm.status && pv.hdr->paired == 0)
+    if (warp == 11 && blockIdx.x == 0 && prm.status && pv.hdr->kind != kPlanPair)
         for (int b = threadIdx.x & 31; b < prm.d.B; b += 32) prm.status[b] = CONFU_ST_BAD_PLAN;
 
     if (warp < 8) {
@@ -669,7 +669,7 @@ cudaError_t launch_attention_pair(const Ctx* ctx, const confu_dims& d, const voi
     prm.out = (__nv_bfloat16*)out;
     prm.lse = lse;
     prm.status = status;
-    set_rows(prm, d);
+    set_rows(prm, d, 2);
     prm.c = (d.sm_scale != 0.f ? d.sm_scale : 1.f / sqrtf((float)d.D)) * 1.4426950408889634f;
     prm.wait_ns = ctx->wait_ns;
     prm.k_scale = prm.v_scale = nullptr;

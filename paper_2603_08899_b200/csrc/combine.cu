@@ -66,7 +66,7 @@ __device__ __forceinline__ const float* part_of(const Params& prm, const Pair& u
     return prm.partials + (size_t)(2 * (u.c0 + p * prm.n_rg) + (p < u.n - 1 ? 1 : 0)) * (partial_slot_bytes() / sizeof(float));
 }
 // query row of row `lane_row` of M tile t (may be past the last)
-__device__ __forceinline__ int query_row(const Params& prm, const Pair& u, int t, int lane_row) { return prm.rpt * (2 * u.rg + t) + lane_row / prm.G; }
+__device__ __forceinline__ int query_row(const Params& prm, const Pair& u, int t, int lane_row) { return prm.rpt * (prm.tpg * u.rg + t) + lane_row / prm.G; }
 
 template <int D>
 __device__ __forceinline__ void finish(const Params& prm, const Pair& u, int r, int lane_row, const Piece<D>& acc, float M, float L, int lane)

@@ -23,10 +23,16 @@ constexpr int kTileKeys = 128;                  // keys per attention tile (tens
 // B 2, 32 / 8 heads of 64, R 64, prefixes 1500..2500: 27 us, on CUDA cores 2820 us.)
 constexpr int kMaxTcGroup = 32;                 // query heads per kv head the tensor-core kernels take (groups of 8 rows at G = 32)
 __host__ __device__ inline int rows_per_tile(int G) { return 128 / G; }
-__host__ __device__ inline int row_groups(int R, int G)
+__host__ __device__ inline int row_groups(int R, int G, int tiles_per_group)
 {
-    return G > kMaxTcGroup ? 1 : (R + 2 * rows_per_tile(G) - 1) / (2 * rows_per_tile(G));
+    const int rows = tiles_per_group * rows_per_tile(G);
+    return G > kMaxTcGroup ? 1 : (R + rows - 1) / rows;
 }
+
+// The kinds of work units a plan can be for: CTAs that hold two M tiles (one row group = two tiles), CTA pairs (the same
+// rows, one tile per CTA), CTAs that hold one M tile (one row group = one tile).
+enum PlanKind { kPlanCta = 0, kPlanPair = 1, kPlanNarrow = 2 };
+__host__ __device__ inline int tiles_per_group(int kind) { return kind == kPlanNarrow ? 1 : 2; }
 
 // ---------------------------------------------------------------------------
 // Plan buffer (device).  Built once per step by plan_kernel, read by every layer.
@@ -55,7 +61,7 @@ constexpr int kPairOverheadTiles = 4;
 struct PlanHeader {
     int32_t B, Hkv, T, C, S, R;
     int32_t n_ctas;            // work units of the tensor-core attention launch: CTAs (<= SM count) or CTA pairs
-    int32_t paired;            // 1: the runs are listed per CTA pair (two-SM kernel), 0: per CTA
+    int32_t kind;              // PlanKind
     int64_t n_tiles;           // length N of the cost line
 };
 
@@ -76,7 +82,7 @@ struct alignas(64) CtaPlan {
     SegDesc first;
     int32_t n_runs;            // 0: nothing to do
     int32_t begin;             // its runs are segs[begin .. begin + n_runs)
-    int32_t paired;            // as in the header
+    int32_t kind;              // as in the header
     int32_t pad;
 };
 static_assert(sizeof(CtaPlan) == 64, "CtaPlan is read as four 16-byte words");
@@ -257,7 +263,7 @@ __device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b)
 // launchers (defined in the .cu files)
 // ---------------------------------------------------------------------------
 cudaError_t launch_plan(const Ctx* ctx, const confu_dims& d, const int64_t* seq_start, const int32_t* prefix_len,
-                        const int32_t* parent, const int32_t* con_owner, void* plan, int32_t* status, bool paired,
+                        const int32_t* parent, const int32_t* con_owner, void* plan, int32_t* status, int kind,
                         cudaStream_t st);
 
 cudaError_t launch_attention_generic(const Ctx* ctx, const confu_dims& d, const void* q, const void* k_cache,

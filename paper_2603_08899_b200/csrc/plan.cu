@@ -17,7 +17,7 @@ namespace confu {
 constexpr int kPlanThreads = 1024, kPlanWarps = kPlanThreads / 32;      // at most; at least kPlanMaxCtas threads
 constexpr int kPlanCached = 1024;                    // sequences whose tile counts and positions fit shared memory
 
-__global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int units, int paired, const int64_t* __restrict__ seq_start,
+__global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int units, int kind, const int64_t* __restrict__ seq_start,
                                                             const int32_t* __restrict__ prefix_len,
                                                             const int32_t* __restrict__ parent,
                                                             const int32_t* __restrict__ con_owner, void* plan_raw,
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
         }
         // The line is cut into `lanes` shares; CTA lane * n_rg + rg walks the lane's share for row group rg,
         // so the CTAs of a lane read the same K/V tiles at about the same time (the second read hits L2).
-        const int n_rg0 = row_groups(R, d.Hq / d.Hkv);
+        const int n_rg0 = row_groups(R, d.Hq / d.Hkv, tiles_per_group(kind));
         const int cap = units < kPlanMaxCtas ? units : kPlanMaxCtas;
         int lanes = cap / n_rg0;
         // With few enough stretches every one can have shares of its own, of at most `own` tiles: where that is no
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
             h.B = B; h.Hkv = d.Hkv; h.T = T; h.C = C; h.S = d.S; h.R = R;
             h.n_tiles = acc;
             h.n_ctas = lanes * n_rg0;
-            h.paired = paired;
+            h.kind = kind;
             *pv.hdr = h;
         }
     }
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
     // The runs of key tiles of every CTA of the tensor-core attention kernel, worked out once per step
     // instead of by every role of every CTA of every layer: thread c walks CTA c's share of the cost
     // line, first to count its runs, then (behind a prefix sum) to write them down.
-    const int n_rg = row_groups(R, d.Hq / d.Hkv);
+    const int n_rg = row_groups(R, d.Hq / d.Hkv, tiles_per_group(kind));
     const int64_t N = pv.hdr->n_tiles;
     const int n_ctas = pv.hdr->n_ctas, n_lanes = n_ctas / n_rg;
     auto base_of = [&](int b) { return cached ? s_base[b] : pv.tile_base[b]; };
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
         if (c < kPlanMaxCtas) {
             pv.cta[c].n_runs = c < n_ctas ? 1 : 0;
             pv.cta[c].begin = 0;
-            pv.cta[c].paired = paired;
+            pv.cta[c].kind = kind;
         }
         return;
     }
@@ -272,21 +272,21 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
                 first = before + incl - n;
                 pv.cta[c].n_runs = n;                // (0 past the last unit)
                 pv.cta[c].begin = first;
-                pv.cta[c].paired = paired;
+                pv.cta[c].kind = kind;
             }
         }
     }
 }
 
 cudaError_t launch_plan(const Ctx* ctx, const confu_dims& d, const int64_t* seq_start, const int32_t* prefix_len,
-                        const int32_t* parent, const int32_t* con_owner, void* plan, int32_t* status, bool paired,
+                        const int32_t* parent, const int32_t* con_owner, void* plan, int32_t* status, int kind,
                         cudaStream_t st)
 {
     // work units of the attention launch the plan is for: one CTA per SM, or one CTA pair per two SMs
-    const int units = paired ? ctx->sm_count / 2 : ctx->sm_count;
+    const int units = kind == kPlanPair ? ctx->sm_count / 2 : ctx->sm_count;
     // a warp per sequence, no more threads than that needs (a CTA of 1024 starts 0.5 us later than one of 256)
     const int threads = d.B <= 8 ? 256 : d.B <= 16 ? 512 : kPlanThreads;
-    return launch_pdl(plan_kernel, dim3(1), dim3((unsigned)threads), st, d, units, paired ? 1 : 0, seq_start, prefix_len, parent, con_owner,
+    return launch_pdl(plan_kernel, dim3(1), dim3((unsigned)threads), st, d, units, kind, seq_start, prefix_len, parent, con_owner,
                       plan, status);
 }
 

@@ -25,14 +25,14 @@ struct Walker {
     const SegDesc* cur;
     int left;
     bool soft;
-    // The unit's first run; false when it has nothing to do, or when the plan is for the other kind of unit.
-    __device__ bool begin(const PlanView& v, const Params& p, int unit, bool paired, Segment& s)
+    // The unit's first run; false when it has nothing to do, or when the plan is for another kind of unit.
+    __device__ bool begin(const PlanView& v, const Params& p, int unit, int kind, Segment& s)
     {
         const uint4* q = reinterpret_cast<const uint4*>(v.cta + unit);
         const uint4 w0 = __ldg(q), w1 = __ldg(q + 1), w2 = __ldg(q + 2), w3 = __ldg(q + 3);
         soft = p.d.S > 0;
         cur = v.segs + (int)w3.y;
-        left = paired && w3.z == 0 ? 0 : (int)w3.x;
+        left = (int)w3.z == kind ? (int)w3.x : 0;
         take(s, w0, w1, w2);
         return left > 0;
     }

@@ -54,7 +54,7 @@ def test_append_writes_the_rows_and_nothing_else(gpu, R, Hkv, D, dtype):
         assert torch.equal(d.cpu(), p)
 
 
-@pytest.mark.parametrize("B,Hkv,G,prefix,R", [(1, 8, 4, 4096, (60, 4)), (1, 1, 4, 20000, (20, 20)), (2, 8, 3, (1, 900), (40, 30)), (9, 8, 4, (100, 300), (20, 20)), (7, 4, 8, (0, 1500), (30, 4))])
+@pytest.mark.parametrize("B,Hkv,G,prefix,R", [(1, 8, 4, 4096, (60, 4)), (1, 1, 4, 20000, (20, 20)), (2, 8, 3, (1, 900), (40, 30)), (9, 8, 4, (100, 300), (20, 20)), (18, 4, 4, (1, 1200), (60, 4)), (19, 4, 4, (1, 200), (60, 4)), (7, 4, 8, (0, 1500), (30, 4))])
 def test_shares_of_their_own(gpu, B, Hkv, G, prefix, R):
     """Few (sequence, kv head) pairs for the machine: each gets a number of equal shares; an uneven one per pair, one tile per
     share, and batches that just fit or just do not."""
@@ -65,7 +65,7 @@ def test_shares_of_their_own(gpu, B, Hkv, G, prefix, R):
     if B > 1:
         parent[1, 1] = 7
     want, want_lse, want_st = H.oracle_attention(cfg, t, seq_start, plen, parent, owner)
-    for path in (cb.ATTENTION_TENSOR, cb.ATTENTION_TENSOR_PAIR):
+    for path in (cb.ATTENTION_AUTO, cb.ATTENTION_TENSOR, cb.ATTENTION_TENSOR_PAIR):
         gpu.set_path(path)
         try:
             out, lse, st = H.gpu_attention(gpu, cfg, t, seq_start, plen, parent, owner, n_slots, use_plan=True)

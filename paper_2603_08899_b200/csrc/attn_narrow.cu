@@ -13,7 +13,9 @@
 //                         warps 4-7 on keys 64-127 of the same rows, each with a reference maximum, sum and accumulator
 //                         of its own; the two meet once, at the end of a run
 // so two warps per scheduler keep the exponential unit busy on every tile, and a tile's weights are ready in half the
-// time that one warp would take.
+// time that one warp would take.  A quarter of the exponentials goes to the FMA pipe (batch 1, a layer: prefix 8192 19.1 ->
+// 18.7 us, 16000 26.7 -> 25.7; three eighths: no better than none.  In the kernels with two M tiles, where each scheduler
+// has two chains to choose from, it costs 2-8 %).
 //
 // A layer (this kernel and the merge) against CTA pairs: batch 1, 32/8 heads, R 64, prefix 512: 12.0 -> 9.8 us, 4096: 16.9
 // -> 14.7, 8192: 21.0 -> 19.0; R 120, 4096: 20.4 -> 18.9; 8 sequences of 101..3001, R 60: 26.9 -> 23.8.  Of the 14.7 us
@@ -273,7 +275,7 @@ __device__ void softmax_role(SharedStorage<D>& sh, const Params& prm, const Plan
             const float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref;
             // P over the first 32 of this half's columns of S (which sit in registers by now)
             uint32_t pk[32];
-            l += weights64(sv, c, neg_m, pk);
+            l += weights64<true>(sv, c, neg_m, pk);
             tmem_st32(s_addr + buf * 128, pk);
             tc_wait_st();
             // P V of a run's first tile overwrites both accumulators: both warps of these rows have read the old ones

@@ -259,6 +259,28 @@ __device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b)
     return r;
 }
 
+// 2^x of a pair on the FMA pipe, for x >= -126 (smaller arguments give 2^-126): x = n + f with n the nearest integer,
+// a polynomial of degree 5 for 2^f (interpolated at the Chebyshev nodes of [-1/2, 1/2]; relative error 2.2e-7, the
+// exponential unit's own is 1.2e-7), n into the exponent field.
+__device__ __forceinline__ void ex2_pair_fma(float& x0, float& x1)
+{
+    const uint64_t x = f2_pack(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
+    const uint64_t big = f2_pack(12582912.f, 12582912.f), nbig = f2_pack(-12582912.f, -12582912.f), neg1 = f2_pack(-1.f, -1.f);
+    const uint64_t t = f2_add(x, big);
+    const uint64_t f = f2_fma(f2_add(t, nbig), neg1, x);
+    auto c = [](float v) { return f2_pack(v, v); };
+    uint64_t p = f2_fma(f, c(0.0013390863f), c(0.009676032f));
+    p = f2_fma(p, f, c(0.05550357f));
+    p = f2_fma(p, f, c(0.24022107f));
+    p = f2_fma(p, f, c(0.6931472f));
+    p = f2_fma(p, f, c(1.0000001f));
+    float t0, t1, p0, p1;
+    f2_unpack(t, t0, t1);
+    f2_unpack(p, p0, p1);
+    x0 = __uint_as_float(__float_as_uint(p0) + (__float_as_uint(t0) << 23));
+    x1 = __uint_as_float(__float_as_uint(p1) + (__float_as_uint(t1) << 23));
+}
+
 // ---------------------------------------------------------------------------
 // launchers (defined in the .cu files)
 // ---------------------------------------------------------------------------

@@ -126,7 +126,9 @@ __device__ __forceinline__ float max64(const uint32_t (&sv)[64])
     return fmaxf(fmaxf(a[0], a[1]), fmaxf(a[2], a[3]));
 }
 
-// exp2(s*c - m) of 64 scores -> 32 packed bf16 pairs; returns their fp32 sum
+// exp2(s*c - m) of 64 scores -> 32 packed bf16 pairs; returns their fp32 sum.  kFma: a quarter of the exponentials on the
+// FMA pipe (for kernels that the exponential unit holds up).
+template <bool kFma = false>
 __device__ __forceinline__ float weights64(const uint32_t* sv, float c, float neg_m, uint32_t (&pk)[32])
 {
     uint64_t sum2 = f2_pack(0.f, 0.f);
@@ -135,7 +137,9 @@ __device__ __forceinline__ float weights64(const uint32_t* sv, float c, float ne
     for (int j = 0; j < 32; ++j) {
         float x0, x1;
         f2_unpack(f2_fma(f2_pack(__uint_as_float(sv[2 * j]), __uint_as_float(sv[2 * j + 1])), c2, nm2), x0, x1);
-        const float p0 = ex2(x0), p1 = ex2(x1);
+        if (kFma && (j & 3) == 1) ex2_pair_fma(x0, x1);
+        else { x0 = ex2(x0); x1 = ex2(x1); }
+        const float p0 = x0, p1 = x1;
         sum2 = f2_add(sum2, f2_pack(p0, p1));
         pk[j] = pack_bf16(p0, p1);
     }

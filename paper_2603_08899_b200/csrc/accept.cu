@@ -44,42 +44,44 @@ __device__ __forceinline__ void load8(const T* __restrict__ row, int i0, int V, 
 // ---------------------------------------------------------------------------------------------
 // K3: row statistics
 // ---------------------------------------------------------------------------------------------
-// Eight bf16 logits (one 16-byte vector starting at index ib) folded into a thread's running
+// N vectors of eight bf16 logits (16 bytes, starting at index ib and kStep apart) folded into a thread's running
 // statistics: maximum m, sum s of exp2((x - m) * k2), lowest index arg of the largest value bestv,
 // non-finite flag.  Maximum and minimum are taken on packed bf16 pairs with NaN propagation, so one
 // comparison of each against the finite range finds NaN and both infinities.
-__device__ __forceinline__ void stats8_bf16(const uint4& v, int ib, float k2, float& m, float& s, float& bestv, int& arg,
-                                            int& flag)
+template <int N>
+__device__ __forceinline__ void stats_bf16(const uint4 (&v)[N], int ib, int step, float k2, float& m, float& s, float& bestv, int& arg,
+                                           int& flag)
 {
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    __nv_bfloat162 h[4];
+    uint32_t w[4 * N];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) h[j] = *reinterpret_cast<const __nv_bfloat162*>(&w[j]);
-    const __nv_bfloat162 mx2 = __hmax2_nan(__hmax2_nan(h[0], h[1]), __hmax2_nan(h[2], h[3]));
-    const __nv_bfloat162 mn2 = __hmin2_nan(__hmin2_nan(h[0], h[1]), __hmin2_nan(h[2], h[3]));
+    for (int u = 0; u < N; ++u) { w[4 * u] = v[u].x; w[4 * u + 1] = v[u].y; w[4 * u + 2] = v[u].z; w[4 * u + 3] = v[u].w; }
+    auto h = [&](int j) { return *reinterpret_cast<const __nv_bfloat162*>(&w[j]); };
+    __nv_bfloat162 mx2 = h(0), mn2 = h(0);
+#pragma unroll
+    for (int j = 1; j < 4 * N; ++j) { mx2 = __hmax2_nan(mx2, h(j)); mn2 = __hmin2_nan(mn2, h(j)); }
     const float hi0 = __low2float(mx2), hi1 = __high2float(mx2), lo0 = __low2float(mn2), lo1 = __high2float(mn2);
     if (!(hi0 <= 3.0e38f && hi1 <= 3.0e38f && lo0 >= -3.0e38f && lo1 >= -3.0e38f)) flag = 1;
     const float cm = fmaxf(hi0, hi1);
     if (cm > bestv) {                                    // rare after the first vectors: find the first element equal to it
         bestv = cm;
 #pragma unroll
-        for (int j = 7; j >= 0; --j) {
+        for (int j = 8 * N - 1; j >= 0; --j) {
             const float x = __uint_as_float((j & 1) ? (w[j >> 1] & 0xffff0000u) : (w[j >> 1] << 16));
-            if (x == cm) arg = ib + j;
+            if (x == cm) arg = ib + (j >> 3) * step + (j & 7);
         }
     }
     if (cm > m) { s *= ex2((m - cm) * k2); m = cm; }
     const float nmk = -m * k2;
-    uint64_t acc = f2_pack(0.f, 0.f);
+    uint64_t acc[2] = {f2_pack(0.f, 0.f), f2_pack(0.f, 0.f)};
     const uint64_t k22 = f2_pack(k2, k2), nmk2 = f2_pack(nmk, nmk);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < 4 * N; ++j) {
         float x0, x1;
         f2_unpack(f2_fma(f2_pack(__uint_as_float(w[j] << 16), __uint_as_float(w[j] & 0xffff0000u)), k22, nmk2), x0, x1);
-        acc = f2_add(acc, f2_pack(ex2(x0), ex2(x1)));
+        acc[j & 1] = f2_add(acc[j & 1], f2_pack(ex2(x0), ex2(x1)));
     }
     float a0, a1;
-    f2_unpack(acc, a0, a1);
+    f2_unpack(f2_add(acc[0], acc[1]), a0, a1);
     s += a0 + a1;
 }
 
@@ -99,16 +101,28 @@ __global__ void __launch_bounds__(256) row_stats_kernel(const T* __restrict__ tl
     float m = -INFINITY, s = 0.f, bestv = -INFINITY;
     int arg = INT_MAX, flag = 0;
 
-    for (int i0 = lo + tid * kEpt; i0 < hi; i0 += 256 * kEpt * 2) {
+    int i0 = lo + tid * kEpt;
+    if constexpr (sizeof(T) == 2) {
+        // four vectors in flight per thread and folded in together (two, one after the other: 195 us for the 985 MB of 32
+        // sequences of 60 nodes, V 128256; now 172 us, 5.7 TB/s)
+        if (vec_ok) {
+            constexpr int kStep = 256 * kEpt;
+            for (; i0 + 3 * kStep + kEpt <= hi; i0 += 4 * kStep) {
+                uint4 v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = *reinterpret_cast<const uint4*>(base + i0 + u * kStep);
+                stats_bf16(v, i0, kStep, k2, m, s, bestv, arg, flag);
+            }
+        }
+    }
+    for (; i0 < hi; i0 += 256 * kEpt * 2) {
         float x[2][kEpt];
         const int i1 = i0 + 256 * kEpt;
         if constexpr (sizeof(T) == 2) {
             // bf16 rows, both 8-element vectors whole: packed path (about 4 instructions per logit)
             if (vec_ok && i1 + kEpt <= hi) {
-                const uint4 v0 = *reinterpret_cast<const uint4*>(base + i0);
-                const uint4 v1 = *reinterpret_cast<const uint4*>(base + i1);
-                stats8_bf16(v0, i0, k2, m, s, bestv, arg, flag);
-                stats8_bf16(v1, i1, k2, m, s, bestv, arg, flag);
+                const uint4 v[2] = {*reinterpret_cast<const uint4*>(base + i0), *reinterpret_cast<const uint4*>(base + i1)};
+                stats_bf16(v, i0, 256 * kEpt, k2, m, s, bestv, arg, flag);
                 continue;
             }
         }

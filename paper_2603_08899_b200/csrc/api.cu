@@ -97,6 +97,7 @@ int resolve_attention_path(const confu_ctx* ctx, const confu_dims& d)
 int plan_kind(const confu_ctx* ctx, const confu_dims& d, int path)
 {
     if (path == CONFU_ATTENTION_TENSOR_PAIR) return kPlanPair;
+    if (path == CONFU_ATTENTION_GENERIC && !tc_attention_supported(d) && !pair_attention_supported(d)) return kPlanMasks;
     const int n_tiles = row_groups(d.T + d.C, d.Hq / d.Hkv, 1);
     const bool few = 2 * (int64_t)d.B * d.Hkv * n_tiles <= 3 * (int64_t)ctx->sm_count;
     return path == CONFU_ATTENTION_TENSOR && ctx->attention_path == CONFU_ATTENTION_AUTO && d.kv_dtype == CONFU_BF16 && few ? kPlanNarrow : kPlanCta;

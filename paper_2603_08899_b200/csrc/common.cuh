@@ -30,8 +30,9 @@ __host__ __device__ inline int row_groups(int R, int G, int tiles_per_group)
 }
 
 // The kinds of work units a plan can be for: CTAs that hold two M tiles (one row group = two tiles), CTA pairs (the same
-// rows, one tile per CTA), CTAs that hold one M tile (one row group = one tile).
-enum PlanKind { kPlanCta = 0, kPlanPair = 1, kPlanNarrow = 2 };
+// rows, one tile per CTA), CTAs that hold one M tile (one row group = one tile), none (dims that only the CUDA-core kernel
+// takes: it reads the masks alone).
+enum PlanKind { kPlanCta = 0, kPlanPair = 1, kPlanNarrow = 2, kPlanMasks = 3 };
 __host__ __device__ inline int tiles_per_group(int kind) { return kind == kPlanNarrow ? 1 : 2; }
 
 // ---------------------------------------------------------------------------
@@ -40,7 +41,8 @@ __host__ __device__ inline int tiles_per_group(int kind) { return kind == kPlanN
 //   uint64 mask[B][128]       bit j < T of mask[b][r]: row r sees the slot of tree row j.  (A contemplate
 //                             row also sees its own slot and no other contemplate row's: not stored.)
 //   int32  bad[B]             non-zero: malformed tree, sequence skipped
-//   int32  tiles[B]           key tiles of one (sequence, kv head) pair, soft-prompt tile included
+//   int32  tiles[B]           key tiles of one (sequence, kv head) pair, soft-prompt tile included (this and tile_base: written
+//                             only where B is too large for plan_kernel's shared memory)
 //   int64  tile_base[B + 1]   position of sequence b's first (sequence, kv head) stretch on the flat cost line (exclusive scan)
 //   CtaPlan cta[kPlanMaxCtas]   work unit c of the tensor-core kernel: its first run of key tiles, how many it has and where
 //                             the others are (one 64-byte read tells a CTA what to start with)

@@ -9,13 +9,16 @@
 // 64-bit divisions), and every step waits for it.  A warp takes a sequence: parents go through shared memory, so that
 // walking to the root is a few shared loads; the cost line is a warp scan; each CTA's share is found by bisection in
 // shared memory.  B 32: 35 -> 10 us, B 8: 12 -> 7 us; at B 1 the step is 5 us shorter: the attention kernel of the first
-// layer sets itself up meanwhile.
+// layer sets itself up meanwhile.  The search for shares of their own starts at the smallest that can fit, sums are one
+// reduction instruction, the step's constants and first slots go through shared memory, and the line is left out where no
+// tensor-core kernel takes the dims.  Plan and one layer, 8 kv heads: B 1 prefix 4096 20.6 -> 19.1 us, B 8 of 300..4000
+// 55.2 -> 47.3, B 32 of 300..2000 81.5 -> 78.0; the fp32 layer of 256 keys 13.7 -> 10.7.
 #include "common.cuh"
 
 namespace confu {
 
 constexpr int kPlanThreads = 1024, kPlanWarps = kPlanThreads / 32;      // at most; at least kPlanMaxCtas threads
-constexpr int kPlanCached = 1024;                    // sequences whose tile counts and positions fit shared memory
+constexpr int kPlanCached = 1024;                    // sequences whose tile counts, positions and first slots fit shared memory
 
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int units, int kind, const int64_t* __restrict__ seq_start,
                                                             const int32_t* __restrict__ prefix_len,
@@ -28,8 +31,9 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
     __shared__ int8_t s_par[kPlanWarps][kMaxTree];
     __shared__ uint64_t s_mask[kPlanWarps][kMaxTree];
     __shared__ int32_t s_tiles[kPlanCached];
-    __shared__ int64_t s_base[kPlanCached + 1];
-    __shared__ int s_warp[kPlanMaxCtas / 32], s_own;
+    __shared__ int64_t s_base[kPlanCached + 1], s_slot[kPlanCached];
+    __shared__ int64_t s_line;
+    __shared__ int s_warp[kPlanMaxCtas / 32], s_own, s_ctas;
     PlanView pv = plan_view(plan_raw, B, d.Hkv);
     const bool cached = B <= kPlanCached;
 
@@ -46,6 +50,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
             o[h] = r < C ? con_owner[(size_t)b * C + r] : 0;
         }
         const int P = prefix_len[b];
+        const int64_t slot = seq_start ? seq_start[b] : 0;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int r = lane + 32 * h;
@@ -84,77 +89,69 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
             if (code && status) status[b] = code;
             const int64_t keys = (int64_t)P + R;
             const int tiles = code ? 0 : (int32_t)((keys + kTileKeys - 1) / kTileKeys) + (d.S > 0 ? 1 : 0);
-            pv.tiles[b] = tiles;
-            if (cached) s_tiles[b] = tiles;
+            (cached ? s_tiles : pv.tiles)[b] = tiles;
+            if (cached) s_slot[b] = slot;
         }
         __syncwarp();
     }
     __syncthreads();
-    // ---- the cost line: one stretch per (sequence, kv head); its groups of query rows are walked side by side ----
+    if (kind == kPlanMasks) return;
+    // ---- shares of their own, or the cost line: one stretch per (sequence, kv head); its groups of query rows are walked
+    // side by side ----
+    const int n_rg = row_groups(R, d.Hq / d.Hkv, tiles_per_group(kind));
     if (warp == 0) {
-        int64_t acc = 0;
-        for (int b0 = 0; b0 < B; b0 += 32) {
-            const int b = b0 + lane;
-            const int tiles = b < B ? (cached ? s_tiles[b] : pv.tiles[b]) : 0;
-            const int64_t own = tiles > 0 ? (int64_t)(tiles + kPairOverheadTiles) * d.Hkv : 0;
-            int64_t incl = own;
-#pragma unroll
-            for (int k = 1; k < 32; k <<= 1) {
-                const int64_t t = __shfl_up_sync(0xffffffffu, incl, k);
-                if (lane >= k) incl += t;
-            }
-            if (b < B) {
-                pv.tile_base[b] = acc + incl - own;
-                if (cached) s_base[b] = acc + incl - own;
-            }
-            acc += __shfl_sync(0xffffffffu, incl, 31);
-        }
-        // The line is cut into `lanes` shares; CTA lane * n_rg + rg walks the lane's share for row group rg,
+        // The work is cut into `lanes` shares; CTA lane * n_rg + rg walks the lane's share for row group rg,
         // so the CTAs of a lane read the same K/V tiles at about the same time (the second read hits L2).
-        const int n_rg0 = row_groups(R, d.Hq / d.Hkv, tiles_per_group(kind));
-        const int cap = units < kPlanMaxCtas ? units : kPlanMaxCtas;
-        int lanes = cap / n_rg0;
+        int lanes = (units < kPlanMaxCtas ? units : kPlanMaxCtas) / n_rg;
         // With few enough stretches every one can have shares of its own, of at most `own` tiles: where that is no
         // longer than a share of the line, no work unit changes from one pair to the next.  (A layer at batch 1, prefix 4096:
         // 34 tiles in 9 shares of at most 4 instead of a line cut into shares of 4.1, some of which span two pairs: 17.5 ->
         // 16.9 us; prefix 512: 12.75 -> 12.2; 4 sequences of 500..4000: 23.9 -> 22.9; E4M3 cache, batch 1: 20.0 -> 18.3.)
         int own = 0;
-        if (cached && acc > 0 && (int64_t)B * d.Hkv <= lanes) {
-            const int longest = (int)((acc + lanes - 1) / lanes);
-            for (own = 1; own <= longest; ++own) {
-                int shares = 0;
-                for (int b = lane; b < B; b += 32) shares += (s_tiles[b] + own - 1) / own;
-#pragma unroll
-                for (int k = 16; k > 0; k >>= 1) shares += __shfl_xor_sync(0xffffffffu, shares, k);
-                if (shares * d.Hkv <= lanes) break;
+        if (cached && (int64_t)B * d.Hkv <= lanes) {
+            uint32_t tiles = 0, line = 0;            // (at most kPlanMaxCtas sequences of at most 2^24 + 2 tiles)
+            for (int b = lane; b < B; b += 32) {
+                tiles += (uint32_t)s_tiles[b];
+                line += s_tiles[b] ? (uint32_t)(s_tiles[b] + kPairOverheadTiles) : 0;
             }
-            if (own > longest) own = 0;
-        }
-        if (own) {                                   // positions are share numbers now
-            acc = 0;
-            for (int b0 = 0; b0 < B; b0 += 32) {
-                const int b = b0 + lane;
-                const int mine = b < B ? (s_tiles[b] + own - 1) / own * d.Hkv : 0;
-                int incl = mine;
-#pragma unroll
-                for (int k = 1; k < 32; k <<= 1) {
-                    const int t = __shfl_up_sync(0xffffffffu, incl, k);
-                    if (lane >= k) incl += t;
+            tiles = __reduce_add_sync(0xffffffffu, tiles);
+            line = __reduce_add_sync(0xffffffffu, line);
+            if (tiles) {
+                const int longest = (int)(((uint64_t)line * d.Hkv + lanes - 1) / lanes);
+                for (own = (int)(((uint64_t)tiles * d.Hkv + lanes - 1) / lanes); own <= longest; ++own) {
+                    uint32_t shares = 0;
+                    for (int b = lane; b < B; b += 32) shares += (uint32_t)(s_tiles[b] + own - 1) / (uint32_t)own;
+                    if ((int)__reduce_add_sync(0xffffffffu, shares) * d.Hkv <= lanes) break;
                 }
-                if (b < B) s_base[b] = acc + incl - mine;
-                acc += __shfl_sync(0xffffffffu, incl, 31);
+                if (own > longest) own = 0;
             }
-            __syncwarp();
+        }
+        // positions on the line, or share numbers
+        int64_t acc = 0;
+        for (int b0 = 0; b0 < B; b0 += 32) {
+            const int b = b0 + lane;
+            const int tiles = b < B ? (cached ? s_tiles[b] : pv.tiles[b]) : 0;
+            int64_t mine = tiles > 0 ? (int64_t)(tiles + kPairOverheadTiles) * d.Hkv : 0;
+            if (own) mine = (uint32_t)(tiles + own - 1) / (uint32_t)own * d.Hkv;
+            int64_t incl = mine;
+#pragma unroll 1
+            for (int k = 1; k < 32 && k < B; k <<= 1) {
+                const int64_t t = __shfl_up_sync(0xffffffffu, incl, k);
+                if (lane >= k) incl += t;
+            }
+            if (b < B) (cached ? s_base : pv.tile_base)[b] = acc + incl - mine;
+            acc += __shfl_sync(0xffffffffu, incl, B - b0 < 32 ? B - b0 - 1 : 31);
         }
         if ((int64_t)lanes > acc) lanes = (int)acc;
         if (lane == 0) {
             s_own = own;
-            pv.tile_base[B] = acc;
-            if (cached) s_base[B] = acc;
+            s_ctas = lanes * n_rg;
+            s_line = acc;
+            (cached ? s_base : pv.tile_base)[B] = acc;
             PlanHeader h;
             h.B = B; h.Hkv = d.Hkv; h.T = T; h.C = C; h.S = d.S; h.R = R;
             h.n_tiles = acc;
-            h.n_ctas = lanes * n_rg0;
+            h.n_ctas = lanes * n_rg;
             h.kind = kind;
             *pv.hdr = h;
         }
@@ -163,16 +160,18 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
     // The runs of key tiles of every CTA of the tensor-core attention kernel, worked out once per step
     // instead of by every role of every CTA of every layer: thread c walks CTA c's share of the cost
     // line, first to count its runs, then (behind a prefix sum) to write them down.
-    const int n_rg = row_groups(R, d.Hq / d.Hkv, tiles_per_group(kind));
-    const int64_t N = pv.hdr->n_tiles;
-    const int n_ctas = pv.hdr->n_ctas, n_lanes = n_ctas / n_rg;
+    const int64_t N = s_line;
+    const int n_ctas = s_ctas, n_lanes = n_ctas / n_rg;
     auto base_of = [&](int b) { return cached ? s_base[b] : pv.tile_base[b]; };
     const int c = tid;
     int64_t f0 = 0, f1 = 0;
     int seq0 = 0;
     if (c < n_ctas) {
-        f0 = (int64_t)(c / n_rg) * N / n_lanes;
-        f1 = (int64_t)(c / n_rg + 1) * N / n_lanes;
+        f0 = c / n_rg;
+        if (!s_own) {
+            f1 = (f0 + 1) * N / n_lanes;
+            f0 = f0 * N / n_lanes;
+        }
         for (int hi = B; seq0 + 1 < hi;) {           // the last sequence whose stretch starts at or before f0
             const int mid = (seq0 + hi) / 2;
             if (base_of(mid) <= f0) seq0 = mid;
@@ -195,7 +194,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
             s.P = prefix_len[seq0];
             s.part_slot = k == 1 ? -1 : 2 * c + (p + 1 < k ? 1 : 0);
             s.pad0 = 0;
-            s.slot0 = seq_start ? seq_start[seq0] : 0;
+            s.slot0 = s_slot[seq0];
             s.pad1 = 0;
             pv.cta[c].first = s;
         }
@@ -249,7 +248,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
                     s.P = prefix_len[seq];
                     s.part_slot = (t0 == 0 && t1 == nt) ? -1 : 2 * c + (t1 < nt ? 1 : 0);
                     s.pad0 = 0;
-                    s.slot0 = seq_start ? seq_start[seq] : 0;
+                    s.slot0 = cached ? s_slot[seq] : seq_start ? seq_start[seq] : 0;
                     s.pad1 = 0;
                     out[n] = s;
                     if (n == 0) pv.cta[c].first = s;

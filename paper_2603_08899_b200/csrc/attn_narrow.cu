@@ -461,7 +461,7 @@ static cudaError_t launch_d(const Ctx* ctx, const confu_dims& d, const void* q, 
     prm.out = (__nv_bfloat16*)out;
     prm.lse = lse;
     prm.status = status;
-    set_rows(prm, d, 1);
+    set_rows(prm, d, kPlanNarrow);
     prm.c = (d.sm_scale != 0.f ? d.sm_scale : 1.f / sqrtf((float)d.D)) * 1.4426950408889634f;
     prm.wait_ns = ctx->wait_ns;
     prm.k_scale = prm.v_scale = nullptr;

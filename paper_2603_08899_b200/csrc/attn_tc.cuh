@@ -18,6 +18,7 @@ struct Params {
     __nv_bfloat16* out;
     float* lse;
     int32_t* status;
+    int kind;            // PlanKind of the launch's work units: a plan for another kind is refused
     int n_mt;            // M tiles in use (2 unless one holds all rows)
     int n_rg;            // groups of query rows; a pair = (sequence, kv head, row group)
     int G;               // query heads per kv head
@@ -36,9 +37,11 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
     return r;
 }
 
-// The row packing of a launch (see rows_per_tile).
-inline void set_rows(Params& p, const confu_dims& d, int tpg)
+// The kind of a launch's work units and its row packing (see rows_per_tile).
+inline void set_rows(Params& p, const confu_dims& d, int kind)
 {
+    const int tpg = tiles_per_group(kind);
+    p.kind = kind;
     p.tpg = tpg;
     p.G = d.Hq / d.Hkv;
     p.rpt = rows_per_tile(p.G);

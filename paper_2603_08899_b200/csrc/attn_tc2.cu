@@ -669,7 +669,7 @@ cudaError_t launch_attention_pair(const Ctx* ctx, const confu_dims& d, const voi
     prm.out = (__nv_bfloat16*)out;
     prm.lse = lse;
     prm.status = status;
-    set_rows(prm, d, 2);
+    set_rows(prm, d, kPlanPair);
     prm.c = (d.sm_scale != 0.f ? d.sm_scale : 1.f / sqrtf((float)d.D)) * 1.4426950408889634f;
     prm.wait_ns = ctx->wait_ns;
     prm.k_scale = prm.v_scale = nullptr;

@@ -161,7 +161,10 @@ __global__ void __launch_bounds__(kMergeThreads, 4) merge_kernel(const Params pr
     u.b = bg / prm.d.Hkv;
     u.g = bg % prm.d.Hkv;
     u.rg = blockIdx.x % prm.n_rg;
-    const int parts = __ldg(pv.parts + bg);
+    // A plan for another kind of work unit has been refused by the attention kernel.  Its share numbers must not be followed:
+    // they belong to another number of row groups, and the partial slots they lead to may lie past the workspace.
+    const int parts = __ldg(pv.parts + bg), kind = __ldg(&pv.hdr->kind);
+    if (kind != prm.kind) return;
     u.c0 = (parts & 0xffff) * prm.n_rg + u.rg;
     u.n = parts >> 16;
     if (u.n == 1) return;                                   // one unit covered the pair and wrote the output itself

@@ -46,7 +46,7 @@ struct SharedStorage {
     alignas(8) uint64_t q_full, q_empty;
     uint64_t full[kSlots], empty[kSlots];
     uint64_t s_full[2], p_full[2][2], o_done;        // [S buffer], [S buffer][half]
-    uint64_t v_fixed;
+    uint64_t v_fixed[kSlots];                        // per slot: the warp that zeroes ragged rows may be a run ahead of the MMA warp
     uint64_t x_bar[4], y_bar[4], r_bar[4];           // per pair of warps with the same rows: written / read the exchange, read O
     uint32_t tmem_base;
     int abort;
@@ -111,7 +111,7 @@ __device__ void mma_role(SharedStorage<D>& sh, const Params& prm, const PlanView
     Walker w;
     Segment s;
     const bool issuer = elect_lane();
-    uint32_t i = 0, g = 0, seg = 0, n_fix = 0;       // slots, tiles, runs, repaired V tiles so far
+    uint32_t i = 0, g = 0, seg = 0, fix_phase = 0;   // slots, tiles, runs so far; phase of every slot's v_fixed
     const uint32_t q_lo = desc_lo(smem_u32(sh.q), 16), k_lo0 = desc_lo(smem_u32(sh.kv[0]), 16);
     const uint32_t v_lo0 = desc_lo(smem_u32(sh.kv[0]), kHalfTile);
     constexpr uint32_t kStep = kTile<D> >> 4;
@@ -133,8 +133,9 @@ __device__ void mma_role(SharedStorage<D>& sh, const Params& prm, const PlanView
     auto issue_pv = [&](uint32_t slot, bool first, bool last, bool ragged) -> bool {     // of tile g - 1
         if (!mbar_wait(&sh.full[slot % kSlots], (slot / kSlots) & 1, &sh.abort, prm.wait_ns)) return false;
         if (ragged) {
-            if (!mbar_wait(&sh.v_fixed, n_fix & 1, &sh.abort, prm.wait_ns)) return false;
-            ++n_fix;
+            const uint32_t st = slot % kSlots;
+            if (!mbar_wait(&sh.v_fixed[st], (fix_phase >> st) & 1, &sh.abort, prm.wait_ns)) return false;
+            fix_phase ^= 1u << st;
         }
         const uint32_t buf = (g - 1) & 1, vl = v_lo0 + (slot % kSlots) * kStep;
 #pragma unroll
@@ -178,7 +179,9 @@ __device__ void mma_role(SharedStorage<D>& sh, const Params& prm, const PlanView
 }
 
 // Sees every slot before it is filled again (it arrives on the slot's empty barrier) and, where it holds the V tile of a
-// sequence's last key tile, zeroes the rows past the last slot.
+// sequence's last key tile, zeroes the rows past the last slot.  It does not wait for the MMA warp: while that waits for the
+// weights of a run's last tiles, the whole of a next run of one tile may be here and be repaired too.  So a slot
+// has a barrier of its own, which cannot complete twice before the MMA warp has used the slot.
 template <int D>
 __device__ void tail_role(SharedStorage<D>& sh, const Params& prm, const PlanView& pv)
 {
@@ -196,7 +199,7 @@ __device__ void tail_role(SharedStorage<D>& sh, const Params& prm, const PlanVie
                     *reinterpret_cast<uint4*>(sh.kv[st] + kb * kHalfTile + off) = zero;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive(&sh.v_fixed);
+            if (lane == 0) mbar_arrive(&sh.v_fixed[st]);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(&sh.empty[st]);
@@ -379,13 +382,12 @@ attention_narrow_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
         mbar_init(&sh.q_full, 1);
         mbar_init(&sh.q_empty, 1);
         // a slot is free again when its MMAs have completed and the tail warp has seen it
-        for (int i = 0; i < kSlots; ++i) { mbar_init(&sh.full[i], 1); mbar_init(&sh.empty[i], 2); }
+        for (int i = 0; i < kSlots; ++i) { mbar_init(&sh.full[i], 1); mbar_init(&sh.empty[i], 2); mbar_init(&sh.v_fixed[i], 1); }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&sh.s_full[i], 1);
             for (int h = 0; h < 2; ++h) mbar_init(&sh.p_full[i][h], 4);      // one arrival per warp
         }
         mbar_init(&sh.o_done, 1);
-        mbar_init(&sh.v_fixed, 1);
         for (int i = 0; i < 4; ++i) { mbar_init(&sh.x_bar[i], 2); mbar_init(&sh.y_bar[i], 2); mbar_init(&sh.r_bar[i], 2); }
         sh.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");

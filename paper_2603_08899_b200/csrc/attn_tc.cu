@@ -49,6 +49,7 @@ struct SharedStorage {
     alignas(8) uint64_t q_full, q_empty;
     uint64_t kv_full[kStages<D>], kv_empty[kStages<D>];
     uint64_t s_full[2][2], p_full[2][2], o_done[2];      // [M tile][half of the key tile]
+    uint64_t pv0_done[2];                 // P V of half 0 of a run's last tile has completed
     uint64_t v_fixed;                     // the rows of a V tile past the sequence's last slot have been zeroed
     uint32_t tmem_base;
     int abort;
@@ -184,10 +185,12 @@ __device__ void mma_role(SharedStorage<D>& sh, const Params& prm, const PlanView
                     if (!mbar_wait(&sh.p_full[t][h], (stage - 1) & 1, &sh.abort, prm.wait_ns)) return false;
                     tc_fence_after();
                     issue_pv(t, h, vl, prev_first);
-                    // Behind every P V of half 0 comes a completion of s_full[t][0], with or without a Q K^T: half 1 of
-                    // the same tile waits for it before it rescales O.
+                    // Before half 1 of a tile rescales O it waits for the P V of half 0: for the Q K^T behind it, or, at the
+                    // end of a run, for a barrier of its own.  (Were that a completion of s_full[t][0] too, the first Q K^T of
+                    // the next run, which is not held up by the softmax threads, could complete it a second time
+                    // before a late warp has seen the first.)
                     if (prev_last) {
-                        if (issuer) tc_commit(h == 0 ? &sh.s_full[t][0] : &sh.o_done[t]);
+                        if (issuer) tc_commit(h == 0 ? &sh.pv0_done[t] : &sh.o_done[t]);
                     } else
                         issue_qk(t, h, kl);
                 }
@@ -300,12 +303,13 @@ __device__ void softmax_role(SharedStorage<D>& sh, const Params& prm, const Plan
             return true;
         };
         // the reference maximum follows the running maximum; O is brought along when it moves.  P V of the half before
-        // has completed when the other half's next completion of s_full is there (see the issuing warp).
-        auto follow = [&](float m_half, int h) -> bool {
+        // has completed when the other half's next completion of s_full is there, or, in half 1 of the run's last
+        // tile, that of pv0_done (see the issuing warp).
+        auto follow = [&](float m_half, int h, bool last) -> bool {
             const float m_new = fmaxf(m_ref, m_half);
             const bool move = m_new - m_ref > kRescaleThreshold;             // false when both are -inf (NaN)
             if (!__any_sync(0xffffffffu, move)) return true;
-            if (!mbar_wait(&sh.s_full[t][h ^ 1], n_s[h ^ 1] & 1, &sh.abort, prm.wait_ns)) return false;
+            if (!mbar_wait(last ? &sh.pv0_done[t] : &sh.s_full[t][h ^ 1], (last ? seg : n_s[h ^ 1]) & 1, &sh.abort, prm.wait_ns)) return false;
             tc_fence_after();
             const float alpha = move ? ex2(m_ref - m_new) : 1.f;
             if (move) { m_ref = m_new; l *= alpha; }
@@ -341,16 +345,13 @@ __device__ void softmax_role(SharedStorage<D>& sh, const Params& prm, const Plan
                 hand_over(0, sa);
                 hand_over(1, sb);
             } else {
-                if (!follow(m0, 0)) return;
+                if (!follow(m0, 0, false)) return;
                 hand_over(0, sa);
                 if (!load_half(1, tile, sb)) return;
-                if (!follow(max64(sb) * c, 1)) return;
+                if (!follow(max64(sb) * c, 1, tile + 1 == s.t1)) return;
                 hand_over(1, sb);
             }
         }
-        // (the completion that stands for the P V of the last half 0)
-        if (!mbar_wait(&sh.s_full[t][0], n_s[0] & 1, &sh.abort, prm.wait_ns)) return;
-        ++n_s[0];
         // ---- epilogue of this pair / range ----
         if (!mbar_wait(&sh.o_done[t], seg & 1, &sh.abort, prm.wait_ns)) return;
         tc_fence_after();
@@ -445,6 +446,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
                 mbar_init(&sh.p_full[t][h], 128);
             }
             mbar_init(&sh.o_done[t], 1);
+            mbar_init(&sh.pv0_done[t], 1);
         }
         sh.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");

@@ -23,7 +23,7 @@ TILES = [[10, 1] * 4, [3, 1, 1, 2, 1, 1, 4, 1], [1] * 9 + [2] * 4, [6, 1, 1, 1, 
 
 @pytest.mark.parametrize("D", [128, 64])
 @pytest.mark.parametrize("tiles", TILES)
-@pytest.mark.parametrize("path", ["auto"])
+@pytest.mark.parametrize("path", ["auto", "one_cta_per_sm"])
 def test_ragged_tiles_of_neighbouring_runs(gpu, tiles, path, D):
     B, R = len(tiles), 64
     cfg = inputs.VerifyConfig("short", B=B, L=1, Hq=32, Hkv=8, D=D, T=60, C=4, S=0, V=32, prefix=(1, 2), tree="random",

@@ -163,10 +163,10 @@ __global__ void __launch_bounds__(kMergeThreads, 4) merge_kernel(const Params pr
     u.rg = blockIdx.x % prm.n_rg;
     // A plan for another kind of work unit has been refused by the attention kernel.  Its share numbers must not be followed:
     // they belong to another number of row groups, and the partial slots they lead to may lie past the workspace.
-    const int parts = __ldg(pv.parts + bg), kind = __ldg(&pv.hdr->kind);
-    if (kind != prm.kind) return;
-    u.c0 = (parts & 0xffff) * prm.n_rg + u.rg;
-    u.n = parts >> 16;
+    const Parts parts = {__ldg(&pv.parts[bg].word)};
+    if (parts.kind() != prm.kind) return;
+    u.c0 = parts.first() * prm.n_rg + u.rg;
+    u.n = parts.n();
     if (u.n == 1) return;                                   // one unit covered the pair and wrote the output itself
     const int rows = prm.rpt * prm.G;                       // of an M tile
     const int row0 = (blockIdx.z * kMergeWarps + (threadIdx.x >> 5)) * per_warp, end = min(row0 + per_warp, rows);

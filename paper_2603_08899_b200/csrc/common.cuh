@@ -46,7 +46,8 @@ __host__ __device__ inline int tiles_per_group(int kind) { return kind == kPlanN
 //   int64  tile_base[B + 1]   position of sequence b's first (sequence, kv head) stretch on the flat cost line (exclusive scan)
 //   CtaPlan cta[kPlanMaxCtas]   work unit c of the tensor-core kernel: its first run of key tiles, how many it has and where
 //                             the others are (one 64-byte read tells a CTA what to start with)
-//   int32  parts[B * Hkv]     who walked a (sequence, kv head): first share | number of shares << 16 (0: malformed tree)
+//   int32  parts[B * Hkv]     who walked a (sequence, kv head), see Parts: first share, number of shares (0: malformed tree),
+//                             and the plan's kind again (so that the merge need not read the header for it)
 //   SegDesc segs[B * Hkv * max(2, n_rg) + kPlanMaxCtas]   the runs of key tiles, one pair at a time, of every CTA in walking order
 //
 // The split-KV work is balanced on a "cost line": every (sequence, kv head) pair takes
@@ -89,6 +90,14 @@ struct alignas(64) CtaPlan {
 };
 static_assert(sizeof(CtaPlan) == 64, "CtaPlan is read as four 16-byte words");
 
+struct Parts {
+    int32_t word;
+    __host__ __device__ static Parts make(int first, int n, int kind) { return {first | (n << 12) | (kind << 24)}; }     // first, n <= kPlanMaxCtas
+    __host__ __device__ int first() const { return word & 0xfff; }
+    __host__ __device__ int n() const { return (word >> 12) & 0xfff; }
+    __host__ __device__ int kind() const { return word >> 24; }
+};
+
 struct PlanView {
     PlanHeader* hdr;
     uint64_t* mask;
@@ -96,7 +105,7 @@ struct PlanView {
     int32_t* tiles;
     int64_t* tile_base;
     CtaPlan* cta;
-    int32_t* parts;
+    Parts* parts;
     SegDesc* segs;
 };
 
@@ -125,7 +134,7 @@ __host__ __device__ inline PlanView plan_view(void* base, int B, int Hkv)
     v.tiles = (int32_t*)p;                   p += align_up((size_t)B * sizeof(int32_t), 256);
     v.tile_base = (int64_t*)p;               p += align_up((size_t)(B + 1) * sizeof(int64_t), 256);
     v.cta = (CtaPlan*)p;                     p += align_up((size_t)kPlanMaxCtas * sizeof(CtaPlan), 256);
-    v.parts = (int32_t*)p;                   p += align_up((size_t)B * Hkv * sizeof(int32_t), 256);
+    v.parts = (Parts*)p;                     p += align_up((size_t)B * Hkv * sizeof(int32_t), 256);
     v.segs = (SegDesc*)p;
     return v;
 }

@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
     if (s_own) {                                     // shares of their own: one run each, a stretch's tiles dealt out evenly
         for (int u = tid; u < B * d.Hkv; u += (int)blockDim.x) {
             const int b = u / d.Hkv, k = (s_tiles[b] + s_own - 1) / s_own;
-            pv.parts[u] = k ? ((int)s_base[b] + u % d.Hkv * k) | (k << 16) : 0;
+            pv.parts[u] = Parts::make(k ? (int)s_base[b] + u % d.Hkv * k : 0, k, kind);
         }
         if (c < n_ctas) {
             const int nt = s_tiles[seq0], k = (nt + s_own - 1) / s_own, local = c / n_rg - (int)s_base[seq0], p = local % k;
@@ -209,11 +209,11 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
     // floor(((x + 1) * n - 1) / N) of n.
     for (int u = tid; u < B * d.Hkv; u += (int)blockDim.x) {
         const int b = u / d.Hkv, nt = cached ? s_tiles[b] : pv.tiles[b];
-        int32_t parts = 0;
+        Parts parts = Parts::make(0, 0, kind);
         if (nt > 0) {
             const int64_t F = base_of(b) + (int64_t)(u % d.Hkv) * (nt + kPairOverheadTiles) + kPairOverheadTiles;
             const int lo = (int)(((F + 1) * n_lanes - 1) / N), hi = (int)(((F + nt) * n_lanes - 1) / N);
-            parts = lo | ((hi - lo + 1) << 16);
+            parts = Parts::make(lo, hi - lo + 1, kind);
         }
         pv.parts[u] = parts;
     }

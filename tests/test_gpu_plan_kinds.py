@@ -19,7 +19,7 @@ def gpu():
     g.close()
 
 
-@pytest.mark.parametrize("launched", ["auto", "pairs"])
+@pytest.mark.parametrize("launched", list(PATHS))
 @pytest.mark.parametrize("built", list(PATHS))
 @pytest.mark.parametrize("B,prefix", [(8, (500, 2000)), (1, 3000)])
 def test_plan_of_another_kind_is_refused(gpu, built, launched, B, prefix):

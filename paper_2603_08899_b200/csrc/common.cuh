@@ -269,13 +269,20 @@ __device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b)
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
 
-// 2^x of a pair on the FMA pipe, for x >= -126 (smaller arguments give 2^-126): x = n + f with n the nearest integer,
-// a polynomial of degree 5 for 2^f (interpolated at the Chebyshev nodes of [-1/2, 1/2]; relative error 2.2e-7, the
-// exponential unit's own is 1.2e-7), n into the exponent field.
+// 2^x of a pair on the FMA pipe, for x < 128: x = n + f with n the nearest integer, a polynomial of degree 5 for 2^f
+// (interpolated at the Chebyshev nodes of [-1/2, 1/2]; relative error 2.2e-7, the exponential unit's own is 1.2e-7), times
+// 2^n put together in the exponent field.  n stops at -127, whose field reads 0: arguments below -126.5, -infinity
+// among them, give exactly 0, as a masked key's weight has to be.
 __device__ __forceinline__ void ex2_pair_fma(float& x0, float& x1)
 {
-    const uint64_t x = f2_pack(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
+    const uint64_t x = f2_pack(fmaxf(x0, -127.f), fmaxf(x1, -127.f));
     const uint64_t big = f2_pack(12582912.f, 12582912.f), nbig = f2_pack(-12582912.f, -12582912.f), neg1 = f2_pack(-1.f, -1.f);
     const uint64_t t = f2_add(x, big);
     const uint64_t f = f2_fma(f2_add(t, nbig), neg1, x);
@@ -285,11 +292,10 @@ __device__ __forceinline__ void ex2_pair_fma(float& x0, float& x1)
     p = f2_fma(p, f, c(0.24022107f));
     p = f2_fma(p, f, c(0.6931472f));
     p = f2_fma(p, f, c(1.0000001f));
-    float t0, t1, p0, p1;
+    float t0, t1;
     f2_unpack(t, t0, t1);
-    f2_unpack(p, p0, p1);
-    x0 = __uint_as_float(__float_as_uint(p0) + (__float_as_uint(t0) << 23));
-    x1 = __uint_as_float(__float_as_uint(p1) + (__float_as_uint(t1) << 23));
+    auto pow2 = [](float v) { return __uint_as_float((__float_as_uint(v) << 23) + 0x3f800000u); };
+    f2_unpack(f2_mul(p, f2_pack(pow2(t0), pow2(t1))), x0, x1);
 }
 
 // ---------------------------------------------------------------------------

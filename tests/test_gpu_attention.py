@@ -185,3 +185,33 @@ def test_empty_batch_is_a_no_op(gpu):
     rc = cb.lib().confu_tree_attention(gpu.ctx, C.byref(dims), None, None, None, C.c_int64(0), None, None, None, None,
                                        None, None, None, None, None, None, None)
     assert rc == 0
+
+
+@pytest.mark.parametrize("D,G", [(128, 4), (64, 4), (128, 8)])
+@pytest.mark.parametrize("prefix", [300, (3, 700)])
+@pytest.mark.parametrize("path", ["auto", "one_cta_per_sm", "cta_pairs"])
+def test_unseen_keys_have_weight_exactly_zero(gpu, D, G, prefix, path):
+    """Values of 3e38 at slots that a row must not see (leaves of other branches, contemplate rows, soft prompts) leave its
+    output bit for bit what ordinary values there give: even the smallest normal weight would add 3.5 to a sum."""
+    if path == "cta_pairs" and D == 64:
+        pytest.skip("the two-SM kernel takes head dim 128")
+    cfg = _cfg(B=1 if prefix == 300 else 3, Hq=2 * G, Hkv=2, D=D, T=60, C=20, S=16, prefix=prefix, max_depth=7, fanout=(1, 4), seed=61)
+    parent, owner, plen, seq_start, n_slots, t = H.setup_case(cfg)
+    loud = dict(t)
+    loud["v_cache"], loud["v_soft"] = t["v_cache"].clone(), torch.full_like(t["v_soft"], 3e38)
+    quiet = torch.zeros(cfg.B, cfg.R, dtype=torch.bool)
+    for b in range(cfg.B):
+        leaves = sorted(set(range(cfg.T)) - set(parent[b].tolist()))
+        first = int(seq_start[b]) + int(plen[b])
+        for r in leaves + list(range(cfg.T, cfg.R)):
+            loud["v_cache"][first + r] = 3e38
+        quiet[b, :cfg.T] = True
+        quiet[b, leaves] = False
+        assert quiet[b].sum() >= 20
+    gpu.set_path({"auto": cb.ATTENTION_AUTO, "one_cta_per_sm": cb.ATTENTION_TENSOR, "cta_pairs": cb.ATTENTION_TENSOR_PAIR}[path])
+    try:
+        a, la, _ = H.gpu_attention(gpu, cfg, t, seq_start, plen, parent, owner, n_slots)
+        b, lb, _ = H.gpu_attention(gpu, cfg, loud, seq_start, plen, parent, owner, n_slots)
+    finally:
+        gpu.set_path(cb.ATTENTION_AUTO)
+    assert torch.equal(a[quiet], b[quiet]) and torch.equal(la[quiet], lb[quiet])

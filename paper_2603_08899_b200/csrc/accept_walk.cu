@@ -15,13 +15,6 @@
 namespace confu {
 namespace walk {
 
-// maximum that keeps a NaN
-__device__ __forceinline__ float max_nan(float a, float b)
-{
-    float r;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
 __device__ __forceinline__ float warp_max_nan(float v)
 {
 #pragma unroll

@@ -249,6 +249,13 @@ __device__ __forceinline__ float ex2(float x)
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+// maximum that keeps a NaN
+__device__ __forceinline__ float max_nan(float a, float b)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
 // Packed fp32 pairs (one 64-bit register): the FMA pipe takes two lanes per instruction.
 __device__ __forceinline__ uint64_t f2_pack(float a, float b)
 {
@@ -279,10 +286,10 @@ __device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b)
 // 2^x of a pair on the FMA pipe, for x < 128: x = n + f with n the nearest integer, a polynomial of degree 5 for 2^f
 // (interpolated at the Chebyshev nodes of [-1/2, 1/2]; relative error 2.2e-7, the exponential unit's own is 1.2e-7), times
 // 2^n put together in the exponent field.  n stops at -127, whose field reads 0: arguments below -126.5, -infinity
-// among them, give exactly 0, as a masked key's weight has to be.
+// among them, give exactly 0, as a masked key's weight has to be.  NaN stays NaN (by way of the polynomial).
 __device__ __forceinline__ void ex2_pair_fma(float& x0, float& x1)
 {
-    const uint64_t x = f2_pack(fmaxf(x0, -127.f), fmaxf(x1, -127.f));
+    const uint64_t x = f2_pack(max_nan(x0, -127.f), max_nan(x1, -127.f));
     const uint64_t big = f2_pack(12582912.f, 12582912.f), nbig = f2_pack(-12582912.f, -12582912.f), neg1 = f2_pack(-1.f, -1.f);
     const uint64_t t = f2_add(x, big);
     const uint64_t f = f2_fma(f2_add(t, nbig), neg1, x);

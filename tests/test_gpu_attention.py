@@ -215,3 +215,26 @@ def test_unseen_keys_have_weight_exactly_zero(gpu, D, G, prefix, path):
     finally:
         gpu.set_path(cb.ATTENTION_AUTO)
     assert torch.equal(a[quiet], b[quiet]) and torch.equal(la[quiet], lb[quiet])
+
+
+@pytest.mark.parametrize("D,G", [(128, 4), (64, 4), (128, 8)])
+@pytest.mark.parametrize("path", ["auto", "one_cta_per_sm", "cta_pairs"])
+def test_nan_in_a_visible_key_shows(gpu, D, G, path):
+    """One NaN key of the prefix makes every row that sees it NaN, whichever place of its tile it has (neighbouring places take
+    different ways to their weight); rows of other sequences stay as they are."""
+    if path == "cta_pairs" and D == 64:
+        pytest.skip("the two-SM kernel takes head dim 128")
+    cfg = _cfg(B=2, Hq=2 * G, Hkv=2, D=D, T=60, C=4, S=4, prefix=300, max_depth=7, fanout=(1, 4), seed=62)
+    parent, owner, plen, seq_start, n_slots, t = H.setup_case(cfg)
+    gpu.set_path({"auto": cb.ATTENTION_AUTO, "one_cta_per_sm": cb.ATTENTION_TENSOR, "cta_pairs": cb.ATTENTION_TENSOR_PAIR}[path])
+    try:
+        a, _, _ = H.gpu_attention(gpu, cfg, t, seq_start, plen, parent, owner, n_slots)
+        for j in list(range(8)) + [64 + 3, 128 + 66, 299]:
+            broken = dict(t, k_cache=t["k_cache"].clone())
+            broken["k_cache"][int(seq_start[1]) + j, 1] = float("nan")
+            b, lse, st = H.gpu_attention(gpu, cfg, broken, seq_start, plen, parent, owner, n_slots)
+            assert st.tolist() == [0, 0]
+            assert torch.equal(a[0], b[0]) and torch.equal(a[1, :, :G], b[1, :, :G])
+            assert b[1, :, G:].isnan().all() and lse[1, :, G:].isnan().all(), f"key {j}"
+    finally:
+        gpu.set_path(cb.ATTENTION_AUTO)

@@ -61,3 +61,8 @@ def test_exact_at_whole_numbers_and_zero_below(exp2_pair):
     assert np.all(np.abs(exp2_pair(n) / np.exp2(n) - 1) <= 2.0 ** -23)
     x = np.array([-126.51, -127, -127.3, -130, -500, -3e38, -np.inf, -np.inf], dtype=np.float32)
     assert np.all(exp2_pair(x).view(np.uint32) == 0)
+
+
+def test_nan_stays_nan(exp2_pair):
+    x = np.array([np.nan, -3.0, 1.5, np.nan, np.nan, -np.inf, -np.inf, np.nan], dtype=np.float32)
+    assert np.array_equal(np.isnan(exp2_pair(x)), np.isnan(x))

@@ -265,8 +265,7 @@ __global__ void __launch_bounds__(M / 4 * kGroupThreads<M>, 1) attention_generic
         for (int c = 0; c < kPieces; ++c) sum[c] = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int c = 0; c < n_ranks; ++c) {
             const float m_c = *cluster.map_shared_rank(&sh.m[i], c);
-            if (m_c == -INFINITY) continue;          // this rank saw no key of the row
-            const float w = expf(m_c - mm);
+            const float w = expf(m_c - mm);          // a rank that saw no key of the row: 0 (and 0 times its sums; NaN if it saw only NaN)
             l = fmaf(w, *cluster.map_shared_rank(&sh.l[i], c), l);
 #pragma unroll
             for (int cc = 0; cc < kPieces; ++cc) {

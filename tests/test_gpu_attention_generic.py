@@ -38,3 +38,22 @@ def test_generic_matches_oracle(gpu, cfg):
     want, want_lse, _ = H.oracle_attention(cfg, t, seq_start, plen, parent, owner)
     assert st.tolist() == [0] * cfg.B
     H.assert_attention_close(out, lse, want, want_lse, cfg.kv_dtype, cfg.name)
+
+
+@pytest.mark.parametrize("where", ["root", "tile"])
+def test_nan_that_is_all_a_cta_sees_of_a_row_shows(gpu, where):
+    """The keys are dealt out over a cluster; a CTA may see nothing of a row but NaN: the root's row in the tile of the tree
+    slots, or any row in a tile of 64 NaN keys."""
+    cfg = inputs.VerifyConfig("generic", B=1, L=1, Hq=4, Hkv=2, D=64, T=8, C=2, S=2, V=32, prefix=256 - 2, tree="chain",
+                              kv_dtype=torch.float32, logit_dtype=torch.float32, sigma_logit=1.0, draft="independent",
+                              temperatures=(1.0,), seed=570)
+    parent, owner, plen, seq_start, n_slots, t = H.setup_case(cfg)       # soft prompts and prefix: four whole tiles of 64 keys
+    at = int(seq_start[0]) + int(plen[0])
+    if where == "root":
+        t["k_cache"][at, 1] = float("nan")
+    else:
+        t["k_cache"][at - 64:at, 1] = float("nan")
+    out, lse, st = H.gpu_attention(gpu, cfg, t, seq_start, plen, parent, owner, n_slots)
+    assert st.tolist() == [0]
+    assert out[0, :, :2].isfinite().all() and lse[0, :, :2].isfinite().all()
+    assert out[0, :, 2:].isnan().all() and lse[0, :, 2:].isnan().all()

@@ -481,9 +481,6 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
             else mma_role<D, false>(sh, prm, pv, tmem);
         } else if (warp == 10) {
             tail_role(sh, prm, pv);
-        } else if (blockIdx.x == 0 && prm.status && pv.hdr->kind != kPlanCta) {
-            // a plan for another kind of work unit is refused: no role finds anything to do
-            for (int b = threadIdx.x & 31; b < prm.d.B; b += 32) prm.status[b] = CONFU_ST_BAD_PLAN;
         }
         __syncwarp();
     }

@@ -164,7 +164,10 @@ __global__ void __launch_bounds__(kMergeThreads, 4) merge_kernel(const Params pr
     // A plan for another kind of work unit has been refused by the attention kernel.  Its share numbers must not be followed:
     // they belong to another number of row groups, and the partial slots they lead to may lie past the workspace.
     const Parts parts = {__ldg(&pv.parts[bg].word)};
-    if (parts.kind() != prm.kind) return;
+    if (parts.kind() != prm.kind) {
+        if (prm.status && threadIdx.x == 0 && u.g == 0 && u.rg == 0 && blockIdx.y == 0 && blockIdx.z == 0) prm.status[u.b] = CONFU_ST_BAD_PLAN;
+        return;
+    }
     u.c0 = parts.first() * prm.n_rg + u.rg;
     u.n = parts.n();
     if (u.n == 1) return;                                   // one unit covered the pair and wrote the output itself

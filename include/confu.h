@@ -205,7 +205,8 @@ int confu_tree_plan(confu_ctx* ctx, const confu_dims* dims,
  * [S][Hkv][D] (NULL if S == 0); lse: optional [B][R][Hq] fp32 natural-log softmax
  * denominators.  plan: a buffer filled by confu_tree_plan for these dims, lengths
  * and trees, or NULL to have the call build one in the workspace (then parent,
- * con_owner are read; otherwise they may be NULL).  Accumulation is fp32; bf16
+ * con_owner are read; otherwise they may be NULL).  Accumulation is fp32; softmax weights are rounded to bf16
+ * on the tensor-core path where D = 128 and Hq/Hkv <= 4 (and always by _TENSOR_PAIR), and keep 16 bits elsewhere; bf16
  * inputs use the tensor-core path when Hq/Hkv <= 32 and S <= 128; it takes the
  * query rows in groups of 2 * (128 / (Hq/Hkv)), so more rows than that stream the keys once
  * per group (the groups walk the same keys at the same time: the later reads are served by L2).

@@ -105,7 +105,7 @@ __device__ void producer_role(SharedStorage<D>& sh, const Params& prm, const Pla
 // Slot order: Q K^T of tile g before P V of tile g - 1 (whose weights are being worked on meanwhile); where tile g starts a
 // run, after it: the new Q lands while the old run's last weights are worked on.  Instructions of one thread reach the
 // pipe in order, so Q K^T of tile g may overwrite the buffer that P V of tile g - 2 read.
-template <int D>
+template <int D, bool kSplit>
 __device__ void mma_role(SharedStorage<D>& sh, const Params& prm, const PlanView& pv, uint32_t tmem)
 {
     Walker w;
@@ -144,8 +144,8 @@ __device__ void mma_role(SharedStorage<D>& sh, const Params& prm, const PlanView
             tc_fence_after();
             if (!issuer) continue;
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                mma_ts(tmem + kColO + h * 128, tmem + buf * 128 + h * 64 + j * 8, vl + (4 * h + j) * (2048u >> 4),
+            for (int j = 0; j < (kSplit ? 8 : 4); ++j)           // (4..7: what bf16 leaves of the weights, 32 columns on)
+                mma_ts(tmem + kColO + h * 128, tmem + buf * 128 + h * 64 + j * 8, vl + (4 * h + j % 4) * (2048u >> 4),
                        D == 128 ? kIdescPV : kIdescPV64, (first && j == 0) ? 0u : 1u);
         }
         if (issuer) {
@@ -217,7 +217,7 @@ __device__ void tail_role(SharedStorage<D>& sh, const Params& prm, const PlanVie
     if (prev >= 0) see(prev);
 }
 
-template <int D>
+template <int D, bool kSplit>
 __device__ void softmax_role(SharedStorage<D>& sh, const Params& prm, const PlanView& pv, uint32_t tmem)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -276,10 +276,8 @@ __device__ void softmax_role(SharedStorage<D>& sh, const Params& prm, const Plan
                 }
             }
             const float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref;
-            // P over the first 32 of this half's columns of S (which sit in registers by now)
-            uint32_t pk[32];
-            l += weights64<true>(sv, c, neg_m, pk);
-            tmem_st32(s_addr + buf * 128, pk);
+            // P over this half's columns of S (which sit in registers by now)
+            l += store_weights64<kSplit, true>(sv, c, neg_m, s_addr + buf * 128);
             tc_wait_st();
             // P V of a run's first tile overwrites both accumulators: both warps of these rows have read the old ones
             if (tile == s.t0 && seg > 0 && !wait_warp(sh, &sh.r_bar[wq], (seg - 1) & 1, prm.wait_ns)) return;
@@ -326,7 +324,7 @@ __device__ void softmax_role(SharedStorage<D>& sh, const Params& prm, const Plan
             }
         }
         if (whole && half == 0 && row_valid && prm.lse)
-            prm.lse[((size_t)s.b * R + r) * Hq + h] = (m_row + log2f(l_row)) * 0.6931471805599453f;
+            prm.lse[((size_t)s.b * R + r) * Hq + h] = natural_lse(m_row, l_row);
         if (!wait_warp(sh, &sh.y_bar[wq], seg & 1, prm.wait_ns)) return;     // the exchange has been read: its place is free
         if (!wait_warp(sh, &sh.o_done, seg & 1, prm.wait_ns)) return;
         tc_fence_after();
@@ -368,7 +366,7 @@ __device__ void softmax_role(SharedStorage<D>& sh, const Params& prm, const Plan
     }
 }
 
-template <int D>
+template <int D, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
 attention_narrow_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                         const __grid_constant__ CUtensorMap v_map, const __grid_constant__ CUtensorMap ks_map,
@@ -406,11 +404,11 @@ attention_narrow_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
     // global memory is read and written from here on: the kernels before this one have completed
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const PlanView pv = plan_view(const_cast<void*>(prm.plan), prm.d.B, prm.d.Hkv);
-    if (warp < 8) softmax_role(sh, prm, pv, tmem);
+    if (warp < 8) softmax_role<D, kSplit>(sh, prm, pv, tmem);
     else if (warp == 8) {
         if ((threadIdx.x & 31) == 0) producer_role(sh, prm, pv, &q_map, &k_map, &v_map, &ks_map, &vs_map);
     } else if (warp == 9)
-        mma_role(sh, prm, pv, tmem);
+        mma_role<D, kSplit>(sh, prm, pv, tmem);
     else if (warp == 10)
         tail_role(sh, prm, pv);
     else if (blockIdx.x == 0 && prm.status && pv.hdr->kind != kPlanNarrow)
@@ -439,7 +437,7 @@ bool make_tile_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t h
 
 }  // namespace tc
 
-template <int D>
+template <int D, bool kSplit>
 static cudaError_t launch_d(const Ctx* ctx, const confu_dims& d, const void* q, const void* k_cache, const void* v_cache,
                             int64_t n_slots, const SlotMap& map, const int32_t* prefix_len, const void* k_soft,
                             const void* v_soft, const void* plan, void* partials, void* out, float* lse, int32_t* status,
@@ -470,7 +468,7 @@ static cudaError_t launch_d(const Ctx* ctx, const confu_dims& d, const void* q, 
     const size_t smem = sizeof(SharedStorage<D>) + 1024;
     static OncePerDevice attr_done;
     cudaError_t e = attr_done.run([&] {
-        return cudaFuncSetAttribute(attention_narrow_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        return cudaFuncSetAttribute(attention_narrow_kernel<D, kSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     });
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute pdl[1];
@@ -483,7 +481,7 @@ static cudaError_t launch_d(const Ctx* ctx, const confu_dims& d, const void* q, 
     cfg.stream = st;
     cfg.attrs = pdl;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, attention_narrow_kernel<D>, q_map, k_map, v_map, ks_map, vs_map, prm);
+    e = cudaLaunchKernelEx(&cfg, attention_narrow_kernel<D, kSplit>, q_map, k_map, v_map, ks_map, vs_map, prm);
     if (e != cudaSuccess) return e;
     return launch_combine(prm, ctx->sm_count / 2, st);
 }
@@ -493,7 +491,8 @@ cudaError_t launch_attention_narrow(const Ctx* ctx, const confu_dims& d, const v
                                     const int32_t* prefix_len, const void* k_soft, const void* v_soft, const void* plan,
                                     void* partials, void* out, float* lse, int32_t* status, cudaStream_t st)
 {
-    return (d.D == 64 ? launch_d<64> : launch_d<128>)(ctx, d, q, k_cache, v_cache, n_slots, map, prefix_len, k_soft, v_soft, plan,
+    auto launch = d.D == 64 ? launch_d<64, true> : tc::split_weights(d) ? launch_d<128, true> : launch_d<128, false>;
+    return launch(ctx, d, q, k_cache, v_cache, n_slots, map, prefix_len, k_soft, v_soft, plan,
                                                       partials, out, lse, status, st);
 }
 

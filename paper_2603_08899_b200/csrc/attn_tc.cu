@@ -127,7 +127,7 @@ __device__ void producer_role(SharedStorage<D>& sh, const Params& prm, const Pla
 // descriptors are made of can live in uniform registers: with a lone thread the same loop took 12 % longer,
 // and the kernel 2-3 % at 32 sequences.)  Per stage g: P V of key tile g-1 for both M tiles (each
 // as soon as its P is there), Q K^T of key tile g for both, then the stage is released.
-template <int D, bool kTwo>
+template <int D, bool kSplit, bool kTwo>
 __device__ void mma_role(SharedStorage<D>& sh, const Params& prm, const PlanView& pv, uint32_t tmem)
 {
     constexpr int kMt = kTwo ? 2 : 1;
@@ -157,8 +157,8 @@ __device__ void mma_role(SharedStorage<D>& sh, const Params& prm, const PlanView
     auto issue_pv = [&](int t, int h, uint32_t vl, bool first_of_segment) {
         if (!issuer) return;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            mma_ts(tmem + 256 + t * 128, tmem + t * 128 + h * 64 + i * 8, vl + (4 * h + i) * (2048u >> 4), kIdescO,
+        for (int i = 0; i < (kSplit ? 8 : 4); ++i)           // (4..7: what bf16 leaves of the weights, 32 columns on)
+            mma_ts(tmem + 256 + t * 128, tmem + t * 128 + h * 64 + i * 8, vl + (4 * h + i % 4) * (2048u >> 4), kIdescO,
                    (first_of_segment && h == 0 && i == 0) ? 0u : 1u);
     };
     // one stage: P V of the previous key tile (if any), Q K^T of the current one (if any), half by half: while the
@@ -264,7 +264,7 @@ __device__ void tail_role(SharedStorage<D>& sh, const Params& prm, const PlanVie
     if (have_prev) run_stage(0);
 }
 
-template <int D>
+template <int D, bool kSplit>
 __device__ void softmax_role(SharedStorage<D>& sh, const Params& prm, const PlanView& pv, uint32_t tmem, int t /*M tile*/)
 {
     const int lane_row = threadIdx.x & 127;                 // row of the M tile = TMEM lane
@@ -324,13 +324,11 @@ __device__ void softmax_role(SharedStorage<D>& sh, const Params& prm, const Plan
             }
             return true;
         };
-        // P over the first 32 columns of the half (whose scores sit in registers by now); masked scores are -inf
-        // and get weight exactly 0
+        // P over the columns of the half (whose scores sit in registers by now); masked scores are -inf and get weight
+        // exactly 0
         auto hand_over = [&](int h, const uint32_t (&sv)[64]) {
             const float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref;
-            uint32_t pk[32];
-            l += weights64(sv, c, neg_m, pk);
-            tmem_st32(s_addr + h * 64, pk);
+            l += store_weights64<kSplit>(sv, c, neg_m, s_addr + h * 64);
             tc_wait_st();
             tc_fence_before();
             mbar_arrive(&sh.p_full[t][h]);
@@ -411,7 +409,7 @@ __device__ void softmax_role(SharedStorage<D>& sh, const Params& prm, const Plan
         }
         if (whole) {
             if (row_valid && prm.lse)
-                prm.lse[((size_t)s.b * R + r) * Hq + h] = (m_ref + log2f(l)) * 0.6931471805599453f;
+                prm.lse[((size_t)s.b * R + r) * Hq + h] = natural_lse(m_ref, l);
         } else {
             float* ml = prm.partials + (size_t)s.part_slot * (partial_slot_bytes() / sizeof(float)) + (size_t)kPartRows * kPartD;
             ml[t * 128 + lane_row] = m_ref;
@@ -424,7 +422,7 @@ __device__ void softmax_role(SharedStorage<D>& sh, const Params& prm, const Plan
     }
 }
 
-template <int D>
+template <int D, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
 attention_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                     const __grid_constant__ CUtensorMap v_map, const __grid_constant__ CUtensorMap ks_map,
@@ -471,14 +469,14 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
     if (warp < 8) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
         const int t = warp >> 2;
-        if (t < prm.n_mt) softmax_role(sh, prm, pv, tmem, t);
+        if (t < prm.n_mt) softmax_role<D, kSplit>(sh, prm, pv, tmem, t);
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         if (warp == 8) {
             if ((threadIdx.x & 31) == 0) producer_role(sh, prm, pv, &q_map, &k_map, &v_map, &ks_map, &vs_map);
         } else if (warp == 9) {
-            if (prm.n_mt > 1) mma_role<D, true>(sh, prm, pv, tmem);
-            else mma_role<D, false>(sh, prm, pv, tmem);
+            if (prm.n_mt > 1) mma_role<D, kSplit, true>(sh, prm, pv, tmem);
+            else mma_role<D, kSplit, false>(sh, prm, pv, tmem);
         } else if (warp == 10) {
             tail_role(sh, prm, pv);
         }
@@ -542,7 +540,7 @@ bool tc_attention_supported(const confu_dims& d)
     return d.kv_dtype == CONFU_BF16 && G <= kMaxTcGroup && d.S <= 128;
 }
 
-template <int D>
+template <int D, bool kSplit>
 static cudaError_t launch_tc(const Ctx* ctx, const confu_dims& d, const void* q, const void* k_cache,
                              const void* v_cache, int64_t n_slots, const SlotMap& map, const int32_t* prefix_len,
                              const void* k_soft, const void* v_soft, const void* plan, void* partials, void* out,
@@ -573,7 +571,7 @@ static cudaError_t launch_tc(const Ctx* ctx, const confu_dims& d, const void* q,
     static OncePerDevice attr_done;
     {
         cudaError_t e = attr_done.run([&] {
-            return cudaFuncSetAttribute(attention_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            return cudaFuncSetAttribute(attention_tc_kernel<D, kSplit>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         });
         if (e != cudaSuccess) return e;
     }
@@ -591,7 +589,7 @@ static cudaError_t launch_tc(const Ctx* ctx, const confu_dims& d, const void* q,
     cfg.stream = st;
     cfg.attrs = pdl;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, attention_tc_kernel<D>, q_map, k_map, v_map, ks_map, vs_map, prm);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, attention_tc_kernel<D, kSplit>, q_map, k_map, v_map, ks_map, vs_map, prm);
     if (e != cudaSuccess) return e;
     return launch_combine(prm, ctx->sm_count, st);
 }
@@ -601,7 +599,8 @@ cudaError_t launch_attention_tc(const Ctx* ctx, const confu_dims& d, const void*
                                 const int32_t* prefix_len, const void* k_soft, const void* v_soft, const void* plan,
                                 void* partials, void* out, float* lse, int32_t* status, cudaStream_t st)
 {
-    return (d.D == 64 ? launch_tc<64> : launch_tc<128>)(ctx, d, q, k_cache, v_cache, n_slots, map, prefix_len, k_soft, v_soft,
+    auto launch = d.D == 64 ? launch_tc<64, true> : tc::split_weights(d) ? launch_tc<128, true> : launch_tc<128, false>;
+    return launch(ctx, d, q, k_cache, v_cache, n_slots, map, prefix_len, k_soft, v_soft,
                                                         plan, partials, out, lse, status, st);
 }
 

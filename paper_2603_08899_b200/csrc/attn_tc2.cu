@@ -530,7 +530,7 @@ __device__ void softmax_role(SharedStorage& sh, const Params& prm, const PlanVie
         if (half == 0) {
             if (whole) {
                 if (row_valid && prm.lse)
-                    prm.lse[((size_t)s.b * R + r) * Hq + h] = (m_ref + log2f(l_row)) * 0.6931471805599453f;
+                    prm.lse[((size_t)s.b * R + r) * Hq + h] = natural_lse(m_ref, l_row);
             } else {
                 float* ml = prm.partials + (size_t)s.part_slot * (partial_slot_bytes() / sizeof(float)) + (size_t)kPartRows * kPartD;
                 ml[rank * 128 + lane_row] = m_ref;

@@ -73,7 +73,7 @@ __device__ __forceinline__ void finish(const Params& prm, const Pair& u, int r, 
 {
     const size_t row = ((size_t)u.b * (prm.d.T + prm.d.C) + r) * prm.d.Hq + u.g * prm.G + lane_row % prm.G;
     acc.store(prm.out + row * D, lane, 1.f / L);
-    if (prm.lse && lane == 0) prm.lse[row] = (M + log2f(L)) * 0.6931471805599453f;
+    if (prm.lse && lane == 0) prm.lse[row] = natural_lse(M, L);
 }
 
 // NR rows (row0, row0 + 1, ... below `rows`) of up to NP parts each, all loads in flight at once

@@ -148,5 +148,52 @@ __device__ __forceinline__ float weights64(const uint32_t* sv, float c, float ne
     return s0 + s1;
 }
 
+// The same for 32 scores, each weight as the sum of two bf16 numbers, 16 bits of it: hi and, for what the first leaves, lo.
+template <bool kFma = false>
+__device__ __forceinline__ float split_weights32(const uint32_t* sv, float c, float neg_m, uint32_t (&hi)[16], uint32_t (&lo)[16])
+{
+    uint64_t sum2 = f2_pack(0.f, 0.f);
+    const uint64_t c2 = f2_pack(c, c), nm2 = f2_pack(neg_m, neg_m), neg1 = f2_pack(-1.f, -1.f);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        float x0, x1;
+        f2_unpack(f2_fma(f2_pack(__uint_as_float(sv[2 * j]), __uint_as_float(sv[2 * j + 1])), c2, nm2), x0, x1);
+        if (kFma && (j & 3) == 1) ex2_pair_fma(x0, x1);
+        else { x0 = ex2(x0); x1 = ex2(x1); }
+        const uint64_t p = f2_pack(x0, x1);
+        sum2 = f2_add(sum2, p);
+        hi[j] = pack_bf16(x0, x1);
+        float r0, r1;
+        f2_unpack(f2_fma(f2_pack(__uint_as_float(hi[j] << 16), __uint_as_float(hi[j] & 0xffff0000u)), neg1, p), r0, r1);
+        lo[j] = pack_bf16(r0, r1);
+    }
+    float s0, s1;
+    f2_unpack(sum2, s0, s1);
+    return s0 + s1;
+}
+
+// 64 scores of a thread's row -> weights in tensor memory at `addr` (over the scores' own columns): bf16 in the first 32, and
+// with kSplit what they leave in the next 32.  Returns their fp32 sum.
+template <bool kSplit, bool kFma = false>
+__device__ __forceinline__ float store_weights64(const uint32_t* sv, float c, float neg_m, uint32_t addr)
+{
+    if constexpr (!kSplit) {
+        uint32_t pk[32];
+        const float sum = weights64<kFma>(sv, c, neg_m, pk);
+        tmem_st32(addr, pk);
+        return sum;
+    } else {
+        float sum = 0.f;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            uint32_t hi[16], lo[16];
+            sum += split_weights32<kFma>(sv + 32 * q, c, neg_m, hi, lo);
+            tmem_st16(addr + 16 * q, hi);
+            tmem_st16(addr + 32 + 16 * q, lo);
+        }
+        return sum;
+    }
+}
+
 }  // namespace tc
 }  // namespace confu

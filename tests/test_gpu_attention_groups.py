@@ -45,3 +45,25 @@ def test_groups_match_oracle(gpu, G, D, T, C, prefix):
             gpu.set_path(cb.ATTENTION_AUTO)
         assert st.tolist() == [0] * cfg.B
         H.assert_attention_close(out, lse, want, want_lse, cfg.kv_dtype, f"G {G} D {D} path {path}")
+
+
+@pytest.mark.parametrize("G,D", [(1, 64), (4, 64), (8, 64), (5, 128), (8, 128), (32, 128)])
+@pytest.mark.parametrize("path", ["auto", "one_cta_per_sm"])
+def test_weights_keep_more_than_bf16(gpu, G, D, path):
+    """Head dim 64 and more than four heads per kv head: weights travel as two bf16 numbers, 16 bits or more of each, so the error against 64 bits is
+    that of rounding the output to bf16 (2^-9 at most, 2^-17 from the weights: together at most 1 + 2^-8 times the first, and
+    far less in the 2-norm; with weights of 8 bits it is 1.03 to 1.4 times).  lse, in absolute terms: fp32 rounding of a number near 8."""
+    cfg = inputs.VerifyConfig("split", B=2, L=1, Hq=2 * G, Hkv=2, D=D, T=30, C=10, S=5, V=32, prefix=(200, 1500), tree="random",
+                              kv_dtype=torch.bfloat16, logit_dtype=torch.float32, sigma_logit=1.0, draft="independent",
+                              temperatures=(1.0,), seed=650 + G + D, max_depth=7, fanout=(1, 4))
+    parent, owner, plen, seq_start, n_slots, t = H.setup_case(cfg)
+    want, want_lse, _ = H.oracle_attention(cfg, t, seq_start, plen, parent, owner)
+    gpu.set_path(cb.ATTENTION_AUTO if path == "auto" else cb.ATTENTION_TENSOR)
+    try:
+        out, lse, st = H.gpu_attention(gpu, cfg, t, seq_start, plen, parent, owner, n_slots)
+    finally:
+        gpu.set_path(cb.ATTENTION_AUTO)
+    assert st.tolist() == [0, 0]
+    rounding = (want.to(torch.bfloat16).double() - want).norm().item()
+    assert (out.double() - want).norm().item() <= 1.001 * rounding
+    assert (lse.double() - want_lse).abs().max().item() <= 4e-6

@@ -41,6 +41,7 @@ struct RatioShared {
     double p[kMaxTree], q[kMaxTree];                 // of every node's token in its parent's rows
     int act, x, nonfinite, degenerate, owner;
     float cs, iZ;
+    double iZ64[2];                                  // statistics on demand: inverse normalisers of the current node's rows
     double off, target, total;
 };
 
@@ -56,6 +57,7 @@ __global__ void __launch_bounds__(kThreads, 1) ratio_walk_kernel(const Args a, c
     const Span sp = span_of<T>(a.V, rank, n);
     const double inv_temp = 1.0 / (double)a.temperature;
     const float k2 = (float)inv_temp * kLog2e;
+    const double k64 = inv_temp * 1.4426950408889634;
     const T* tl_b = tl + (size_t)b * a.T * a.V;
     const T* dl_b = dl + (size_t)b * a.T * a.V;
 
@@ -65,7 +67,7 @@ __global__ void __launch_bounds__(kThreads, 1) ratio_walk_kernel(const Args a, c
     prefetch_slice<T, E>(dl_b, sp);
     int flag = 0;
     if (!kLazy) {
-        // chunk statistics of all rows, half a warp to a row (fp32 exponentials as in the chunks' own sums, fp64 sum)
+        // chunk statistics of all rows, half a warp to a row, joined in fp64
         constexpr int kRounds = 2 * kMaxTree / (2 * kWarps);
         const int c = lane & 15, half = 2 * warp + (lane >> 4);
         uint4 v[kRounds];
@@ -84,10 +86,11 @@ __global__ void __launch_bounds__(kThreads, 1) ratio_walk_kernel(const Args a, c
             float mm = m;
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
-            double z = m > -INFINITY ? (double)(__uint_as_float(v[k].y) * ex2((m - mm) * k2)) : 0.0;
+            double z = m > -INFINITY ? (double)__uint_as_float(v[k].y) : 0.0;
+            z *= joint(m - mm, k64);
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-            if (c == 0 && row < 2 * a.T) { sh.M[row / a.T][row % a.T] = mm; sh.iZ_row[row / a.T][row % a.T] = 1.f / (float)z; }
+            if (c == 0 && row < 2 * a.T) { sh.M[row / a.T][row % a.T] = mm; sh.iZ_row[row / a.T][row % a.T] = (float)(1.0 / z); }
         }
     }
     if (tid == 0) { sh.nonfinite = 0; sh.degenerate = 0; }
@@ -141,21 +144,29 @@ __global__ void __launch_bounds__(kThreads, 1) ratio_walk_kernel(const Args a, c
             const bool any_bad = __any_sync(0xffffffffu, bad);
             exchange(sh.ex, parity, rank, n, make_uint4(__float_as_uint(any_bad ? NAN : wt), __float_as_uint(st), __float_as_uint(wd), __float_as_uint(sd)));
             if (warp == 0) {
+                // eight warps' parts per lane, relative to the lane's own maxima first
                 const int r = lane >> 1;
-                float mt = -INFINITY, md = -INFINITY;
-                if (r < n)
+                const uint4* slot = &sh.ex.slot[parity][r < n ? r : 0][(lane & 1) * (kWarps / 2)];
+                float lt = -INFINITY, ld = -INFINITY;
+                double zt = 0.0, zd = 0.0;
+                if (r < n) {
                     for (int w = 0; w < kWarps / 2; ++w) {
-                        const uint4 v = sh.ex.slot[parity][r][(lane & 1) * (kWarps / 2) + w];
-                        mt = max_nan(mt, __uint_as_float(v.x));
-                        md = fmaxf(md, __uint_as_float(v.z));
+                        lt = max_nan(lt, __uint_as_float(slot[w].x));
+                        ld = fmaxf(ld, __uint_as_float(slot[w].z));
                     }
-                mt = warp_max_nan(mt);
-                md = warp_max(md);
-                const double zt = sum_ranks(rank_totals(sh.ex, parity, n, [&](const uint4& v) { return (double)(__uint_as_float(v.y) * ex2((__uint_as_float(v.x) - mt) * k2)); }));
-                const double zd = sum_ranks(rank_totals(sh.ex, parity, n, [&](const uint4& v) { return (double)(__uint_as_float(v.w) * ex2((__uint_as_float(v.z) - md) * k2)); }));
+                    const float bt2 = lt == -INFINITY ? 0.f : lt, bd2 = ld == -INFINITY ? 0.f : ld;
+                    for (int w = 0; w < kWarps / 2; ++w) {
+                        zt += (double)(__uint_as_float(slot[w].y) * ex2((__uint_as_float(slot[w].x) - bt2) * k2));
+                        zd += (double)(__uint_as_float(slot[w].w) * ex2((__uint_as_float(slot[w].z) - bd2) * k2));
+                    }
+                }
+                const float mt = warp_max_nan(lt), md = warp_max(ld);
+                zt = warp_sum(zt * joint(lt - mt, k2));
+                zd = warp_sum(zd * joint(ld - md, k2));
                 if (lane == 0) {
                     sh.M[0][cur] = mt; sh.M[1][cur] = md;
-                    sh.iZ_row[0][cur] = 1.f / (float)zt; sh.iZ_row[1][cur] = 1.f / (float)zd;
+                    sh.iZ64[0] = 1.0 / zt; sh.iZ64[1] = 1.0 / zd;
+                    sh.iZ_row[0][cur] = (float)sh.iZ64[0]; sh.iZ_row[1][cur] = (float)sh.iZ64[1];
                     sh.nonfinite = !(mt == mt);
                 }
             }
@@ -189,7 +200,7 @@ __global__ void __launch_bounds__(kThreads, 1) ratio_walk_kernel(const Args a, c
         // weights of the row itself (no rejection): p, with q = 0
         auto target_weights = [&]() {
             if (kLazy) {
-                const float f = ex2((wt - Mt()) * k2) * iZt();
+                const float f = (float)(joint(wt - Mt(), k2) * sh.iZ64[0]);
 #pragma unroll
                 for (int e = 0; e < E; ++e) p[e] *= f;
             } else {
@@ -231,7 +242,7 @@ __global__ void __launch_bounds__(kThreads, 1) ratio_walk_kernel(const Args a, c
                         } else {
                             ++tr.hits;
                             sh.x = tr.tok[c];
-                            sh.cs = rem > 0.0 ? 1.f / (float)rem : 0.f;
+                            sh.cs = rem > 0.0 ? (float)(1.0 / rem) : 0.f;
                         }
                     }
                 }
@@ -247,7 +258,7 @@ __global__ void __launch_bounds__(kThreads, 1) ratio_walk_kernel(const Args a, c
             rejected = true;
             target_weights();
             if (kLazy) {
-                const float f = ex2((wd - sh.M[1][cur]) * k2) * sh.iZ_row[1][cur];
+                const float f = (float)(joint(wd - sh.M[1][cur], k2) * sh.iZ64[1]);
 #pragma unroll
                 for (int e = 0; e < E; ++e) q[e] *= f;
             } else {
@@ -261,7 +272,7 @@ __global__ void __launch_bounds__(kThreads, 1) ratio_walk_kernel(const Args a, c
                 if (warp == 0) {
                     const double Z = sum_ranks(rank_totals(sh.ex, parity ^ 1, n, [](const uint4& v) { return quad_double(v); }));
                     if (Z > 0.0) {
-                        const float iz = 1.f / (float)Z;
+                        const float iz = (float)(1.0 / Z);
                         if (lane == 0) sh.iZ = iz;
                         p0 = fmax(p0 - q0, 0.0) * (double)iz;
                         p1 = fmax(p1 - q1, 0.0) * (double)iz;
@@ -451,7 +462,7 @@ __global__ void __launch_bounds__(kThreads, 1) match_walk_kernel(const Args a, c
                 if (lane == 0) sh.x = best;
             } else {
                 const double mine = rank_totals(sh.ex, parity, n, [&](const uint4& v) {
-                    return quad_double(make_uint4(v.z, v.w, 0u, 0u)) * (double)ex2((__uint_as_float(v.x) - M) * k2);
+                    return quad_double(make_uint4(v.z, v.w, 0u, 0u)) * (double)joint_f32(__uint_as_float(v.x) - M, k2);
                 });
                 const double total = sum_ranks(mine);
                 double before;
@@ -463,7 +474,7 @@ __global__ void __launch_bounds__(kThreads, 1) match_walk_kernel(const Args a, c
         if (sh.code) break;
         if (!greedy) {
             if (sh.owner == rank) {
-                const float f = ex2((m - sh.M) * k2);
+                const float f = joint_f32(m - sh.M, k2);
                 bool found;
                 double lo = 0.0, hi = 0.0;
                 const int pick = locate<E>(sh.sr, sp, sh.off, sh.target, [&](int e) { return w[e] * f; }, found, lo, hi);

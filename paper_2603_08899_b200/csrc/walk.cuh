@@ -163,6 +163,46 @@ __device__ __forceinline__ uint4 as_quad(double d)
 }
 __device__ __forceinline__ double quad_double(const uint4& q) { return __longlong_as_double((long long)(((uint64_t)q.y << 32) | q.x)); }
 
+// 2^(d k) for d <= 0 (0 for -infinity): the factor between two parts of a row whose weights are relative to maxima d apart.  A
+// second exponential of the exponential unit's precision on top of the entry's own would double a weight's error, so the
+// sums of a row's parts are joined in fp64.  The power series of 2^f = e^(f ln 2) to the 9th power (|f| <= 1/2: within 7e-12), by
+// hand so that several go side by side (statistics and ratio rule at batch 1: 27.3 us with ex2, 28.4 with calls
+// of exp2, 27.8 so).
+__device__ __forceinline__ double joint(float d, double k)
+{
+    const double a = fmax((double)d * k, -1100.0), t = a + 6755399441055744.0;      // 1.5 * 2^52: a, rounded, in the low word
+    const int n = __double2loint(t);
+    const double f = (a - (t - 6755399441055744.0)) * 0.69314718055994531;
+    double p = fma(f, 1.0 / 362880.0, 1.0 / 40320.0);
+    p = fma(p, f, 1.0 / 5040.0);
+    p = fma(p, f, 1.0 / 720.0);
+    p = fma(p, f, 1.0 / 120.0);
+    p = fma(p, f, 1.0 / 24.0);
+    p = fma(p, f, 1.0 / 6.0);
+    p = fma(p, f, 0.5);
+    p = fma(p, f, 1.0);
+    p = fma(p, f, 1.0);
+    return n < -1000 ? 0.0 : __hiloint2double(__double2hiint(p) + (n << 20), __double2loint(p));
+}
+
+// The same rounded to fp32 (within 0.6 units in the last place), for where a lane has eight of them on the critical path
+// (sample-and-match, B 16, V 151936: 25.3 us with ex2, 25.9 so, 26.6 and more in fp64): the argument and its product with ln 2 as sums of two fp32 numbers, then the power series of e^t to
+// the 7th power (|t| <= ln 2 / 2: within 5e-9).
+__device__ __forceinline__ float joint_f32(float d, float k2)
+{
+    const float ah = d * k2, al = fmaf(d, k2, -ah), n = rintf(ah), r = ah - n;
+    constexpr float kLn2 = 0.69314718f, kLn2Lo = -1.9046543e-9f;                 // their sum is ln 2 to 2^-50
+    const float t = r * kLn2, tl = fmaf(r, kLn2, -t) + fmaf(al, kLn2, r * kLn2Lo);
+    float p = fmaf(t, 1.f / 5040.f, 1.f / 720.f);
+    p = fmaf(p, t, 1.f / 120.f);
+    p = fmaf(p, t, 1.f / 24.f);
+    p = fmaf(p, t, 1.f / 6.f);
+    p = fmaf(p, t, 0.5f);
+    const float pt = p * t, u = fmaf(fmaf(pt, t, t), tl, tl);                      // e^t tl
+    p = 1.f + (t + fmaf(pt, t, u));
+    return n < -126.f ? 0.f : p * __int_as_float(((int)n + 127) << 23);
+}
+
 // One warp: the CTAs' totals, rank c's in lanes 2 c and 2 c + 1 (0 past the last rank); f turns a slot into its
 // share.  The order of every sum is fixed.
 template <typename F>

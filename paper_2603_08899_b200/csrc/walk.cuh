@@ -185,9 +185,9 @@ __device__ __forceinline__ double joint(float d, double k)
     return n < -1000 ? 0.0 : __hiloint2double(__double2hiint(p) + (n << 20), __double2loint(p));
 }
 
-// The same rounded to fp32 (within 0.6 units in the last place), for where a lane has eight of them on the critical path
-// (sample-and-match, B 16, V 151936: 25.3 us with ex2, 25.9 so, 26.6 and more in fp64): the argument and its product with ln 2 as sums of two fp32 numbers, then the power series of e^t to
-// the 7th power (|t| <= ln 2 / 2: within 5e-9).
+// The same rounded to fp32 (error at most 1.3 * 2^-24), for where a lane has eight of them on the critical path (sample-and-match, B 16,
+// V 151936: 25.3 us with ex2, 25.9 so, 26.6 and more in fp64): the argument and its product with ln 2 as sums of two fp32
+// numbers, then the power series of e^t to the 7th power (|t| <= ln 2 / 2: within 5e-9).
 __device__ __forceinline__ float joint_f32(float d, float k2)
 {
     const float ah = d * k2, al = fmaf(d, k2, -ah), n = rintf(ah), r = ah - n;

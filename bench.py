@@ -95,6 +95,7 @@ def measured_peaks():
 
 KERNEL_SOURCES = {"attention_fp8_kernel": ("attn_fp8.cu", "tc_walk.cuh", "tc_ptx.cuh", "attn_tc.cuh"),
                   "attention_pair_kernel": ("attn_tc2.cu", "tc_walk.cuh", "tc_ptx.cuh", "attn_tc.cuh"),
+                  "attention_narrow_kernel": ("attn_narrow.cu", "tc_walk.cuh", "tc_ptx.cuh", "attn_tc.cuh"),
                   "attention_tc_kernel": ("attn_tc.cu", "tc_walk.cuh", "tc_ptx.cuh", "attn_tc.cuh"),
                   "attention_generic_kernel": ("attn_generic.cu",)}
 

@@ -133,13 +133,16 @@ int confu_set_paging(confu_ctx* ctx, const int32_t* block_table, int32_t max_pag
  *                             as _TENSOR, D = 128, and more than 32 or 128 / (Hq/Hkv) query rows).  A path that does not
  *                             support the dims makes the calls return CONFU_ERR_UNSUPPORTED.  Set
  *                             it before confu_tree_plan: a plan only fits the path it was built
- *                             for (status CONFU_ST_BAD_PLAN otherwise).
+ *                             for (status CONFU_ST_BAD_PLAN otherwise), as confu_attention_path names it.  For small
+ *                             batches _AUTO takes a form of its own of _TENSOR, _TENSOR_NARROW (one
+ *                             M tile of query rows per CTA), which cannot be set.
  *   CONFU_OPT_WAIT_LIMIT_NS   wall-clock limit of every wait on a barrier inside the tensor-core
  *                             kernels (default 2 s; 1 us .. 10 s).  A wait that runs out makes the
  *                             kernel release what it holds and report CONFU_ST_TIMEOUT.
  */
 enum { CONFU_OPT_ATTENTION_PATH = 1, CONFU_OPT_WAIT_LIMIT_NS = 2 };
-enum { CONFU_ATTENTION_AUTO = 0, CONFU_ATTENTION_GENERIC = 1, CONFU_ATTENTION_TENSOR = 2, CONFU_ATTENTION_TENSOR_PAIR = 3 };
+enum { CONFU_ATTENTION_AUTO = 0, CONFU_ATTENTION_GENERIC = 1, CONFU_ATTENTION_TENSOR = 2, CONFU_ATTENTION_TENSOR_PAIR = 3,
+       CONFU_ATTENTION_TENSOR_NARROW = 4 };   /* _TENSOR_NARROW: only returned by confu_attention_path */
 int confu_set_option(confu_ctx* ctx, int32_t option, int64_t value);
 
 /*

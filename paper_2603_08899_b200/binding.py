@@ -20,7 +20,7 @@ ACCEPT_LAZY = 0x100          # or-ed into sibling_mode: row statistics on demand
 BF16, F32, FP8_E4M3 = 0, 1, 2
 OK = 0
 OPT_ATTENTION_PATH, OPT_WAIT_LIMIT_NS = 1, 2
-ATTENTION_AUTO, ATTENTION_GENERIC, ATTENTION_TENSOR, ATTENTION_TENSOR_PAIR = 0, 1, 2, 3
+ATTENTION_AUTO, ATTENTION_GENERIC, ATTENTION_TENSOR, ATTENTION_TENSOR_PAIR, ATTENTION_TENSOR_NARROW = 0, 1, 2, 3, 4
 ST_TIMEOUT, ST_BAD_PATH, ST_BAD_PLAN = 6, 9, 10
 
 EXPORTS = [

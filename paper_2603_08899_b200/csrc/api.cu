@@ -69,7 +69,7 @@ cudaError_t launch_attention_tc(const Ctx* ctx, const confu_dims& d, const void*
 namespace {
 
 // Which attention kernel serves these dims under the context's option: a CONFU_ATTENTION_* value
-// (never _AUTO), or a negative error code when a forced path cannot take them.
+// (never _AUTO, nor _TENSOR_NARROW, see plan_kind), or a negative error code when a forced path cannot take them.
 int resolve_attention_path(const confu_ctx* ctx, const confu_dims& d)
 {
     // (a share of the work is walked by one CTA, or CTA pair, per group of query rows: at least that many of them)
@@ -193,7 +193,8 @@ int confu_attention_path(const confu_ctx* ctx, const confu_dims* dims)
     if (!ctx) return CONFU_ERR_ARG;
     const int rc = check_dims(dims);
     if (rc != CONFU_OK) return rc;
-    return resolve_attention_path(ctx, *dims);
+    const int path = resolve_attention_path(ctx, *dims);
+    return path == CONFU_ATTENTION_TENSOR && plan_kind(ctx, *dims, path) == kPlanNarrow ? (int)CONFU_ATTENTION_TENSOR_NARROW : path;
 }
 
 int confu_selftest_bounded_wait(confu_ctx* ctx, int64_t limit_ns, int32_t* status, void* stream)

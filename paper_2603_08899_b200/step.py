@@ -139,11 +139,13 @@ class VerifyStep:
             return "attention_generic_kernel"
         if path == cb.ATTENTION_TENSOR_PAIR:
             return "attention_pair_kernel"
+        if path == cb.ATTENTION_TENSOR_NARROW:
+            return "attention_narrow_kernel"
         return "attention_fp8_kernel" if self.cfg.kv_dtype == torch.float8_e4m3fn else "attention_tc_kernel"
 
     def attention_kernels_per_layer(self):
         """The tensor-core kernels are followed by the merge of the split pairs; the generic path is one kernel."""
-        return 2 if self.attention_path() in (cb.ATTENTION_TENSOR, cb.ATTENTION_TENSOR_PAIR) else 1
+        return 1 if self.attention_path() == cb.ATTENTION_GENERIC else 2
 
 
 def sm_count(step):

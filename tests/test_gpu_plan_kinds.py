@@ -52,3 +52,36 @@ def test_plan_of_another_kind_is_refused(gpu, built, launched, B, prefix):
     assert gpu.ws_intact()
     assert status.cpu().tolist() == [cb.ST_BAD_PLAN] * B
     assert (out == 7.0).all() and (lse == 7.0).all()
+
+
+@pytest.mark.parametrize("B,G,narrow", [(1, 4, True), (13, 4, True), (14, 4, False), (6, 8, True), (7, 8, False)])
+def test_path_tells_which_plans_fit(gpu, B, G, narrow):
+    """Up to three M tiles of query rows per two SMs (148 of them: 222) the automatic choice is one tile per CTA: confu_attention_path
+    says so, and a plan built under AUTO fits a forced _TENSOR exactly when both paths have the same name."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if sms != 148:
+        pytest.skip("the batches are those on either side of the rule for 148 SMs")
+    cfg = inputs.VerifyConfig("paths", B=B, L=1, Hq=8 * G, Hkv=8, D=128, T=60, C=4, S=0, V=32, prefix=(1, 200), tree="random",
+                              kv_dtype=torch.bfloat16, logit_dtype=torch.float32, sigma_logit=1.0, draft="independent",
+                              temperatures=(1.0,), seed=710 + B, max_depth=7, fanout=(1, 4))
+    dims = H.dims_of(cfg)
+    parent, owner, plen, seq_start, n_slots, t = H.setup_case(cfg)
+    gpu.ensure_ws(dims)
+    plan = torch.empty(cb.confu_plan_bytes(gpu.ctx, dims), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(B, dtype=torch.int32, device="cuda")
+    ss, pl = seq_start.cuda(), plen.cuda()
+    auto = cb.confu_attention_path(gpu.ctx, dims)
+    assert auto == (cb.ATTENTION_TENSOR_NARROW if narrow else cb.ATTENTION_TENSOR)
+    cb.confu_tree_plan(gpu.ctx, dims, ss, pl, parent.cuda(), owner.cuda(), plan, status)
+    try:
+        gpu.set_path(cb.ATTENTION_TENSOR)
+        assert cb.confu_attention_path(gpu.ctx, dims) == cb.ATTENTION_TENSOR
+        out = torch.zeros_like(t["q"])
+        cb.confu_tree_attention(gpu.ctx, dims, t["q"], t["k_cache"], t["v_cache"], n_slots, ss, pl, None, None, None, None, plan, out,
+                                None, status)
+        torch.cuda.synchronize()
+        with pytest.raises(cb.ConfuError):
+            gpu.set_path(cb.ATTENTION_TENSOR_NARROW)
+    finally:
+        gpu.set_path(cb.ATTENTION_AUTO)
+    assert status.cpu().tolist() == [cb.ST_BAD_PLAN if narrow else 0] * B

@@ -92,14 +92,14 @@ int resolve_attention_path(const confu_ctx* ctx, const confu_dims& d)
 // where pairs are few: every CTA has a short run or a few, and what counts is the way from its start to its last
 // store.  Two read K and V half as often and need half as many runs.  (8 kv heads, R 64: two M tiles a pair; us per layer, one
 // tile against two.  8 sequences of 300..4000: 39.5 / 43.9; 10 of 300..6000: 48.0 / 54.9, of 15..300: 18.8 / 20.0; 16 of
-// 300..6000: 75 / 82, but of 15..300: 25.0 / 22.3; 32 of 600..12000: 227 / 209.)  A path that the caller has chosen is
-// taken as it is named.
+// 300..6000: 75 / 82, but of 15..300: 25.0 / 22.3; 32 of 600..12000: 227 / 209.)  As with two, a share is walked by a CTA per
+// row group: there have to be that many.  A path that the caller has chosen is taken as it is named.
 int plan_kind(const confu_ctx* ctx, const confu_dims& d, int path)
 {
     if (path == CONFU_ATTENTION_TENSOR_PAIR) return kPlanPair;
     if (path == CONFU_ATTENTION_GENERIC && !tc_attention_supported(d) && !pair_attention_supported(d)) return kPlanMasks;
     const int n_tiles = row_groups(d.T + d.C, d.Hq / d.Hkv, 1);
-    const bool few = 2 * (int64_t)d.B * d.Hkv * n_tiles <= 3 * (int64_t)ctx->sm_count;
+    const bool few = 2 * (int64_t)d.B * d.Hkv * n_tiles <= 3 * (int64_t)ctx->sm_count && ctx->sm_count >= n_tiles;
     return path == CONFU_ATTENTION_TENSOR && ctx->attention_path == CONFU_ATTENTION_AUTO && d.kv_dtype == CONFU_BF16 && few ? kPlanNarrow : kPlanCta;
 }
 

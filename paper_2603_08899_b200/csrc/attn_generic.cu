@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(M / 4 * kGroupThreads<M>, 1) attention_generic
     Smem<D, M>& sh = *reinterpret_cast<Smem<D, M>*>(smem_raw);
     cg::cluster_group cluster = cg::this_cluster();
     const int n_ranks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-    const int g = blockIdx.y % dm.Hkv, block = blockIdx.y / dm.Hkv, b = blockIdx.z;
+    const int unit = (int)blockIdx.x / n_ranks, g = unit % dm.Hkv, block = unit / dm.Hkv, b = blockIdx.y;
     const int R = dm.T + dm.C, Hq = dm.Hq, Hkv = dm.Hkv, G = Hq / Hkv;
     const int tid = threadIdx.x, tx = tid % X, ty = tid / X, row0 = 4 * ty;
     // row i of the block is query row (block * M + i) / G, head (block * M + i) % G of the group
@@ -301,7 +301,7 @@ cudaError_t launch_m(int ranks, const confu_dims& d, const void* q, const void* 
     attrs[1].val.clusterDim.x = (unsigned)ranks;
     attrs[1].val.clusterDim.y = attrs[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)ranks, (unsigned)blocks, (unsigned)d.B);
+    cfg.gridDim = dim3((unsigned)(ranks * blocks), (unsigned)d.B);     // (x holds 2^31 of them, y 65535)
     cfg.blockDim = dim3(M / 4 * kGroupThreads<M>);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;

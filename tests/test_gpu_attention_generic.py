@@ -57,3 +57,26 @@ def test_nan_that_is_all_a_cta_sees_of_a_row_shows(gpu, where):
     assert st.tolist() == [0]
     assert out[0, :, :2].isfinite().all() and lse[0, :, :2].isfinite().all()
     assert out[0, :, 2:].isnan().all() and lse[0, :, 2:].isnan().all()
+
+
+def test_more_blocks_than_a_grid_dimension_holds(gpu):
+    """33000 kv heads and 65 rows: two blocks of rows per head, 66000 of them."""
+    heads, D, T, C, P = 33000, 64, 33, 32, 3
+    R = T + C
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    q, k, v = (torch.randn((1, n, heads, D), generator=g, device="cuda") for n in (R, P + R, P + R))
+    dims = cb.make_dims(1, heads, heads, D, T, C, 0, torch.float32)
+    gpu.ensure_ws(dims)
+    parent, owner = torch.arange(-1, T - 1, dtype=torch.int32).cuda(), torch.arange(C, dtype=torch.int32).cuda()
+    out, status = torch.empty_like(q), torch.zeros(1, dtype=torch.int32, device="cuda")
+    cb.confu_tree_attention(gpu.ctx, dims, q, k[0], v[0], P + R, torch.zeros(1, dtype=torch.int64, device="cuda"),
+                            torch.tensor([P], dtype=torch.int32, device="cuda"), None, None, parent, owner, None, out, None, status)
+    assert status.tolist() == [0]
+    row, key = torch.arange(R, device="cuda")[:, None], torch.arange(P + R, device="cuda")[None, :] - P
+    depth = torch.where(row < T, row, row - T)       # a chain: row r sees rows 0..r, contemplate row k rows 0..k and itself
+    sees = (key <= depth) & (key < T) | (key == row)
+    for h in (0, 1, 16383, 32767, 32768, heads - 1):
+        s = (q[0, :, h].double() @ k[0, :, h].double().T) * D ** -0.5
+        want = torch.softmax(s.masked_fill(~sees, float("-inf")), dim=-1) @ v[0, :, h].double()
+        assert (out[0, :, h].double() - want).abs().max().item() <= 1e-5 * want.abs().max().item()

@@ -90,8 +90,12 @@ struct Reader {
         PyBuffer_Release(&view);
         return ok ? p : nullptr;
     }
-    confu_ctx* ctx()
+    confu_ctx* ctx()                                 // None: a null context, which the call refuses
     {
+        if (ok && at < n && args[at] == Py_None) {
+            ++at;
+            return nullptr;
+        }
         void* p = memory(sizeof(void*));
         return p ? *static_cast<confu_ctx**>(p) : nullptr;
     }

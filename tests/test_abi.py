@@ -34,3 +34,22 @@ def test_status_strings_and_host_side_argument_errors():
     assert L.confu_set_workspace(None, None, 0) == -1
     assert L.confu_accept_workspace_bytes(4, 60, 128256) > 0
     assert L.confu_accept_workspace_bytes(-1, 60, 128256) == 0
+
+
+def test_calls_refuse_a_missing_context_as_the_library_does():
+    import pytest
+    import torch
+
+    class Stream:
+        cuda_stream = 0
+
+    build.build()
+    dims = binding.make_dims(1, 4, 2, 64, 8, 2, 2, torch.float32)
+    for call in (lambda s: binding.confu_tree_plan(None, dims, None, None, None, None, None, None, s),
+                 lambda s: binding.confu_tree_attention(None, dims, None, None, None, 0, None, None, None, None, None, None, None, None, None, None, s),
+                 lambda s: binding.confu_tree_accept(None, 1, 8, 2, 100, torch.float32, None, None, None, None, None, None, 1.0, 1, None, None,
+                                                     None, None, None, None, None, s),
+                 lambda s: binding.confu_kv_append(None, dims, None, None, None, None, None, None, s)):
+        with pytest.raises(binding.ConfuError) as e:
+            call(Stream())
+        assert e.value.code == -1

@@ -716,12 +716,16 @@ static cudaError_t match_e(int n, int B, const Args& a, const T* tl, cudaStream_
 // vocabulary takes 16 CTAs a sequence (B 1, V 128256, ratio rule: 15-20 us against 24-28 us with 8; sample-and-match 6.7
 // against 8.1 us): up to 7 sequences, because 7 clusters of 16 run at once on 148 SMs (32 sequences: 78 against 61 us).
 // A small vocabulary gains nothing (V 1000: 13.9 against 12.1 us), and one above 163840 entries needs the 16 CTAs to
-// fit the registers.
+// fit the registers.  Two CTAs share an SM: more sequences than that holds at 8 take fewer CTAs each, as long as a thread keeps 16
+// entries or less (greedy sample-and-match, 256 sequences of V 1000: 8 CTAs 98.8 us, one 14.3; of V 32000: 8 102.9, 4 56.2;
+// ratio rule 154 / 33 and 377 / 276).
 template <typename F>
 static cudaError_t by_vocabulary(int B, int V, F f)
 {
     const bool wide = (V > 8 * kStrip && B <= 7) || V > 8 * 5 * kStrip;
-    const int n = wide ? 16 : 8, strips = (V + n * kStrip - 1) / (n * kStrip);
+    int n = wide ? 16 : 8;
+    while (n > 1 && B * n > 2 * 148 && V <= n / 2 * 2 * kStrip) n /= 2;
+    const int strips = (V + n * kStrip - 1) / (n * kStrip);
     switch (strips) {
         case 0: case 1: return f(std::integral_constant<int, 8>(), n);
         case 2: return f(std::integral_constant<int, 16>(), n);

@@ -19,7 +19,9 @@ def gpu():
 
 
 @pytest.mark.parametrize("B,V", [(2, 1), (2, 9), (2, 32768), (2, 32769), (1, 65544), (2, 131073), (8, 65540), (8, 98312), (8, 131080),
-                                 (8, 163840), (8, 163848), (1, 262144)])
+                                 (8, 163840), (8, 163848), (1, 262144),
+                                 # many sequences: 4, 2 and 1 CTAs each, either side of what 16 entries per thread hold
+                                 (38, 32768), (38, 32769), (75, 16384), (75, 16385), (149, 8192), (149, 8193), (300, 1000), (297, 37)])
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 def test_slice_edges(gpu, B, V, dtype):
     T = 1 if V < 9 else 6

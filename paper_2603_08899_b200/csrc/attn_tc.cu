@@ -237,6 +237,7 @@ __device__ void tail_role(SharedStorage<D>& sh, const Params& prm, const PlanVie
     Segment s;
     const int R = prm.d.T + prm.d.C, lane = threadIdx.x & 31;
     uint32_t stage = 0;
+    int fixed = -1;                     // stage of the last repair
     int prev_valid = 0;                 // > 0: the previous tile's V needs rows [prev_valid, 128) zeroed
     bool have_prev = false;
     auto run_stage = [&](int cur_valid) -> bool {
@@ -249,6 +250,11 @@ __device__ void tail_role(SharedStorage<D>& sh, const Params& prm, const PlanVie
                     *reinterpret_cast<uint4*>(sh.kv[st][0] + half * kHalfTile + off) = zero;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
+            // One barrier for every repair: the issuing warp has to be done with the last one before the next is announced, or
+            // it could miss a phase.  (Where the stage itself has come round since, it is.)
+            if (fixed >= 0 && (int)stage < fixed + (int)kStages<D> &&
+                !mbar_wait(&sh.kv_empty[fixed % kStages<D>], (fixed / kStages<D>) & 1, &sh.abort, prm.wait_ns)) return false;
+            fixed = (int)stage;
             if (lane == 0) mbar_arrive(&sh.v_fixed);
         }
         __syncwarp();

@@ -92,7 +92,9 @@ int resolve_attention_path(const confu_ctx* ctx, const confu_dims& d)
 // where pairs are few: every CTA has a short run or a few, and what counts is the way from its start to its last
 // store.  Two read K and V half as often and need half as many runs.  (8 kv heads, R 64: two M tiles a pair; us per layer, one
 // tile against two.  8 sequences of 300..4000: 39.5 / 43.9; 10 of 300..6000: 48.0 / 54.9, of 15..300: 18.8 / 20.0; 16 of
-// 300..6000: 75 / 82, but of 15..300: 25.0 / 22.3; 32 of 600..12000: 227 / 209.)  As with two, a share is walked by a CTA per
+// 300..6000: 75 / 82, but of 15..300: 25.0 / 22.3; 32 of 600..12000: 227 / 209.  Inside the rule the order is the same with 1 to 16
+// tiles a pair, at the most pairs it lets in: G 8, 4 tiles, 6 sequences of 300..6000: 65.1 / 82.9; G 32, 16 tiles, 1 kv head, 12 of
+// 300..3000: 39.3 / 44.3; G 1, 1 tile, head dim 64, 24 of 300..3000: 36.2 / 49.8.)  As with two, a share is walked by a CTA per
 // row group: there have to be that many.  A path that the caller has chosen is taken as it is named.
 int plan_kind(const confu_ctx* ctx, const confu_dims& d, int path)
 {

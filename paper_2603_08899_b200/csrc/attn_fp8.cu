@@ -16,8 +16,9 @@
 //   - the per-head V scale multiplies the output rows (or the partial results) at the end of a run;
 //   - a key tile is worked on in two halves of 64 keys: E4M3 products take half the time of bf16 ones, so the serial
 //     chain S -> weights -> P V -> next S of an M tile was mostly waiting (1200 of 3800 cycles per tile for S); now the
-//     tensor pipe serves one half of the chain while the softmax threads work on the other.  About 3450 cycles per tile and
-//     SM now; a layer of 32 sequences, prefixes 512..16384: 292 -> 264 us.
+//     tensor pipe serves one half of the chain while the softmax threads work on the other.  About 3560 active cycles per tile
+//     and SM now; a layer of 32 sequences, prefixes 512..16384: 292 -> 264 us.  What is left is the latency of the softmax warps'
+//     own chain, two of them per scheduler: no unit is above 54 % and 31 % of the issue slots are used.
 #include "tc_walk.cuh"
 
 namespace confu {

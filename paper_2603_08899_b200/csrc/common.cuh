@@ -19,8 +19,8 @@ constexpr int kTileKeys = 128;                  // keys per attention tile (tens
 // side in an M tile of 128, so a tile holds 128 / G query rows, and a pass over a pair's keys (two M
 // tiles) a group of twice as many.  (Filling the tile whatever G is, instead of 32 rows x G heads,
 // halves the tensor and exponential work of a group of 64 rows at G <= 2 and is what lets G > 4 in.  One
-// layer, own plan, bf16: B 4, 64 / 8 heads of 128, R 64, prefixes 500..4000: 49 us, on CUDA cores 15270 us;
-// B 2, 32 / 8 heads of 64, R 64, prefixes 1500..2500: 27 us, on CUDA cores 2820 us.)
+// layer, own plan, bf16: B 4, 64 / 8 heads of 128, R 64, prefixes 500..4000: 39.8 us, on CUDA cores 15270 us;
+// B 2, 32 / 8 heads of 64, R 64, prefixes 1500..2500: 18.7 us, on CUDA cores 2820 us.)
 constexpr int kMaxTcGroup = 32;                 // query heads per kv head the tensor-core kernels take (groups of 8 rows at G = 32)
 __host__ __device__ inline int rows_per_tile(int G) { return 128 / G; }
 __host__ __device__ inline int row_groups(int R, int G, int tiles_per_group)

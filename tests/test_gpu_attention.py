@@ -72,9 +72,9 @@ def _takes_tensor_cores(cfg):
 @pytest.mark.parametrize("use_plan", [False, True])
 @pytest.mark.parametrize("path", ["auto", "one_cta_per_sm", "cta_pairs"])
 def test_attention_matches_oracle(gpu, name, use_plan, path):
-    """path auto: the library's own choice (CUDA cores, one CTA per SM with tcgen05, or CTA pairs with
-    the two-SM instructions, by dims and batch size); the two tensor-core kernels are also forced, each
-    for every case it can take."""
+    """path auto: the library's own choice (CUDA cores, or tcgen05 with one or two M tiles per CTA, by dims and
+    batch size); the two-M-tile kernel and CTA pairs with the two-SM instructions are also forced, for every case with
+    head dim 128 and up to four heads per kv head (the others: test_gpu_attention_groups.py)."""
     cfg = CASES[name]
     if path == "one_cta_per_sm" and not _takes_tensor_cores(cfg):
         pytest.skip("not a tensor-core case")

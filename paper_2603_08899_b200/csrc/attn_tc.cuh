@@ -45,7 +45,8 @@ __device__ __forceinline__ float natural_lse(float m, float l) { return (float)(
 // four query heads per kv head: on CUDA cores these dims have fp32 weights, and 16 bits of a weight keep that precision: the
 // error against 64 bits is 1.000001 times that of rounding the output to bf16 (prefixes 100..6000, every G; with weights of 8 bits
 // 1.25-1.4 times).  It costs twice the instructions of P V and four more per pair of weights: one layer with its own
-// plan, B 4, 64 / 8 heads of 128, prefixes 500..4000: 36.0 -> 39.8 us; B 2, 32 / 8 heads of 64, 1500..2500: 17.7 -> 18.7.
+// plan, B 4, 64 / 8 heads of 128, prefixes 500..4000: 36.0 -> 39.8 us; B 2, 32 / 8 heads of 64, 1500..2500: 17.7 -> 18.7; where
+// the tensor pipe is busy more: B 32, 64 / 8 heads of 128, 500..4000 174 -> 248; B 48, 32 / 8 heads of 64 112 -> 145.
 inline bool split_weights(const confu_dims& d) { return d.D == 64 || d.Hq / d.Hkv > 4; }
 
 // The kind of a launch's work units and its row packing (see rows_per_tile).

@@ -57,8 +57,8 @@ __host__ __device__ inline int tiles_per_group(int kind) { return kind == kPlanN
 // key tile q - kPairOverheadTiles, so a share that ends inside a pair's overhead zone takes none of
 // its tiles.  With n_rg groups of query rows (row_groups above) there are n = n_ctas / n_rg shares and
 // CTA c * n_rg + rg walks share c for row group rg: the CTAs of a share read the same K/V tiles at
-// about the same time, so that only the first read of a tile goes to DRAM.  Where there are no more pairs than shares,
-// and it makes no share longer, the pairs get whole numbers of equal shares instead (plan.cu).
+// about the same time, so that only the first read of a tile goes to DRAM.  Where it makes no share much longer, long
+// pairs are cut into equal shares of their own instead, and short ones share one whole (plan.cu).
 // ---------------------------------------------------------------------------
 constexpr int kPairOverheadTiles = 4;
 struct PlanHeader {

@@ -12,13 +12,37 @@
 // layer sets itself up meanwhile.  The search for shares of their own starts at the smallest that can fit, sums are one
 // reduction instruction, the step's constants and first slots go through shared memory, and the line is left out where no
 // tensor-core kernel takes the dims.  Plan and one layer, 8 kv heads: B 1 prefix 4096 20.6 -> 19.1 us, B 8 of 300..4000
-// 55.2 -> 47.3, B 32 of 300..2000 81.5 -> 78.0; the fp32 layer of 256 keys 13.7 -> 10.7.
+// 55.2 -> 47.3, B 32 of 300..2000 81.5 -> 78.0; the fp32 layer of 256 keys 13.7 -> 10.7.  The search has one copy of the test in a
+// loop that is not unrolled: code that is fetched once is paid for in full (B 2: three copies and 4 KB more of shared memory
+// +1.4 us).
 #include "common.cuh"
 
 namespace confu {
 
 constexpr int kPlanThreads = 1024, kPlanWarps = kPlanThreads / 32;      // at most; at least kPlanMaxCtas threads
 constexpr int kPlanCached = 1024;                    // sequences whose tile counts, positions and first slots fit shared memory
+
+// Shares of their own, none longer than `own` where a run weighs its tiles + kRunOverheadTiles: a sequence's (sequence, kv head)
+// stretches are cut into equal pieces, one to a share, or, where they are short, several whole ones make up a share.  (A change of run
+// takes 3000 to 4800 cycles, a key tile 1750 with one M tile and 3600 with two.  Slack of 1, 2, 4 tiles against the line: 1 is 2-6 %
+// slower at 6 to 12 sequences, 4 is the same or 2 % slower.)
+constexpr int kRunOverheadTiles = 2;
+struct Shares {
+    int pieces;                                      // shares of a stretch
+    int whole;                                       // stretches of a share (1 where they are cut)
+    int total;                                       // shares of the sequence
+};
+__device__ __forceinline__ Shares shares_of(int tiles, int own, int Hkv)
+{
+    if (tiles == 0) return {0, 1, 0};
+    if (tiles + kRunOverheadTiles > own) {
+        const int pieces = (int)((uint32_t)(tiles + own - kRunOverheadTiles - 1) / (uint32_t)(own - kRunOverheadTiles));
+        return {pieces, 1, (int)min((int64_t)pieces * Hkv, (int64_t)kPlanMaxCtas + 1)};
+    }
+    const int whole = min((int)((uint32_t)own / (uint32_t)(tiles + kRunOverheadTiles)), min(Hkv, 1 << 14));
+    if (whole == 1) return {1, 1, min(Hkv, kPlanMaxCtas + 1)};
+    return {1, whole, (int)min((uint32_t)(Hkv + whole - 1) / (uint32_t)whole, (uint32_t)kPlanMaxCtas + 1)};
+}
 
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int units, int kind, const int64_t* __restrict__ seq_start,
                                                             const int32_t* __restrict__ prefix_len,
@@ -34,6 +58,9 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
     __shared__ int64_t s_base[kPlanCached + 1], s_slot[kPlanCached];
     __shared__ int64_t s_line;
     __shared__ int s_warp[kPlanMaxCtas / 32], s_own, s_ctas;
+    // shares of their own: pieces of a stretch, whole stretches of a share (in the place of the masks, which are done by then)
+    short2* s_cut = reinterpret_cast<short2*>(s_mask);
+    static_assert(sizeof(s_mask) >= kPlanCached * sizeof(short2), "s_cut");
     PlanView pv = plan_view(plan_raw, B, d.Hkv);
     const bool cached = B <= kPlanCached;
 
@@ -103,27 +130,40 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
         // The work is cut into `lanes` shares; CTA lane * n_rg + rg walks the lane's share for row group rg,
         // so the CTAs of a lane read the same K/V tiles at about the same time (the second read hits L2).
         int lanes = (units < kPlanMaxCtas ? units : kPlanMaxCtas) / n_rg;
-        // With few enough stretches every one can have shares of its own, of at most `own` tiles: where that is no
-        // longer than a share of the line, no work unit changes from one pair to the next.  (A layer at batch 1, prefix 4096:
-        // 34 tiles in 9 shares of at most 4 instead of a line cut into shares of 4.1, some of which span two pairs: 17.5 ->
-        // 16.9 us; prefix 512: 12.75 -> 12.2; 4 sequences of 500..4000: 23.9 -> 22.9; E4M3 cache, batch 1: 20.0 -> 18.3.)
+        // Every run costs its CTA a load of Q, a drain and output rows, or partial rows that the merge reads again: shares of
+        // their own (above) have one run or whole ones, where the line's have the end of one stretch and the beginning of another.
+        // They are taken where the longest is not over the line's share by more than what a run weighs.  (A layer with its append
+        // and merge, 8 kv heads, paged, 8 sequences of 101..3001, R 60: 27.7 -> 25.4 us, 72 instead of 144 CTAs with partial rows;
+        // 4 sequences of 500..4000, 64 / 8 heads, own plan: 40.0 -> 39.1; batch 1, prefix 4096: 34 tiles in 9 shares of 4
+        // instead of a line cut into shares of 4.1: 17.5 -> 16.9.  32 sequences of 512..16384: no such shares, the line.)
         int own = 0;
-        if (cached && (int64_t)B * d.Hkv <= lanes) {
-            uint32_t tiles = 0, line = 0;            // (at most kPlanMaxCtas sequences of at most 2^24 + 2 tiles)
+        if (cached && lanes > 0) {
+            bool huge = false;
+            uint32_t tiles = 0, line = 0;
             for (int b = lane; b < B; b += 32) {
+                huge = huge || s_tiles[b] >= (1 << 20);
                 tiles += (uint32_t)s_tiles[b];
                 line += s_tiles[b] ? (uint32_t)(s_tiles[b] + kPairOverheadTiles) : 0;
             }
             tiles = __reduce_add_sync(0xffffffffu, tiles);
             line = __reduce_add_sync(0xffffffffu, line);
-            if (tiles) {
-                const int longest = (int)(((uint64_t)line * d.Hkv + lanes - 1) / lanes);
-                for (own = (int)(((uint64_t)tiles * d.Hkv + lanes - 1) / lanes); own <= longest; ++own) {
-                    uint32_t shares = 0;
-                    for (int b = lane; b < B; b += 32) shares += (uint32_t)(s_tiles[b] + own - 1) / (uint32_t)own;
-                    if ((int)__reduce_add_sync(0xffffffffu, shares) * d.Hkv <= lanes) break;
+            // (32 bits hold these sums, and the products with the heads but for absurd numbers of them)
+            if (!__any_sync(0xffffffffu, huge) && tiles && (uint64_t)line * d.Hkv < (1u << 30)) {
+                const uint32_t L = (uint32_t)lanes, H = (uint32_t)d.Hkv;
+                int lo = (int)((tiles * H + L - 1) / L) + kRunOverheadTiles;         // no share is shorter than the mean
+                const int longest = (int)((line * H + L - 1) / L) + kRunOverheadTiles;
+#pragma unroll 1
+                for (int hi = longest + 1, at = lo; ; at = (lo + hi) / 2) {          // the shortest that fits
+                    if (lo >= hi) {
+                        own = hi <= longest ? hi : 0;
+                        break;
+                    }
+                    uint32_t n = 0;
+#pragma unroll 1
+                    for (int b = lane; b < B; b += 32) n += (uint32_t)shares_of(s_tiles[b], at, d.Hkv).total;
+                    if ((int)__reduce_add_sync(0xffffffffu, n) <= lanes) hi = at;
+                    else lo = at + 1;
                 }
-                if (own > longest) own = 0;
             }
         }
         // positions on the line, or share numbers
@@ -132,7 +172,11 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
             const int b = b0 + lane;
             const int tiles = b < B ? (cached ? s_tiles[b] : pv.tiles[b]) : 0;
             int64_t mine = tiles > 0 ? (int64_t)(tiles + kPairOverheadTiles) * d.Hkv : 0;
-            if (own) mine = (uint32_t)(tiles + own - 1) / (uint32_t)own * d.Hkv;
+            if (own) {
+                const Shares sh = shares_of(tiles, own, d.Hkv);
+                mine = sh.total;
+                if (b < B) s_cut[b] = make_short2((short)sh.pieces, (short)sh.whole);
+            }
             int64_t incl = mine;
 #pragma unroll 1
             for (int k = 1; k < 32 && k < B; k <<= 1) {
@@ -178,29 +222,36 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(confu_dims d, int un
             else hi = mid;
         }
     }
-    if (s_own) {                                     // shares of their own: one run each, a stretch's tiles dealt out evenly
+    if (s_own) {
         for (int u = tid; u < B * d.Hkv; u += (int)blockDim.x) {
-            const int b = u / d.Hkv, k = (s_tiles[b] + s_own - 1) / s_own;
-            pv.parts[u] = Parts::make(k ? (int)s_base[b] + u % d.Hkv * k : 0, k, kind);
+            const int b = u / d.Hkv, h = u % d.Hkv, pieces = s_cut[b].x, whole = s_cut[b].y;
+            pv.parts[u] = Parts::make(pieces ? (int)s_base[b] + (whole > 1 ? h / whole : h * pieces) : 0, pieces, kind);
         }
+        int n_runs = 0, begin = 0;
         if (c < n_ctas) {
-            const int nt = s_tiles[seq0], k = (nt + s_own - 1) / s_own, local = c / n_rg - (int)s_base[seq0], p = local % k;
+            const int nt = s_tiles[seq0], local = c / n_rg - (int)s_base[seq0], pieces = s_cut[seq0].x, whole = s_cut[seq0].y;
+            const int head = pieces > 1 ? local / pieces : local, p = local - head * pieces, head0 = head * whole;
+            n_runs = min(whole, d.Hkv - head0);
+            begin = (seq0 * d.Hkv + head0) * n_rg + c % n_rg * n_runs;       // (a share's runs have its stretches' places)
             SegDesc s;
             s.b = seq0;
-            s.g_rg = (local / k) | ((c % n_rg) << 16);
-            s.t0 = p * nt / k;
-            s.t1 = (p + 1) * nt / k;
+            s.t0 = pieces > 1 ? p * nt / pieces : 0;             // (256 pieces of 2^20 tiles at most)
+            s.t1 = pieces > 1 ? (p + 1) * nt / pieces : nt;
             s.nt = nt;
             s.P = prefix_len[seq0];
-            s.part_slot = k == 1 ? -1 : 2 * c + (p + 1 < k ? 1 : 0);
+            s.part_slot = pieces == 1 ? -1 : 2 * c + (p + 1 < pieces ? 1 : 0);
             s.pad0 = 0;
             s.slot0 = s_slot[seq0];
             s.pad1 = 0;
-            pv.cta[c].first = s;
+            for (int i = 0; i < n_runs; ++i) {
+                s.g_rg = (head0 + i) | ((c % n_rg) << 16);
+                if (i == 0) pv.cta[c].first = s;
+                else pv.segs[begin + i] = s;
+            }
         }
         if (c < kPlanMaxCtas) {
-            pv.cta[c].n_runs = c < n_ctas ? 1 : 0;
-            pv.cta[c].begin = 0;
+            pv.cta[c].n_runs = n_runs;
+            pv.cta[c].begin = begin;
             pv.cta[c].kind = kind;
         }
         return;

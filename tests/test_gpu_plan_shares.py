@@ -1,0 +1,105 @@
+"""Shares of a plan that hold several whole (sequence, kv head) stretches or one piece of a stretch: every key tile is walked
+exactly once, the merge is told who walked it, and attention over such plans agrees with the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2603_08899_b200 import binding as cb
+from paper_2603_08899_b200 import inputs
+from tests import harness as H
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gpu():
+    g = H.Gpu()
+    yield g
+    g.close()
+
+
+def _config(tiles, Hkv, G, T=60, C=4, S=0, D=128):
+    return inputs.VerifyConfig("shares", B=len(tiles), L=1, Hq=Hkv * G, Hkv=Hkv, D=D, T=T, C=C, S=S, V=32, prefix=(1, 2),
+                               tree="random", kv_dtype=torch.bfloat16, logit_dtype=torch.float32, sigma_logit=1.0,
+                               draft="independent", temperatures=(1.0,), seed=760 + len(tiles) + Hkv, max_depth=7, fanout=(1, 4))
+
+
+def _prefix(tiles, R):
+    return torch.tensor([max(128 * n - R - 3 * b, 1) for b, n in enumerate(tiles)], dtype=torch.int32)
+
+
+def _up(x):
+    return (x + 255) // 256 * 256
+
+
+def _runs(plan, B, Hkv):
+    """The runs of every work unit, and the words that tell the merge who walked a stretch."""
+    raw = plan.cpu().numpy()
+    at = 256 + _up(B * 128 * 8) + 2 * _up(B * 4) + _up((B + 1) * 8)
+    cta = raw[at:at + 256 * 64].view(np.int32).reshape(256, 16)
+    at += _up(256 * 64)
+    parts = raw[at:at + B * Hkv * 4].view(np.int32)
+    at += _up(B * Hkv * 4)
+    segs = raw[at:at + (raw.size - at) // 48 * 48].view(np.int32).reshape(-1, 12)
+    return [[cta[c, :12]] + [segs[cta[c, 13] + i] for i in range(1, cta[c, 12])] if cta[c, 12] else [] for c in range(256)], parts
+
+
+LENGTHS = [[22, 3, 18, 11, 6, 8, 5, 3], [40, 1, 1, 2, 1], [9, 2, 2, 1], [1] * 30, [30, 1] * 3, [2], [5, 5, 4, 4, 3], [17] * 7, [60, 3, 1] * 5]
+
+
+@pytest.mark.parametrize("Hkv,G,S", [(8, 4, 16), (3, 8, 0), (5, 3, 0), (1, 32, 0), (12, 1, 5)])
+@pytest.mark.parametrize("tiles", LENGTHS)
+def test_every_tile_once(gpu, tiles, Hkv, G, S):
+    cfg = _config(tiles, Hkv, G, S=S)
+    B, R = cfg.B, cfg.R
+    parent, owner = inputs.trees(cfg)
+    if B > 2:
+        parent[1, 5] = 7                             # a malformed tree in between: no shares
+    plen = _prefix(tiles, R)
+    seq_start, _ = inputs.cache_layout(cfg, plen)
+    dims = cb.make_dims(B, cfg.Hq, Hkv, cfg.D, cfg.T, cfg.C, S, cfg.kv_dtype)
+    plan = torch.zeros(cb.confu_plan_bytes(gpu.ctx, dims), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(B, dtype=torch.int32, device="cuda")
+    cb.confu_tree_plan(gpu.ctx, dims, seq_start.cuda(), plen.cuda(), parent.cuda(), owner.cuda(), plan, status)
+    torch.cuda.synchronize()
+    per_tile = 128 // G * (1 if cb.confu_attention_path(gpu.ctx, dims) == cb.ATTENTION_TENSOR_NARROW else 2)
+    n_rg = (R + per_tile - 1) // per_tile
+    runs, parts = _runs(plan, B, Hkv)
+    seen, walkers = {}, {}
+    for c, of_c in enumerate(runs):
+        slots = [int(r[6]) for r in of_c if r[6] >= 0]
+        assert len(slots) == len(set(slots)) <= 2 and all(s // 2 == c for s in slots)
+        for r in of_c:
+            b, g, rg, t0, t1, nt, P = int(r[0]), int(r[1]) & 0xffff, int(r[1]) >> 16, int(r[2]), int(r[3]), int(r[4]), int(r[5])
+            assert rg == c % n_rg and P == int(plen[b]) and nt == (P + R + 127) // 128 + (S > 0) and 0 <= t0 < t1 <= nt
+            assert (r[6] < 0) == (t0 == 0 and t1 == nt)
+            if r[6] >= 0:
+                assert int(r[6]) == 2 * c + (t1 < nt)
+            walkers.setdefault((b, g, rg), []).append(c)
+            for t in range(t0, t1):
+                assert (b, g, rg, t) not in seen
+                seen[b, g, rg, t] = c
+    good = [b for b in range(B) if not (B > 2 and b == 1)]
+    assert len(seen) == sum((int(plen[b]) + R + 127) // 128 + (S > 0) for b in good) * Hkv * n_rg
+    for u, word in enumerate(parts.tolist()):
+        b, g = divmod(u, Hkv)
+        first, n = word & 0xfff, (word >> 12) & 0xfff
+        assert n == (0 if b not in good else len(walkers[b, g, 0]))
+        for rg in range(n_rg if b in good else 0):
+            assert walkers[b, g, rg] == [(first + p) * n_rg + rg for p in range(n)]
+
+
+@pytest.mark.parametrize("tiles,Hkv,G,D", [([22, 3, 9, 11, 1, 2], 8, 4, 128), ([9, 2, 2, 1], 3, 8, 128), ([14, 1, 1, 2, 1], 8, 4, 64)])
+def test_attention_over_packed_shares(gpu, tiles, Hkv, G, D):
+    cfg = _config(tiles, Hkv, G, S=16, D=D)
+    parent, owner = inputs.trees(cfg)
+    plen = _prefix(tiles, cfg.R)
+    seq_start, n_slots = inputs.cache_layout(cfg, plen)
+    t = inputs.layer_tensors(cfg, 0, n_slots, device="cuda", seq_start=seq_start, prefix_len=plen)
+    want, want_lse, _ = H.oracle_attention(cfg, t, seq_start, plen, parent, owner)
+    for path in (cb.ATTENTION_AUTO, cb.ATTENTION_TENSOR):
+        gpu.set_path(path)
+        out, lse, st = H.gpu_attention(gpu, cfg, t, seq_start, plen, parent, owner, n_slots, use_plan=True)
+        gpu.set_path(cb.ATTENTION_AUTO)
+        assert st.tolist() == [0] * cfg.B
+        H.assert_attention_close(out, lse, want, want_lse, cfg.kv_dtype, f"{tiles}")

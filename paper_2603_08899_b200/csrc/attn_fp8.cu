@@ -550,11 +550,12 @@ attention_fp8_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sh.tmem_base;
-    // Everything above touches only this kernel's own shared and tensor memory, so it runs while the
-    // kernel before this one in the stream drains.  From here on global memory is read and written:
+    const PlanView pv = plan_view(const_cast<void*>(prm.plan), prm.d.B, prm.d.Hkv);
+    if (prm.prefetch && threadIdx.x == 11 * 32) prefetch_first<kD, kD>(prm, pv, &q_map, &k_map);
+    // Everything above touches only this kernel's own shared and tensor memory (but for that hint), so it runs while
+    // the kernel before this one in the stream drains.  From here on global memory is read and written:
     // every CTA waits until the kernels before this one have completed.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const PlanView pv = plan_view(const_cast<void*>(prm.plan), prm.d.B, prm.d.Hkv);
 
     if (warp < 8) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
@@ -647,6 +648,7 @@ cudaError_t launch_attention_fp8(const Ctx* ctx, const confu_dims& d, const void
     prm.map = map;
     prm.prefix_len = prefix_len;
     prm.plan = plan;
+    prm.prefetch = plan != ctx->workspace;           // (where a call's own plan lies)
     prm.partials = (float*)partials;
     prm.out = (__nv_bfloat16*)out;
     prm.lse = lse;

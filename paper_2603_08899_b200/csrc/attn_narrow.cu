@@ -401,9 +401,10 @@ attention_narrow_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sh.tmem_base;
+    const PlanView pv = plan_view(const_cast<void*>(prm.plan), prm.d.B, prm.d.Hkv);
+    if (prm.prefetch && threadIdx.x == 11 * 32) prefetch_first<D, 64>(prm, pv, &q_map, &k_map);
     // global memory is read and written from here on: the kernels before this one have completed
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const PlanView pv = plan_view(const_cast<void*>(prm.plan), prm.d.B, prm.d.Hkv);
     if (warp < 8) softmax_role<D, kSplit>(sh, prm, pv, tmem);
     else if (warp == 8) {
         if ((threadIdx.x & 31) == 0) producer_role(sh, prm, pv, &q_map, &k_map, &v_map, &ks_map, &vs_map);
@@ -457,6 +458,7 @@ static cudaError_t launch_d(const Ctx* ctx, const confu_dims& d, const void* q, 
     prm.map = map;
     prm.prefix_len = prefix_len;
     prm.plan = plan;
+    prm.prefetch = plan != ctx->workspace;           // (where a call's own plan lies)
     prm.partials = (float*)partials;
     prm.out = (__nv_bfloat16*)out;
     prm.lse = lse;

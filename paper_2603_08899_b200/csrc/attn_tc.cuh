@@ -28,6 +28,7 @@ struct Params {
     unsigned long long wait_ns;   // limit of every wait on an mbarrier (wall clock)
     const float* k_scale;         // E4M3 cache: value = code * scale[kv head] (device, [Hkv]); unused otherwise
     const float* v_scale;
+    int prefetch;                 // 1: the plan was made by an earlier call, what it says can be fetched ahead of time
 };
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)

@@ -665,6 +665,7 @@ cudaError_t launch_attention_pair(const Ctx* ctx, const confu_dims& d, const voi
     prm.map = map;
     prm.prefix_len = prefix_len;
     prm.plan = plan;
+    prm.prefetch = 0;
     prm.partials = (float*)partials;
     prm.out = (__nv_bfloat16*)out;
     prm.lse = lse;

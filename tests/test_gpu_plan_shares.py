@@ -103,3 +103,44 @@ def test_attention_over_packed_shares(gpu, tiles, Hkv, G, D):
         gpu.set_path(cb.ATTENTION_AUTO)
         assert st.tolist() == [0] * cfg.B
         H.assert_attention_close(out, lse, want, want_lse, cfg.kv_dtype, f"{tiles}")
+
+
+@pytest.mark.parametrize("path", ["auto", "one_cta_per_sm"])
+def test_plan_rewritten_between_layers(gpu, path):
+    """One plan buffer, plans of other lengths and attention calls right behind one another: what a CTA fetches ahead of time by the
+    plan before must not be what it works with."""
+    cfg = _config([9, 3, 5], 8, 4, S=16)
+    parent, owner = (x.cuda() for x in inputs.trees(cfg))
+    gpu.set_path(cb.ATTENTION_AUTO if path == "auto" else cb.ATTENTION_TENSOR)
+    dims = cb.make_dims(cfg.B, cfg.Hq, cfg.Hkv, cfg.D, cfg.T, cfg.C, cfg.S, cfg.kv_dtype)
+    gpu.ensure_ws(dims)
+    room = _prefix([9, 9, 9], cfg.R)
+    seq_start, n_slots = inputs.cache_layout(cfg, room)
+    t = inputs.layer_tensors(cfg, 0, n_slots, device="cuda", seq_start=seq_start, prefix_len=room)
+    ss = seq_start.cuda()
+    lengths = [_prefix(x, cfg.R).cuda() for x in ([9, 3, 5], [1, 9, 2], [4, 4, 9])]
+    plan = torch.zeros(cb.confu_plan_bytes(gpu.ctx, dims), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(cfg.B, dtype=torch.int32, device="cuda")
+
+    def step(n, out):
+        cb.confu_tree_plan(gpu.ctx, dims, ss, n, parent, owner, plan, status)
+        cb.confu_tree_attention(gpu.ctx, dims, t["q"], t["k_cache"], t["v_cache"], n_slots, ss, n, t["k_soft"], t["v_soft"], None, None,
+                                plan, out, None, status)
+
+    try:
+        alone = [torch.empty_like(t["q"]) for _ in lengths]
+        for n, out in zip(lengths, alone):
+            step(n, out)
+            torch.cuda.synchronize()
+            want, _, _ = H.oracle_attention(cfg, t, seq_start, n.cpu(), parent.cpu(), owner.cpu())
+            H.assert_attention_close(out.cpu(), None, want, None, cfg.kv_dtype)
+        outs = [[torch.empty_like(t["q"]) for _ in lengths] for _ in range(5)]
+        for o in outs:
+            for n, out in zip(lengths, o):
+                step(n, out)
+        torch.cuda.synchronize()
+        assert status.tolist() == [0] * cfg.B
+        for o in outs:
+            assert all(torch.equal(a, b) for a, b in zip(o, alone))
+    finally:
+        gpu.set_path(cb.ATTENTION_AUTO)

@@ -18,9 +18,9 @@ size_t accept_workspace_bytes(int B, int T, int /*V*/)
 }
 
 template <typename T>
-__device__ __forceinline__ void load8(const T* __restrict__ row, int i0, int V, bool vec_ok, float (&x)[kEpt])
+__device__ __forceinline__ void load8(const T* __restrict__ row, int i0, int V, float (&x)[kEpt])
 {
-    if (vec_ok && i0 + kEpt <= V) {
+    if (i0 + kEpt <= V) {
         if constexpr (sizeof(T) == 2) {
             const uint4 v = *reinterpret_cast<const uint4*>(row + i0);
             const uint32_t w[4] = {v.x, v.y, v.z, v.w};
@@ -93,26 +93,37 @@ __global__ void __launch_bounds__(256) row_stats_kernel(const T* __restrict__ tl
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int row = blockIdx.x, chunk = blockIdx.y, mat = blockIdx.z;
-    const T* base = (mat == 0 ? tl : dl) + (size_t)row * V;
-    const bool vec_ok = ((size_t)V * sizeof(T)) % 16 == 0;
-    const int lo = chunk * chunk_elems, hi = min(V, lo + chunk_elems);
+    // counted from the 16-byte boundary at or before the row's first entry, which has place `shift` (a chunk that is left without
+    // entries of its row writes the statistics of none)
+    const T* first = (mat == 0 ? tl : dl) + (size_t)row * V;
+    const int shift = (int)((reinterpret_cast<uintptr_t>(first) & 15u) / sizeof(T));
+    const T* base = first - shift;
+    const int lo = chunk * chunk_elems, hi = min(V + shift, lo + chunk_elems);
     const int tid = threadIdx.x;
 
     float m = -INFINITY, s = 0.f, bestv = -INFINITY;
     int arg = INT_MAX, flag = 0;
 
     int i0 = lo + tid * kEpt;
+    if (i0 < shift) {                                    // the vector that holds the row's first entries
+        for (int i = shift; i < min(kEpt, hi); ++i) {
+            const float v = to_f32(base[i]);
+            if (!(fabsf(v) <= 3.0e38f)) flag = 1;
+            if (v > bestv) { bestv = v; arg = i; }
+            if (v > m) { s *= ex2((m - v) * k2); m = v; }
+            s += ex2((v - m) * k2);
+        }
+        i0 += 256 * kEpt;
+    }
     if constexpr (sizeof(T) == 2) {
         // four vectors in flight per thread and folded in together (two, one after the other: 195 us for the 985 MB of 32
         // sequences of 60 nodes, V 128256; now 172 us, 5.7 TB/s)
-        if (vec_ok) {
-            constexpr int kStep = 256 * kEpt;
-            for (; i0 + 3 * kStep + kEpt <= hi; i0 += 4 * kStep) {
-                uint4 v[4];
+        constexpr int kStep = 256 * kEpt;
+        for (; i0 + 3 * kStep + kEpt <= hi; i0 += 4 * kStep) {
+            uint4 v[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) v[u] = *reinterpret_cast<const uint4*>(base + i0 + u * kStep);
-                stats_bf16(v, i0, kStep, k2, m, s, bestv, arg, flag);
-            }
+            for (int u = 0; u < 4; ++u) v[u] = *reinterpret_cast<const uint4*>(base + i0 + u * kStep);
+            stats_bf16(v, i0, kStep, k2, m, s, bestv, arg, flag);
         }
     }
     for (; i0 < hi; i0 += 256 * kEpt * 2) {
@@ -120,14 +131,14 @@ __global__ void __launch_bounds__(256) row_stats_kernel(const T* __restrict__ tl
         const int i1 = i0 + 256 * kEpt;
         if constexpr (sizeof(T) == 2) {
             // bf16 rows, both 8-element vectors whole: packed path (about 4 instructions per logit)
-            if (vec_ok && i1 + kEpt <= hi) {
+            if (i1 + kEpt <= hi) {
                 const uint4 v[2] = {*reinterpret_cast<const uint4*>(base + i0), *reinterpret_cast<const uint4*>(base + i1)};
                 stats_bf16(v, i0, 256 * kEpt, k2, m, s, bestv, arg, flag);
                 continue;
             }
         }
-        load8(base, i0, hi, vec_ok, x[0]);
-        if (i1 < hi) load8(base, i1, hi, vec_ok, x[1]);
+        load8(base, i0, hi, x[0]);
+        if (i1 < hi) load8(base, i1, hi, x[1]);
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const int ib = u == 0 ? i0 : i1;
@@ -174,7 +185,7 @@ __global__ void __launch_bounds__(256) row_stats_kernel(const T* __restrict__ tl
     if (tid == 0) {
         for (int w = 1; w < 8; ++w) merge(sm[w], ss[w], sv[w], sa[w], sf[w]);
         RowStat r;
-        r.m = m; r.s = s; r.arg = arg; r.flag = flag;
+        r.m = m; r.s = s; r.arg = arg == INT_MAX ? arg : arg - shift; r.flag = flag;
         stats[((size_t)mat * n_rows + row) * kStatChunksMax + chunk] = r;
     }
     (void)nch;
@@ -195,9 +206,10 @@ static cudaError_t launch_accept_t(int sm_count, int B, int Tn, int C, int V, co
     // enough CTAs to fill the machine a few times over, chunks a multiple of the vector width
     int nch = (sm_count * 8 + n_rows * nmat - 1) / (n_rows * nmat);
     nch = nch < 1 ? 1 : (nch > kStatChunksMax ? kStatChunksMax : nch);
-    int chunk_elems = (V + nch - 1) / nch;
+    const int all = ((size_t)V * sizeof(T)) % 16 == 0 ? V : V + 16 / (int)sizeof(T) - 1;      // places of a row, whatever its shift
+    int chunk_elems = (all + nch - 1) / nch;
     chunk_elems = (chunk_elems + 15) / 16 * 16;
-    nch = (V + chunk_elems - 1) / chunk_elems;
+    nch = (all + chunk_elems - 1) / chunk_elems;
     const float k2 = (greedy ? 1.f : 1.f / temperature) * kLog2e;
     RowStat* stats = (RowStat*)workspace;
     if (!lazy) {

@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(kThreads, 1) ratio_walk_kernel(const Args a, c
     const cg::cluster_group cluster = cg::this_cluster();
     const int n = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), b = blockIdx.x / n;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const Span sp = span_of<T>(a.V, rank, n);
+    Span sp = span_of<T>(a.V, rank, n);
     const double inv_temp = 1.0 / (double)a.temperature;
     const float k2 = (float)inv_temp * kLog2e;
     const double k64 = inv_temp * 1.4426950408889634;
@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(kThreads, 1) ratio_walk_kernel(const Args a, c
 
     cluster_arrive();                                // the peers' shared memory exists: waited for before the first exchange
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    to_row(sp, tl_b, a.V);
     prefetch_slice<T, E>(tl_b, sp);                  // the root's rows travel while the tree is fetched and checked
     prefetch_slice<T, E>(dl_b, sp);
     int flag = 0;
@@ -119,6 +120,7 @@ __global__ void __launch_bounds__(kThreads, 1) ratio_walk_kernel(const Args a, c
     for (;;) {
         Raw<T, E> xt, xd;
         float p[E], q[E];
+        to_row(sp, tl_b + (size_t)cur * a.V, a.V);   // (both matrices are aligned alike)
         xt.load(tl_b + (size_t)cur * a.V, sp);
         xd.load(dl_b + (size_t)cur * a.V, sp);
         // ---- maxima and normalisers of the node's two rows ----
@@ -408,13 +410,14 @@ __global__ void __launch_bounds__(kThreads, 1) match_walk_kernel(const Args a, c
     const cg::cluster_group cluster = cg::this_cluster();
     const int n = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), b = blockIdx.x / n;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const Span sp = span_of<T>(a.V, rank, n);
+    Span sp = span_of<T>(a.V, rank, n);
     const bool greedy = !(a.temperature > 0.f);
     const float k2 = (greedy ? 1.f : 1.f / a.temperature) * kLog2e;
     const T* tl_b = tl + (size_t)b * a.T * a.V;
 
     cluster_arrive();
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    to_row(sp, tl_b, a.V);
     prefetch_slice<T, E>(tl_b, sp);                  // the root's row travels while the tree is fetched and checked
     load_tree(tr, a, b, false);
     if (tid == 0) { sh.code = tr.code == INT_MAX ? 0 : tr.code; sh.done = 0; }
@@ -423,6 +426,7 @@ __global__ void __launch_bounds__(kThreads, 1) match_walk_kernel(const Args a, c
     int parity = 0, cur = 0, next = -1;
     while (!sh.code) {
         Raw<T, E> x;
+        to_row(sp, tl_b + (size_t)cur * a.V, a.V);
         x.load(tl_b + (size_t)cur * a.V, sp);
         // ---- the row's maximum and, when sampling, the sum of its weights 2^((x - maximum) k2) ----
         const bool bad = __any_sync(0xffffffffu, nonfinite(x, sp));
@@ -617,7 +621,7 @@ __global__ void __launch_bounds__(kThreads, 1) greedy_lazy_walk_kernel(const Arg
     const cg::cluster_group cluster = cg::this_cluster();
     const int n = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), b = blockIdx.x / n;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const Span sp = span_of<T>(a.V, rank, n);
+    Span sp = span_of<T>(a.V, rank, n);
 
     cluster_arrive();
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -630,6 +634,7 @@ __global__ void __launch_bounds__(kThreads, 1) greedy_lazy_walk_kernel(const Arg
     // argmax of a node's target row, into sh.best (all CTAs of the cluster take the same branches)
     auto need = [&](int node) {
         Raw<T, E> x;
+        to_row(sp, tl + ((size_t)b * a.T + node) * a.V, a.V);
         x.load(tl + ((size_t)b * a.T + node) * a.V, sp);
         const bool bad = __any_sync(0xffffffffu, nonfinite(x, sp));
         float m;
@@ -738,12 +743,12 @@ static cudaError_t by_vocabulary(int B, int V, F f)
 template <typename T>
 static cudaError_t walk_t(int B, const Args& a, const void* tl, const void* dl, int nch, const RowStat* stats, cudaStream_t st)
 {
-    return by_vocabulary(B, a.V, [&](auto e, int n) { return walk_e<T, decltype(e)::value>(n, B, a, (const T*)tl, (const T*)dl, nch, stats, st); });
+    return by_vocabulary(B, places<T>(a.V), [&](auto e, int n) { return walk_e<T, decltype(e)::value>(n, B, a, (const T*)tl, (const T*)dl, nch, stats, st); });
 }
 template <typename T>
 static cudaError_t match_t(int B, const Args& a, const void* tl, cudaStream_t st)
 {
-    return by_vocabulary(B, a.V, [&](auto e, int n) { return match_e<T, decltype(e)::value>(n, B, a, (const T*)tl, st); });
+    return by_vocabulary(B, places<T>(a.V), [&](auto e, int n) { return match_e<T, decltype(e)::value>(n, B, a, (const T*)tl, st); });
 }
 
 }  // namespace walk

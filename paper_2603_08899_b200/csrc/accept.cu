@@ -45,12 +45,12 @@ __device__ __forceinline__ void load8(const T* __restrict__ row, int i0, int V, 
 // K3: row statistics
 // ---------------------------------------------------------------------------------------------
 // N vectors of eight bf16 logits (16 bytes, starting at index ib and kStep apart) folded into a thread's running
-// statistics: maximum m, sum s of exp2((x - m) * k2), lowest index arg of the largest value bestv,
-// non-finite flag.  Maximum and minimum are taken on packed bf16 pairs with NaN propagation, so one
+// statistics: maximum m, non-finite flag, and what the walk behind it reads: sampling the sum s of exp2((x - m) * k2), greedy the lowest
+// index arg of the maximum.  (A search for the index is long, and with 32 lanes and a chunk of a few batches some lane finds a
+// new maximum in nearly every one.)  Maximum and minimum are taken on packed bf16 pairs with NaN propagation, so one
 // comparison of each against the finite range finds NaN and both infinities.
-template <int N>
-__device__ __forceinline__ void stats_bf16(const uint4 (&v)[N], int ib, int step, float k2, float& m, float& s, float& bestv, int& arg,
-                                           int& flag)
+template <int N, bool kGreedy>
+__device__ __forceinline__ void stats_bf16(const uint4 (&v)[N], int ib, int step, float k2, float& m, float& s, int& arg, int& flag)
 {
     uint32_t w[4 * N];
 #pragma unroll
@@ -62,15 +62,18 @@ __device__ __forceinline__ void stats_bf16(const uint4 (&v)[N], int ib, int step
     const float hi0 = __low2float(mx2), hi1 = __high2float(mx2), lo0 = __low2float(mn2), lo1 = __high2float(mn2);
     if (!(hi0 <= 3.0e38f && hi1 <= 3.0e38f && lo0 >= -3.0e38f && lo1 >= -3.0e38f)) flag = 1;
     const float cm = fmaxf(hi0, hi1);
-    if (cm > bestv) {                                    // rare after the first vectors: find the first element equal to it
-        bestv = cm;
+    if (cm > m) {
+        if (!kGreedy) s *= ex2((m - cm) * k2);
+        m = cm;
+        if (kGreedy) {                                   // the first element equal to it
 #pragma unroll
-        for (int j = 8 * N - 1; j >= 0; --j) {
-            const float x = __uint_as_float((j & 1) ? (w[j >> 1] & 0xffff0000u) : (w[j >> 1] << 16));
-            if (x == cm) arg = ib + (j >> 3) * step + (j & 7);
+            for (int j = 8 * N - 1; j >= 0; --j) {
+                const float x = __uint_as_float((j & 1) ? (w[j >> 1] & 0xffff0000u) : (w[j >> 1] << 16));
+                if (x == cm) arg = ib + (j >> 3) * step + (j & 7);
+            }
         }
     }
-    if (cm > m) { s *= ex2((m - cm) * k2); m = cm; }
+    if (kGreedy) return;
     const float nmk = -m * k2;
     uint64_t acc[2] = {f2_pack(0.f, 0.f), f2_pack(0.f, 0.f)};
     const uint64_t k22 = f2_pack(k2, k2), nmk2 = f2_pack(nmk, nmk);
@@ -85,110 +88,150 @@ __device__ __forceinline__ void stats_bf16(const uint4 (&v)[N], int ib, int step
     s += a0 + a1;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) row_stats_kernel(const T* __restrict__ tl, const T* __restrict__ dl, int V,
-                                                        int n_rows, int nch, int chunk_elems, float k2,
-                                                        RowStat* __restrict__ stats)
+// A warp's statistics in every lane: the maximum (as an integer of the same order: one reduction instruction), the sums
+// brought to it once, the lowest index that has it.  Values that are not there are (-inf, 0, INT_MAX).
+template <bool kGreedy>
+__device__ __forceinline__ void warp_stats(float k2, float& m, float& s, int& arg, int& flag)
+{
+    auto order = [](int i) { return i ^ ((i >> 31) & 0x7fffffff); };
+    const float M = __int_as_float(order(__reduce_max_sync(0xffffffffu, order(__float_as_int(m)))));
+    if (kGreedy) arg = __reduce_min_sync(0xffffffffu, m == M ? arg : INT_MAX);
+    else s = warp_sum(m == M ? s : s * ex2((m - M) * k2));
+    flag = __any_sync(0xffffffffu, flag);
+    m = M;
+}
+
+// W warps work on an item, a chunk of a row, then on the next; the launch is as many warps as the GPU holds at once.  HBM bound: what
+// counts is that enough loads are in flight (four vectors a lane) and that nothing else takes time: rounds of equal items that come
+// out even (see the launch) and a handful of reductions at the end of an item.
+constexpr int kStatWarps = 8;
+constexpr int kStatBlocks = 5;                            // per SM
+template <typename T, int W, bool kGreedy>
+__global__ void __launch_bounds__(32 * kStatWarps, kStatBlocks) row_stats_kernel(const T* __restrict__ tl, const T* __restrict__ dl, int V, int n_rows,
+                                                                       int items, int nch, int chunk_elems, float k2,
+                                                                       RowStat* __restrict__ stats)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int row = blockIdx.x, chunk = blockIdx.y, mat = blockIdx.z;
-    // counted from the 16-byte boundary at or before the row's first entry, which has place `shift` (a chunk that is left without
-    // entries of its row writes the statistics of none)
-    const T* first = (mat == 0 ? tl : dl) + (size_t)row * V;
-    const int shift = (int)((reinterpret_cast<uintptr_t>(first) & 15u) / sizeof(T));
-    const T* base = first - shift;
-    const int lo = chunk * chunk_elems, hi = min(V + shift, lo + chunk_elems);
-    const int tid = threadIdx.x;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int leader = warp / W * W;
+    __shared__ float sm[2][kStatWarps], ss[2][kStatWarps];
+    __shared__ int sa[2][kStatWarps], sf[2][kStatWarps];
+    int turn = 0;
+    for (int item = blockIdx.x * (kStatWarps / W) + warp / W; item < items; item += gridDim.x * (kStatWarps / W)) {
+        const int both = item / nch, chunk = item - both * nch, mat = both >= n_rows, row = both - (mat ? n_rows : 0);
+        // counted from the 16-byte boundary at or before the row's first entry, which has place `shift` (a chunk that is left without
+        // entries of its row writes the statistics of none)
+        const T* first = (mat == 0 ? tl : dl) + (size_t)row * V;
+        const int shift = (int)((reinterpret_cast<uintptr_t>(first) & 15u) / sizeof(T));
+        const T* base = first - shift;
+        const int lo = chunk * chunk_elems, hi = min(V + shift, lo + chunk_elems);
+        const int tid = (warp % W) * 32 + lane;
+        constexpr int kStep = W * 32 * kEpt;
 
-    float m = -INFINITY, s = 0.f, bestv = -INFINITY;
-    int arg = INT_MAX, flag = 0;
+        float m = -INFINITY, s = 0.f;
+        int arg = INT_MAX, flag = 0;
 
-    int i0 = lo + tid * kEpt;
-    if (i0 < shift) {                                    // the vector that holds the row's first entries
-        for (int i = shift; i < min(kEpt, hi); ++i) {
-            const float v = to_f32(base[i]);
-            if (!(fabsf(v) <= 3.0e38f)) flag = 1;
-            if (v > bestv) { bestv = v; arg = i; }
-            if (v > m) { s *= ex2((m - v) * k2); m = v; }
-            s += ex2((v - m) * k2);
+        int i0 = lo + tid * kEpt;
+        if (i0 < shift) {                                    // the vector that holds the row's first entries
+            for (int i = shift; i < min(kEpt, hi); ++i) {
+                const float v = to_f32(base[i]);
+                if (!(fabsf(v) <= 3.0e38f)) flag = 1;
+                if (v > m) { if (!kGreedy) s *= ex2((m - v) * k2); m = v; arg = i; }
+                if (!kGreedy) s += ex2((v - m) * k2);
+            }
+            i0 += kStep;
         }
-        i0 += 256 * kEpt;
-    }
-    if constexpr (sizeof(T) == 2) {
-        // four vectors in flight per thread and folded in together (two, one after the other: 195 us for the 985 MB of 32
-        // sequences of 60 nodes, V 128256; now 172 us, 5.7 TB/s)
-        constexpr int kStep = 256 * kEpt;
-        for (; i0 + 3 * kStep + kEpt <= hi; i0 += 4 * kStep) {
-            uint4 v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) v[u] = *reinterpret_cast<const uint4*>(base + i0 + u * kStep);
-            stats_bf16(v, i0, kStep, k2, m, s, bestv, arg, flag);
-        }
-    }
-    for (; i0 < hi; i0 += 256 * kEpt * 2) {
-        float x[2][kEpt];
-        const int i1 = i0 + 256 * kEpt;
         if constexpr (sizeof(T) == 2) {
-            // bf16 rows, both 8-element vectors whole: packed path (about 4 instructions per logit)
-            if (i1 + kEpt <= hi) {
-                const uint4 v[2] = {*reinterpret_cast<const uint4*>(base + i0), *reinterpret_cast<const uint4*>(base + i1)};
-                stats_bf16(v, i0, 256 * kEpt, k2, m, s, bestv, arg, flag);
-                continue;
+            for (; i0 + 3 * kStep + kEpt <= hi; i0 += 4 * kStep) {
+                uint4 v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = *reinterpret_cast<const uint4*>(base + i0 + u * kStep);
+                stats_bf16<4, kGreedy>(v, i0, kStep, k2, m, s, arg, flag);
             }
         }
-        load8(base, i0, hi, x[0]);
-        if (i1 < hi) load8(base, i1, hi, x[1]);
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int ib = u == 0 ? i0 : i1;
-            if (ib >= hi) break;
-            float lm = x[u][0];
-#pragma unroll
-            for (int j = 1; j < kEpt; ++j) lm = fmaxf(lm, x[u][j]);
-            if (lm > m) { s *= exp2f((m - lm) * k2); m = lm; }
-            float acc = 0.f;
-#pragma unroll
-            for (int j = 0; j < kEpt; ++j) {
-                const float v = x[u][j];
-                const bool in = ib + j < hi;
-                if (in && !(fabsf(v) <= 3.0e38f)) flag = 1;
-                acc += exp2f((v - m) * k2);                      // out-of-range entries are -inf -> 0
-                if (v > bestv) { bestv = v; arg = ib + j; }
+        for (; i0 < hi; i0 += 2 * kStep) {
+            float x[2][kEpt];
+            const int i1 = i0 + kStep;
+            if constexpr (sizeof(T) == 2) {
+                // bf16 rows, both 8-element vectors whole: packed path (about 4 instructions per logit)
+                if (i1 + kEpt <= hi) {
+                    const uint4 v[2] = {*reinterpret_cast<const uint4*>(base + i0), *reinterpret_cast<const uint4*>(base + i1)};
+                    stats_bf16<2, kGreedy>(v, i0, kStep, k2, m, s, arg, flag);
+                    continue;
+                }
             }
-            s += acc;
+            load8(base, i0, hi, x[0]);
+            if (i1 < hi) load8(base, i1, hi, x[1]);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int ib = u == 0 ? i0 : i1;
+                if (ib >= hi) break;
+                float lm = x[u][0];
+#pragma unroll
+                for (int j = 1; j < kEpt; ++j) lm = fmaxf(lm, x[u][j]);
+                if (lm > m) {
+                    if (!kGreedy) s *= ex2((m - lm) * k2);
+                    m = lm;
+                    if (kGreedy) {
+#pragma unroll
+                        for (int j = kEpt - 1; j >= 0; --j)
+                            if (x[u][j] == lm) arg = ib + j;
+                    }
+                }
+                float acc = 0.f;
+#pragma unroll
+                for (int j = 0; j < kEpt; ++j) {
+                    const float v = x[u][j];
+                    if (ib + j < hi && !(fabsf(v) <= 3.0e38f)) flag = 1;
+                    if (!kGreedy) acc += ex2((v - m) * k2);                        // out-of-range entries are -inf -> 0
+                }
+                s += acc;
+            }
+        }
+        warp_stats<kGreedy>(k2, m, s, arg, flag);
+        if constexpr (W > 1) {
+            if (lane == 0) { sm[turn][warp] = m; ss[turn][warp] = s; sa[turn][warp] = arg; sf[turn][warp] = flag; }
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + warp / W), "r"(32 * W) : "memory");
+            m = -INFINITY; s = 0.f; arg = INT_MAX; flag = 0;
+            if (lane < W) { m = sm[turn][leader + lane]; s = ss[turn][leader + lane]; arg = sa[turn][leader + lane]; flag = sf[turn][leader + lane]; }
+            if (warp == leader) warp_stats<kGreedy>(k2, m, s, arg, flag);
+            turn ^= 1;                               // (the next item's are written elsewhere: one barrier an item)
+        }
+        if (lane == 0 && warp == leader) {
+            RowStat r;
+            r.m = m; r.s = s; r.arg = arg == INT_MAX ? arg : arg - shift; r.flag = flag;
+            stats[(size_t)both * kStatChunksMax + chunk] = r;
         }
     }
-    // block reduction of (m, s), (bestv, arg), flag
-    auto merge = [&](float m2, float s2, float v2, int a2, int f2) {
-        const float mm = fmaxf(m, m2);
-        const float c1 = (m == mm) ? 1.f : exp2f((m - mm) * k2);
-        const float c2 = (m2 == mm) ? 1.f : exp2f((m2 - mm) * k2);
-        s = s * c1 + s2 * c2;
-        m = mm;
-        if (v2 > bestv || (v2 == bestv && a2 < arg)) { bestv = v2; arg = a2; }
-        flag |= f2;
-    };
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float m2 = __shfl_xor_sync(0xffffffffu, m, o);
-        const float s2 = __shfl_xor_sync(0xffffffffu, s, o);
-        const float v2 = __shfl_xor_sync(0xffffffffu, bestv, o);
-        const int a2 = __shfl_xor_sync(0xffffffffu, arg, o);
-        const int f2 = __shfl_xor_sync(0xffffffffu, flag, o);
-        merge(m2, s2, v2, a2, f2);
-    }
-    __shared__ float sm[8], ss[8], sv[8];
-    __shared__ int sa[8], sf[8];
-    if ((tid & 31) == 0) { sm[tid >> 5] = m; ss[tid >> 5] = s; sv[tid >> 5] = bestv; sa[tid >> 5] = arg; sf[tid >> 5] = flag; }
-    __syncthreads();
-    if (tid == 0) {
-        for (int w = 1; w < 8; ++w) merge(sm[w], ss[w], sv[w], sa[w], sf[w]);
-        RowStat r;
-        r.m = m; r.s = s; r.arg = arg == INT_MAX ? arg : arg - shift; r.flag = flag;
-        stats[((size_t)mat * n_rows + row) * kStatChunksMax + chunk] = r;
-    }
-    (void)nch;
+}
+
+// The statistics of all rows.  Chunks per row and warps per chunk: so that the rounds that a warp makes come out even, by what a round
+// takes it: its share of the entries, and what the end of an item stands for (some 0.3 us, of which a warp reads one entry per
+// nanosecond).  A block of 8 warps per row or chunk of a row, maximum's index and sum both, parts merged as a tree with two exponentials a
+// step -> so, us with the walk behind it, T 60: sampling, bf16, V 128256, B 1 28.7 -> 26.6, 3 43.5 -> 40.6, 8 81 -> 77, 16 123 -> 119, 32
+// 213 -> 215; V 32000, B 2 24.6 -> 22.7, 8 36.9 -> 32.2, 32 87 -> 84; fp32, V 128256, B 8 127 -> 118; greedy, bf16, V 128256, B 16 53.3 -> 45.
+// Blocks per SM (registers against warps) 3, 4, 5, 6, 8 at B 16: 132, 132, 119, 126, 134; the next four vectors loaded ahead: 120 -> 132.
+template <typename T, bool kGreedy>
+static cudaError_t launch_stats(int sm_count, int n_rows, int nmat, int V, const T* tl, const T* dl, float k2, RowStat* stats, int& nch, cudaStream_t st)
+{
+    const int all = ((size_t)V * sizeof(T)) % 16 == 0 ? V : V + 16 / (int)sizeof(T) - 1;      // places of a row, whatever its shift
+    const int64_t rows = (int64_t)n_rows * nmat, room = (int64_t)sm_count * kStatBlocks * kStatWarps;
+    int W = 1;
+    int64_t least = INT64_MAX;
+    for (int c = 1; c <= kStatChunksMax; ++c)
+        for (int w = 1; w <= kStatWarps; w *= 2) {
+            const int64_t groups = room / w, rounds = (rows * c + groups - 1) / groups;
+            const int64_t cost = rounds * ((all + c - 1) / c / w + (w > 1 ? 384 : 256));
+            if (cost < least && (c == 1 || rows * c < (1 << 30))) { least = cost; nch = c; W = w; }
+        }
+    int chunk_elems = (all + nch - 1) / nch;
+    chunk_elems = (chunk_elems + 15) / 16 * 16;
+    nch = (all + chunk_elems - 1) / chunk_elems;
+    const int64_t items = rows * nch, per = kStatWarps / W, want = (items + per - 1) / per, most = (int64_t)sm_count * kStatBlocks;
+    const int64_t blocks = want < most ? want : most;
+    auto kernel = W == 1 ? row_stats_kernel<T, 1, kGreedy> : W == 2 ? row_stats_kernel<T, 2, kGreedy> : W == 4 ? row_stats_kernel<T, 4, kGreedy> : row_stats_kernel<T, 8, kGreedy>;
+    return launch_pdl(kernel, dim3((unsigned)blocks), dim3(32 * kStatWarps), st, tl, dl, V, n_rows, (int)items, nch, chunk_elems, k2, stats);
 }
 
 template <typename T>
@@ -203,18 +246,12 @@ static cudaError_t launch_accept_t(int sm_count, int B, int Tn, int C, int V, co
     const bool greedy = !(temperature > 0.f);
     const int n_rows = B * Tn;
     const int nmat = greedy ? 1 : 2;
-    // enough CTAs to fill the machine a few times over, chunks a multiple of the vector width
-    int nch = (sm_count * 8 + n_rows * nmat - 1) / (n_rows * nmat);
-    nch = nch < 1 ? 1 : (nch > kStatChunksMax ? kStatChunksMax : nch);
-    const int all = ((size_t)V * sizeof(T)) % 16 == 0 ? V : V + 16 / (int)sizeof(T) - 1;      // places of a row, whatever its shift
-    int chunk_elems = (all + nch - 1) / nch;
-    chunk_elems = (chunk_elems + 15) / 16 * 16;
-    nch = (all + chunk_elems - 1) / chunk_elems;
+    int nch = 0;
     const float k2 = (greedy ? 1.f : 1.f / temperature) * kLog2e;
     RowStat* stats = (RowStat*)workspace;
     if (!lazy) {
-        const cudaError_t e = launch_pdl(row_stats_kernel<T>, dim3(n_rows, nch, nmat), dim3(256), st, (const T*)tl, (const T*)dl, V,
-                                         n_rows, nch, chunk_elems, k2, stats);
+        const cudaError_t e = greedy ? launch_stats<T, true>(sm_count, n_rows, nmat, V, (const T*)tl, (const T*)dl, k2, stats, nch, st)
+                                     : launch_stats<T, false>(sm_count, n_rows, nmat, V, (const T*)tl, (const T*)dl, k2, stats, nch, st);
         if (e != cudaSuccess) return e;
     }
     return launch_walk(sizeof(T) == 4 ? CONFU_F32 : CONFU_BF16, B, Tn, C, V, tl, dl, tokens, parent, con_owner, uniforms, temperature,

@@ -10,8 +10,8 @@ constexpr float kLog2e = 1.4426950408889634f;
 
 struct alignas(16) RowStat {
     float m;        // max raw logit of the chunk
-    float s;        // sum over the chunk of exp((x - m) / temperature)
-    int32_t arg;    // lowest index of the max
+    float s;        // sampling: sum over the chunk of exp((x - m) / temperature)
+    int32_t arg;    // greedy: lowest index of the max
     int32_t flag;   // 1: a non-finite logit was met
 };
 

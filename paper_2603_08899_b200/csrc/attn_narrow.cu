@@ -245,7 +245,7 @@ __device__ void softmax_role(SharedStorage<D>& sh, const Params& prm, const Plan
             tmem_ld32(s_addr + buf * 128, *reinterpret_cast<uint32_t(*)[32]>(&sv[0]));
             tmem_ld32(s_addr + buf * 128 + 32, *reinterpret_cast<uint32_t(*)[32]>(&sv[32]));
             tc_wait_ld();
-            if (tile >= s.nkt || (int64_t)(tile + 1) * kTileKeys > s.P) {
+            if (tile >= s.masked) {
                 uint64_t lo, hi;
                 visible_bits(s, tile, R, T, S, r, row_valid, mask, lo, hi);
                 const uint64_t vis = half ? hi : lo;

@@ -44,27 +44,13 @@ __device__ __forceinline__ void load8(const T* __restrict__ row, int i0, int V, 
 // ---------------------------------------------------------------------------------------------
 // K3: row statistics
 // ---------------------------------------------------------------------------------------------
-// The weight of a logit and the factor of a sum whose maximum moves from a to b.  bf16 rows: 2^(x k2 - m k2) as one fused operation, with
-// the rounded product m k2 that the whole sum has in common; what it is off, 2^-24 of m k2, would be in every weight, so the
-// end of an item takes it out again (`settled`; max error of a row's sum 1.3e-6 without, 2e-7 with it).  fp32 rows: the difference first.
-template <typename T> __device__ __forceinline__ float weight(float x, float m, float k2)
-{
-    return sizeof(T) == 2 ? ex2(fmaf(x, k2, -__fmul_rn(m, k2))) : ex2((x - m) * k2);
-}
-template <typename T> __device__ __forceinline__ float moved(float a, float b, float k2)
-{
-    return sizeof(T) == 2 ? ex2(__fsub_rn(__fmul_rn(a, k2), __fmul_rn(b, k2))) : ex2((a - b) * k2);
-}
-template <typename T> __device__ __forceinline__ float settled(float s, float m, float k2)
-{
-    return sizeof(T) == 2 && m > -INFINITY ? s * ex2(-fmaf(m, k2, -__fmul_rn(m, k2))) : s;
-}
-
 // N vectors of eight bf16 logits (16 bytes, starting at index ib and kStep apart) folded into a thread's running
 // statistics: maximum m, non-finite flag, and what the walk behind it reads: sampling the sum s of exp2((x - m) * k2), greedy the lowest
 // index arg of the maximum.  (A search for the index is long, and with 32 lanes and a chunk of a few batches some lane finds a
 // new maximum in nearly every one.)  Maximum and minimum are taken on packed bf16 pairs with NaN propagation, so one
-// comparison of each against the finite range finds NaN and both infinities.
+// comparison of each against the finite range finds NaN and both infinities.  The exponent is (x - m) * k2, the difference first: as one
+// fused operation with m * k2 it is wrong where that product leaves fp32 (a row mostly masked with -2.5e38) or is rounded by
+// more than the exponents (temperature 1e-9), and no faster (B 32, T 60, V 128256: 217.4 us with the walk, 214.7 so).
 template <int N, bool kGreedy>
 __device__ __forceinline__ void stats_bf16(const uint4 (&v)[N], int ib, int step, float k2, float& m, float& s, int& arg, int& flag)
 {
@@ -79,7 +65,7 @@ __device__ __forceinline__ void stats_bf16(const uint4 (&v)[N], int ib, int step
     if (!(hi0 <= 3.0e38f && hi1 <= 3.0e38f && lo0 >= -3.0e38f && lo1 >= -3.0e38f)) flag = 1;
     const float cm = fmaxf(hi0, hi1);
     if (cm > m) {
-        if (!kGreedy) s *= moved<__nv_bfloat16>(m, cm, k2);
+        if (!kGreedy) s *= ex2((m - cm) * k2);
         m = cm;
         if (kGreedy) {                                   // the first element equal to it
 #pragma unroll
@@ -90,13 +76,12 @@ __device__ __forceinline__ void stats_bf16(const uint4 (&v)[N], int ib, int step
         }
     }
     if (kGreedy) return;
-    const float nmk = -__fmul_rn(m, k2);
     uint64_t acc[2] = {f2_pack(0.f, 0.f), f2_pack(0.f, 0.f)};
-    const uint64_t k22 = f2_pack(k2, k2), nmk2 = f2_pack(nmk, nmk);
+    const uint64_t k22 = f2_pack(k2, k2), nm2 = f2_pack(-m, -m);
 #pragma unroll
     for (int j = 0; j < 4 * N; ++j) {
         float x0, x1;
-        f2_unpack(f2_fma(f2_pack(__uint_as_float(w[j] << 16), __uint_as_float(w[j] & 0xffff0000u)), k22, nmk2), x0, x1);
+        f2_unpack(f2_mul(f2_add(f2_pack(__uint_as_float(w[j] << 16), __uint_as_float(w[j] & 0xffff0000u)), nm2), k22), x0, x1);
         acc[j & 1] = f2_add(acc[j & 1], f2_pack(ex2(x0), ex2(x1)));
     }
     float a0, a1;
@@ -153,8 +138,8 @@ __global__ void __launch_bounds__(32 * kStatWarps, kStatBlocks) row_stats_kernel
             for (int i = shift; i < min(kEpt, hi); ++i) {
                 const float v = to_f32(base[i]);
                 if (!(fabsf(v) <= 3.0e38f)) flag = 1;
-                if (v > m) { if (!kGreedy) s *= moved<T>(m, v, k2); m = v; arg = i; }
-                if (!kGreedy) s += weight<T>(v, m, k2);
+                if (v > m) { if (!kGreedy) s *= ex2((m - v) * k2); m = v; arg = i; }
+                if (!kGreedy) s += ex2((v - m) * k2);
             }
             i0 += kStep;
         }
@@ -187,7 +172,7 @@ __global__ void __launch_bounds__(32 * kStatWarps, kStatBlocks) row_stats_kernel
 #pragma unroll
                 for (int j = 1; j < kEpt; ++j) lm = fmaxf(lm, x[u][j]);
                 if (lm > m) {
-                    if (!kGreedy) s *= moved<T>(m, lm, k2);
+                    if (!kGreedy) s *= ex2((m - lm) * k2);
                     m = lm;
                     if (kGreedy) {
 #pragma unroll
@@ -200,12 +185,11 @@ __global__ void __launch_bounds__(32 * kStatWarps, kStatBlocks) row_stats_kernel
                 for (int j = 0; j < kEpt; ++j) {
                     const float v = x[u][j];
                     if (ib + j < hi && !(fabsf(v) <= 3.0e38f)) flag = 1;
-                    if (!kGreedy) acc += weight<T>(v, m, k2);                        // out-of-range entries are -inf -> 0
+                    if (!kGreedy) acc += ex2((v - m) * k2);                          // out-of-range entries are -inf -> 0
                 }
                 s += acc;
             }
         }
-        if (!kGreedy) s = settled<T>(s, m, k2);
         warp_stats<kGreedy>(k2, m, s, arg, flag);
         if constexpr (W > 1) {
             if (lane == 0) { sm[turn][warp] = m; ss[turn][warp] = s; sa[turn][warp] = arg; sf[turn][warp] = flag; }

@@ -44,15 +44,31 @@ __device__ __forceinline__ void load8(const T* __restrict__ row, int i0, int V, 
 // ---------------------------------------------------------------------------------------------
 // K3: row statistics
 // ---------------------------------------------------------------------------------------------
+// A lane's running sum, with what its additions have lost so far (Kahan's summation).  A warp that has a row or a chunk of one to itself
+// makes hundreds of them, and beside a weight of 1 each can drop half a unit in the last place: fp32, V 151936, 16 sequences
+// of 60 rows, one logit 18.75 above all others: 1.1e-5 of a row's sum (256 threads to a chunk: 4.5e-6), so 1.2e-7; deviation 5: root mean
+// square 3.3e-7 (1.7e-7), so 4.8e-8; bf16 3.0e-6 (1.2e-6) and 9.8e-8 (3.3e-7), so 1.1e-7 and 5.2e-8.  (That ex2 flushes weights below
+// 2^-126 of the lane's largest changes no sum: exp2f gave the same bits.)
+struct Sum {
+    float s = 0.f, over = 0.f;                       // over: by how much s is above the exact sum
+    __device__ __forceinline__ void add(float a)
+    {
+        const float y = a - over, t = s + y;
+        over = (t - s) - y;
+        s = t;
+    }
+    __device__ __forceinline__ void scale(float f) { s *= f; over *= f; }
+};
+
 // N vectors of eight bf16 logits (16 bytes, starting at index ib and kStep apart) folded into a thread's running
-// statistics: maximum m, non-finite flag, and what the walk behind it reads: sampling the sum s of exp2((x - m) * k2), greedy the lowest
+// statistics: maximum m, non-finite flag, and what the walk behind it reads: sampling the sum of exp2((x - m) * k2), greedy the lowest
 // index arg of the maximum.  (A search for the index is long, and with 32 lanes and a chunk of a few batches some lane finds a
 // new maximum in nearly every one.)  Maximum and minimum are taken on packed bf16 pairs with NaN propagation, so one
 // comparison of each against the finite range finds NaN and both infinities.  The exponent is (x - m) * k2, the difference first: as one
 // fused operation with m * k2 it is wrong where that product leaves fp32 (a row mostly masked with -2.5e38) or is rounded by
 // more than the exponents (temperature 1e-9), and no faster (B 32, T 60, V 128256: 217.4 us with the walk, 214.7 so).
 template <int N, bool kGreedy>
-__device__ __forceinline__ void stats_bf16(const uint4 (&v)[N], int ib, int step, float k2, float& m, float& s, int& arg, int& flag)
+__device__ __forceinline__ void stats_bf16(const uint4 (&v)[N], int ib, int step, float k2, float& m, Sum& sum, int& arg, int& flag)
 {
     uint32_t w[4 * N];
 #pragma unroll
@@ -65,7 +81,7 @@ __device__ __forceinline__ void stats_bf16(const uint4 (&v)[N], int ib, int step
     if (!(hi0 <= 3.0e38f && hi1 <= 3.0e38f && lo0 >= -3.0e38f && lo1 >= -3.0e38f)) flag = 1;
     const float cm = fmaxf(hi0, hi1);
     if (cm > m) {
-        if (!kGreedy) s *= ex2((m - cm) * k2);
+        if (!kGreedy) sum.scale(exp2f((m - cm) * k2));   // (with ex2 the kernel spills registers)
         m = cm;
         if (kGreedy) {                                   // the first element equal to it
 #pragma unroll
@@ -86,7 +102,7 @@ __device__ __forceinline__ void stats_bf16(const uint4 (&v)[N], int ib, int step
     }
     float a0, a1;
     f2_unpack(f2_add(acc[0], acc[1]), a0, a1);
-    s += a0 + a1;
+    sum.add(a0 + a1);
 }
 
 // A warp's statistics in every lane: the maximum (as an integer of the same order: one reduction instruction), the sums
@@ -130,7 +146,8 @@ __global__ void __launch_bounds__(32 * kStatWarps, kStatBlocks) row_stats_kernel
         const int tid = (warp % W) * 32 + lane;
         constexpr int kStep = W * 32 * kEpt;
 
-        float m = -INFINITY, s = 0.f;
+        float m = -INFINITY;
+        Sum sum;
         int arg = INT_MAX, flag = 0;
 
         int i0 = lo + tid * kEpt;
@@ -138,8 +155,8 @@ __global__ void __launch_bounds__(32 * kStatWarps, kStatBlocks) row_stats_kernel
             for (int i = shift; i < min(kEpt, hi); ++i) {
                 const float v = to_f32(base[i]);
                 if (!(fabsf(v) <= 3.0e38f)) flag = 1;
-                if (v > m) { if (!kGreedy) s *= ex2((m - v) * k2); m = v; arg = i; }
-                if (!kGreedy) s += ex2((v - m) * k2);
+                if (v > m) { if (!kGreedy) sum.scale(ex2((m - v) * k2)); m = v; arg = i; }
+                if (!kGreedy) sum.add(ex2((v - m) * k2));
             }
             i0 += kStep;
         }
@@ -148,7 +165,7 @@ __global__ void __launch_bounds__(32 * kStatWarps, kStatBlocks) row_stats_kernel
                 uint4 v[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) v[u] = *reinterpret_cast<const uint4*>(base + i0 + u * kStep);
-                stats_bf16<4, kGreedy>(v, i0, kStep, k2, m, s, arg, flag);
+                stats_bf16<4, kGreedy>(v, i0, kStep, k2, m, sum, arg, flag);
             }
         }
         for (; i0 < hi; i0 += 2 * kStep) {
@@ -158,7 +175,7 @@ __global__ void __launch_bounds__(32 * kStatWarps, kStatBlocks) row_stats_kernel
                 // bf16 rows, both 8-element vectors whole: packed path (about 4 instructions per logit)
                 if (i1 + kEpt <= hi) {
                     const uint4 v[2] = {*reinterpret_cast<const uint4*>(base + i0), *reinterpret_cast<const uint4*>(base + i1)};
-                    stats_bf16<2, kGreedy>(v, i0, kStep, k2, m, s, arg, flag);
+                    stats_bf16<2, kGreedy>(v, i0, kStep, k2, m, sum, arg, flag);
                     continue;
                 }
             }
@@ -172,7 +189,7 @@ __global__ void __launch_bounds__(32 * kStatWarps, kStatBlocks) row_stats_kernel
 #pragma unroll
                 for (int j = 1; j < kEpt; ++j) lm = fmaxf(lm, x[u][j]);
                 if (lm > m) {
-                    if (!kGreedy) s *= ex2((m - lm) * k2);
+                    if (!kGreedy) sum.scale(ex2((m - lm) * k2));
                     m = lm;
                     if (kGreedy) {
 #pragma unroll
@@ -187,9 +204,10 @@ __global__ void __launch_bounds__(32 * kStatWarps, kStatBlocks) row_stats_kernel
                     if (ib + j < hi && !(fabsf(v) <= 3.0e38f)) flag = 1;
                     if (!kGreedy) acc += ex2((v - m) * k2);                          // out-of-range entries are -inf -> 0
                 }
-                s += acc;
+                if (!kGreedy) sum.add(acc);
             }
         }
+        float s = sum.s - sum.over;
         warp_stats<kGreedy>(k2, m, s, arg, flag);
         if constexpr (W > 1) {
             if (lane == 0) { sm[turn][warp] = m; ss[turn][warp] = s; sa[turn][warp] = arg; sf[turn][warp] = flag; }

@@ -43,3 +43,52 @@ def test_masked_rows(gpu, V, dtype, mask, temperature):
         got = H.gpu_accept(gpu, cfg, tl, dl, tok, parent, owner, u, temperature, 1 | lazy)
         assert got["status"].tolist() == want["status"].tolist()
         assert H.compare_accept(got, want) == (cfg.B, 0)
+
+
+def _row_sums(gpu, tl, dl, temperature):
+    """Sum of exp((x - maximum) / temperature) of every target and draft row, from the statistics that the call leaves in its workspace:
+    16 entries of 16 bytes a row (maximum of a chunk, its sum, two integers), the first ones used."""
+    B, T, V = tl.shape
+    ws = torch.zeros(cb.confu_accept_workspace_bytes(B, T, V), dtype=torch.uint8, device="cuda")
+    ws.view(torch.float32)[0::4] = -float("inf")
+    i32 = dict(dtype=torch.int32, device="cuda")
+    out = [torch.zeros(n, **i32) for n in ((B,), (B, cb.MAX_DEPTH + 1), (B,), (B,), (B, 4))]
+    tokens = torch.arange(T, **i32).expand(B, T).contiguous()
+    parent = torch.arange(-1, T - 1, **i32).expand(B, T).contiguous()
+    uniforms = torch.full((B, T), 0.5, device="cuda")
+    status = torch.zeros(B, **i32)
+    cb.confu_tree_accept(gpu.ctx, B, T, 0, V, tl.dtype, tl, dl, tokens, parent, None, uniforms, temperature, 1, *out, ws, status)
+    torch.cuda.synchronize()
+    assert not status.any()
+    part = ws.view(torch.float32)[:2 * B * T * 64].view(2 * B * T, 16, 4).double()
+    m, s = part[..., 0], part[..., 1]
+    top = m.max(1, keepdim=True).values
+    return top[:, 0], (s * torch.exp((m - top) / temperature)).sum(1)
+
+
+# A warp to a row, to a chunk of a row (two rounds of them in the last case), two and eight warps to a chunk (148 SMs).  Half of the rows:
+# one logit far above all others, read among the first, so that its lane's sum takes in hundreds of weights that are next to
+# nothing beside it (eight of an fp32 row, 32 of a bf16 row at a time: a little less than half a unit in its last place).  The other
+# half: deviation 5.
+@pytest.mark.parametrize("dtype,low", [(torch.bfloat16, -20.125), (torch.float32, -18.75)])
+@pytest.mark.parametrize("B,T,V", [(49, 60, 48003), (3, 60, 128256), (2, 47, 5000), (1, 5, 151937), (37, 32, 4099)])
+def test_error_of_sums(gpu, B, T, V, dtype, low):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(B + V)
+    x = torch.randn((2, B, T, V), generator=g, device="cuda") * 5
+    x[:, :, ::2] = low
+    at = torch.randint(0, min(V, 256), (2, B, T, 1), generator=g, device="cuda")
+    x[:, :, ::2] = x[:, :, ::2].scatter(3, at[:, :, ::2], 0.0)
+    x = x.to(dtype)
+    top, got = _row_sums(gpu, x[0].clone(), x[1].clone(), 1.0)
+    rows = x.view(2 * B * T, V)
+    want = torch.stack([torch.exp(r.double() - t).sum() for r, t in zip(rows, top)])
+    assert torch.equal(top, rows.max(1).values.double())
+    err = (got / want - 1).abs()
+    # In units of 2^-24 of the sum: 8 + 2 for the additions in front of a lane's sum, 1 for that sum with its correction, 5 and 3 for a
+    # warp's and a chunk's (fp64 after that); a weight's own error is the exponential unit's 2 and, of its argument a, |a| ln 2 twice:
+    # next to nothing where the sum is its largest weight (|a| of the mean weight some 4 at deviation 5, and as often up as down).
+    lone = torch.arange(2 * B * T, device="cuda") % T % 2 == 0
+    assert err[lone].max().item() <= 19 * 2.0 ** -24
+    assert err[~lone].max().item() <= (19 + 2 + 6) * 2.0 ** -24
+    assert err[~lone].square().mean().sqrt().item() <= 4 * 2.0 ** -24

@@ -194,7 +194,9 @@ struct OncePerDevice {
 
 // Launch as a programmatic dependent: the kernel's blocks may be scheduled while the kernel before it in the stream
 // drains.  Every kernel launched like this executes griddepcontrol.wait in all its threads before it touches global
-// memory, so that ordinary stream order holds, transitively (1-1.5 us per launch of a chain of short kernels).
+// memory, so that ordinary stream order holds, transitively (1-1.5 us per launch of a chain of short kernels).  One thing comes
+// before the wait: an attention kernel reads its plan record, and a block-table entry that this names, to ask for what it will
+// read first (tc_walk.cuh, prefetch_lane); whatever is there at that moment only decides what is fetched into L2.
 template <typename... P, typename... A>
 inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args)
 {

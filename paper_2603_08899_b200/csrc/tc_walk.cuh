@@ -74,7 +74,7 @@ private:
 // 27 of 39..794, 9 layers, E4M3: 393 -> 389.  V of the first tile too: the same; K and V of four tiles: +4 %; batch 1, 8 / 8 heads,
 // prefix 14054: +0.4 %.
 template <int D, int kXStep>
-__device__ __forceinline__ void prefetch_first(const Params& p, const PlanView& v, const CUtensorMap* q_map, const CUtensorMap* k_map)
+__device__ __forceinline__ void prefetch_lane(const Params& p, const PlanView& v, const CUtensorMap* q_map, const CUtensorMap* k_map)
 {
     const int4* w = reinterpret_cast<const int4*>(v.cta + blockIdx.x);
     const int4 w0 = __ldcg(w), w1 = __ldcg(w + 1), w2 = __ldcg(w + 2);
@@ -88,6 +88,13 @@ __device__ __forceinline__ void prefetch_first(const Params& p, const PlanView& 
     for (int mt = 0; mt < p.n_mt; ++mt)
 #pragma unroll
         for (int x = 0; x < D; x += 64) tma_prefetch_3d(q_map, x, g * p.G, b * (p.d.T + p.d.C) + p.rpt * (p.tpg * rg + mt));
+}
+// The same by a whole warp, which is together again behind it: setmaxnreg comes next.
+template <int D, int kXStep>
+__device__ __forceinline__ void prefetch_first(const Params& p, const PlanView& v, const CUtensorMap* q_map, const CUtensorMap* k_map)
+{
+    if ((threadIdx.x & 31) == 0) prefetch_lane<D, kXStep>(p, v, q_map, k_map);
+    __syncwarp();
 }
 
 // Slots of key tile `tile` that belong to the sequence when the tile is its last key tile and

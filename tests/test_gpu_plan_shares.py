@@ -144,3 +144,58 @@ def test_plan_rewritten_between_layers(gpu, path):
             assert all(torch.equal(a, b) for a, b in zip(o, alone))
     finally:
         gpu.set_path(cb.ATTENTION_AUTO)
+
+
+@pytest.mark.parametrize("kv", [torch.bfloat16, torch.float8_e4m3fn])
+@pytest.mark.parametrize("paged", [False, True])
+def test_fetch_ahead_by_a_stale_record(gpu, kv, paged):
+    """Plan and block table rewritten in stream order between attention calls right behind one another: the record that a CTA reads ahead
+    of time, and the table's entry that it names, may be those of the call before (or of none: the first plan is zeros)."""
+    fp8 = kv == torch.float8_e4m3fn
+    cfg = inputs.VerifyConfig("stale", B=3, L=1, Hq=32, Hkv=8, D=128, T=60, C=4, S=16, V=32, prefix=(1, 2), tree="random", kv_dtype=kv,
+                              logit_dtype=torch.float32, sigma_logit=1.0, draft="independent", temperatures=(1.0,), seed=771, max_depth=7,
+                              fanout=(1, 4))
+    parent, owner = (x.cuda() for x in inputs.trees(cfg))
+    dims = cb.make_dims(cfg.B, cfg.Hq, cfg.Hkv, cfg.D, cfg.T, cfg.C, cfg.S, torch.uint8 if fp8 else kv)
+    pages, max_pages = 27, 9                         # of 128 slots, nine to a sequence
+    t = inputs.layer_tensors(cfg, 0, pages * 128, device="cuda")
+    seq_start = torch.arange(3, device="cuda") * max_pages * 128
+    packed = torch.arange(pages, dtype=torch.int32, device="cuda").view(3, max_pages)
+    lengths = [_prefix(x, cfg.R).cuda() for x in ([9, 3, 5], [1, 9, 2], [4, 4, 9])]
+    order = [torch.from_numpy(np.random.default_rng(i).permutation(pages)).cuda() for i in range(3)]
+    # pool i holds page p of the packed one at order[i][p]
+    pools = [{n: torch.empty_like(t[n]).view(pages, 128, 8, 128).index_copy_(0, o, t[n].view(pages, 128, 8, 128)).view_as(t[n])
+              for n in ("k_cache", "v_cache")} if paged else t for o in order]
+    tables = [o.to(torch.int32)[packed.long()].contiguous() for o in order]
+    table = torch.zeros_like(packed)
+    if fp8:
+        cb.confu_set_kv_scales(gpu.ctx, t["k_scale"], t["v_scale"])
+    gpu.ensure_ws(dims)
+    plan = torch.zeros(cb.confu_plan_bytes(gpu.ctx, dims), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(cfg.B, dtype=torch.int32, device="cuda")
+
+    def step(i, pool, ss, out):
+        cb.confu_tree_plan(gpu.ctx, dims, ss, lengths[i], parent, owner, plan, status)
+        cb.confu_tree_attention(gpu.ctx, dims, t["q"], pool["k_cache"], pool["v_cache"], pages * 128, ss, lengths[i], t["k_soft"], t["v_soft"],
+                                None, None, plan, out, None, status)
+
+    try:
+        alone = [torch.empty_like(t["q"]) for _ in lengths]          # packed, one call at a time: tested against the oracle elsewhere
+        for i, out in enumerate(alone):
+            step(i, t, seq_start, out)
+            torch.cuda.synchronize()
+        if paged:
+            cb.confu_set_paging(gpu.ctx, table, max_pages)
+        plan.zero_()
+        outs = [[torch.empty_like(t["q"]) for _ in lengths] for _ in range(5)]
+        for o in outs:
+            for i, out in enumerate(o):
+                table.copy_(tables[i])
+                step(i, pools[i], None if paged else seq_start, out)
+        torch.cuda.synchronize()
+        assert status.tolist() == [0] * cfg.B
+        for o in outs:
+            assert all(torch.equal(a, b) for a, b in zip(o, alone))
+    finally:
+        cb.confu_set_paging(gpu.ctx, None)
+        cb.confu_set_kv_scales(gpu.ctx, None, None)

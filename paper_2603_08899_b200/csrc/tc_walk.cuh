@@ -71,8 +71,11 @@ private:
 // it is read past L1, and a box that lies outside its tensor is not fetched.  One lane of a warp that has nothing else to do, before
 // griddepcontrol.wait (the producer's own lane would start its loads late: prefix 8192 +0.7 %).  A step of 28 layers at batch 1,
 // prefix 2048: 395 -> 388 us; 32 layers, prefix 4096: 505 -> 501; 8 sequences of 101..3001, 32 layers with their appends: 855 -> 837;
-// 27 of 39..794, 9 layers, E4M3: 393 -> 389.  V of the first tile too: the same; K and V of four tiles: +4 %; batch 1, 8 / 8 heads,
-// prefix 14054: +0.4 %.
+// 27 of 39..794, 9 layers, E4M3: 393 -> 389.  V of the first tile too: the same; K and V of four tiles: +4 %.
+// A box of Q with fewer than 64 rows inside the tensor is not asked for: most of a box outside holds the TMA unit up, and with it
+// the K tile behind.  16 layers at batch 1, prefix 3000, 8 / 8 heads, us without any fetch, with Q and K, with K alone: 10 rows 218, 234, 212; 48
+// 221, 224, 215; 64 220, 212, 213; 32 / 8 heads, 40 rows 215, 216, 208; 64 214, 206, 208; 4 sequences, 24 rows 260, 287, 257.
+constexpr int kQRowsFetched = 64;
 template <int D, int kXStep>
 __device__ __forceinline__ void prefetch_lane(const Params& p, const PlanView& v, const CUtensorMap* q_map, const CUtensorMap* k_map)
 {
@@ -85,9 +88,13 @@ __device__ __forceinline__ void prefetch_lane(const Params& p, const PlanView& v
     const int z = (int)(page * kTileKeys + (p.map.block_table ? 0u : (uint32_t)w2.x));
 #pragma unroll
     for (int x = 0; x < D; x += kXStep) tma_prefetch_3d(k_map, x, g, z);
-    for (int mt = 0; mt < p.n_mt; ++mt)
+    const int R = p.d.T + p.d.C, rows = p.d.B * R;
+    for (int mt = 0; mt < p.n_mt; ++mt) {
+        const int at = b * R + p.rpt * (p.tpg * rg + mt);
+        if ((int64_t)(rows - at) * p.G < kQRowsFetched) continue;
 #pragma unroll
-        for (int x = 0; x < D; x += 64) tma_prefetch_3d(q_map, x, g * p.G, b * (p.d.T + p.d.C) + p.rpt * (p.tpg * rg + mt));
+        for (int x = 0; x < D; x += 64) tma_prefetch_3d(q_map, x, g * p.G, at);
+    }
 }
 // The same by a whole warp, which is together again behind it: setmaxnreg comes next.
 template <int D, int kXStep>

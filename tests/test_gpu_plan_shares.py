@@ -199,3 +199,40 @@ def test_fetch_ahead_by_a_stale_record(gpu, kv, paged):
     finally:
         cb.confu_set_paging(gpu.ctx, None)
         cb.confu_set_kv_scales(gpu.ctx, None, None)
+
+
+@pytest.mark.parametrize("kv", [torch.bfloat16, torch.float8_e4m3fn])
+@pytest.mark.parametrize("B,Hkv,G,T,C", [(1, 8, 1, 4, 0), (1, 8, 1, 60, 3), (1, 8, 1, 60, 4), (3, 2, 1, 20, 4), (1, 2, 3, 20, 1), (1, 2, 3, 20, 2),
+                                         (1, 2, 4, 15, 0), (1, 2, 4, 16, 0), (2, 2, 8, 7, 0), (1, 2, 4, 60, 60), (2, 2, 3, 50, 10)])
+def test_few_rows_of_q(gpu, kv, B, Hkv, G, T, C):
+    """Boxes of Q with 63, 64 and other few rows inside the tensor, under a plan made beforehand (what is asked for ahead of time depends on
+    them) and under the call's own (nothing is)."""
+    fp8 = kv == torch.float8_e4m3fn
+    if fp8 and G > 4:
+        pytest.skip("E4M3 caches: up to four query heads per kv head")
+    cfg = inputs.VerifyConfig("few", B=B, L=1, Hq=Hkv * G, Hkv=Hkv, D=128, T=T, C=C, S=3, V=32, prefix=(100, 900), tree="chain", kv_dtype=kv,
+                              logit_dtype=torch.float32, sigma_logit=1.0, draft="independent", temperatures=(1.0,), seed=780 + T)
+    parent, owner, plen, seq_start, n_slots, t = H.setup_case(cfg)
+    parent, owner, plen, seq_start = parent.cuda(), owner.cuda() if C else None, plen.cuda(), seq_start.cuda()
+    dims = cb.make_dims(B, cfg.Hq, Hkv, 128, T, C, 3, torch.uint8 if fp8 else kv)
+    gpu.ensure_ws(dims)
+    if fp8:
+        cb.confu_set_kv_scales(gpu.ctx, t["k_scale"], t["v_scale"])
+    plan = torch.zeros(cb.confu_plan_bytes(gpu.ctx, dims), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(B, dtype=torch.int32, device="cuda")
+    outs = [torch.empty_like(t["q"]) for _ in range(3)]
+    try:
+        for path in (cb.ATTENTION_AUTO, cb.ATTENTION_TENSOR):
+            gpu.set_path(path)
+            cb.confu_tree_plan(gpu.ctx, dims, seq_start, plen, parent, owner, plan, status)
+            for out, own in zip(outs, (False, False, True)):
+                cb.confu_tree_attention(gpu.ctx, dims, t["q"], t["k_cache"], t["v_cache"], n_slots, seq_start, plen, t["k_soft"], t["v_soft"],
+                                        parent if own else None, owner if own else None, None if own else plan, out, None, status)
+            torch.cuda.synchronize()
+            assert not status.any() and all(torch.equal(outs[0], x) for x in outs[1:])
+            if not fp8:
+                want, _, _ = H.oracle_attention(cfg, t, seq_start.cpu(), plen.cpu(), parent.cpu(), owner.cpu() if C else torch.zeros((B, 0)))
+                H.assert_attention_close(outs[0].cpu(), None, want, None, kv)
+    finally:
+        gpu.set_path(cb.ATTENTION_AUTO)
+        cb.confu_set_kv_scales(gpu.ctx, None, None)

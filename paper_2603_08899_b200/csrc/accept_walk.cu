@@ -45,7 +45,7 @@ struct RatioShared {
     double off, target, total;
 };
 
-template <typename T, int E, bool kLazy>
+template <typename T, int E, bool kRagged, bool kLazy>
 __global__ void __launch_bounds__(kThreads, 1) ratio_walk_kernel(const Args a, const T* __restrict__ tl, const T* __restrict__ dl, int nch,
                                                               int n_rows, const RowStat* __restrict__ stats)
 {
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kThreads, 1) ratio_walk_kernel(const Args a, c
 
     cluster_arrive();                                // the peers' shared memory exists: waited for before the first exchange
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    to_row(sp, tl_b, a.V);
+    to_row<kRagged>(sp, tl_b, a.V);
     prefetch_slice<T, E>(tl_b, sp);                  // the root's rows travel while the tree is fetched and checked
     prefetch_slice<T, E>(dl_b, sp);
     int flag = 0;
@@ -118,9 +118,9 @@ __global__ void __launch_bounds__(kThreads, 1) ratio_walk_kernel(const Args a, c
     int parity = 0, cur = 0;
     bool again = false;                              // a node whose residual had no mass: drawn from its target row after all
     for (;;) {
-        Raw<T, E> xt, xd;
+        Raw<T, E, kRagged> xt, xd;
         float p[E], q[E];
-        to_row(sp, tl_b + (size_t)cur * a.V, a.V);   // (both matrices are aligned alike)
+        to_row<kRagged>(sp, tl_b + (size_t)cur * a.V, a.V);   // (both matrices are aligned alike)
         xt.load(tl_b + (size_t)cur * a.V, sp);
         xd.load(dl_b + (size_t)cur * a.V, sp);
         // ---- maxima and normalisers of the node's two rows ----
@@ -382,8 +382,8 @@ __device__ __forceinline__ void best_slot(const Exchange& ex, int parity, int n,
     if (__any_sync(0xffffffffu, bad)) m = NAN;
 }
 // A warp's largest entry and its lowest index (INT_MAX: no entry); every lane gets both.
-template <typename T, int E>
-__device__ __forceinline__ void warp_best(const Raw<T, E>& x, const Span& sp, float& m, int& arg)
+template <typename T, int E, bool kRagged>
+__device__ __forceinline__ void warp_best(const Raw<T, E, kRagged>& x, const Span& sp, float& m, int& arg)
 {
     m = -INFINITY;
 #pragma unroll
@@ -402,7 +402,7 @@ __device__ __forceinline__ void warp_best(const Raw<T, E>& x, const Span& sp, fl
     }
 }
 
-template <typename T, int E>
+template <typename T, int E, bool kRagged>
 __global__ void __launch_bounds__(kThreads, 1) match_walk_kernel(const Args a, const T* __restrict__ tl)
 {
     __shared__ MatchShared sh;
@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(kThreads, 1) match_walk_kernel(const Args a, c
 
     cluster_arrive();
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    to_row(sp, tl_b, a.V);
+    to_row<kRagged>(sp, tl_b, a.V);
     prefetch_slice<T, E>(tl_b, sp);                  // the root's row travels while the tree is fetched and checked
     load_tree(tr, a, b, false);
     if (tid == 0) { sh.code = tr.code == INT_MAX ? 0 : tr.code; sh.done = 0; }
@@ -425,8 +425,8 @@ __global__ void __launch_bounds__(kThreads, 1) match_walk_kernel(const Args a, c
     cluster_wait();
     int parity = 0, cur = 0, next = -1;
     while (!sh.code) {
-        Raw<T, E> x;
-        to_row(sp, tl_b + (size_t)cur * a.V, a.V);
+        Raw<T, E, kRagged> x;
+        to_row<kRagged>(sp, tl_b + (size_t)cur * a.V, a.V);
         x.load(tl_b + (size_t)cur * a.V, sp);
         // ---- the row's maximum and, when sampling, the sum of its weights 2^((x - maximum) k2) ----
         const bool bad = __any_sync(0xffffffffu, nonfinite(x, sp));
@@ -613,7 +613,7 @@ struct GreedyShared {
     int code;
 };
 
-template <typename T, int E>
+template <typename T, int E, bool kRagged>
 __global__ void __launch_bounds__(kThreads, 1) greedy_lazy_walk_kernel(const Args a, const T* __restrict__ tl)
 {
     __shared__ GreedyShared sh;
@@ -633,8 +633,8 @@ __global__ void __launch_bounds__(kThreads, 1) greedy_lazy_walk_kernel(const Arg
     int parity = 0;
     // argmax of a node's target row, into sh.best (all CTAs of the cluster take the same branches)
     auto need = [&](int node) {
-        Raw<T, E> x;
-        to_row(sp, tl + ((size_t)b * a.T + node) * a.V, a.V);
+        Raw<T, E, kRagged> x;
+        to_row<kRagged>(sp, tl + ((size_t)b * a.T + node) * a.V, a.V);
         x.load(tl + ((size_t)b * a.T + node) * a.V, sp);
         const bool bad = __any_sync(0xffffffffu, nonfinite(x, sp));
         float m;
@@ -702,19 +702,19 @@ static cudaError_t launch_cluster(void (*kernel)(P...), OncePerDevice& attr_done
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-template <typename T, int E>
+template <typename T, int E, bool kRagged>
 static cudaError_t walk_e(int n, int B, const Args& a, const T* tl, const T* dl, int nch, const RowStat* stats, cudaStream_t st)
 {
     static OncePerDevice once[3];
-    if (!(a.temperature > 0.f)) return launch_cluster(greedy_lazy_walk_kernel<T, E>, once[0], B, n, st, a, tl);
-    if (stats) return launch_cluster(ratio_walk_kernel<T, E, false>, once[1], B, n, st, a, tl, dl, nch, B * a.T, stats);
-    return launch_cluster(ratio_walk_kernel<T, E, true>, once[2], B, n, st, a, tl, dl, nch, B * a.T, stats);
+    if (!(a.temperature > 0.f)) return launch_cluster(greedy_lazy_walk_kernel<T, E, kRagged>, once[0], B, n, st, a, tl);
+    if (stats) return launch_cluster(ratio_walk_kernel<T, E, kRagged, false>, once[1], B, n, st, a, tl, dl, nch, B * a.T, stats);
+    return launch_cluster(ratio_walk_kernel<T, E, kRagged, true>, once[2], B, n, st, a, tl, dl, nch, B * a.T, stats);
 }
-template <typename T, int E>
+template <typename T, int E, bool kRagged>
 static cudaError_t match_e(int n, int B, const Args& a, const T* tl, cudaStream_t st)
 {
     static OncePerDevice once;
-    return launch_cluster(match_walk_kernel<T, E>, once, B, n, st, a, tl);
+    return launch_cluster(match_walk_kernel<T, E, kRagged>, once, B, n, st, a, tl);
 }
 
 // CTAs per sequence and entries per thread.  A walk is as fast as its slices are small, so a small batch with a large
@@ -743,12 +743,19 @@ static cudaError_t by_vocabulary(int B, int V, F f)
 template <typename T>
 static cudaError_t walk_t(int B, const Args& a, const void* tl, const void* dl, int nch, const RowStat* stats, cudaStream_t st)
 {
-    return by_vocabulary(B, places<T>(a.V), [&](auto e, int n) { return walk_e<T, decltype(e)::value>(n, B, a, (const T*)tl, (const T*)dl, nch, stats, st); });
+    return by_vocabulary(B, places<T>(a.V), [&](auto e, int n) {
+        constexpr int E = decltype(e)::value;
+        return places<T>(a.V) == a.V ? walk_e<T, E, false>(n, B, a, (const T*)tl, (const T*)dl, nch, stats, st)
+                                     : walk_e<T, E, true>(n, B, a, (const T*)tl, (const T*)dl, nch, stats, st);
+    });
 }
 template <typename T>
 static cudaError_t match_t(int B, const Args& a, const void* tl, cudaStream_t st)
 {
-    return by_vocabulary(B, places<T>(a.V), [&](auto e, int n) { return match_e<T, decltype(e)::value>(n, B, a, (const T*)tl, st); });
+    return by_vocabulary(B, places<T>(a.V), [&](auto e, int n) {
+        constexpr int E = decltype(e)::value;
+        return places<T>(a.V) == a.V ? match_e<T, E, false>(n, B, a, (const T*)tl, st) : match_e<T, E, true>(n, B, a, (const T*)tl, st);
+    });
 }
 
 }  // namespace walk

@@ -51,7 +51,10 @@ struct Search {
 // slices
 // ---------------------------------------------------------------------------------------------
 // A row is counted from the 16-byte boundary at or before its first entry, `shift` places earlier, so that vectors can be loaded
-// whatever the vocabulary size is (rows that start anywhere, entry by entry: B 3, V 77777, ratio rule with statistics 49 us, now 35).
+// whatever the vocabulary size is (rows that start anywhere, entry by entry: B 3, V 77777, ratio rule with statistics 49 us, now 31).
+// kRagged: a row's bytes are no multiple of 16, so shifts differ from row to row.  Kernels of their own: where all rows are aligned the code for
+// ends of rows, never run, cost registers (spill loads of the ratio rule at V 128256 156 -> 196 bytes, now 132; B 8 on demand 40.8 us
+// without it, 41.5 with it, 40.8 so; B 32 with statistics 217.5 -> 211.5).
 // CTA `rank` of n owns places [rank * chunk, (rank + 1) * chunk), chunk a multiple of 8; run s of thread t starts at place
 // rank * chunk + s * kStrip + 8 t.
 struct Span {
@@ -71,16 +74,17 @@ __device__ __forceinline__ Span span_of(int V, int rank, int n)
     s.end = s.lim;
     return s;
 }
-template <typename T>
+template <bool kRagged, typename T>
 __device__ __forceinline__ void to_row(Span& s, const T* row, int V)
 {
+    if (!kRagged) return;
     s.shift = (int)((reinterpret_cast<uintptr_t>(row) & 15u) / sizeof(T));
     s.end = min(s.lim, V + s.shift);
 }
 
 // E entries of a row as they lie in memory (bf16: two to a word); places outside the slice or the row are -inf.
-template <typename T, int E> struct Raw;
-template <int E> struct Raw<__nv_bfloat16, E> {
+template <typename T, int E, bool kRagged> struct Raw;
+template <int E, bool kRagged> struct Raw<__nv_bfloat16, E, kRagged> {
     uint32_t w[E / 2];
     __device__ __forceinline__ void load(const __nv_bfloat16* row, const Span& sp)
     {
@@ -89,10 +93,10 @@ template <int E> struct Raw<__nv_bfloat16, E> {
 #pragma unroll
         for (int s = 0; s < E / kRun; ++s) {
             uint4 v = make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
-            if ((s > 0 || i >= sp.shift) && i + s * kStrip + kRun <= sp.end) v = *reinterpret_cast<const uint4*>(r + i + s * kStrip);
+            if ((!kRagged || s > 0 || i >= sp.shift) && i + s * kStrip + kRun <= sp.end) v = *reinterpret_cast<const uint4*>(r + i + s * kStrip);
             w[4 * s] = v.x; w[4 * s + 1] = v.y; w[4 * s + 2] = v.z; w[4 * s + 3] = v.w;
         }
-        if ((sp.shift | sp.end % kRun) == 0) return;
+        if (!kRagged || (sp.shift | sp.end % kRun) == 0) return;
         // the vectors that hold the row's first and last entries
         auto piece = [&](int k, int j) {
             const int a = k + 2 * j;
@@ -115,7 +119,7 @@ template <int E> struct Raw<__nv_bfloat16, E> {
     }
     __device__ __forceinline__ float at(int e) const { return __uint_as_float((e & 1) ? (w[e >> 1] & 0xffff0000u) : (w[e >> 1] << 16)); }
 };
-template <int E> struct Raw<float, E> {
+template <int E, bool kRagged> struct Raw<float, E, kRagged> {
     float x[E];
     __device__ __forceinline__ void load(const float* row, const Span& sp)
     {
@@ -125,10 +129,10 @@ template <int E> struct Raw<float, E> {
         for (int h = 0; h < E / 4; ++h) {
             const int k = i + h / 2 * kStrip + h % 2 * 4;
             float4 v = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-            if ((h > 0 || i >= sp.shift) && k + 4 <= sp.end) v = *reinterpret_cast<const float4*>(r + k);
+            if ((!kRagged || h > 0 || i >= sp.shift) && k + 4 <= sp.end) v = *reinterpret_cast<const float4*>(r + k);
             x[4 * h] = v.x; x[4 * h + 1] = v.y; x[4 * h + 2] = v.z; x[4 * h + 3] = v.w;
         }
-        if ((sp.shift | sp.end % 4) == 0) return;
+        if (!kRagged || (sp.shift | sp.end % 4) == 0) return;
         auto piece = [&](int k) { return k >= sp.shift && k < sp.end ? r[k] : -INFINITY; };
         if (i < sp.shift) {
 #pragma unroll
@@ -160,8 +164,8 @@ __device__ __forceinline__ void prefetch_slice(const T* row, const Span& sp)
 __device__ __forceinline__ int entry(const Span& sp, int e) { return sp.base - sp.shift + (e / kRun) * kStrip + (int)threadIdx.x * kRun + e % kRun; }
 
 // an entry that belongs to the slice and is not a finite number (padding is -inf and does not count)
-template <typename T, int E>
-__device__ __forceinline__ bool nonfinite(const Raw<T, E>& r, const Span& sp)
+template <typename T, int E, bool kRagged>
+__device__ __forceinline__ bool nonfinite(const Raw<T, E, kRagged>& r, const Span& sp)
 {
     bool bad = false;
 #pragma unroll

@@ -702,19 +702,45 @@ static cudaError_t launch_cluster(void (*kernel)(P...), OncePerDevice& attr_done
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-template <typename T, int E, bool kRagged>
+// Where all rows are aligned a walk without the code for ends of rows (kRagged) is taken if it is the faster one, us with it -> without: ratio
+// rule, bf16, statistics given, 16 sequences of V 4096 (8 entries a thread) 18.9 -> 18.6, of 128256 (32) 60.0 -> 57.0, on demand 23.1 ->
+// 22.4, 38.7 -> 38.4; fp32, 5 of 151936 (24) 91.8 -> 89.8, but 9 of them (40) 71.0 -> 72.7; argmax on demand up to 16 entries, fp32, V
+// 4096 12.0 -> 11.8, but bf16, 16 of 128256 17.9 -> 18.5; sample-and-match from 24 on, bf16, 9 of 151936 14.2 -> 13.8, but 4 of 32000 (8)
+// 13.1 -> 14.0.
+template <bool kTight, typename F>
+static cudaError_t by_alignment(bool aligned, F f)
+{
+    if constexpr (kTight) {
+        if (aligned) return f(std::false_type());
+    }
+    return f(std::true_type());
+}
+template <typename T, int E>
 static cudaError_t walk_e(int n, int B, const Args& a, const T* tl, const T* dl, int nch, const RowStat* stats, cudaStream_t st)
 {
-    static OncePerDevice once[3];
-    if (!(a.temperature > 0.f)) return launch_cluster(greedy_lazy_walk_kernel<T, E, kRagged>, once[0], B, n, st, a, tl);
-    if (stats) return launch_cluster(ratio_walk_kernel<T, E, kRagged, false>, once[1], B, n, st, a, tl, dl, nch, B * a.T, stats);
-    return launch_cluster(ratio_walk_kernel<T, E, kRagged, true>, once[2], B, n, st, a, tl, dl, nch, B * a.T, stats);
+    const bool aligned = places<T>(a.V) == a.V;
+    if (!(a.temperature > 0.f))
+        return by_alignment<E <= 16>(aligned, [&](auto ragged) {
+            static OncePerDevice once;
+            return launch_cluster(greedy_lazy_walk_kernel<T, E, decltype(ragged)::value>, once, B, n, st, a, tl);
+        });
+    if (!stats)
+        return by_alignment<true>(aligned, [&](auto ragged) {
+            static OncePerDevice once;
+            return launch_cluster(ratio_walk_kernel<T, E, decltype(ragged)::value, true>, once, B, n, st, a, tl, dl, nch, B * a.T, stats);
+        });
+    return by_alignment<(sizeof(T) * E < 160)>(aligned, [&](auto ragged) {
+        static OncePerDevice once;
+        return launch_cluster(ratio_walk_kernel<T, E, decltype(ragged)::value, false>, once, B, n, st, a, tl, dl, nch, B * a.T, stats);
+    });
 }
-template <typename T, int E, bool kRagged>
+template <typename T, int E>
 static cudaError_t match_e(int n, int B, const Args& a, const T* tl, cudaStream_t st)
 {
-    static OncePerDevice once;
-    return launch_cluster(match_walk_kernel<T, E, kRagged>, once, B, n, st, a, tl);
+    return by_alignment<E >= 24>(places<T>(a.V) == a.V, [&](auto ragged) {
+        static OncePerDevice once;
+        return launch_cluster(match_walk_kernel<T, E, decltype(ragged)::value>, once, B, n, st, a, tl);
+    });
 }
 
 // CTAs per sequence and entries per thread.  A walk is as fast as its slices are small, so a small batch with a large
@@ -744,18 +770,13 @@ template <typename T>
 static cudaError_t walk_t(int B, const Args& a, const void* tl, const void* dl, int nch, const RowStat* stats, cudaStream_t st)
 {
     return by_vocabulary(B, places<T>(a.V), [&](auto e, int n) {
-        constexpr int E = decltype(e)::value;
-        return places<T>(a.V) == a.V ? walk_e<T, E, false>(n, B, a, (const T*)tl, (const T*)dl, nch, stats, st)
-                                     : walk_e<T, E, true>(n, B, a, (const T*)tl, (const T*)dl, nch, stats, st);
+        return walk_e<T, decltype(e)::value>(n, B, a, (const T*)tl, (const T*)dl, nch, stats, st);
     });
 }
 template <typename T>
 static cudaError_t match_t(int B, const Args& a, const void* tl, cudaStream_t st)
 {
-    return by_vocabulary(B, places<T>(a.V), [&](auto e, int n) {
-        constexpr int E = decltype(e)::value;
-        return places<T>(a.V) == a.V ? match_e<T, E, false>(n, B, a, (const T*)tl, st) : match_e<T, E, true>(n, B, a, (const T*)tl, st);
-    });
+    return by_vocabulary(B, places<T>(a.V), [&](auto e, int n) { return match_e<T, decltype(e)::value>(n, B, a, (const T*)tl, st); });
 }
 
 }  // namespace walk

@@ -52,9 +52,8 @@ struct Search {
 // ---------------------------------------------------------------------------------------------
 // A row is counted from the 16-byte boundary at or before its first entry, `shift` places earlier, so that vectors can be loaded
 // whatever the vocabulary size is (rows that start anywhere, entry by entry: B 3, V 77777, ratio rule with statistics 49 us, now 31).
-// kRagged: a row's bytes are no multiple of 16, so shifts differ from row to row.  Kernels of their own: where all rows are aligned the code for
-// ends of rows, never run, cost registers (spill loads of the ratio rule at V 128256 156 -> 196 bytes, now 132; B 8 on demand 40.8 us
-// without it, 41.5 with it, 40.8 so; B 32 with statistics 217.5 -> 211.5).
+// kRagged: a row's bytes are no multiple of 16, so shifts differ from row to row.  Without it the code for ends of rows, which aligned rows
+// never run, is left out: it costs registers (ratio rule, bf16, 32 entries a thread: spill loads 196 bytes with it, 132 without).
 // CTA `rank` of n owns places [rank * chunk, (rank + 1) * chunk), chunk a multiple of 8; run s of thread t starts at place
 // rank * chunk + s * kStrip + 8 t.
 struct Span {

@@ -226,27 +226,33 @@ __global__ void __launch_bounds__(32 * kStatWarps, kStatBlocks) row_stats_kernel
 }
 
 // The statistics of all rows.  Chunks per row and warps per chunk: so that the rounds that a warp makes come out even, by what a round
-// takes it: its share of the entries, and what the end of an item stands for (some 0.3 us, of which a warp reads one entry per
-// nanosecond).  A block of 8 warps per row or chunk of a row, maximum's index and sum both, parts merged as a tree with two exponentials a
-// step -> so, us with the walk behind it, T 60: sampling, bf16, V 128256, B 1 28.7 -> 26.6, 3 43.5 -> 40.6, 8 81 -> 77, 16 123 -> 119, 32
-// 213 -> 215; V 32000, B 2 24.6 -> 22.7, 8 36.9 -> 32.2, 32 87 -> 84; fp32, V 128256, B 8 127 -> 118; greedy, bf16, V 128256, B 16 53.3 -> 45.
+// takes it: its share of the entries, the end of an item (some 256 entries' time), and a last batch that is not whole: its vectors
+// come a few at a time, each after the one before, half a batch's time, or a whole one's where other items wait.  So chunks of
+// whole batches are on offer too; several warps to a chunk keep less in flight (5/4).  With the walk behind it, us, chunks of any length ->
+// so: bf16, T 64, V 128256, B 31 240 -> 217, T 45, V 90000, B 40 177 -> 162, T 60, V 128256, B 3 39.4 -> 35.7, 8 73.0 -> 67.9, 16 117 -> 113;
+// V 32000, B 32 81.3 -> 78.7; greedy, T 64, V 12000, B 32 13.6 -> 10.2; fp32, greedy, T 64, V 151936, B 5 44.3 -> 35.7.  Against a block
+// of 8 warps per row or chunk, maximum's index and sum both, parts merged as a tree: 217, 164, 40.2, 78.0, 123, 84.3, 16.9, 42.3.
 // Blocks per SM (registers against warps) 3, 4, 5, 6, 8 at B 16: 132, 132, 119, 126, 134; the next four vectors loaded ahead: 120 -> 132.
 template <typename T, bool kGreedy>
 static cudaError_t launch_stats(int sm_count, int n_rows, int nmat, int V, const T* tl, const T* dl, float k2, RowStat* stats, int& nch, cudaStream_t st)
 {
     const int all = ((size_t)V * sizeof(T)) % 16 == 0 ? V : V + 16 / (int)sizeof(T) - 1;      // places of a row, whatever its shift
     const int64_t rows = (int64_t)n_rows * nmat, room = (int64_t)sm_count * kStatBlocks * kStatWarps;
-    int W = 1;
+    constexpr int kBatch = 32 * kEpt * (sizeof(T) == 2 ? 4 : 2);                             // entries that a warp loads at a time
+    int W = 1, chunk_elems = 0;
     int64_t least = INT64_MAX;
-    for (int c = 1; c <= kStatChunksMax; ++c)
-        for (int w = 1; w <= kStatWarps; w *= 2) {
-            const int64_t groups = room / w, rounds = (rows * c + groups - 1) / groups;
-            const int64_t cost = rounds * ((all + c - 1) / c / w + (w > 1 ? 384 : 256));
-            if (cost < least && (c == 1 || rows * c < (1 << 30))) { least = cost; nch = c; W = w; }
-        }
-    int chunk_elems = (all + nch - 1) / nch;
-    chunk_elems = (chunk_elems + 15) / 16 * 16;
-    nch = (all + chunk_elems - 1) / chunk_elems;
+    auto offer = [&](int share, int w, bool whole) {
+        const int unit = whole ? kBatch : 16, n = (share + unit - 1) / unit * unit;
+        const int64_t parts = (all + n - 1) / n, groups = room / w, rounds = (rows * parts + groups - 1) / groups;
+        const int tail = (rounds > 1 ? 2 : n < kBatch ? 0 : 1) * kBatch / 2;
+        const int64_t cost = rounds * (w > 1 ? n / w * 5 / 4 + 512 : whole ? n + 512 : n + 256 + tail);
+        if (cost < least && (parts == 1 || rows * parts < (1 << 30))) { least = cost; nch = (int)parts; W = w; chunk_elems = n; }
+    };
+    for (int c = 1; c <= kStatChunksMax; ++c) {
+        const int share = (all + c - 1) / c;
+        for (int w = 1; w <= kStatWarps; w *= 2) offer(share, w, false);
+        offer(share, 1, true);
+    }
     const int64_t items = rows * nch, per = kStatWarps / W, want = (items + per - 1) / per, most = (int64_t)sm_count * kStatBlocks;
     const int64_t blocks = want < most ? want : most;
     auto kernel = W == 1 ? row_stats_kernel<T, 1, kGreedy> : W == 2 ? row_stats_kernel<T, 2, kGreedy> : W == 4 ? row_stats_kernel<T, 4, kGreedy> : row_stats_kernel<T, 8, kGreedy>;

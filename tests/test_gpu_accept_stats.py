@@ -66,12 +66,13 @@ def _row_sums(gpu, tl, dl, temperature):
     return top[:, 0], (s * torch.exp((m - top) / temperature)).sum(1)
 
 
-# A warp to a row, to a chunk of a row (two rounds of them in the last case), two and eight warps to a chunk (148 SMs).  Half of the rows:
-# one logit far above all others, read among the first, so that its lane's sum takes in hundreds of weights that are next to
+# A warp to a row, to chunks of whole and of broken batches, in one round and in two, two and eight warps to a chunk (148 SMs).  Half of the
+# rows: one logit far above all others, read among the first, so that its lane's sum takes in hundreds of weights that are next to
 # nothing beside it (eight of an fp32 row, 32 of a bf16 row at a time: a little less than half a unit in its last place).  The other
 # half: deviation 5.
 @pytest.mark.parametrize("dtype,low", [(torch.bfloat16, -20.125), (torch.float32, -18.75)])
-@pytest.mark.parametrize("B,T,V", [(49, 60, 48003), (3, 60, 128256), (2, 47, 5000), (1, 5, 151937), (37, 32, 4099)])
+@pytest.mark.parametrize("B,T,V", [(49, 60, 48003), (3, 60, 128256), (2, 47, 5000), (1, 5, 151937), (37, 32, 4099), (32, 3, 12878),
+                                   (55, 8, 171133)])
 def test_error_of_sums(gpu, B, T, V, dtype, low):
     g = torch.Generator(device="cuda")
     g.manual_seed(B + V)

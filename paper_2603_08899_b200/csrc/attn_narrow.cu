@@ -403,7 +403,7 @@ attention_narrow_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_
     tc_fence_after();
     const uint32_t tmem = sh.tmem_base;
     const PlanView pv = plan_view(const_cast<void*>(prm.plan), prm.d.B, prm.d.Hkv);
-    if (prm.prefetch && warp == 11) prefetch_first<D, 64>(prm, pv, &q_map, &k_map);
+    prefetch_first<D, 64>(prm, pv, &q_map, &k_map);
     // global memory is read and written from here on: the kernels before this one have completed
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (warp < 8) softmax_role<D, kSplit>(sh, prm, pv, tmem);

@@ -467,7 +467,7 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
     tc_fence_after();
     const uint32_t tmem = sh.tmem_base;
     const PlanView pv = plan_view(const_cast<void*>(prm.plan), prm.d.B, prm.d.Hkv);
-    if (prm.prefetch && warp == 11) prefetch_first<D, 64>(prm, pv, &q_map, &k_map);
+    prefetch_first<D, 64>(prm, pv, &q_map, &k_map);
     // Everything above touches only this kernel's own shared and tensor memory (but for that hint), so it runs while
     // the kernel before this one in the stream drains.  From here on global memory is read and written:
     // every CTA waits until the kernels before this one have completed.

@@ -89,6 +89,7 @@ __device__ __forceinline__ void prefetch_lane(const Params& p, const PlanView& v
 #pragma unroll
     for (int x = 0; x < D; x += kXStep) tma_prefetch_3d(k_map, x, g, z);
     const int R = p.d.T + p.d.C, rows = p.d.B * R;
+#pragma unroll 1
     for (int mt = 0; mt < p.n_mt; ++mt) {
         const int at = b * R + p.rpt * (p.tpg * rg + mt);
         if ((int64_t)(rows - at) * p.G < kQRowsFetched) continue;
@@ -96,11 +97,13 @@ __device__ __forceinline__ void prefetch_lane(const Params& p, const PlanView& v
         for (int x = 0; x < D; x += 64) tma_prefetch_3d(q_map, x, g * p.G, at);
     }
 }
-// The same by a whole warp, which is together again behind it: setmaxnreg comes next.
+// By one lane of warp 11, if the plan was there before this call; every warp is together again behind it: setmaxnreg comes next.  (With the
+// warp, not the thread, as the outer condition: 4 sequences of 500..4000, 64 / 8 heads, plan made beforehand, 29.7 -> 30.6 us, the same
+// spills.)
 template <int D, int kXStep>
 __device__ __forceinline__ void prefetch_first(const Params& p, const PlanView& v, const CUtensorMap* q_map, const CUtensorMap* k_map)
 {
-    if ((threadIdx.x & 31) == 0) prefetch_lane<D, kXStep>(p, v, q_map, k_map);
+    if (p.prefetch && threadIdx.x == 11 * 32) prefetch_lane<D, kXStep>(p, v, q_map, k_map);
     __syncwarp();
 }
 
